@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "xk_bcr.cuh"
 
@@ -31,7 +32,6 @@ namespace xk {
 
 namespace {
 
-constexpr int kLeafWarpsUsed = 16;   // warps of the leaf inversion: 16 x 50 elements per thread
 constexpr int kMvThreads = 256;
 constexpr int kMvRows = 64;
 constexpr int kArrD = 0, kArrINV = 1, kArrTMP = 2, kArrCP = 3, kArrPQ = 4, kArrays = 5;
@@ -45,199 +45,275 @@ __device__ __forceinline__ bool stop(const int *skip, const Ctl *ctl)
 int split_of(int n) { return 32 * ((n + 63) / 64); }
 
 // ---------------------------------------------------------------------------
-// Gauss-Jordan inversion with partial pivoting of one block per CTA, the block
-// held in registers: warp v owns columns v + 16 b (b < 10) and lane l owns rows
-// l + 32 a (a < 5), so column c belongs to one whole warp and, with the column
-// loop unrolled over b, to a fixed register.  Pivoting is implicit: rows never
-// move; the pivot of column c is the unused row p(c) of largest |value|, and
-// the in-place elimination leaves row p(k) holding row k of (P M)^-1, so
-// M^-1[k][p(c)] = W[p(k)][c].
+// Gauss-Jordan inversion with partial pivoting of one N x N block per CTA
+// (N = 32 RG <= 160), in panels of 8 columns with look-ahead.  Pivoting is
+// implicit: rows never move; the pivot of column c is the unused row p(c) of
+// largest |value|, and the in-place elimination leaves row p(k) holding row k
+// of (P M)^-1, so M^-1[k][p(c)] = W[p(k)][c].
 //
-// One barrier per column.  After it every warp reads the pivot row index, the
-// pivot and the column's multipliers from shared memory and takes the pivot
-// row's entries in its own columns from the lane that holds them (a warp
-// shuffle).  The warp owning the next column updates that column first, picks
-// its pivot (redux.sync maximum of |value| over the unused rows, the lowest
-// row on ties) and publishes it before updating its other columns
-// (look-ahead); shared buffers alternate between columns.
+// Warp 0 factors the panels: lane l holds rows l + 32 a of the panel's 8
+// columns in registers, a column costs one warp reduction (the pivot), one
+// shared-memory broadcast (the pivot row) and 8 RG FMAs, and no block barrier.
+// Its result G (N x 8) turns the other columns by one rank-8 update,
+//   W[r][j] <- W[r][j] + sum_l G[r][l] U[l][j],   U the panel's pivot rows,
+// (the pivot rows themselves without their old value), which the other 15
+// warps apply one panel behind: warp w owns whole columns, NC of them, so the
+// pivot rows it needs are its own, and the only block barrier is one per
+// panel.  Warp 0 applies the previous panel's update to its next panel itself.
+//
+// What bounds it: the 8 N-long chains of dependent columns on warp 0 and the
+// 2 N^3 flop of one SM's FP32 pipe are about equal at N = 160 (a panel is 2,000
+// to 2,500 clocks on either side), which is why the panel is 8 wide: 16 makes
+// the chain longer than the updates, 4 doubles the updates' loads.
 // ---------------------------------------------------------------------------
-constexpr int kLeafRowGroups = (kBcrLeafMax + 31) / 32;                         // 5
-
-// Row groups: element a of a lane's rows selected by a runtime index.
-__device__ __forceinline__ float leaf_pick(const float (&col)[kLeafRowGroups], int a)
+constexpr int kLeafPanel = 8;
+constexpr int kLeafTrail = 15;                                // warps of the trailing update
+constexpr int kLeafThreads = 32 * (kLeafTrail + 1);
+constexpr int leaf_cols(int N) { return (N + kLeafTrail - 1) / kLeafTrail; }
+constexpr int leaf_ucols(int N) { return (leaf_cols(N) + 3) / 4 * 4; }
+// the block (odd row stride), G and the raw panels (two buffers each), U per warp, the pivot rows
+// of warp 0's panel, two pivot-row broadcasts
+constexpr size_t leaf_smem(int N)
 {
-    float v = col[0];
-#pragma unroll
-    for (int q = 1; q < kLeafRowGroups; ++q)
-        if (a == q) v = col[q];
-    return v;
+    return sizeof(float) * ((size_t)N * (N + 1) + 4 * kLeafPanel * N + (size_t)kLeafTrail * kLeafPanel * leaf_ucols(N) +
+                            kLeafPanel * kLeafPanel + 2 * kLeafPanel);
 }
 
-struct LeafPivot {
-    int p;
-    float v;
-};
-
-// Pivot of one column (its values in this lane's rows: col[a]) over the unused rows of the warp.
-__device__ __forceinline__ LeafPivot leaf_argmax(const float (&col)[kLeafRowGroups], unsigned used, int ln, int n)
+// Calls f(A) with the constant A equal to pa (< RG), so that arrays indexed by A stay in registers.
+template <int RG, typename F>
+__device__ __forceinline__ void leaf_with_group(int pa, F f)
 {
-    unsigned key = 0u;
-    int br = 0x7fffffff;
-#pragma unroll
-    for (int a = 0; a < kLeafRowGroups; ++a) {
-        const float v = fabsf(col[a]);
-        const unsigned k = (((used >> a) & 1u) || !(v == v)) ? 0u : __float_as_uint(v) + 1u;
-        if (k > key) { key = k; br = ln + 32 * a; }
+    switch (pa) {
+    case 0: f(std::integral_constant<int, 0>()); break;
+    case 1: if constexpr (RG > 1) f(std::integral_constant<int, 1>()); break;
+    case 2: if constexpr (RG > 2) f(std::integral_constant<int, 2>()); break;
+    case 3: if constexpr (RG > 3) f(std::integral_constant<int, 3>()); break;
+    default: if constexpr (RG > 4) f(std::integral_constant<int, 4>()); break;
     }
-    const unsigned m = __reduce_max_sync(0xffffffffu, key);
-    int p = (int)__reduce_min_sync(0xffffffffu, (key == m && m != 0u) ? (unsigned)br : 0x7fffffffu);
-    if (m == 0u || p >= n) p = 0;       // no candidate left: a singular block
-    const float val = __shfl_sync(0xffffffffu, leaf_pick(col, p >> 5), p & 31);
-    return LeafPivot{p, val};
 }
 
-template <int kLeafWarps>
-__global__ void __launch_bounds__(kLeafWarps * 32, 1) k_leaf_inverse(const BcrLeaf *tasks, const int *skip, const Ctl *ctl)
+// Store the 8 values of one row (row group pa of this lane) and clear it.
+template <int RG>
+__device__ __forceinline__ void leaf_take_row(float (&x)[RG][kLeafPanel], int pa, float *dst)
 {
-    constexpr int kLeafColGroups = (kBcrLeafMax + kLeafWarps - 1) / kLeafWarps;
+    leaf_with_group<RG>(pa, [&](auto A) {
+        constexpr int a = decltype(A)::value;
+        *(float4 *)dst = make_float4(x[a][0], x[a][1], x[a][2], x[a][3]);
+        *(float4 *)(dst + 4) = make_float4(x[a][4], x[a][5], x[a][6], x[a][7]);
+#pragma unroll
+        for (int j = 0; j < kLeafPanel; ++j) x[a][j] = 0.0f;
+    });
+}
+
+template <int RG>
+__global__ void __launch_bounds__(kLeafThreads, 1) k_leaf_inverse(const BcrLeaf *tasks, const int *skip, const Ctl *ctl)
+{
+    constexpr int N = 32 * RG, NP = kLeafPanel, NPAN = N / NP, NC = leaf_cols(N), UC = leaf_ucols(N), LD = N + 1;
     if (stop(skip, ctl)) return;
     const BcrLeaf t = tasks[blockIdx.x];
-    __shared__ float fcol[2][kBcrLeafMax];
-    __shared__ float pval[2];
-    __shared__ int piv[2];
-    __shared__ int perm[kBcrLeafMax], iperm[kBcrLeafMax];
-    const int n = t.n;
+    extern __shared__ __align__(16) float sm[];
+    float *tile = sm;                          // [N][LD]
+    float *G = tile + N * LD;                  // [2][NP][N]
+    float *raw = G + 2 * NP * N;               // [2][NP][N]: panel columns as the trailing warps left them
+    float *U = raw + 2 * NP * N;               // [kLeafTrail][NP][UC]
+    float *pu = U + kLeafTrail * NP * UC;      // [NP][NP]: the previous panel's pivot rows in this panel
+    float *rowb = pu + NP * NP;                // [2][NP]
+    __shared__ int piv[2][NP], perm[N];
     const int ln = threadIdx.x & 31, wv = threadIdx.x >> 5;
-    float w[kLeafColGroups][kLeafRowGroups];        // w[b][a] = W[ln + 32 a][wv + 16 b]
-    unsigned used = 0;
-#pragma unroll
-    for (int a = 0; a < kLeafRowGroups; ++a) {
-        const int r = ln + 32 * a;
-#pragma unroll
-        for (int b = 0; b < kLeafColGroups; ++b) {
-            const int j = wv + kLeafWarps * b;
-            w[b][a] = (r < n && j < n) ? t.in[(long long)r * t.ldin + j] : 0.0f;
-        }
-        if (r >= n) used |= 1u << a;
-    }
-    // column 0: its owner (warp 0) publishes the first pivot
-    if (wv == 0) {
-        const LeafPivot pv = leaf_argmax(w[0], used, ln, n);
-#pragma unroll
-        for (int a = 0; a < kLeafRowGroups; ++a) {
-            const int r = ln + 32 * a;
-            if (r < n) fcol[0][r] = w[0][a];
-        }
-        if (ln == 0) { piv[0] = pv.p; pval[0] = pv.v; perm[0] = pv.p; iperm[pv.p] = 0; }
+#pragma unroll 10
+    for (int e = threadIdx.x; e < N * N; e += kLeafThreads) {
+        const int r = e / N, j = e - r * N;
+        tile[r * LD + j] = t.in[(long long)r * t.ldin + j];
     }
     __syncthreads();
+    if (wv == 0) {
+        float g[RG][NP];                       // G of the previous panel, rows ln + 32 a
+        unsigned used = 0;
+        for (int p = 0; p <= NPAN; ++p) {
+            if (p < NPAN) {
+                float x[RG][NP];
+                if (p < 2) {
 #pragma unroll
-    for (int bc = 0; bc < kLeafColGroups; ++bc) {
-        for (int cw = 0; cw < kLeafWarps; ++cw) {
-            const int c = kLeafWarps * bc + cw;
-            if (c >= n) break;
-            const int buf = c & 1;
-            const int p = piv[buf];
-            const int pa = p >> 5, pl = p & 31;
-            float pivv = pval[buf];
-            if (pivv == 0.0f) pivv = 1e-30f;    // singular block: the FP64 Krylov solve sees a poor preconditioner
-            const float inv = 1.0f / pivv;
-            float f[kLeafRowGroups];
+                    for (int a = 0; a < RG; ++a)
 #pragma unroll
-            for (int a = 0; a < kLeafRowGroups; ++a) {
-                const int r = ln + 32 * a;
-                f[a] = (r < n) ? fcol[buf][r] : 0.0f;
-            }
-            if (ln == pl) used |= 1u << pa;          // row p is a pivot from now on
-            const bool own = (wv == cw);             // this warp owns column c
-            // the pivot row in this warp's columns (lane pl, row group pa: uniform over the warp), scaled;
-            // the column-c entry becomes 1 / pivot
-            float pr[kLeafColGroups];
-            switch (pa) {
-#define XK_LEAF_ROW(A)                                                                            \
-    case A:                                                                                       \
-        _Pragma("unroll") for (int b = 0; b < kLeafColGroups; ++b) pr[b] =                     \
-            __shfl_sync(0xffffffffu, w[b][A], pl);                                                \
-        break;
-                XK_LEAF_ROW(0) XK_LEAF_ROW(1) XK_LEAF_ROW(2) XK_LEAF_ROW(3) XK_LEAF_ROW(4)
-#undef XK_LEAF_ROW
-            }
+                        for (int j = 0; j < NP; ++j) x[a][j] = tile[(ln + 32 * a) * LD + p * NP + j];
+                } else {
+                    const float *src = raw + (p & 1) * NP * N + ln;
 #pragma unroll
-            for (int b = 0; b < kLeafColGroups; ++b) pr[b] *= inv;
-            if (own) pr[bc] = inv;
-            // update of one column b: every row w - f pr (column c: -f / pivot); the pivot row is
-            // then overwritten by its scaled values (fix_pivot)
-            auto update = [&](float (&col)[kLeafRowGroups], float prb, bool is_c) {
+                    for (int a = 0; a < RG; ++a)
 #pragma unroll
-                for (int a = 0; a < kLeafRowGroups; ++a) col[a] = is_c ? -f[a] * inv : fmaf(-f[a], prb, col[a]);
-            };
-            auto fix_pivot = [&](float (&col)[kLeafRowGroups], float prb) {
-                if (ln == pl) {
-                    switch (pa) {
-                    case 0: col[0] = prb; break;
-                    case 1: col[1] = prb; break;
-                    case 2: col[2] = prb; break;
-                    case 3: col[3] = prb; break;
-                    default: col[4] = prb; break;
+                        for (int j = 0; j < NP; ++j) x[a][j] = src[j * N + 32 * a];
+                }
+                if (p > 0) {
+                    const int *pp = piv[(p - 1) & 1];
+#pragma unroll
+                    for (int l = 0; l < NP; ++l) {
+                        const int row = pp[l];
+                        if (ln == (row & 31)) leaf_take_row<RG>(x, row >> 5, pu + l * NP);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int l = 0; l < NP; ++l) {
+                        const float4 u0 = *(const float4 *)(pu + l * NP), u1 = *(const float4 *)(pu + l * NP + 4);
+                        const float u[NP] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+#pragma unroll
+                        for (int j = 0; j < NP; ++j)
+#pragma unroll
+                            for (int a = 0; a < RG; ++a) x[a][j] = fmaf(g[a][l], u[j], x[a][j]);
                     }
                 }
-            };
-            // look-ahead: the owner of column c + 1 updates it, picks its pivot and publishes it first
-            const int cn = c + 1;
-            const int nw = cn % kLeafWarps;
-            const bool next_here = cn < n && wv == nw;
-            if (next_here) {
-                if (cw + 1 < kLeafWarps) {
-                    update(w[bc], pr[bc], false);
-                    fix_pivot(w[bc], pr[bc]);
-                    const LeafPivot pv = leaf_argmax(w[bc], used, ln, n);
 #pragma unroll
-                    for (int a = 0; a < kLeafRowGroups; ++a) {
-                        const int r = ln + 32 * a;
-                        if (r < n) fcol[buf ^ 1][r] = w[bc][a];
+                for (int c = 0; c < NP; ++c) {
+                    // pivot: the unused row of largest |value| (its float bits without the low eight, which
+                    // hold the row so that one reduction finds both; the lowest row among near-equals)
+                    unsigned key = 0u;
+#pragma unroll
+                    for (int a = 0; a < RG; ++a) {
+                        const unsigned m = __float_as_uint(x[a][c]) & 0x7fffffffu;
+                        const unsigned k = ((m > 0x7f800000u ? 0u : m) & 0xffffff00u) | (unsigned)(255 - (ln + 32 * a));
+                        if (!((used >> a) & 1u)) key = max(key, k);
                     }
-                    if (ln == 0) { piv[buf ^ 1] = pv.p; pval[buf ^ 1] = pv.v; perm[cn] = pv.p; iperm[pv.p] = cn; }
-                } else if (bc + 1 < kLeafColGroups) {
-                    update(w[bc + 1], pr[bc + 1], false);
-                    fix_pivot(w[bc + 1], pr[bc + 1]);
-                    const LeafPivot pv = leaf_argmax(w[bc + 1], used, ln, n);
-#pragma unroll
-                    for (int a = 0; a < kLeafRowGroups; ++a) {
-                        const int r = ln + 32 * a;
-                        if (r < n) fcol[buf ^ 1][r] = w[bc + 1][a];
+                    key = __reduce_max_sync(0xffffffffu, key);
+                    const int row = 255 - (int)(key & 0xffu);
+                    const bool mine = ln == (row & 31);
+                    float *rb = rowb + (c & 1) * NP;
+                    if (mine) {
+                        used |= 1u << (row >> 5);
+                        leaf_take_row<RG>(x, row >> 5, rb);
                     }
-                    if (ln == 0) { piv[buf ^ 1] = pv.p; pval[buf ^ 1] = pv.v; perm[cn] = pv.p; iperm[pv.p] = cn; }
-                }
-            }
+                    __syncwarp();
+                    const float4 r0 = *(const float4 *)rb, r1 = *(const float4 *)(rb + 4);
+                    float pr[NP] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+                    // singular block: the FP64 Krylov solve sees a poor preconditioner
+                    const float inv = 1.0f / (pr[c] == 0.0f ? 1e-30f : pr[c]);
 #pragma unroll
-            for (int b = 0; b < kLeafColGroups; ++b) {
-                const bool done_early = next_here && ((cw + 1 < kLeafWarps) ? (b == bc) : (b == bc + 1));
-                if (!done_early) update(w[b], pr[b], own && b == bc);
-            }
-            if (ln == pl) {
-                switch (pa) {
-#define XK_LEAF_FIX(A)                                                                           \
-    case A:                                                                                      \
-        _Pragma("unroll") for (int b = 0; b < kLeafColGroups; ++b) w[b][A] = pr[b];             \
-        break;
-                    XK_LEAF_FIX(0) XK_LEAF_FIX(1) XK_LEAF_FIX(2) XK_LEAF_FIX(3) XK_LEAF_FIX(4)
-#undef XK_LEAF_FIX
+                    for (int j = 0; j < NP; ++j) pr[j] = j == c ? inv : pr[j] * inv;
+                    // the pivot row is now zero: a multiplier of -1 leaves it as the scaled row, exactly
+#pragma unroll
+                    for (int a = 0; a < RG; ++a) {
+                        const float f = mine && a == (row >> 5) ? -1.0f : x[a][c];
+#pragma unroll
+                        for (int q = 1; q < NP; ++q) {
+                            const int j = (c + q) % NP;
+                            x[a][j] = fmaf(-f, pr[j], x[a][j]);
+                        }
+                        x[a][c] = -f * inv;
+                    }
+                    if (ln == 0) {
+                        piv[p & 1][c] = row;
+                        perm[p * NP + c] = row;
+                    }
                 }
+                float *dst = G + (p & 1) * NP * N + ln;
+#pragma unroll
+                for (int a = 0; a < RG; ++a)
+#pragma unroll
+                    for (int j = 0; j < NP; ++j) {
+                        dst[j * N + 32 * a] = x[a][j];
+                        g[a][j] = x[a][j];
+                    }
             }
             __syncthreads();
         }
-    }
-    // M^-1[k][p(c)] = W[p(k)][c]: row r = p(k) of W goes to row iperm[r] of the output
+    } else {
+        const int tw = wv - 1, j0 = tw * NC;
+        float w[NC][RG];                       // w[b][a] = W[ln + 32 a][j0 + b]
 #pragma unroll
-    for (int a = 0; a < kLeafRowGroups; ++a) {
-        const int r = ln + 32 * a;
-        if (r >= n) continue;
-        float *o = t.out + (long long)iperm[r] * t.ldout;
+        for (int b = 0; b < NC; ++b)
 #pragma unroll
-        for (int b = 0; b < kLeafColGroups; ++b) {
-            const int j = wv + kLeafWarps * b;
-            if (j < n) o[perm[j]] = w[b][a];
+            for (int a = 0; a < RG; ++a) w[b][a] = j0 + b < N ? tile[(ln + 32 * a) * LD + j0 + b] : 0.0f;
+        float *uw = U + tw * NP * UC;
+        for (int p = 0; p <= NPAN; ++p) {
+            if (p > 0) {
+                const float *gq = G + ((p - 1) & 1) * NP * N + ln;
+                const int *pp = piv[(p - 1) & 1];
+                // the pivot rows of panel p - 1 in this warp's columns; they start from zero in the update
+#pragma unroll
+                for (int l = 0; l < NP; ++l) {
+                    const int row = pp[l];
+                    if (ln == (row & 31)) {
+                        leaf_with_group<RG>(row >> 5, [&](auto A) {
+                            constexpr int a = decltype(A)::value;
+#pragma unroll
+                            for (int b = 0; b < NC; ++b) {
+                                uw[l * UC + b] = w[b][a];
+                                w[b][a] = 0.0f;
+                            }
+                        });
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int l = 0; l < NP; ++l) {
+                    float gl[RG], ul[UC];
+#pragma unroll
+                    for (int a = 0; a < RG; ++a) gl[a] = gq[l * N + 32 * a];
+#pragma unroll
+                    for (int b = 0; b < UC; b += 4) {
+                        const float4 v = *(const float4 *)(uw + l * UC + b);
+                        ul[b] = v.x; ul[b + 1] = v.y; ul[b + 2] = v.z; ul[b + 3] = v.w;
+                    }
+#pragma unroll
+                    for (int b = 0; b < NC; ++b)
+#pragma unroll
+                        for (int a = 0; a < RG; ++a) w[b][a] = fmaf(gl[a], ul[b], w[b][a]);
+                }
+                // panel p - 1's own columns are G; panel p + 1's go to warp 0
+#pragma unroll
+                for (int b = 0; b < NC; ++b) {
+                    const int j = j0 + b, pj = j / NP;
+                    if (j < N && pj == p - 1) {
+#pragma unroll
+                        for (int a = 0; a < RG; ++a) w[b][a] = gq[(j % NP) * N + 32 * a];
+                    } else if (j < N && pj == p + 1) {
+                        float *dst = raw + (pj & 1) * NP * N + (j % NP) * N + ln;
+#pragma unroll
+                        for (int a = 0; a < RG; ++a) dst[32 * a] = w[b][a];
+                    }
+                }
+                __syncwarp();
+            }
+            __syncthreads();
         }
+        // M^-1[k][p(c)] = W[p(k)][c]: columns permuted here, rows on the way out
+#pragma unroll
+        for (int b = 0; b < NC; ++b)
+            if (j0 + b < N) {
+                const int c = perm[j0 + b];
+#pragma unroll
+                for (int a = 0; a < RG; ++a) tile[(ln + 32 * a) * LD + c] = w[b][a];
+            }
+    }
+    __syncthreads();
+#pragma unroll 10
+    for (int e = threadIdx.x; e < N * N; e += kLeafThreads) {
+        const int k = e / N, j = e - k * N;
+        t.out[(long long)k * t.ldout + j] = tile[perm[k] * LD + j];
+    }
+}
+
+template <int RG>
+cudaError_t launch_leaf_rg(const BcrLeaf *tasks, int count, const int *skip, const Ctl *ctl, cudaStream_t st)
+{
+    constexpr size_t smem = leaf_smem(32 * RG);
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_leaf_inverse<RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr != cudaSuccess) return attr;
+    count_launches(1);
+    k_leaf_inverse<RG><<<count, kLeafThreads, smem, st>>>(tasks, skip, ctl);
+    return cudaGetLastError();
+}
+
+// One CTA per block; every block of a launch has the same n, a multiple of 32 up to kBcrLeafMax.
+cudaError_t launch_leaf(const BcrLeaf *tasks, int count, int n, const int *skip, const Ctl *ctl, cudaStream_t st)
+{
+    switch (n / 32) {
+    case 1: return launch_leaf_rg<1>(tasks, count, skip, ctl, st);
+    case 2: return launch_leaf_rg<2>(tasks, count, skip, ctl, st);
+    case 3: return launch_leaf_rg<3>(tasks, count, skip, ctl, st);
+    case 4: return launch_leaf_rg<4>(tasks, count, skip, ctl, st);
+    case 5: return launch_leaf_rg<5>(tasks, count, skip, ctl, st);
+    default: return cudaErrorInvalidValue;
     }
 }
 
@@ -527,7 +603,7 @@ struct Builder {
     {
         const int B = (int)zin.size();
         if (n <= kBcrLeafMax) {
-            BcrStage s{kBcrLeafStage, (int)p.leaf.size(), B, 0, level};
+            BcrStage s{kBcrLeafStage, (int)p.leaf.size(), B, n, level};
             for (int b = 0; b < B; ++b)
                 p.leaf.push_back(BcrLeaf{ptr(in.arr, zin[b], in.r0, in.c0), ptr(out.arr, zout[b], out.r0, out.c0),
                                          cols(in.arr), cols(out.arr), n});
@@ -833,12 +909,13 @@ cudaError_t bcr_factor(const BcrPlan &p, const int *skip, Ctl *ctl, cudaStream_t
 {
     for (const BcrStage &s : p.fac) {
         switch (s.kind) {
-        case kBcrLeafStage:
+        case kBcrLeafStage: {
             if (timer) timer->begin(s.kind);
-            count_launches(1);
-            k_leaf_inverse<kLeafWarpsUsed><<<s.count, kLeafWarpsUsed * 32, 0, st>>>(p.leaf_d + s.off, skip, ctl);
+            cudaError_t e = launch_leaf(p.leaf_d + s.off, s.count, s.tiles, skip, ctl, st);
             if (timer) timer->end(s.kind);
+            if (e != cudaSuccess) return e;
             break;
+        }
         case kBcrGemm: {
             if (timer) timer->begin(s.kind);
             cudaError_t e = launch_tc_gemm(p.gemm_d + s.off, s.count, s.tiles, p.maps_d, skip, ctl, st);

@@ -30,7 +30,7 @@ struct BcrMv {
 struct BcrStage {
     int kind;          // BcrKind
     int off, count;    // range in the task list of that kind
-    int tiles;         // GEMM: output tiles of the launch
+    int tiles;         // GEMM: output tiles of the launch; leaf inversions: the blocks' order n
     int level;         // the reduction level it belongs to
 };
 enum BcrKind { kBcrLeafStage = 0, kBcrGemm = 1, kBcrLevel0 = 2, kBcrMv = 3, kBcrFwd0 = 4, kBcrIn = 5, kBcrOut = 6 };
