@@ -41,6 +41,10 @@ struct xk_ctx {
     bool have_net = false, have_photo = false, have_atm = false;
     bool rates_valid = false;      // k_f, k_r of the loaded network and atmosphere are in the workspace
     // host index structures
+    std::vector<int> sgp, sent, spart, ssp, dgp, dent, dpart, dsp, jto, jtg, jgc, jge, jrt, jit;
+    std::vector<unsigned short> jterm;
+    int nsub = 0;
+    std::vector<uint4> rx;
     std::vector<int> yp, yent, jp, jcol, jtp, jrs, jdq, abs_sp;
     std::vector<int> pg_p, pg_v, pg_s, pg_code;   // reaction graph of the pathway analyser
     std::vector<int> eq_sp, eq_se, eq_ep, eq_ey, eq_eij;   // sparse element structure (equilibrium)
@@ -177,6 +181,42 @@ struct Bump {
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
+// Lists cut into sublists of nearly equal length, one lane each, 32 of similar length to a group (see
+// Col::sgp); returns the number of sublists.
+int build_sublists(const std::vector<std::vector<int>> &lists, std::vector<int> &gp, std::vector<int> &ent,
+                   std::vector<int> &part, std::vector<int> &sp)
+{
+    struct Sub {
+        int list, e0, n, part;
+    };
+    std::vector<Sub> subs;
+    size_t total = 0;
+    for (const auto &l : lists) total += l.size();
+    // at most about 8192 besides one per list
+    const size_t sub_max = kSubMax * std::max<size_t>(1, (total + kSubMax * 8192 - 1) / (kSubMax * 8192));
+    sp.assign(lists.size() + 1, 0);
+    for (size_t y = 0; y < lists.size(); ++y) {
+        const size_t n = lists[y].size(), m = (n + sub_max - 1) / sub_max;
+        for (size_t q = 0; q < m; ++q) {
+            const size_t a = n * q / m, b = n * (q + 1) / m;
+            subs.push_back(Sub{(int)y, (int)a, (int)(b - a), (int)subs.size()});
+        }
+        sp[y + 1] = (int)subs.size();
+    }
+    std::stable_sort(subs.begin(), subs.end(), [](const Sub &a, const Sub &b) { return a.n > b.n; });
+    gp.assign(1, 0);
+    ent.clear();
+    part.clear();
+    for (size_t g = 0; g < subs.size(); g += 32) {
+        for (int l = 0; l < 32; ++l) part.push_back(g + l < subs.size() ? subs[g + l].part : -1);
+        for (int q = 0; q < subs[g].n; ++q)
+            for (int l = 0; l < 32; ++l)
+                ent.push_back(g + l < subs.size() && q < subs[g + l].n ? lists[subs[g + l].list][subs[g + l].e0 + q] : -1);
+        gp.push_back((int)ent.size() / 32);
+    }
+    return (int)subs.size();
+}
+
 // Index structures built once per network (symbolic, no arithmetic of the method).
 void build_indices(xk_ctx *c)
 {
@@ -195,6 +235,33 @@ void build_indices(xk_ctx *c)
     for (int y = 0; y < S; ++y) {
         c->yent.insert(c->yent.end(), ys[y].begin(), ys[y].end());
         c->yp[y + 1] = (int)c->yent.size();
+    }
+    // species sums: each species' entries; diagonal entries: the terms of the species' own column
+    std::vector<std::vector<int>> lists(S);
+    for (int y = 0; y < S; ++y)
+        for (int e = c->yp[y]; e < c->yp[y + 1]; ++e)
+            lists[y].push_back((c->yent[e] >> 4) << 1 | ((c->yent[e] & 15) < 8 ? 1 : 0));
+    c->nsub = build_sublists(lists, c->sgp, c->sent, c->spart, c->ssp);
+    for (auto &l : lists) l.clear();
+    for (int r = 0; r < R; ++r)
+        for (int side = 0; side < 2; ++side)
+            for (int s = 0; s < 3; ++s) {
+                const int j = side == 0 ? c->reac[3 * r + s] : c->prod[3 * r + s];
+                if (j < 0) continue;
+                for (int q = 0; q < 3; ++q) {
+                    if (c->reac[3 * r + q] == j) lists[j].push_back((r * 6 + side * 3 + s) << 1 | 1);
+                    if (c->prod[3 * r + q] == j) lists[j].push_back((r * 6 + side * 3 + s) << 1);
+                }
+            }
+    c->nsub = std::max(c->nsub, build_sublists(lists, c->dgp, c->dent, c->dpart, c->dsp));
+    c->rx.assign(R, uint4{});
+    for (int r = 0; r < R; ++r) {
+        unsigned short v[8] = {};
+        for (int s = 0; s < 3; ++s) {
+            v[s] = (unsigned short)(c->reac[3 * r + s] >= 0 ? c->reac[3 * r + s] : S);
+            v[3 + s] = (unsigned short)(c->prod[3 * r + s] >= 0 ? c->prod[3 * r + s] : S);
+        }
+        memcpy(&c->rx[r], v, sizeof v);
     }
     // Jacobian rows: for r, side, slot s (column j), then each reactant (+) / product (-) row
     std::vector<std::vector<std::pair<int, int>>> rows(S);
@@ -237,6 +304,58 @@ void build_indices(xk_ctx *c)
         if (!ent.empty()) c->jtp.push_back((int)c->jrs.size());
         c->jp[i + 1] = (int)c->jcol.size();
     }
+    // the dense assembly's tiles: each occurrence of species i contributes its reaction's derivative in
+    // every slot to the column of that slot's species
+    c->jto.clear(); c->jtg.clear(); c->jgc.clear(); c->jge.clear(); c->jterm.clear(); c->jit.clear();
+    c->jrt.assign(S + 1, 0);
+    std::vector<std::pair<int, unsigned short>> terms;
+    std::vector<int> light, heavy;
+    for (int i = 0; i < S; ++i) {
+        const int nocc = c->yp[i + 1] - c->yp[i];
+        const int tile = nocc <= kJacOcc ? kJacOcc : kJacHeavyOcc;
+        (nocc <= kJacOcc ? light : heavy).push_back(i);
+        for (int e0 = c->yp[i]; e0 < c->yp[i + 1]; e0 += tile) {
+            const int e1 = std::min(e0 + tile, c->yp[i + 1]);
+            terms.clear();
+            for (int e = e0; e < e1; ++e) {
+                const int r = c->yent[e] >> 4, plus = (c->yent[e] & 15) < 8;
+                for (int s = 0; s < 6; ++s) {
+                    const int j = s < 3 ? c->reac[3 * r + s] : c->prod[3 * r + s - 3];
+                    if (j >= 0) terms.push_back({j, (unsigned short)((((e - e0) * 6 + s) << 1) | plus)});
+                }
+            }
+            std::stable_sort(terms.begin(), terms.end(),
+                             [](const auto &a, const auto &b) { return a.first < b.first; });
+            c->jto.push_back(e0);
+            c->jtg.push_back((int)c->jgc.size());
+            // the tile's columns, longest first: the lanes of a warp get columns of similar length
+            std::vector<std::pair<int, int>> cols;      // (terms, first)
+            for (int t = 0; t < (int)terms.size(); ++t) {
+                if (t == 0 || terms[t].first != terms[t - 1].first) cols.push_back({0, t});
+                ++cols.back().first;
+            }
+            std::stable_sort(cols.begin(), cols.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
+            for (const auto &g : cols) {
+                c->jgc.push_back(terms[g.second].first);
+                c->jge.push_back((int)c->jterm.size());
+                for (int t = 0; t < g.first; ++t) c->jterm.push_back(terms[g.second + t].second);
+            }
+        }
+        c->jrt[i + 1] = (int)c->jto.size();
+    }
+    c->jto.push_back((int)c->yent.size());
+    c->jtg.push_back((int)c->jgc.size());
+    c->jge.push_back((int)c->jterm.size());
+    // heavy rows first (the longest), then the light ones eight to an item, longest first
+    auto longer = [&](int a, int b) { return c->yp[a + 1] - c->yp[a] > c->yp[b + 1] - c->yp[b]; };
+    std::stable_sort(heavy.begin(), heavy.end(), longer);
+    std::stable_sort(light.begin(), light.end(), longer);
+    for (int i : heavy) {
+        c->jit.push_back(i);
+        for (int q = 1; q < kJacWarps; ++q) c->jit.push_back(-2);
+    }
+    for (size_t q = 0; q < light.size(); q += kJacWarps)
+        for (int w = 0; w < kJacWarps; ++w) c->jit.push_back(q + w < light.size() ? light[q + w] : -1);
     // absorbers with a non-zero cross section somewhere
     c->abs_sp.clear();
     c->sig_abs_c.clear();
@@ -357,10 +476,23 @@ size_t layout(xk_ctx *c, char *base)
     t.rtype = b.take<int>(R); t.reac = b.take<int>(3 * (size_t)R); t.prod = b.take<int>(3 * (size_t)R);
     t.form = b.take<int>(R); t.prow = b.take<int>(R);
     t.yp = b.take<int>(S + 1); t.yent = b.take<int>(std::max<size_t>(1, c->yent.size()));
+    t.sgp = b.take<int>(c->sgp.size()); t.ssp = b.take<int>(S + 1);
+    t.sent = b.take<int>(std::max<size_t>(1, c->sent.size())); t.spart = b.take<int>(std::max<size_t>(1, c->spart.size()));
+    t.nsg = (int)c->sgp.size() - 1;
+    t.dgp = b.take<int>(c->dgp.size()); t.dsp = b.take<int>(S + 1);
+    t.dent = b.take<int>(std::max<size_t>(1, c->dent.size())); t.dpart = b.take<int>(std::max<size_t>(1, c->dpart.size()));
+    t.ndg = (int)c->dgp.size() - 1;
+    t.nsub = c->nsub;
+    t.rx = b.take<uint4>(std::max(R, 1));
     t.jp = b.take<int>(S + 1); t.jcol = b.take<int>(std::max<size_t>(1, c->jcol.size()));
     t.jtp = b.take<int>(std::max<size_t>(1, c->jtp.size()));
     t.jrs = b.take<int>(std::max<size_t>(1, c->jrs.size()));
     t.jdq = b.take<int>(S);
+    t.jto = b.take<int>(c->jto.size()); t.jtg = b.take<int>(c->jtg.size());
+    t.jgc = b.take<int>(std::max<size_t>(1, c->jgc.size())); t.jge = b.take<int>(c->jge.size());
+    t.jterm = b.take<unsigned short>(std::max<size_t>(1, c->jterm.size()));
+    t.jrt = b.take<int>(S + 1); t.jit = b.take<int>(c->jit.size());
+    t.nji = (int)c->jit.size() / kJacWarps;
     t.J0 = b.take<double>(std::max(W, 1)); t.dlam = b.take<double>(std::max(W, 1));
     t.sigma = b.take<double>(std::max<size_t>(1, (size_t)Rph * W));
     t.sig_abs = b.take<double>(std::max<size_t>(1, (size_t)Sabs * W));
@@ -408,7 +540,7 @@ size_t layout(xk_ctx *c, char *base)
     c->h1 = b.take<double>(kMaxBasis + 1);
     c->h2 = b.take<double>(kMaxBasis + 1);
     c->red = b.take<double>(8);
-    c->partials = b.take<double>((size_t)kGmPartialBlocks * (kMaxBasis + 1));
+    c->partials = b.take<double>((size_t)std::max(kGmPartialBlocks, 2 * L) * (kMaxBasis + 1));
     c->counter = b.take<unsigned>(8);
     c->gm = b.take<GmState>(1);
     if (c->cfg.precision == XK_PREC_FP64) {
@@ -457,7 +589,7 @@ size_t layout(xk_ctx *c, char *base)
     c->dinv = b.take<double>(32 * 32);
     c->ymid = b.take<double>(2 * (size_t)S);
     c->bar = b.take<unsigned>(8);
-    c->bcr.bar = c->bar ? c->bar + 4 : nullptr;      // words 4-5: the reduction's solve
+    c->bcr.bar = c->bar ? c->bar + 4 : nullptr;      // words 4-5: the reduction's solve and FGMRES
     c->ctl = b.take<Ctl>(1);
     c->ctl_aux = b.take<Ctl>(1);
     // Lagrangian parcel scheme
@@ -649,19 +781,19 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
         c->rates_valid = true;
     }
     { PhaseMark m(c, XK_PH_PHOTO); launch_photolysis(col, n, st); }
-    { PhaseMark m(c, XK_PH_REACTION); launch_reaction_terms(col, n, st); }
-    { PhaseMark m(c, XK_PH_RESIDUAL); launch_residual(col, n, col.F, ctl, c->cfg.f_floor, st); }
     cudaError_t e;
     const long long N = (long long)c->L * c->S;
     const int refine = std::max(c->cfg.refine_max_iter, 0);
+    {
+        // equations divided by their diagonal: residuals in units of relative change per species
+        PhaseMark m(c, XK_PH_RESIDUAL);
+        const bool equilibrate = c->cfg.precision != XK_PREC_FP64 || refine > 0;
+        launch_layer_terms(col, n, col.F, ctl, c->cfg.f_floor, equilibrate ? c->rowd : nullptr, c->bhat, st);
+    }
     if (c->cfg.precision == XK_PREC_FP64) {
         {
             PhaseMark m(c, XK_PH_JACOBIAN);
-            launch_jacobian64(col, n, ctl, dt_override, 1, c->A64, c->lo64, c->up64, st);
-            if (refine > 0) {
-                launch_diag(col, ctl, c->rowd, st);
-                launch_rowdiv(N, col.b, c->rowd, c->bhat, st);
-            }
+            launch_jacobian64(col, ctl, dt_override, 1, c->A64, c->lo64, c->up64, st);
         }
         { PhaseMark m(c, XK_PH_FACTOR); e = launch_factor<double>(sys64(c), c->plan, ctl, st); }
         if (e != cudaSuccess) return fail(c, XK_ECUDA, "factor launch: %s", cudaGetErrorString(e));
@@ -677,11 +809,8 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
         const int *skip32 = &ctl->skip32;
         {
             PhaseMark m(c, XK_PH_JACOBIAN);
-            launch_jacobian32(col, n, ctl, c->A32, c->lo32, c->up32, nullptr, st, skip32,
+            launch_jacobian32(col, ctl, c->A32, c->lo32, c->up32, st, skip32,
                               c->use_bcr ? (long long)c->bcr.Sp * c->bcr.Sp : 0);
-            // equations divided by their diagonal: residuals in units of relative change per species
-            launch_diag(col, ctl, c->rowd, st);
-            launch_rowdiv(N, col.b, c->rowd, c->bhat, st);
         }
         {
             PhaseMark m(c, XK_PH_FACTOR);
@@ -707,7 +836,14 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
         a.precond = [c, ctl, rowd](const double *v, double *z, const int *skip, cudaStream_t s) {
             solve32(c, v, z, ctl, s, rowd, skip);
         };
-        { PhaseMark m(c, XK_PH_SOLVE); enqueue_fgmres(a, st); }
+        if (c->use_bcr && !col.photo_jac) {
+            PhaseMark m(c, XK_PH_SOLVE);
+            e = bcr_fgmres(c->bcr, col, a, rowd, st);
+            if (e != cudaSuccess) return fail(c, XK_ECUDA, "solve launch: %s", cudaGetErrorString(e));
+        } else {
+            PhaseMark m(c, XK_PH_SOLVE);
+            enqueue_fgmres(a, st);
+        }
         // FGMRES around the last FP64 factorization, rescaled to this step's variables
         if (c->cfg.reuse_factorization) {
             launch_reuse_scales(N, rowd, col.s, c->s64, c->pin, c->pout, ctl, st);
@@ -723,7 +859,7 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
         const int *skip64 = &ctl->skip64;
         {
             PhaseMark m(c, XK_PH_FALLBACK);
-            launch_jacobian64(col, n, ctl, 0.0, 1, c->A64, c->lo64, c->up64, st, skip64);
+            launch_jacobian64(col, ctl, 0.0, 1, c->A64, c->lo64, c->up64, st, skip64);
             e = launch_factor<double>(sys64(c), c->plan64, ctl, st, skip64);
             if (e == cudaSuccess) {
                 launch_after_refactor(N, col.s, c->s64, ctl, st);
@@ -1141,7 +1277,12 @@ int xk_set_workspace(xk_ctx *c, void *dptr, size_t bytes)
     up(c, k.mass, c->mass); up(c, k.nasa, c->nasa); up(c, k.dcoef, c->dcoef);
     up(c, k.arr, c->arr); up(c, k.troe, c->troe); up(c, k.rtype, c->rtype); up(c, k.reac, c->reac);
     up(c, k.prod, c->prod); up(c, k.form, c->form); up(c, k.prow, c->prow);
-    up(c, k.yp, c->yp); up(c, k.yent, c->yent); up(c, k.jp, c->jp); up(c, k.jcol, c->jcol); up(c, k.jtp, c->jtp); up(c, k.jrs, c->jrs);
+    up(c, k.yp, c->yp); up(c, k.yent, c->yent);
+    up(c, k.jto, c->jto); up(c, k.jtg, c->jtg); up(c, k.jgc, c->jgc); up(c, k.jge, c->jge); up(c, k.jterm, c->jterm);
+    up(c, k.jrt, c->jrt); up(c, k.jit, c->jit);
+    up(c, k.sgp, c->sgp); up(c, k.sent, c->sent); up(c, k.spart, c->spart); up(c, k.ssp, c->ssp);
+    up(c, k.dgp, c->dgp); up(c, k.dent, c->dent); up(c, k.dpart, c->dpart); up(c, k.dsp, c->dsp); up(c, k.rx, c->rx);
+    up(c, k.jp, c->jp); up(c, k.jcol, c->jcol); up(c, k.jtp, c->jtp); up(c, k.jrs, c->jrs);
     up(c, k.jdq, c->jdq);
     up(c, k.J0, c->J0); up(c, k.dlam, c->dlam); up(c, k.sigma, c->sigma); up(c, k.sig_abs, c->sig_abs_c);
     up(c, k.abs_sp, c->abs_sp);
@@ -1360,8 +1501,7 @@ int xk_eval_residual(xk_ctx *c, const double *n, double *F)
     if (!n || !F) return fail(c, XK_EINVAL, "null pointer");
     launch_rates(c->col, c->st);
     launch_photolysis(c->col, n, c->st);
-    launch_reaction_terms(c->col, n, c->st);
-    launch_residual(c->col, n, F, nullptr, c->cfg.f_floor, c->st);
+    launch_layer_terms(c->col, n, F, nullptr, c->cfg.f_floor, nullptr, nullptr, c->st);
     return finish_eval(c, "eval_residual");
 }
 
@@ -1374,9 +1514,8 @@ int xk_eval_jacobian(xk_ctx *c, const double *n, double dt, double *A, double *l
     col.ld = c->S;
     launch_rates(col, c->st);
     launch_photolysis(col, n, c->st);
-    launch_reaction_terms(col, n, c->st);
-    launch_residual(col, n, col.F, nullptr, c->cfg.f_floor, c->st);
-    launch_jacobian64(col, n, nullptr, dt, 0, A, lo, up, c->st);
+    launch_layer_terms(col, n, col.F, nullptr, c->cfg.f_floor, nullptr, nullptr, c->st);
+    launch_jacobian64(col, nullptr, dt, 0, A, lo, up, c->st);
     return finish_eval(c, "eval_jacobian");
 }
 
@@ -1423,7 +1562,12 @@ int xk_block_solve32(xk_ctx *c, const double *A, const double *lo, const double 
     cudaMemcpyAsync(c->ctl_aux, c->ctl_host, sizeof(Ctl), cudaMemcpyHostToDevice, c->st);
     cudaError_t e = factor32(c, c->ctl_aux, nullptr);
     if (e != cudaSuccess) return fail(c, XK_ECUDA, "factor launch: %s", cudaGetErrorString(e));
-    e = solve32(c, f, x, c->ctl_aux, c->st, nullptr, nullptr);
+    const double *rhs = f;
+    if (f < x + L * S && x < f + L * S) {        // the solve reads f to its end while it writes x
+        d2d(c, c->bhat, f, L * S * 8);
+        rhs = c->bhat;
+    }
+    e = solve32(c, rhs, x, c->ctl_aux, c->st, nullptr, nullptr);
     if (e != cudaSuccess) return fail(c, XK_ECUDA, "solve launch: %s", cudaGetErrorString(e));
     cudaMemcpyAsync(c->ctl_host, c->ctl_aux, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st);
     if ((rc = finish_eval(c, "block_solve32"))) return rc;

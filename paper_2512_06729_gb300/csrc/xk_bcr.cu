@@ -32,8 +32,6 @@ namespace xk {
 
 namespace {
 
-constexpr int kMvThreads = 256;
-constexpr int kMvRows = 64;
 constexpr int kArrD = 0, kArrINV = 1, kArrTMP = 2, kArrCP = 3, kArrPQ = 4, kArrays = 5;
 
 __device__ __forceinline__ bool stop(const int *skip, const Ctl *ctl)
@@ -347,168 +345,6 @@ __global__ void k_bcr_level0(float *D, const float *INV, float *CP, const float 
     D[(long long)i * blk + e] -= upd;
 }
 
-// Batched y = base + sign M v (one block per blockIdx.y, kMvRows rows per blockIdx.x).
-__global__ void __launch_bounds__(kMvThreads) k_bcr_mv(const BcrMv *tasks, int S, int Sp, const int *skip, const Ctl *ctl)
-{
-    if (stop(skip, ctl)) return;
-    const BcrMv t = tasks[blockIdx.y];
-    extern __shared__ float v[];
-    for (int k = threadIdx.x; k < t.K; k += blockDim.x) {
-        float val;
-        if (k < Sp) {
-            val = t.v0[k];
-            if (k < S) {
-                if (t.d0) val -= t.d0[k] * t.w0[k];
-                if (t.d1) val -= t.d1[k] * t.w1[k];
-            }
-        } else {
-            val = t.v1[k - Sp];
-        }
-        v[k] = val;
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r1 = min(Sp, (int)(blockIdx.x + 1) * kMvRows);
-    for (int r = blockIdx.x * kMvRows + warp; r < r1; r += kMvThreads / 32) {
-        const float4 *row = (const float4 *)(t.M + (long long)r * t.ld);
-        float acc = 0.0f;
-        for (int q = lane; q < t.K / 4; q += 32) {
-            const float4 m = row[q];
-            acc += m.x * v[4 * q] + m.y * v[4 * q + 1] + m.z * v[4 * q + 2] + m.w * v[4 * q + 3];
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) t.y[r] = (t.base ? t.base[r] : 0.0f) + t.sign * acc;
-    }
-}
-
-__global__ void k_bcr_in(const double *b, const double *bscale, float *bw, int L, int S, int Sp, const int *skip,
-                         const Ctl *ctl)
-{
-    if (stop(skip, ctl)) return;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)L * Sp) return;
-    const int k = (int)(e / Sp), y = (int)(e - (long long)k * Sp);
-    float val = 0.0f;
-    if (y < S) {
-        const long long q = (long long)k * S + y;
-        val = (float)(bscale ? b[q] * bscale[q] : b[q]);
-    }
-    bw[e] = val;
-}
-
-__global__ void k_bcr_out(const float *xw, const double *xscale, double *x, int L, int S, int Sp, const int *skip,
-                          const Ctl *ctl)
-{
-    if (stop(skip, ctl)) return;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)L * S) return;
-    const int k = (int)(e / S), y = (int)(e - (long long)k * S);
-    const double val = (double)xw[(long long)k * Sp + y];
-    x[e] = xscale ? val * xscale[e] : val;
-}
-
-// Level-0 right-hand-side update of the kept even layers: b_i -= lo_i t_{i-1} + up_i t_{i+1}.
-__global__ void k_bcr_fwd0(float *bw, const float *tw, const float *lo, const float *up, int L, int S, int Sp,
-                           const int *skip, const Ctl *ctl)
-{
-    if (stop(skip, ctl)) return;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int nk = (L + 1) / 2;
-    if (e >= (long long)nk * S) return;
-    const int i = 2 * (int)(e / S), y = (int)(e % S);
-    float acc = 0.0f;
-    if (i >= 1) acc += lo[(long long)i * S + y] * tw[(long long)(i - 1) * Sp + y];
-    if (i + 1 < L) acc += up[(long long)i * S + y] * tw[(long long)(i + 1) * Sp + y];
-    bw[(long long)i * Sp + y] -= acc;
-}
-
-// The whole solve in one cooperative launch: the stages of the plan in order, each spread over
-// the grid, separated by bounded grid barriers.  A skipped solve costs one early-exiting launch.
-struct SolveArgs {
-    const BcrStage *stages;
-    const BcrMv *mv;
-    const double *b, *bscale, *xscale;
-    double *x;
-    float *bw, *tw, *xw;
-    const float *lo, *up;
-    unsigned *bar;
-    int nstages, L, S, Sp;
-};
-
-__global__ void __launch_bounds__(kMvThreads) k_bcr_solve_all(SolveArgs a, const int *skip, Ctl *ctl)
-{
-    if (stop(skip, ctl)) return;
-    extern __shared__ float v[];
-    const int S = a.S, Sp = a.Sp, L = a.L;
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x, gstride = (long long)gridDim.x * blockDim.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int chunks = (Sp + kMvRows - 1) / kMvRows;
-    for (int si = 0; si < a.nstages; ++si) {
-        const BcrStage st = a.stages[si];
-        if (st.kind == kBcrIn) {
-            for (long long e = gtid; e < (long long)L * Sp; e += gstride) {
-                const int k = (int)(e / Sp), y = (int)(e - (long long)k * Sp);
-                float val = 0.0f;
-                if (y < S) {
-                    const long long q = (long long)k * S + y;
-                    val = (float)(a.bscale ? a.b[q] * a.bscale[q] : a.b[q]);
-                }
-                a.bw[e] = val;
-            }
-        } else if (st.kind == kBcrFwd0) {
-            const int nk = (L + 1) / 2;
-            for (long long e = gtid; e < (long long)nk * S; e += gstride) {
-                const int i = 2 * (int)(e / S), y = (int)(e % S);
-                float acc = 0.0f;
-                if (i >= 1) acc += a.lo[(long long)i * S + y] * a.tw[(long long)(i - 1) * Sp + y];
-                if (i + 1 < L) acc += a.up[(long long)i * S + y] * a.tw[(long long)(i + 1) * Sp + y];
-                a.bw[(long long)i * Sp + y] -= acc;
-            }
-        } else if (st.kind == kBcrOut) {
-            for (long long e = gtid; e < (long long)L * S; e += gstride) {
-                const int k = (int)(e / S), y = (int)(e - (long long)k * S);
-                const double val = (double)a.xw[(long long)k * Sp + y];
-                a.x[e] = a.xscale ? val * a.xscale[e] : val;
-            }
-        } else if (st.kind == kBcrMv) {
-            const int items = st.count * chunks;
-            for (int item = blockIdx.x; item < items; item += gridDim.x) {
-                const BcrMv t = a.mv[st.off + item / chunks];
-                const int chunk = item % chunks;
-                __syncthreads();
-                for (int k = threadIdx.x; k < t.K; k += blockDim.x) {
-                    float val;
-                    if (k < Sp) {
-                        val = t.v0[k];
-                        if (k < S) {
-                            if (t.d0) val -= t.d0[k] * t.w0[k];
-                            if (t.d1) val -= t.d1[k] * t.w1[k];
-                        }
-                    } else {
-                        val = t.v1[k - Sp];
-                    }
-                    v[k] = val;
-                }
-                __syncthreads();
-                const int r1 = min(Sp, (chunk + 1) * kMvRows);
-                for (int r = chunk * kMvRows + warp; r < r1; r += kMvThreads / 32) {
-                    const float4 *row = (const float4 *)(t.M + (long long)r * t.ld);
-                    float acc = 0.0f;
-                    for (int q = lane; q < t.K / 4; q += 32) {
-                        const float4 m = row[q];
-                        acc += m.x * v[4 * q] + m.y * v[4 * q + 1] + m.z * v[4 * q + 2] + m.w * v[4 * q + 3];
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    if (lane == 0) t.y[r] = (t.base ? t.base[r] : 0.0f) + t.sign * acc;
-                }
-            }
-        }
-        if (si + 1 < a.nstages && !grid_barrier(a.bar, ctl)) return;
-    }
-}
-
 __global__ void k_bcr_pad(float *D, int L, int S, int Sp)
 {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -750,46 +586,54 @@ struct Builder {
         }
         const int root = lists.back()[0];
         inverse(Sp, Dfull, std::vector<int>{root}, Ifull, std::vector<int>{root}, 0, p.levels);
-        // solve
-        p.sol.push_back(BcrStage{kBcrIn, 0, 0, 0, 0});
+        // solve: right-hand sides are read where they are first needed, and those of the layers kept
+        // at level 0 with the coupling terms to their eliminated neighbours taken off on the way
+        auto rhs0 = [&](int i, int &layer, const float *&c0, const float *&w0, const float *&c1, const float *&w1) {
+            layer = i;
+            if (i >= 1) { c0 = row(p.lo, i); w0 = vec(p.tw, i - 1); }
+            if (i + 1 < L) { c1 = row(p.up, i); w1 = vec(p.tw, i + 1); }
+        };
+        auto mv = [](const float *M, int ld, int K, float sign, float *y) {
+            BcrMv t{};
+            t.M = M; t.ld = ld; t.K = K; t.sign = sign; t.y = y;
+            t.in = t.bin = t.out = -1;
+            return t;
+        };
         for (int l = 0; l < p.levels; ++l) {
             const auto &a = lists[l];
             std::vector<BcrMv> ts;
             for (size_t q = 1; q < a.size(); q += 2) {       // t_j = D_j^-1 b_j
                 const int j = a[q];
-                ts.push_back(BcrMv{ptr(kArrINV, j, 0, 0), vec(p.bw, j), nullptr, nullptr, nullptr, nullptr, nullptr,
-                                   nullptr, vec(p.tw, j), Sp, Sp, 1.0f});
+                BcrMv t = mv(ptr(kArrINV, j, 0, 0), Sp, Sp, 1.0f, vec(p.tw, j));
+                if (l == 0) t.in = j;
+                else if (l == 1) rhs0(j, t.in, t.d0, t.w0, t.d1, t.w1);
+                else t.v0 = vec(p.bw, j);
+                ts.push_back(t);
             }
             mv_stage(ts, l);
+            if (l == 0) continue;
             ts.clear();
-            if (l == 0) {
-                p.sol.push_back(BcrStage{kBcrFwd0, 0, 0, 0, 0});
-                continue;
-            }
             for (size_t q = 0; q < a.size(); q += 2) {       // b_i -= L_i t_l + U_i t_r
                 const int i = a[q];
                 const int cpi = cp_off[l] + (int)q;
                 const bool hl = q >= 1, hr = q + 1 < a.size();
                 if (!hl && !hr) continue;
-                BcrMv t{};
-                t.ld = 2 * Sp;
-                t.sign = -1.0f;
-                t.base = vec(p.bw, i);
-                t.y = vec(p.bw, i);
-                if (hl && hr) {
-                    t.M = ptr(kArrCP, cpi, 0, 0); t.K = 2 * Sp; t.v0 = vec(p.tw, a[q - 1]); t.v1 = vec(p.tw, a[q + 1]);
-                } else if (hl) {
-                    t.M = ptr(kArrCP, cpi, 0, 0); t.K = Sp; t.v0 = vec(p.tw, a[q - 1]);
-                } else {
-                    t.M = ptr(kArrCP, cpi, 0, Sp); t.K = Sp; t.v0 = vec(p.tw, a[q + 1]);
-                }
+                BcrMv t = mv(ptr(kArrCP, cpi, 0, hl ? 0 : Sp), 2 * Sp, hl && hr ? 2 * Sp : Sp, -1.0f, vec(p.bw, i));
+                if (l == 1) rhs0(i, t.bin, t.e0, t.f0, t.e1, t.f1);
+                else t.base = vec(p.bw, i);
+                t.v0 = vec(p.tw, hl ? a[q - 1] : a[q + 1]);
+                if (hl && hr) t.v1 = vec(p.tw, a[q + 1]);
                 ts.push_back(t);
             }
             mv_stage(ts, l);
         }
         {
-            std::vector<BcrMv> ts{BcrMv{ptr(kArrINV, root, 0, 0), vec(p.bw, root), nullptr, nullptr, nullptr, nullptr,
-                                        nullptr, nullptr, vec(p.xw, root), Sp, Sp, 1.0f}};
+            BcrMv t = mv(ptr(kArrINV, root, 0, 0), Sp, Sp, 1.0f, vec(p.xw, root));
+            if (p.levels == 0) t.in = root;
+            else if (p.levels == 1) rhs0(root, t.in, t.d0, t.w0, t.d1, t.w1);
+            else t.v0 = vec(p.bw, root);
+            t.out = root;
+            std::vector<BcrMv> ts{t};
             mv_stage(ts, p.levels);
         }
         for (int l = p.levels - 1; l >= 0; --l) {
@@ -798,30 +642,23 @@ struct Builder {
             for (size_t q = 1; q < a.size(); q += 2) {
                 const int j = a[q];
                 const bool hr = q + 1 < a.size();
-                BcrMv t{};
-                t.ld = Sp;
-                t.K = Sp;
-                t.y = vec(p.xw, j);
+                BcrMv t;
                 if (l == 0) {      // x_j = D_j^-1 (b_j - lo_j x_{j-1} - up_j x_{j+1})
-                    t.M = ptr(kArrINV, j, 0, 0);
-                    t.v0 = vec(p.bw, j);
+                    t = mv(ptr(kArrINV, j, 0, 0), Sp, Sp, 1.0f, vec(p.xw, j));
+                    t.in = j;
                     t.d0 = row(p.lo, j); t.w0 = vec(p.xw, a[q - 1]);
                     if (hr) { t.d1 = row(p.up, j); t.w1 = vec(p.xw, a[q + 1]); }
-                    t.sign = 1.0f;
                 } else {           // x_j = t_j - [P_j | Q_j] [x_l; x_r]
-                    t.M = ptr(kArrPQ, j, 0, 0);
-                    t.ld = 2 * Sp;
-                    t.K = hr ? 2 * Sp : Sp;
+                    t = mv(ptr(kArrPQ, j, 0, 0), 2 * Sp, hr ? 2 * Sp : Sp, -1.0f, vec(p.xw, j));
                     t.v0 = vec(p.xw, a[q - 1]);
                     t.v1 = hr ? vec(p.xw, a[q + 1]) : nullptr;
                     t.base = vec(p.tw, j);
-                    t.sign = -1.0f;
                 }
+                t.out = j;
                 ts.push_back(t);
             }
             mv_stage(ts, l);
         }
-        p.sol.push_back(BcrStage{kBcrOut, 0, 0, 0, 0});
     }
 };
 
@@ -933,30 +770,6 @@ cudaError_t bcr_factor(const BcrPlan &p, const int *skip, Ctl *ctl, cudaStream_t
         }
     }
     return cudaGetLastError();
-}
-
-cudaError_t bcr_solve(const BcrPlan &p, const double *b, double *x, const double *bscale, const double *xscale,
-                      const int *skip, Ctl *ctl, cudaStream_t st)
-{
-    static int fit = 0;
-    const size_t smem = (size_t)2 * p.Sp * sizeof(float);
-    if (!fit) {
-        int dev = 0, sms = 0, per = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bcr_solve_all, kMvThreads, 2 * 1280 * sizeof(float)) !=
-                cudaSuccess || per < 1)
-            per = 1;
-        fit = sms * std::min(per, 4);
-    }
-    int ctas = p.solve_ctas > 0 ? std::min(p.solve_ctas, fit) : fit;
-    SolveArgs a;
-    a.stages = p.sol_d; a.mv = p.mv_d; a.b = b; a.bscale = bscale; a.xscale = xscale; a.x = x;
-    a.bw = p.bw; a.tw = p.tw; a.xw = p.xw; a.lo = p.lo; a.up = p.up; a.bar = p.bar;
-    a.nstages = (int)p.sol.size(); a.L = p.L; a.S = p.S; a.Sp = p.Sp;
-    void *args[] = {(void *)&a, (void *)&skip, (void *)&ctl};
-    count_launches(1);
-    return cudaLaunchCooperativeKernel((const void *)k_bcr_solve_all, dim3(ctas), dim3(kMvThreads), args, smem, st);
 }
 
 }  // namespace xk

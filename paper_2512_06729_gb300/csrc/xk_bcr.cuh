@@ -17,14 +17,18 @@ struct BcrLeaf {
     int ldin, ldout, n;
 };
 
-// y = base + sign * M v for the rows [0, Sp) of one block: M is Sp x K row-major (ld), v is
-// [v0; v1] (K = Sp or 2 Sp), optionally v0 - d0 w0 - d1 w1 on the first S entries (level 0).
+// y = base + sign * M v for the rows [0, Sp) of one block: M is Sp x K row-major (ld).  v is the
+// right-hand side of layer `in` (in >= 0) or the work vector v0, less d0 w0 and d1 w1 on the first S
+// entries (the diagonal couplings of level 0), and behind it v1 when K = 2 Sp.  The base likewise:
+// layer `bin` of the right-hand side or the vector base, less e0 f0 and e1 f1.  out >= 0: y is also
+// the solution of that layer.
 struct BcrMv {
     const float *M;
-    const float *v0, *v1, *d0, *w0, *d1, *w1, *base;
+    const float *v0, *v1, *d0, *w0, *d1, *w1, *base, *e0, *f0, *e1, *f1;
     float *y;
     int ld, K;
     float sign;
+    int in, bin, out;
 };
 
 struct BcrStage {
@@ -33,7 +37,7 @@ struct BcrStage {
     int tiles;         // GEMM: output tiles of the launch; leaf inversions: the blocks' order n
     int level;         // the reduction level it belongs to
 };
-enum BcrKind { kBcrLeafStage = 0, kBcrGemm = 1, kBcrLevel0 = 2, kBcrMv = 3, kBcrFwd0 = 4, kBcrIn = 5, kBcrOut = 6 };
+enum BcrKind { kBcrLeafStage = 0, kBcrGemm = 1, kBcrLevel0 = 2, kBcrMv = 3 };
 
 // The plan of one column's factorization and solve.  Built on the host once per workspace; the
 // task lists live in the workspace.
@@ -56,8 +60,8 @@ struct BcrPlan {
     std::vector<CUtensorMap> maps;
     int *l0_d = nullptr;
     BcrStage *sol_d = nullptr;     // the solve's stages, walked by one persistent kernel
-    unsigned *bar = nullptr;       // its grid-barrier words (2, zero between calls)
-    int solve_ctas = 0;            // CTAs of that kernel (0: as many as fit on the GPU)
+    unsigned *bar = nullptr;       // its GridSync words (2, zero between calls)
+    int solve_ctas = 0;            // CTAs of that kernel (0: one per SM)
 };
 
 // Sizes of the device arrays and task lists of an L-layer, S-species column (no pointers).
@@ -81,8 +85,14 @@ struct BcrTimer {
 cudaError_t bcr_factor(const BcrPlan &p, const int *skip, Ctl *ctl, cudaStream_t st, BcrTimer *timer = nullptr);
 // Flops of one factorization: 2 m n k over the products, 2 n^3 over the leaves.
 void bcr_work(const BcrPlan &p, double *mma_flops, double *leaf_flops);
-// x = M^-1 (b * bscale) (* xscale) with the factorization, FP64 in and out.
+// x = M^-1 (b * bscale) (* xscale) with the factorization, FP64 in and out (xk_fgmres.cu).
 cudaError_t bcr_solve(const BcrPlan &p, const double *b, double *x, const double *bscale, const double *xscale,
                       const int *skip, Ctl *ctl, cudaStream_t st);
+
+struct GmArgs;
+// The whole FGMRES of enqueue_fgmres preconditioned by the reduction (role 0), in one cooperative
+// launch; its matrix-vector product is launch_jv's with the rows divided by rowd, its preconditioner
+// bcr_solve's with bscale = rowd.  Not for cfg.photo_jacobian, whose product needs launches of its own.
+cudaError_t bcr_fgmres(const BcrPlan &p, const Col &c, const GmArgs &g, const double *rowd, cudaStream_t st);
 
 }  // namespace xk

@@ -7,8 +7,9 @@
 #include <algorithm>
 
 #include <atomic>
+#include <mutex>
 
-#include "xk_internal.cuh"
+#include "xk_layer.cuh"
 
 namespace xk {
 
@@ -303,110 +304,205 @@ __global__ void k_photo_k(Col c)
 // d[slot] = d(k_f prod n_reac)/d n_reac[slot] (slots 0-2) and
 //           -d(k_r prod n_prod)/d n_prod[slot] (slots 3-5)
 // ---------------------------------------------------------------------------
-__global__ void k_reaction_terms(Col c, const double *n)
-{
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)c.L * c.R) return;
-    int k = (int)(idx / c.R), r = (int)(idx % c.R);
-    reaction_terms_at(c, k, r, n + (long long)k * c.S, c.w + idx, c.d + idx * 6);
-}
-
-// F = sum_r nu w_r - (phi_{k+1/2} - phi_{k-1/2}) / dz_k; also the solve scaling
-// s = max(n, f_floor n_gas) and the scaled right-hand side b = F / s.
-__global__ void k_residual(Col c, const double *n, double *F, const Ctl *ctl, double f_floor)
+// Layer k of the step's right-hand side, by one CTA: the reaction rates and derivatives
+// (reaction_terms_at), then F = sum_r nu w_r - (phi_{k+1/2} - phi_{k-1/2}) / dz_k from the rates in
+// shared memory, the solve scaling s = max(n, f_floor n_gas) with b = F / s, and, when diag is
+// given, the rows' equilibration: diag = max(|I/dt - dF/dn|_ii, 1/dt) and bhat = b / diag, the
+// diagonal entry summed from the derivatives just written.  A kernel per quantity with a thread per
+// species took 170 us at 594 species x 150 layers, most of it in the few threads that hold the bath
+// gas's thousands of entries one after the other.
+__global__ void __launch_bounds__(512)
+k_layer_terms(Col c, const double *n, double *F, const Ctl *ctl, double f_floor, double *diag, double *bhat,
+              int rates_in_smem)
 {
     if (ctl && ctl->finished) return;
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    int S = c.S, L = c.L;
-    if (idx >= (long long)L * S) return;
-    int k = (int)(idx / S), y = (int)(idx % S);
-    const double *wk = c.w + (long long)k * c.R;
-    double f = 0.0;
-    for (int e = c.yp[y]; e < c.yp[y + 1]; ++e) {
-        int code = c.yent[e];
-        int r = code >> 4;
-        int nu = (code & 15) - 8;
-        if (nu < 0) f -= wk[r];
-        else f += wk[r];
-    }
-    double nk = n[idx];
-    double upf = 0.0, dnf = 0.0;
-    if (k + 1 < L) upf = c.u[(long long)k * S + y] * nk - c.v[(long long)k * S + y] * n[idx + S];
-    if (k > 0) dnf = c.u[(long long)(k - 1) * S + y] * n[idx - S] - c.v[(long long)(k - 1) * S + y] * nk;
-    f += -(upf - dnf) / c.dz[k];
-    if (c.fshift) f -= c.fshift[idx];
-    F[idx] = f;
-    if (c.s) {
-        double sc = fmax(nk, f_floor * c.ngas[k]);
-        c.s[idx] = sc;
-        c.b[idx] = f / sc;
-        if (c.rs) c.rs[idx] = 1.0 / sc;
+    extern __shared__ double lt_sm[];
+    const int S = c.S, R = c.R, L = c.L;
+    for (int k = blockIdx.x; k < L; k += gridDim.x) {
+        double *sn = lt_sm, *part = sn + S, *w = rates_in_smem ? part + c.nsub : c.w + (long long)k * R;
+        const long long row0 = (long long)k * S;
+        __syncthreads();
+        for (int i = threadIdx.x; i < S; i += blockDim.x) sn[i] = n[row0 + i];
+        __syncthreads();
+        double *dk = c.d + (long long)k * R * 6;
+        for (int r = threadIdx.x; r < R; r += blockDim.x) {
+            double wr, d[6];
+            reaction_terms_at(c, k, r, sn, &wr, d);
+            w[r] = wr;
+            double2 *o = (double2 *)(dk + (long long)r * 6);
+            o[0] = make_double2(d[0], d[1]);
+            o[1] = make_double2(d[2], d[3]);
+            o[2] = make_double2(d[4], d[5]);
+        }
+        __syncthreads();
+        species_parts(c, w, part);
+        __syncthreads();
+        for (int i = threadIdx.x; i < S; i += blockDim.x) {
+            const long long idx = row0 + i;
+            const double nk = sn[i];
+            double f = -species_sum(c, part, i);
+            double upf = 0.0, dnf = 0.0;
+            if (k + 1 < L) upf = c.u[idx] * nk - c.v[idx] * n[idx + S];
+            if (k > 0) dnf = c.u[idx - S] * n[idx - S] - c.v[idx - S] * nk;
+            f += -(upf - dnf) / c.dz[k];
+            if (c.fshift) f -= c.fshift[idx];
+            F[idx] = f;
+            if (c.s) {
+                const double sc = fmax(nk, f_floor * c.ngas[k]);
+                c.s[idx] = sc;
+                c.b[idx] = f / sc;
+                c.rs[idx] = 1.0 / sc;
+            }
+        }
+        if (!diag) continue;
+        __syncthreads();
+        // diagonal entries: the same sublists over the terms of each species' own column
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        for (int g = warp; g < c.ndg; g += nw) {
+            double acc = 0.0;
+            const int q1 = c.dgp[g + 1];
+#pragma unroll 4
+            for (int q = c.dgp[g]; q < q1; ++q) {
+                const int code = c.dent[32 * q + lane];
+                if (code >= 0) acc += signed_by(dk[code >> 1], code & 1);
+            }
+            const int to = c.dpart[32 * g + lane];
+            if (to >= 0) part[to] = acc;
+        }
+        __syncthreads();
+        const double rdt = 1.0 / ctl->dt;
+        for (int i = threadIdx.x; i < S; i += blockDim.x) {
+            const long long idx = row0 + i;
+            double acc = 0.0;
+            for (int q = c.dsp[i]; q < c.dsp[i + 1]; ++q) acc += part[q];
+            const double dg = fmax(fabs(rdt + acc + c.tdg[idx]), rdt);
+            diag[idx] = dg;
+            bhat[idx] = c.b[idx] / dg;
+        }
     }
 }
 
-// Dense diagonal blocks A_k = I/dt - dF_k/dn_k, couplings lo/up; one warp per row.
-// Contributions are summed in a fixed order (deterministic).  scaled != 0 writes
+// Dense diagonal blocks A_k = I/dt - dF_k/dn_k, couplings lo/up.  scaled != 0 writes
 // diag(1/s) A diag(s) and the matching couplings.
+//
+// A row's non-zeros come from the reactions its species is in, about fifty of a network's thousands.
+// A warp loads those reactions' derivatives (48 contiguous bytes each) into shared memory once and
+// its lanes then sum whole columns of the row from there, each in a fixed order, eight rows to a
+// CTA; a species in more than kJacOcc reactions (the bath gas is in thousands) takes a whole CTA.
+// Gathering every term of every entry from global memory instead is bound by its latency: 1,290 us
+// at 594 species x 150 layers.  Bound now by the FP64 additions of the terms (4.2e7, about 75 us at
+// this part's two FP64 operations per clock and SM) beside the write of the blocks (222 MB in FP32,
+// 33 us); only non-zero entries are scaled and converted, which FP64 units do too.
 template <typename T>
-__global__ void k_jacobian(Col c, const double *n, const Ctl *ctl, double dt_override, int scaled,
-                           T *A, T *lo, T *up, double *dout, const int *skip, long long lstride)
+__global__ void __launch_bounds__(kJacWarps * 32)
+k_jacobian(Col c, const Ctl *ctl, double dt_override, int scaled, T *A, T *lo, T *up, const int *skip, long long lstride)
 {
     if ((ctl && ctl->finished) || (skip && *skip)) return;
-    extern __shared__ double sh[];
-    const int S = c.S, L = c.L;
-    const int wpb = blockDim.x >> 5;
+    extern __shared__ __align__(16) unsigned char jac_sm[];
+    const int S = c.S, L = c.L, ld = c.ld;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *rowbuf = sh + (long long)warp * (S + 64);
-    const double dt = dt_override > 0.0 ? dt_override : ctl->dt;
-    for (long long row = (long long)blockIdx.x * wpb + warp; row < (long long)L * S; row += (long long)gridDim.x * wpb) {
-        const int k = (int)(row / S), i = (int)(row % S);
-        __syncwarp();
-        for (int j = lane; j < S; j += 32) rowbuf[j] = 0.0;
-        __syncwarp();
-        const double *dk = c.d + (long long)k * c.R * 6;
-        // each lane owns whole column entries and sums their terms in a fixed order (deterministic)
-        for (int q = c.jp[i] + lane; q < c.jp[i + 1]; q += 32) {
-            double acc = 0.0;
-            for (int t = c.jtp[q]; t < c.jtp[q + 1]; ++t) {
-                const int code = c.jrs[t];
-                const int rs = code >> 1;
-                const double dv = dk[(long long)(rs >> 3) * 6 + (rs & 7)];
-                acc += (code & 1) ? dv : -dv;
+    double *dall = (double *)jac_sm;                                  // kJacHeavyOcc * 6: the tiles' derivatives
+    double *hrow = dall + kJacHeavyOcc * 6;                           // S: a heavy row
+    T *row = (T *)(hrow + S) + (long long)warp * S;                   // S: this warp's light row
+    double *dbuf = dall + warp * kJacOcc * 6;
+    const double rdt = 1.0 / (dt_override > 0.0 ? dt_override : ctl->dt);
+    if (lstride <= 0) lstride = (long long)S * ld;
+
+    // derivatives of tile t's reactions, by nt threads of which this is number id
+    auto load_tile = [&](const double2 *dk, int t, double *dst, int id, int nt) {
+        const int o0 = c.jto[t], n = (c.jto[t + 1] - o0) * 3;
+        for (int b = id; b < n; b += 4 * nt) {
+            double2 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e = min(b + u * nt, n - 1), occ = e / 3;
+                v[u] = dk[3 * (long long)(c.yent[o0 + occ] >> 4) + (e - 3 * occ)];
             }
-            rowbuf[c.jcol[q]] = acc;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (b + u * nt < n) ((double2 *)dst)[b + u * nt] = v[u];
         }
-        __syncwarp();
-        const double *sk = c.s + (long long)k * S;
-        if (lane == 0) {
-            rowbuf[i] += 1.0 / dt + c.tdg[row];
-            if (dout) dout[row] = fmax(fabs(rowbuf[i]), 1.0 / dt);
-            double lov = c.tlo[row];
-            double upv = c.tup[row];
-            if (scaled) {
-                if (k > 0) lov *= c.s[(long long)(k - 1) * S + i] / sk[i];
-                if (k + 1 < L) upv *= c.s[(long long)(k + 1) * S + i] / sk[i];
-            }
-            lo[row] = (T)lov;
-            up[row] = (T)upv;
+    };
+    auto group_sum = [&](const double *src, int g) {
+        double acc = 0.0;
+        const int t1 = c.jge[g + 1];
+#pragma unroll 4
+        for (int t = c.jge[g]; t < t1; ++t) {
+            const int code = c.jterm[t];
+            acc += signed_by(src[code >> 1], code & 1);
         }
-        __syncwarp();
-        T *Ar = A + (long long)k * (lstride > 0 ? lstride : (long long)S * c.ld) + (long long)i * c.ld;
+        return acc;
+    };
+    auto couplings = [&](int k, int i) {
+        const long long q = (long long)k * S + i;
+        double lov = c.tlo[q], upv = c.tup[q];
         if (scaled) {
-            double inv = 1.0 / sk[i];
-            for (int j = lane; j < S; j += 32) Ar[j] = (T)(rowbuf[j] * sk[j] * inv);
-        } else {
-            for (int j = lane; j < S; j += 32) Ar[j] = (T)rowbuf[j];
+            const double ri = c.rs[q];
+            if (k > 0) lov *= c.s[q - S] * ri;
+            if (k + 1 < L) upv *= c.s[q + S] * ri;
         }
-        for (int j = S + lane; j < c.ld; j += 32) Ar[j] = (T)0;
+        lo[q] = (T)lov;
+        up[q] = (T)upv;
+    };
+
+    const long long items = (long long)c.nji * L;
+    for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+        const int q = (int)(it / L), k = (int)(it - (long long)q * L);
+        const double2 *dk = (const double2 *)(c.d + (long long)k * c.R * 6);
+        const double *sk = c.s + (long long)k * S;
+        if (c.jit[kJacWarps * q + 1] != -2) {
+            const int i = c.jit[kJacWarps * q + warp];
+            if (i < 0) continue;
+            for (int j = lane; j < S; j += 32) row[j] = (T)0;
+            const double diag = rdt + c.tdg[(long long)k * S + i];
+            const double inv = scaled ? c.rs[(long long)k * S + i] : 1.0;
+            __syncwarp();
+            const int t = c.jrt[i];
+            if (t < c.jrt[i + 1]) {                       // one tile at most
+                load_tile(dk, t, dbuf, lane, 32);
+                __syncwarp();
+                for (int g = c.jtg[t] + lane; g < c.jtg[t + 1]; g += 32) {
+                    const int j = c.jgc[g];
+                    double v = group_sum(dbuf, g);
+                    if (j == i) v += diag;
+                    if (scaled && j != i) v = v * sk[j] * inv;
+                    row[j] = (T)v;
+                }
+            }
+            if (lane == 0) {
+                if (c.jdq[i] < 0) row[i] = (T)diag;       // no reaction holds it
+                couplings(k, i);
+            }
+            __syncwarp();
+            T *Ar = A + (long long)k * lstride + (long long)i * ld;
+            for (int j = lane; j < ld; j += 32) Ar[j] = j < S ? row[j] : (T)0;
+            __syncwarp();
+        } else {
+            const int i = c.jit[kJacWarps * q];
+            const double diag = rdt + c.tdg[(long long)k * S + i];
+            const double inv = scaled ? c.rs[(long long)k * S + i] : 1.0;
+            __syncthreads();
+            for (int j = threadIdx.x; j < S; j += blockDim.x) hrow[j] = j == i ? diag : 0.0;
+            for (int t = c.jrt[i]; t < c.jrt[i + 1]; ++t) {
+                __syncthreads();
+                load_tile(dk, t, dall, threadIdx.x, blockDim.x);
+                __syncthreads();
+                for (int g = c.jtg[t] + threadIdx.x; g < c.jtg[t + 1]; g += blockDim.x)
+                    hrow[c.jgc[g]] += group_sum(dall, g);
+            }
+            __syncthreads();
+            T *Ar = A + (long long)k * lstride + (long long)i * ld;
+            for (int j = threadIdx.x; j < ld; j += blockDim.x) {
+                double v = j < S ? hrow[j] : 0.0;
+                if (scaled && j < S && j != i) v = v * sk[j] * inv;
+                Ar[j] = (T)v;
+            }
+            if (threadIdx.x == 0) couplings(k, i);
+            __syncthreads();
+        }
     }
 }
 
-// y = diag(1/s) (I/dt - J) diag(s) x, matrix-free from the reaction derivatives (FP64), in two
-// passes.  First the directional derivative of every rate along v = s x:
-//   dw[k][r] = sum over the reaction's slots of d[k][r][slot] v[k][species(slot)]
-// (d holds d(k_f prod n_reac)/dn and -d(k_r prod n_prod)/dn, so dw is the change of w_r);
-// then per species (J v)_i = sum_r nu_ir dw_r through the species-major stoichiometry, a warp
-// per row, plus the transport terms.
 // ---------------------------------------------------------------------------
 // photolysis rates in the Jacobian (cfg.photo_jacobian): the change of k_ph along the physical
 // direction v = s x of J v.  The direct beam J = J0 exp(-tau/mu) changes by -J dtau/mu, with dtau
@@ -494,128 +590,16 @@ __global__ void k_photo_dk(Col c, const Ctl *ctl, const int *skip)
     if (lane == 0) c.pdk[(long long)k * c.Rph + q] = c.tf * s;
 }
 
-// the photolysis rate's extra change along v (0 unless photo_jacobian): dk_ph n_A
-__device__ __forceinline__ double photo_jv_term(const Col &c, int k, int r)
-{
-    if (!c.photo_jac || c.rtype[r] != XK_RX_PHOTO) return 0.0;
-    return c.pdk[(long long)k * c.Rph + c.prow[r]] * c.n[(long long)k * c.S + c.reac[3 * r]];
-}
-
-__global__ void k_jv_rates(Col c, const Ctl *ctl, const double *x, const int *skip)
+// y = diag(1/s) (I/dt - J) diag(s) x, one CTA per layer (xk_layer.cuh)
+__global__ void __launch_bounds__(512) k_jv_layer(Col c, const Ctl *ctl, const double *x, double *y,
+                                                  const double *rowdiv, const int *skip, int rates_in_smem)
 {
     if ((ctl && ctl->finished) || (skip && *skip)) return;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < (long long)c.L * c.R;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(idx / c.R), r = (int)(idx % c.R);
-        const double *d = c.d + idx * 6;
-        const double *sk = c.s + (long long)k * c.S, *xk = x + (long long)k * c.S;
-        double acc = 0.0;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const int i = c.reac[3 * r + q];
-            if (i >= 0) acc += d[q] * sk[i] * xk[i];
-            const int j = c.prod[3 * r + q];
-            if (j >= 0) acc += d[3 + q] * sk[j] * xk[j];
-        }
-        c.dw[idx] = acc + photo_jv_term(c, k, r);
-    }
-}
-
-__device__ __forceinline__ void jv_row(const Col &c, const Ctl *ctl, const double *x, double *y, const double *rowdiv,
-                                       int warp, int lane);
-__device__ __forceinline__ void jv_finish(const Col &c, const Ctl *ctl, const double *x, double *y,
-                                          const double *rowdiv, int k, int i, double acc);
-
-// The same J v in one launch with one CTA per layer: the layer's R directional rate derivatives are
-// formed in shared memory, then each species sums its stoichiometric entries from there (the
-// gathers hit shared memory instead of L1).  For networks whose R doubles fit shared memory.
-__global__ void k_jv_layer(Col c, const Ctl *ctl, const double *x, double *y, const double *rowdiv, const int *skip)
-{
-    if ((ctl && ctl->finished) || (skip && *skip)) return;
-    extern __shared__ double dws[];
-    const int S = c.S, R = c.R;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    extern __shared__ double jv_sm[];
     for (int k = blockIdx.x; k < c.L; k += gridDim.x) {
-        const double *sk = c.s + (long long)k * S, *xk = x + (long long)k * S;
-        const double *dk = c.d + (long long)k * R * 6;
         __syncthreads();
-        for (int r = threadIdx.x; r < R; r += blockDim.x) {
-            const double *d = dk + (long long)r * 6;
-            double acc = 0.0;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int a = c.reac[3 * r + q];
-                if (a >= 0) acc += d[q] * sk[a] * xk[a];
-                const int b = c.prod[3 * r + q];
-                if (b >= 0) acc += d[3 + q] * sk[b] * xk[b];
-            }
-            dws[r] = acc + photo_jv_term(c, k, r);
-        }
-        __syncthreads();
-        for (int i = warp; i < S; i += nw) {
-            double acc = 0.0;
-            for (int e = c.yp[i] + lane; e < c.yp[i + 1]; e += 32) {
-                const int code = c.yent[e];
-                const double v = dws[code >> 4];
-                acc += ((code & 15) - 8 < 0) ? v : -v;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) jv_finish(c, ctl, x, y, rowdiv, k, i, acc);
-        }
+        jv_layer_body(c, ctl, x, y, rowdiv, k, jv_sm, rates_in_smem != 0);
     }
-}
-
-__global__ void k_jv(Col c, const Ctl *ctl, const double *x, double *y, const double *rowdiv, const int *skip)
-{
-    if ((ctl && ctl->finished) || (skip && *skip)) return;
-    const int S = c.S, L = c.L;
-    const int lane = threadIdx.x & 31;
-    const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); warp < L * S; warp += nwarps)
-        jv_row(c, ctl, x, y, rowdiv, warp, lane);
-}
-
-__device__ __forceinline__ void jv_row(const Col &c, const Ctl *ctl, const double *x, double *y, const double *rowdiv,
-                                       int warp, int lane)
-{
-    const int S = c.S, L = c.L;
-    int k = warp / S, i = warp % S;
-    const double *dwk = c.dw + (long long)k * c.R;
-    const double *sk = c.s + (long long)k * S;
-    const double *xk = x + (long long)k * S;
-    double acc = 0.0;
-    for (int e = c.yp[i] + lane; e < c.yp[i + 1]; e += 32) {
-        const int code = c.yent[e];
-        const double v = dwk[code >> 4];
-        acc += ((code & 15) - 8 < 0) ? v : -v;       // -(nu) dw: reactant rows +, product rows -
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) jv_finish(c, ctl, x, y, rowdiv, k, i, acc);
-    (void)sk;
-    (void)xk;
-}
-
-// Row (k, i) of y from the chemistry sum acc = -(J diag(s) x)_i: scaling, I/dt and transport.
-__device__ __forceinline__ void jv_finish(const Col &c, const Ctl *ctl, const double *x, double *y,
-                                          const double *rowdiv, int k, int i, double acc)
-{
-    const int S = c.S, L = c.L;
-    const long long q = (long long)k * S + i;
-    const double ri = c.rs[q];
-    double r = acc * ri + (1.0 / ctl->dt + c.tdg[q]) * x[q];
-    if (k > 0) r += c.tlo[q] * c.s[q - S] * ri * x[q - S];
-    if (k + 1 < L) r += c.tup[q] * c.s[q + S] * ri * x[q + S];
-    if (rowdiv) r /= rowdiv[q];
-    y[q] = r;
-}
-
-// y = x / d (row equilibration of a right-hand side)
-__global__ void k_rowdiv(long long N, const double *x, const double *d, double *y)
-{
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < N) y[idx] = x[idx] / d[idx];
 }
 
 __global__ void k_unscale(Col c, const double *xs, double *delta)
@@ -670,30 +654,6 @@ __global__ void k_route(Ctl *ctl)
     ctl->skip_reuse = reuse ? 0 : 1;
     ctl->skip64 = (ctl->skip32 && !reuse) ? 0 : 1;
     ctl->used_fp64 = ctl->skip32;
-}
-
-// Diagonal of I/dt - dF/dn per (layer, species), from the reaction derivatives and transport.
-__global__ void k_diag(Col c, const Ctl *ctl, double *diag)
-{
-    if (ctl->finished) return;
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    int S = c.S, L = c.L;
-    if (idx >= (long long)L * S) return;
-    int k = (int)(idx / S), i = (int)(idx % S);
-    const double *dk = c.d + (long long)k * c.R * 6;
-    double acc = 0.0;
-    const int q = c.jdq[i];
-    if (q >= 0)
-        for (int t = c.jtp[q]; t < c.jtp[q + 1]; ++t) {
-            const int code = c.jrs[t];
-            const int rs = code >> 1;
-            const double dv = dk[(long long)(rs >> 3) * 6 + (rs & 7)];
-            acc += (code & 1) ? dv : -dv;
-        }
-    double dg = 1.0 / ctl->dt + acc;
-    if (k + 1 < L) dg += c.u[(long long)k * S + i] / c.dz[k];
-    if (k > 0) dg += c.v[(long long)(k - 1) * S + i] / c.dz[k];
-    diag[idx] = fmax(fabs(dg), 1.0 / ctl->dt);
 }
 
 // Scalings of the reused FP64 factorization: input rowd * s / s64, output s64 / s.
@@ -873,37 +833,43 @@ void launch_photolysis(const Col &c, const double *n, cudaStream_t st)
     if (((long long)c.L * c.Rph * 32) > 0) { count_launches(1); k_photo_k<<<nblocks((long long)c.L * c.Rph * 32), kThreads, 0, st>>>(c); }
 }
 
-void launch_reaction_terms(const Col &c, const double *n, cudaStream_t st)
+void launch_layer_terms(const Col &c, const double *n, double *F, const Ctl *ctl, double f_floor, double *diag,
+                        double *bhat, cudaStream_t st)
 {
-    if (((long long)c.L * c.R) > 0) { count_launches(1); k_reaction_terms<<<nblocks((long long)c.L * c.R), kThreads, 0, st>>>(c, n); }
+    if ((long long)c.L * c.S <= 0) return;
+    const bool rates = jv_rates_in_smem(c);
+    const size_t sm = jv_smem_doubles(c, rates) * sizeof(double);
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute(k_layer_terms, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
+    });
+    count_launches(1);
+    k_layer_terms<<<std::min(c.L, kGatedBlocks), 512, sm, st>>>(c, n, F, ctl, f_floor, diag, bhat, rates ? 1 : 0);
 }
 
-void launch_residual(const Col &c, const double *n, double *F, const Ctl *ctl, double f_floor, cudaStream_t st)
+template <typename T>
+static void launch_jacobian_t(const Col &c, const Ctl *ctl, double dt_override, int scaled, T *A, T *lo, T *up,
+                              cudaStream_t st, const int *skip, long long lstride)
 {
-    if (((long long)c.L * c.S) > 0) { count_launches(1); k_residual<<<nblocks((long long)c.L * c.S), kThreads, 0, st>>>(c, n, F, ctl, f_floor); }
+    if ((long long)c.L * c.S <= 0) return;
+    const size_t sm = sizeof(double) * ((size_t)kJacHeavyOcc * 6 + c.S) + sizeof(T) * (size_t)kJacWarps * c.S;
+    cudaFuncSetAttribute(k_jacobian<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const long long items = (long long)c.nji * c.L;
+    count_launches(1);
+    k_jacobian<T><<<(int)std::min<long long>(items, kGatedBlocks), kJacWarps * 32, sm, st>>>(c, ctl, dt_override, scaled, A, lo,
+                                                                                           up, skip, lstride);
 }
 
-static size_t jac_smem(const Col &c, int wpb)
+void launch_jacobian64(const Col &c, const Ctl *ctl, double dt_override, int scaled, double *A, double *lo, double *up,
+                       cudaStream_t st, const int *skip)
 {
-    return (size_t)wpb * ((size_t)(c.S + 64) * sizeof(double));
+    launch_jacobian_t<double>(c, ctl, dt_override, scaled, A, lo, up, st, skip, 0);
 }
 
-void launch_jacobian64(const Col &c, const double *n, const Ctl *ctl, double dt_override, int scaled,
-                       double *A, double *lo, double *up, cudaStream_t st, const int *skip)
+void launch_jacobian32(const Col &c, const Ctl *ctl, float *A, float *lo, float *up, cudaStream_t st, const int *skip,
+                       long long lstride)
 {
-    const int wpb = 4;
-    size_t sm = jac_smem(c, wpb);
-    cudaFuncSetAttribute(k_jacobian<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (((long long)c.L * c.S) > 0) { count_launches(1); k_jacobian<double><<<skip ? gated_blocks((long long)c.L * c.S, wpb) : nblocks((long long)c.L * c.S, wpb), wpb * 32, sm, st>>>(c, n, ctl, dt_override, scaled, A, lo, up, nullptr, skip, 0); }
-}
-
-void launch_jacobian32(const Col &c, const double *n, const Ctl *ctl, float *A, float *lo, float *up, double *diag,
-                       cudaStream_t st, const int *skip, long long lstride)
-{
-    const int wpb = 4;
-    size_t sm = jac_smem(c, wpb);
-    cudaFuncSetAttribute(k_jacobian<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (((long long)c.L * c.S) > 0) { count_launches(1); k_jacobian<float><<<skip ? gated_blocks((long long)c.L * c.S, wpb) : nblocks((long long)c.L * c.S, wpb), wpb * 32, sm, st>>>(c, n, ctl, 0.0, 1, A, lo, up, diag, skip, lstride); }
+    launch_jacobian_t<float>(c, ctl, 0.0, 1, A, lo, up, st, skip, lstride);
 }
 
 void launch_jv(const Col &c, const Ctl *ctl, const double *xs, double *ys, const double *rowdiv, const int *skip,
@@ -917,25 +883,14 @@ void launch_jv(const Col &c, const Ctl *ctl, const double *xs, double *ys, const
         k_photo_dJ<<<nblocks((long long)c.W * 32, 128), 128, 0, st>>>(c, ctl, skip);
         k_photo_dk<<<nblocks((long long)c.L * c.Rph * 32), kThreads, 0, st>>>(c, ctl, skip);
     }
-    const size_t sm = (size_t)std::max(c.R, 1) * sizeof(double);
-    if (sm <= 160 * 1024) {
-        static size_t attr = 0;
-        if (sm > attr) {
-            cudaFuncSetAttribute(k_jv_layer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(160 * 1024));
-            attr = 160 * 1024;
-        }
-        count_launches(1);
-        k_jv_layer<<<std::min(c.L, kGatedBlocks), 512, sm, st>>>(c, ctl, xs, ys, rowdiv, skip);
-        return;
-    }
-    if (((long long)c.L * c.R) > 0) { count_launches(1); k_jv_rates<<<gated_blocks((long long)c.L * c.R), kThreads, 0, st>>>(c, ctl, xs, skip); }
+    const bool rates = jv_rates_in_smem(c);
+    const size_t sm = jv_smem_doubles(c, rates) * sizeof(double);
+    static std::once_flag once;
+    std::call_once(once, [] {
+        cudaFuncSetAttribute(k_jv_layer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
+    });
     count_launches(1);
-    k_jv<<<gated_blocks((long long)c.L * c.S * 32), kThreads, 0, st>>>(c, ctl, xs, ys, rowdiv, skip);
-}
-
-void launch_rowdiv(long long N, const double *x, const double *d, double *y, cudaStream_t st)
-{
-    if (N > 0) { count_launches(1); k_rowdiv<<<nblocks(N), kThreads, 0, st>>>(N, x, d, y); }
+    k_jv_layer<<<std::min(c.L, kGatedBlocks), 512, sm, st>>>(c, ctl, xs, ys, rowdiv, skip, rates ? 1 : 0);
 }
 
 void launch_unscale(const Col &c, const double *xs, double *delta, cudaStream_t st)
@@ -957,12 +912,6 @@ void launch_decide(const Col &c, Ctl *ctl, const Policy &pol, cudaStream_t st)
 void launch_apply(const Col &c, Ctl *ctl, cudaStream_t st)
 {
     if (((long long)c.L * c.S) > 0) { count_launches(1); k_apply<<<nblocks((long long)c.L * c.S), kThreads, 0, st>>>(c, ctl); }
-}
-
-void launch_diag(const Col &c, const Ctl *ctl, double *diag, cudaStream_t st)
-{
-    count_launches(1);
-    k_diag<<<nblocks((long long)c.L * c.S), kThreads, 0, st>>>(c, ctl, diag);
 }
 
 void launch_reuse_scales(long long N, const double *rowd, const double *s, const double *s64, double *pin, double *pout,

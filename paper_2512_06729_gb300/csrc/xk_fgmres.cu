@@ -197,32 +197,32 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// h[i] = <V_i, w>, i < nv, and with nv < 0 h[0] = <w, w>: a warp per basis vector over this CTA's
-// layers, then (after the barrier) every CTA adds the CTAs' parts in the same order.
-// The parts alternate between two buffers: a CTA past the barrier may write its next part while
-// another still adds the last ones.
+// h[i] = <V_i, w>, i < nv, and with nv < 0 h[0] = <w, w>: a warp per basis vector and layer of this
+// CTA, then (after the barrier) every CTA adds the layers' parts in the same order, so that the sums
+// do not depend on how many CTAs the launch has.  The parts alternate between two buffers: a CTA past
+// the barrier may write its next parts while another still adds the last ones.
 __device__ __forceinline__ bool fg_dots(const FgArgs &a, int nv, const double *w, double *h, GridSync &gs, int &buf)
 {
-    double *parts = a.partials + (long long)(buf ^= 1) * gridDim.x * (kMaxBasis + 1);
     const int S = a.c.S, L = a.c.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double *parts = a.partials + (long long)(buf ^= 1) * L * (kMaxBasis + 1);
     const long long N = (long long)L * S;
     const int n = nv < 0 ? 1 : nv;
     __syncthreads();
-    for (int i = warp; i < n; i += kWarps) {
-        const double *vi = nv < 0 ? w : a.V + (long long)i * N;
-        double acc = 0.0;
-        for (int k = blockIdx.x; k < L; k += gridDim.x) {
-            const long long o = (long long)k * S;
+    for (int k = blockIdx.x; k < L; k += gridDim.x) {
+        const long long o = (long long)k * S;
+        for (int i = warp; i < n; i += kWarps) {
+            const double *vi = nv < 0 ? w : a.V + (long long)i * N;
+            double acc = 0.0;
 #pragma unroll 4
             for (int e = lane; e < S; e += 32) acc += vi[o + e] * w[o + e];
+            acc = warp_sum(acc);
+            if (lane == 0) parts[(long long)k * (kMaxBasis + 1) + i] = acc;
         }
-        acc = warp_sum(acc);
-        if (lane == 0) parts[(long long)blockIdx.x * (kMaxBasis + 1) + i] = acc;
     }
     if (!gs.sync()) return false;
     for (int i = warp; i < n; i += kWarps) {
         double acc = 0.0;
-        for (int q = lane; q < (int)gridDim.x; q += 32) acc += parts[(long long)q * (kMaxBasis + 1) + i];
+        for (int k = lane; k < L; k += 32) acc += parts[(long long)k * (kMaxBasis + 1) + i];
         acc = warp_sum(acc);
         if (lane == 0) h[i] = acc;
     }
@@ -400,12 +400,8 @@ int sm_count()
     return n;
 }
 
-// One CTA per SM, or the column's share of them in a batch (two buffers of partial sums per CTA).
-int solve_ctas(const BcrPlan &p)
-{
-    const int all = std::min(sm_count(), kGmPartialBlocks / 2);
-    return p.solve_ctas > 0 ? std::min(p.solve_ctas, all) : all;
-}
+// One CTA per SM, or the column's share of them in a batch.
+int solve_ctas(const BcrPlan &p) { return p.solve_ctas > 0 ? std::min(p.solve_ctas, sm_count()) : sm_count(); }
 
 ApplyArgs apply_args(const BcrPlan &p) { return ApplyArgs{p.sol_d, p.mv_d, (int)p.sol.size(), p.L, p.S, p.Sp}; }
 

@@ -26,7 +26,7 @@ __device__ __forceinline__ double warp_sum(double v)
 
 // Deterministic multi-dot h[i] = <V_i, w>, i < nv (nv <= kMaxBasis), optionally
 // also ||w||^2 into h[nv].  Partial sums per block; the last block to finish
-// adds them in block order.
+// adds them in a fixed order.
 __global__ void k_dots(const double *V, int nv, const double *w, long long N, double *partials,
                        unsigned *counter, double *out, const GmState *gm, int with_norm)
 {
@@ -45,11 +45,13 @@ __global__ void k_dots(const double *V, int nv, const double *w, long long N, do
         if (with_norm) acc[kMaxBasis] += wn * wn;
     }
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // only the sums in use: an FP64 addition costs a warp tens of clocks on this part
 #pragma unroll
-    for (int i = 0; i <= kMaxBasis; ++i) {
-        double v = warp_sum(acc[i]);
-        if (lane == 0) sacc[warp][i] = v;
-    }
+    for (int i = 0; i <= kMaxBasis; ++i)
+        if (i < nv || (with_norm && i == kMaxBasis)) {
+            double v = warp_sum(acc[i]);
+            if (lane == 0) sacc[warp][i] = v;
+        }
     __syncthreads();
     if (threadIdx.x < nout) {
         int i = threadIdx.x < nv ? threadIdx.x : kMaxBasis;
@@ -63,10 +65,12 @@ __global__ void k_dots(const double *V, int nv, const double *w, long long N, do
     __syncthreads();
     if (last) {
         __threadfence();
-        if (threadIdx.x < nout) {
+        // a warp per sum, the blocks' parts strided over its lanes
+        for (int i = warp; i < nout; i += kRedThreads / 32) {
             double s = 0.0;
-            for (int b = 0; b < gridDim.x; ++b) s += partials[(long long)b * (kMaxBasis + 1) + threadIdx.x];
-            out[threadIdx.x] = s;
+            for (int b = lane; b < gridDim.x; b += 32) s += partials[(long long)b * (kMaxBasis + 1) + i];
+            s = warp_sum(s);
+            if (lane == 0) out[i] = s;
         }
         if (threadIdx.x == 0) *counter = 0u;
     }

@@ -29,10 +29,33 @@ struct Col {
     const int *rtype, *reac, *prod, *form, *prow;
     // species-major stoichiometry (residual gather): entries r * 16 + (nu + 8)
     const int *yp, *yent;
+    // the same lists for the species sums of one CTA: cut into sublists of at most kSubMax entries (a
+    // multiple in networks so large that the partial sums would not fit shared memory), one lane each,
+    // 32 of similar length to a group.  Group g's entries are ent[32 q + lane], q = sgp[g] .. sgp[g+1):
+    // (reaction << 1) | (1: reactant row), or -1; lane l of group g leaves its sum in part[spart[32 g + l]]
+    // (-1: none), species y's parts are ssp[y] .. ssp[y+1); nsg groups, nsub parts
+    const int *sgp, *sent, *spart, *ssp;
+    int nsg, nsub;
+    // the diagonal entries' terms in the same form, over d: (reaction * 6 + slot) << 1 | (1: +d)
+    const int *dgp, *dent, *dpart, *dsp;
+    int ndg;
+    // the six species of each reaction (three reactants, three products; S where there is none) as
+    // eight 16-bit values
+    const uint4 *rx;
     // Jacobian pattern by row and column: row i's distinct columns jcol[jp[i] .. jp[i+1]), the terms of
     // column entry q in jrs[jtp[q] .. jtp[q+1]) as (reaction * 8 + slot) << 1 | (1: +d, 0: -d); jdq[i]
     // the diagonal entry of row i (-1: none)
     const int *jp, *jcol, *jtp, *jrs, *jdq;
+    // the same pattern for the dense assembly, by species list: row i is a set of tiles of its
+    // occurrences in yent (light rows one tile of at most kJacOcc, heavy rows tiles of kJacHeavyOcc),
+    // tile t holding the occurrences jto[t] .. jto[t+1); its columns are the groups jtg[t] .. jtg[t+1),
+    // all distinct: column jgc[g], terms jterm[jge[g] .. jge[g+1]), each (occurrence in the tile * 6 +
+    // slot) << 1 | (1: +d, 0: -d).  Row i's tiles: jrt[i] .. jrt[i+1).  Work items of the assembly:
+    // item q is the rows jit[8 q .. 8 q + 8) (-1 padded), or, with jit[8 q + 1] == -2, the heavy row
+    // jit[8 q] alone; nji items
+    const int *jto, *jtg, *jgc, *jge, *jrt, *jit;
+    const unsigned short *jterm;
+    int nji;
     // photolysis
     const double *J0, *dlam, *sigma, *sig_abs;   // sig_abs: Sabs x W
     const int *abs_sp;
@@ -89,6 +112,9 @@ struct Ctl {
     long long fp64_steps;
     double dt_fp64;       // smallest dt at which the FP32-preconditioned solve did not converge
 };
+
+constexpr int kJacWarps = 8, kJacOcc = 128, kJacHeavyOcc = kJacWarps * kJacOcc;
+constexpr int kSubMax = 48;     // entries of a species list summed by one lane
 
 struct Policy {
     double dt_max, rel_reject, rel_target, grow_max, shrink_min, neg_tol, f_floor, dt_min, ss_dt, ss_tol;
@@ -239,6 +265,7 @@ struct ParcelArgs {
 // One global iteration on one CTA (photolysis and rate coefficients already in c).
 cudaError_t launch_parcel_iteration(const Col &c, const ParcelArgs &a, cudaStream_t st);
 
+constexpr unsigned long long kSyncPolls = 1ull << 22;   // polls of GridSync, without a sleep: a second or two
 constexpr unsigned long long kSpinLimit = 1ull << 24;   // polls of a bounded wait: ~1-2 s with the sleep below
 
 // Barrier over the nblk CTAs that share the counter pair bar[0..1] (the whole grid by default).
@@ -282,6 +309,52 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, Ctl *ctl, unsigned n
     return s_go != 0;
 }
 
+// Barrier over all CTAs of a cooperative launch: one counter that only grows during the launch
+// (target: what it reads when every CTA has arrived), one release-add and one polled acquire-load
+// per CTA.  words[0] is the counter and words[1] counts the CTAs that have left; the last one out
+// clears both, so the words are zero between launches.  The wait is bounded as in grid_barrier.
+struct GridSync {
+    unsigned *words;
+    Ctl *ctl;
+    unsigned target = 0;
+    __device__ GridSync(unsigned *w, Ctl *c) : words(w), ctl(c) {}
+    __device__ __forceinline__ bool sync()
+    {
+        __shared__ int s_ok;
+        target += gridDim.x;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int ok = 1;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(words) : "memory");
+            const unsigned long long limit = ctl->wait_polls ? ctl->wait_polls : kSyncPolls;
+            volatile int *vto = &ctl->err_timeout;
+            for (unsigned long long i = 0;; ++i) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(words) : "memory");
+                if ((int)(v - target) >= 0) break;
+                if (i > limit || ((i & 63) == 63 && *vto)) {
+                    atomicExch(&ctl->err_timeout, 1);
+                    ok = 0;
+                    break;
+                }
+            }
+            s_ok = ok;
+        }
+        __syncthreads();
+        return s_ok != 0;
+    }
+    // every CTA calls this once, after its last sync
+    __device__ __forceinline__ void leave()
+    {
+        __syncthreads();
+        if (threadIdx.x == 0 && atomicAdd(words + 1, 1u) == gridDim.x - 1) {
+            words[0] = 0u;
+            words[1] = 0u;
+            __threadfence();
+        }
+    }
+};
+
 // Launch helpers implemented in xk_chem.cu
 void launch_grid(const Col &c, cudaStream_t st);
 void launch_thermo(const Col &c, cudaStream_t st);
@@ -289,18 +362,17 @@ void launch_rates(const Col &c, cudaStream_t st);
 // u, v of Eq. 2 for the eddy profile Kzz (a zero profile leaves the molecular part only)
 void launch_transport_coeffs(const Col &c, const double *Kzz, double *u, double *v, cudaStream_t st);
 void launch_photolysis(const Col &c, const double *n, cudaStream_t st);
-void launch_reaction_terms(const Col &c, const double *n, cudaStream_t st);
-void launch_residual(const Col &c, const double *n, double *F, const Ctl *ctl, double f_floor, cudaStream_t st);
-void launch_jacobian64(const Col &c, const double *n, const Ctl *ctl, double dt_override, int scaled,
+// rates, derivatives, residual F, scaling and b = F / s; with diag also the row equilibration and
+// bhat = b / diag (reads ctl->dt)
+void launch_layer_terms(const Col &c, const double *n, double *F, const Ctl *ctl, double f_floor, double *diag,
+                        double *bhat, cudaStream_t st);
+void launch_jacobian64(const Col &c, const Ctl *ctl, double dt_override, int scaled,
                        double *A, double *lo, double *up, cudaStream_t st, const int *skip = nullptr);
 // lstride: elements between consecutive layers' blocks (0: S * ld)
-void launch_jacobian32(const Col &c, const double *n, const Ctl *ctl, float *A, float *lo, float *up, double *diag,
-                       cudaStream_t st, const int *skip = nullptr, long long lstride = 0);
+void launch_jacobian32(const Col &c, const Ctl *ctl, float *A, float *lo, float *up, cudaStream_t st, const int *skip = nullptr, long long lstride = 0);
 void launch_route(Ctl *ctl, cudaStream_t st);
 void launch_jv(const Col &c, const Ctl *ctl, const double *xs, double *ys, const double *rowdiv, const int *skip,
                cudaStream_t st);
-void launch_rowdiv(long long N, const double *x, const double *d, double *y, cudaStream_t st);
-void launch_diag(const Col &c, const Ctl *ctl, double *diag, cudaStream_t st);
 void launch_reuse_scales(long long N, const double *rowd, const double *s, const double *s64, double *pin, double *pout,
                          const Ctl *ctl, cudaStream_t st);
 void launch_after_refactor(long long N, const double *s, double *s64, Ctl *ctl, cudaStream_t st);

@@ -5,39 +5,38 @@
 
 namespace xk {
 
-// Species sums of one layer over its reactions: for every species, sum over its entries of
-// sign * val[reaction], reactant entries with sign rsign and product entries with -rsign.  A warp
-// takes a chunk (kSpChunk entries, two per lane, or a multiple in networks so large that the chunk
-// sums would not fit shared memory) at a time and leaves the chunk's sum in part[chunk]; chunks
-// bound the longest chain (the bath gas is in thousands of reactions, most
-// species in a few dozen).  The caller adds a species' chunks in order after a block barrier: every
-// sum has a fixed order.
-__device__ __forceinline__ void species_chunks(const Col &c, const double *val, double *part)
+// v or -v by flipping the sign bit: a negation on the FP64 unit would cost as much as an addition
+// (this part issues about two FP64 operations per clock and SM).
+__device__ __forceinline__ double signed_by(double v, bool plus)
+{
+    return __hiloint2double(__double2hiint(v) ^ (plus ? 0 : (int)0x80000000), __double2loint(v));
+}
+
+// Species sums of one layer over its reactions: for every species, the sum over its entries of
+// +val[reaction] for reactant entries and -val[reaction] for product entries.  Each lane sums one
+// sublist serially (Col::sgp): FP64 additions are what this costs, so there are as few as entries,
+// none for padding lanes of a warp-wide tree.  The caller adds a species' parts in order
+// (species_sum) after a block barrier: every sum has a fixed order.
+__device__ __forceinline__ void species_parts(const Col &c, const double *val, double *part)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int q = warp; q < c.nchk; q += nw) {
-        const int e0 = c.cks[q], e1 = c.cks[q + 1];
+    for (int g = warp; g < c.nsg; g += nw) {
         double acc = 0.0;
-        for (int ea = e0 + lane; ea < e1; ea += 64) {
-            const int eb = ea + 32;
-            const int ca = c.yent[ea], cb = eb < e1 ? c.yent[eb] : -1;
-            const double va = val[ca >> 4];
-            acc += ((ca & 15) < 8) ? va : -va;
-            if (cb >= 0) {
-                const double vb = val[cb >> 4];
-                acc += ((cb & 15) < 8) ? vb : -vb;
-            }
+        const int q1 = c.sgp[g + 1];
+#pragma unroll 4
+        for (int q = c.sgp[g]; q < q1; ++q) {
+            const int code = c.sent[32 * q + lane];
+            if (code >= 0) acc += signed_by(val[code >> 1], code & 1);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) part[q] = acc;
+        const int to = c.spart[32 * g + lane];
+        if (to >= 0) part[to] = acc;
     }
 }
 
 __device__ __forceinline__ double species_sum(const Col &c, const double *part, int i)
 {
     double acc = 0.0;
-    for (int q = c.ckp[i]; q < c.ckp[i + 1]; ++q) acc += part[q];
+    for (int q = c.ssp[i]; q < c.ssp[i + 1]; ++q) acc += part[q];
     return acc;
 }
 
@@ -48,11 +47,11 @@ __device__ __forceinline__ double photo_jv_term(const Col &c, int k, int r)
     return c.pdk[(long long)k * c.Rph + c.prow[r]] * c.n[(long long)k * c.S + c.reac[3 * r]];
 }
 
-// Doubles of shared memory that jv_layer_body needs: v = s x of the layer with a zero behind it,
-// the chunk sums, and the rates' changes where they fit (otherwise they go through c.dw).
+// Doubles of shared memory that jv_layer_body needs: v = s x of the layer,
+// the partial sums, and the rates' changes where they fit (otherwise they go through c.dw).
 __host__ __device__ inline size_t jv_smem_doubles(const Col &c, bool rates)
 {
-    return (size_t)c.S + 1 + (size_t)c.nchk + (rates ? (size_t)c.R : 0);
+    return (size_t)c.S + 1 + (size_t)c.nsub + (rates ? (size_t)c.R : 0);
 }
 
 // The rates' changes stay in shared memory up to this size of everything together (R about 20,000);
@@ -69,9 +68,9 @@ __device__ __forceinline__ void jv_layer_body(const Col &c, const Ctl *ctl, cons
                                               const double *rowdiv, int k, double *sm, bool rates_in_smem)
 {
     const int S = c.S, R = c.R, L = c.L;
-    double *sx = sm, *part = sx + S + 1, *dws = rates_in_smem ? part + c.nchk : c.dw + (long long)k * R;
+    double *sx = sm, *part = sx + S + 1, *dws = rates_in_smem ? part + c.nsub : c.dw + (long long)k * R;
     const long long row0 = (long long)k * S;
-    for (int i = threadIdx.x; i <= S; i += blockDim.x) sx[i] = i < S ? c.s[row0 + i] * x[row0 + i] : 0.0;
+    for (int i = threadIdx.x; i < S; i += blockDim.x) sx[i] = c.s[row0 + i] * x[row0 + i];
     __syncthreads();
     const double2 *dk = (const double2 *)(c.d + (long long)k * R * 6);
     // four reactions per thread at a time, all their loads before the first use
@@ -90,18 +89,21 @@ __device__ __forceinline__ void jv_layer_body(const Col &c, const Ctl *ctl, cons
         for (int u = 0; u < 4; ++u) {
             const int r = r0 + u * (int)blockDim.x;
             if (r >= R) break;
-            double acc = d01[u].x * sx[q[u].x & 0xffffu];
-            acc += d23[u].y * sx[q[u].y >> 16];
-            acc += d01[u].y * sx[q[u].x >> 16];
-            acc += d45[u].x * sx[q[u].z & 0xffffu];
-            acc += d23[u].x * sx[q[u].y & 0xffffu];
-            acc += d45[u].y * sx[q[u].z >> 16];
+            // reactions of a kind stand together, so the slots a kind does not use are skipped by whole warps
+            double acc = 0.0;
+            auto slot = [&](double d, unsigned j) { if (j != (unsigned)S) acc += d * sx[j]; };
+            slot(d01[u].x, q[u].x & 0xffffu);
+            slot(d23[u].y, q[u].y >> 16);
+            slot(d01[u].y, q[u].x >> 16);
+            slot(d45[u].x, q[u].z & 0xffffu);
+            slot(d23[u].x, q[u].y & 0xffffu);
+            slot(d45[u].y, q[u].z >> 16);
             if (c.photo_jac) acc += photo_jv_term(c, k, r);
             dws[r] = acc;
         }
     }
     __syncthreads();
-    species_chunks(c, dws, part);
+    species_parts(c, dws, part);
     __syncthreads();
     const double rdt = 1.0 / ctl->dt;
     for (int i = threadIdx.x; i < S; i += blockDim.x) {
