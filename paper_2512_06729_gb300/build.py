@@ -18,7 +18,9 @@ LIB = os.path.join(BUILD, "libxk.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", "-Xptxas", "-warn-spills"]
-SOURCES = ["xk_api.cu", "xk_chem.cu", "xk_factor.cu", "xk_gmres.cu", "xk_noalloc.cu", "xk_cluster.cu", "xk_tc.cu", "xk_bcr.cu", "xk_fgmres.cu", "xk_parcel.cu", "xk_analysis.cu", "xk_bdf.cu"]
+SOURCES = ["xk_api.cu", "xk_chem.cu", "xk_factor.cu", "xk_factor64.cu", "xk_gmres.cu", "xk_cond.cu", "xk_noalloc.cu", "xk_cluster.cu", "xk_tc.cu", "xk_bcr.cu", "xk_fgmres.cu", "xk_parcel.cu", "xk_analysis.cu", "xk_bdf.cu"]
+
+RELOCATABLE = ["xk_cond.cu"]     # calls into the CUDA device runtime
 
 
 def nvcc():
@@ -43,7 +45,8 @@ def build(force=False, verbose=False, extra=()):
 
     def compile_one(src):
         obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = [exe, *ARCH, *FLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+        rdc = ["-rdc=true"] if src in RELOCATABLE else []
+        cmd = [exe, *ARCH, *FLAGS, *rdc, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
         p = subprocess.run(cmd, capture_output=True, text=True)
         if p.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{p.stdout}\n{p.stderr}")
@@ -54,7 +57,7 @@ def build(force=False, verbose=False, extra=()):
     with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
         objs = list(ex.map(compile_one, SOURCES))
     tmp = LIB + f".tmp{os.getpid()}"
-    cmd = [exe, *ARCH, "-shared", "-Xcompiler", "-fPIC", "-o", tmp, *objs]
+    cmd = [exe, *ARCH, "-shared", "-Xcompiler", "-fPIC", "-o", tmp, *objs, "-lcudadevrt"]
     p = subprocess.run(cmd, capture_output=True, text=True)
     if p.returncode != 0:
         raise RuntimeError(f"link failed:\n{p.stdout}\n{p.stderr}")

@@ -40,6 +40,7 @@ struct xk_ctx {
     int diffuse = 0;
     bool have_net = false, have_photo = false, have_atm = false;
     bool rates_valid = false;      // k_f, k_r of the loaded network and atmosphere are in the workspace
+    bool indices_valid = false;    // the index structures below belong to the loaded inputs
     // host index structures
     std::vector<int> sgp, sent, spart, ssp, dgp, dent, dpart, dsp, jto, jtg, jgc, jge, jrt, jit;
     std::vector<unsigned short> jterm;
@@ -100,6 +101,9 @@ struct xk_ctx {
     // captured chunks of controlled steps (cfg.use_graphs), dropped whenever a plan, the workspace
     // or the batch slot changes
     std::vector<StepGraph> graphs;
+    CondStreams cond;                // capture streams of the steps' conditional parts
+    bool follow = false;             // a call that waits anyway: the host reads the device's routing flags
+    int *word_host = nullptr;        // pinned
     cudaStream_t cap_st = nullptr;   // capture stream (the legacy default stream cannot be captured)
     // tracing
     bool prof = false;
@@ -217,9 +221,11 @@ int build_sublists(const std::vector<std::vector<int>> &lists, std::vector<int> 
     return (int)subs.size();
 }
 
-// Index structures built once per network (symbolic, no arithmetic of the method).
+// Index structures built once per network and photolysis inputs (symbolic, no arithmetic of the method).
 void build_indices(xk_ctx *c)
 {
+    if (c->indices_valid) return;
+    c->indices_valid = true;
     const int S = c->S, R = c->R;
     // species-major stoichiometry, in reaction order: for r, for slot s: reactant, then product
     std::vector<std::vector<int>> ys(S);
@@ -561,6 +567,7 @@ size_t layout(xk_ctx *c, char *base)
         q.tw = b.take<float>(z.floats_vec);
         q.xw = b.take<float>(z.floats_vec);
         q.gemm_d = b.take<TcTask>(std::max(z.ngemm, 1));
+        q.tile_task_d = b.take<int>(std::max(z.ntile, 1));
         q.leaf_d = b.take<BcrLeaf>(std::max(z.nleaf, 1));
         q.mv_d = b.take<BcrMv>(std::max(z.nmv, 1));
         q.maps_d = b.take<CUtensorMap>(10);
@@ -745,7 +752,7 @@ int need_ready(xk_ctx *c)
 // FGMRES in FP64 on the exact operator, preconditioned by a fresh FP64 factorization (the plain FP64
 // path, and the mixed path's FP64 route): the right-hand side and residuals are row-equilibrated by
 // c->rowd, which the preconditioner undoes before applying the stored inverses.
-void enqueue_refine64(xk_ctx *c, const Col &col, Ctl *ctl, const FactorPlan &plan, const int *skip, int max_iter)
+cudaError_t enqueue_refine64(xk_ctx *c, const Col &col, Ctl *ctl, const FactorPlan &plan, const int *skip, int max_iter)
 {
     GmArgs a;
     a.N = (long long)c->L * c->S;
@@ -757,6 +764,8 @@ void enqueue_refine64(xk_ctx *c, const Col &col, Ctl *ctl, const FactorPlan &pla
     a.skip_solve = skip;
     a.role = 2;
     a.reuse_max_iters = 0;
+    a.cond = &c->cond;
+    a.host = c->follow ? c->word_host : nullptr;
     const double *rowd = c->rowd;
     a.matvec = [col, ctl, rowd](const double *x, double *y, const int *sk, cudaStream_t s) {
         launch_jv(col, ctl, x, y, rowd, sk, s);
@@ -764,7 +773,7 @@ void enqueue_refine64(xk_ctx *c, const Col &col, Ctl *ctl, const FactorPlan &pla
     a.precond = [c, plan, ctl, rowd](const double *v, double *z, const int *sk, cudaStream_t s) {
         solve64(c, plan, v, z, ctl, s, rowd, sk, nullptr);
     };
-    enqueue_fgmres(a, c->st);
+    return enqueue_fgmres(a, c->st);
 }
 
 // Enqueue thermochemistry, rates, photolysis, residual, Jacobian and the linear solve for state col.n (or n_override),
@@ -799,7 +808,7 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
         if (e != cudaSuccess) return fail(c, XK_ECUDA, "factor launch: %s", cudaGetErrorString(e));
         PhaseMark m(c, XK_PH_SOLVE);
         if (refine > 0)
-            enqueue_refine64(c, col, ctl, c->plan, nullptr, refine);
+            e = enqueue_refine64(c, col, ctl, c->plan, nullptr, refine);
         else
             e = solve64(c, c->plan, col.b, col.x, ctl, st, nullptr, nullptr, nullptr);
         if (e != cudaSuccess) return fail(c, XK_ECUDA, "solve launch: %s", cudaGetErrorString(e));
@@ -825,6 +834,8 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
         a.b = c->bhat; a.x = col.x; a.V = c->V; a.Z = c->Z; a.w = c->gw; a.h1 = c->h1; a.h2 = c->h2;
         a.red = c->red; a.partials = c->partials; a.counter = c->counter; a.gm = c->gm; a.ctl = ctl;
         a.reuse_max_iters = c->cfg.reuse_max_iters > 0 ? c->cfg.reuse_max_iters : 40;
+        a.cond = &c->cond;
+        a.host = c->follow ? c->word_host : nullptr;
         FactorPlan plan64 = c->plan64;
         const double *rowd = c->rowd, *pin = c->pin, *pout = c->pout;
         a.matvec = [col, ctl, rowd](const double *x, double *y, const int *skip, cudaStream_t s) {
@@ -842,7 +853,8 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
             if (e != cudaSuccess) return fail(c, XK_ECUDA, "solve launch: %s", cudaGetErrorString(e));
         } else {
             PhaseMark m(c, XK_PH_SOLVE);
-            enqueue_fgmres(a, st);
+            e = enqueue_fgmres(a, st);
+            if (e != cudaSuccess) return fail(c, XK_ECUDA, "solve enqueue: %s", cudaGetErrorString(e));
         }
         // FGMRES around the last FP64 factorization, rescaled to this step's variables
         if (c->cfg.reuse_factorization) {
@@ -852,24 +864,37 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
             a.precond = [c, plan64, ctl, pin, pout](const double *v, double *z, const int *skip, cudaStream_t s) {
                 solve64(c, plan64, v, z, ctl, s, pin, skip, pout);
             };
-            { PhaseMark m(c, XK_PH_SOLVE); enqueue_fgmres(a, st); }
+            PhaseMark m(c, XK_PH_SOLVE);
+            e = enqueue_fgmres(a, st);
+            if (e != cudaSuccess) return fail(c, XK_ECUDA, "solve enqueue: %s", cudaGetErrorString(e));
         }
         // FP64 factorization, then FGMRES refinement around it (or a direct solve), gated on the
         // device by ctl->skip64
         const int *skip64 = &ctl->skip64;
-        {
+        auto route64 = [&](cudaStream_t inner) {
             PhaseMark m(c, XK_PH_FALLBACK);
-            launch_jacobian64(col, ctl, 0.0, 1, c->A64, c->lo64, c->up64, st, skip64);
-            e = launch_factor<double>(sys64(c), c->plan64, ctl, st, skip64);
+            cudaStream_t own = c->st;
+            c->st = inner;
+            launch_jacobian64(col, ctl, 0.0, 1, c->A64, c->lo64, c->up64, inner, skip64);
+            e = launch_factor<double>(sys64(c), c->plan64, ctl, inner, skip64);
             if (e == cudaSuccess) {
-                launch_after_refactor(N, col.s, c->s64, ctl, st);
+                launch_after_refactor(N, col.s, c->s64, ctl, inner);
                 if (refine > 0)
-                    enqueue_refine64(c, col, ctl, c->plan64, skip64, refine);
+                    e = enqueue_refine64(c, col, ctl, c->plan64, skip64, refine);
                 else
-                    e = solve64(c, c->plan64, col.b, col.x, ctl, st, nullptr, skip64, nullptr);
+                    e = solve64(c, c->plan64, col.b, col.x, ctl, inner, nullptr, skip64, nullptr);
             }
+            c->st = own;
+        };
+        if (c->follow) {
+            e = cudaMemcpyAsync(c->word_host, skip64, sizeof(int), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e == cudaSuccess && *c->word_host == 0) route64(st);
+        } else {
+            cudaError_t ce = enqueue_if(st, &c->cond, skip64, 0, route64);
+            if (e == cudaSuccess) e = ce;
         }
-        if (e != cudaSuccess) return fail(c, XK_ECUDA, "FP64 fallback launch: %s", cudaGetErrorString(e));
+        if (e != cudaSuccess) return fail(c, XK_ECUDA, "FP64 route: %s", cudaGetErrorString(e));
     }
     launch_unscale(col, col.x, delta_out, st);
     return cuda_check(c, "step enqueue");
@@ -1058,9 +1083,11 @@ int xk_create(xk_ctx **out, const xk_config *cfg)
     x->st = (cudaStream_t)c.stream;
     cudaSetDevice(c.device);
     if (cudaMallocHost((void **)&x->ctl_host, sizeof(Ctl)) != cudaSuccess ||
-        cudaMallocHost((void **)&x->parcel_host, sizeof(ParcelState)) != cudaSuccess) {
+        cudaMallocHost((void **)&x->parcel_host, sizeof(ParcelState)) != cudaSuccess ||
+        cudaMallocHost((void **)&x->word_host, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         if (x->ctl_host) cudaFreeHost(x->ctl_host);
+        if (x->parcel_host) cudaFreeHost(x->parcel_host);
         delete x;
         return XK_ECUDA;
     }
@@ -1077,6 +1104,9 @@ int xk_destroy(xk_ctx *ctx)
         for (auto &pr : v) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
     if (ctx->ctl_host) cudaFreeHost(ctx->ctl_host);
     if (ctx->parcel_host) cudaFreeHost(ctx->parcel_host);
+    if (ctx->word_host) cudaFreeHost(ctx->word_host);
+    for (cudaStream_t in : ctx->cond.inner)
+        if (in) cudaStreamDestroy(in);
     delete ctx;
     return XK_OK;
 }
@@ -1118,6 +1148,7 @@ int xk_load_network(xk_ctx *c, int S, int E, int R, const int *elem, const doubl
     c->form.assign(form, form + R);
     c->nasa.assign(nasa, nasa + 15 * (size_t)S);
     c->have_net = true;
+    c->indices_valid = false;
     c->rates_valid = false;
     c->have_photo = false;
     c->ready = false;
@@ -1154,6 +1185,7 @@ int xk_load_photo(xk_ctx *c, int W, int Rph, const int *prow, const double *lamb
     c->sigma_abs.assign(sigma_abs, sigma_abs + (size_t)c->S * W);
     c->mu = mu; c->tf = tf;
     c->have_photo = true;
+    c->indices_valid = false;
     c->ready = false;
     (void)nph;
     return XK_OK;
@@ -1176,6 +1208,7 @@ int xk_load_scattering(xk_ctx *c, int W, const double *sigma_s, double albedo, i
     }
     c->albedo = albedo;
     c->diffuse = diffuse;
+    c->indices_valid = false;
     c->ready = false;
     return XK_OK;
 }
@@ -1587,7 +1620,10 @@ int xk_step_delta(xk_ctx *c, const double *n, double dt, double *delta, int *ite
     *c->ctl_host = init;
     cudaMemcpyAsync(c->ctl_aux, c->ctl_host, sizeof(Ctl), cudaMemcpyHostToDevice, c->st);
     double dto = c->cfg.precision == XK_PREC_FP64 ? dt : 0.0;
-    if ((rc = enqueue_linear_step(c, n, dto, delta, c->ctl_aux))) return rc;
+    c->follow = !c->prof && !capturing(c->st);
+    rc = enqueue_linear_step(c, n, dto, delta, c->ctl_aux);
+    c->follow = false;
+    if (rc) return rc;
     cudaMemcpyAsync(c->ctl_host, c->ctl_aux, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st);
     if ((rc = finish_eval(c, "step_delta"))) return rc;
     if (iters) *iters = c->ctl_host->used_fp64 ? -1 : c->ctl_host->solver_iters;

@@ -23,8 +23,9 @@
 // in the padding, so that every product has dimensions that are multiples of 32.
 #include <cuda_runtime.h>
 
+#include <stdint.h>
+
 #include <algorithm>
-#include <type_traits>
 
 #include "xk_bcr.cuh"
 
@@ -49,238 +50,273 @@ int split_of(int n) { return 32 * ((n + 63) / 64); }
 // largest |value|, and the in-place elimination leaves row p(k) holding row k
 // of (P M)^-1, so M^-1[k][p(c)] = W[p(k)][c].
 //
-// Warp 0 factors the panels: lane l holds rows l + 32 a of the panel's 8
-// columns in registers, a column costs one warp reduction (the pivot), one
-// shared-memory broadcast (the pivot row) and 8 RG FMAs, and no block barrier.
-// Its result G (N x 8) turns the other columns by one rank-8 update,
+// Warps 0 .. RG-1 factor the panels, a row per lane with its 8 entries in
+// registers.  A column costs a warp reduction (the warp's best row), a barrier
+// among these warps (each leaves its best row, already scaled, in shared
+// memory) and 8 FMAs.  The result G (N x 8) turns the other columns by one
+// rank-8 update,
 //   W[r][j] <- W[r][j] + sum_l G[r][l] U[l][j],   U the panel's pivot rows,
-// (the pivot rows themselves without their old value), which the other 15
-// warps apply one panel behind: warp w owns whole columns, NC of them, so the
-// pivot rows it needs are its own, and the only block barrier is one per
-// panel.  Warp 0 applies the previous panel's update to its next panel itself.
+// (the pivot rows themselves without their old value), which the other warps
+// apply one panel behind, in registers: a warp owns quads of columns (all of
+// their rows) and writes them to the block's image in shared memory after each
+// update, where it then reads the next panel's pivot rows; a quad belongs to one
+// panel, and the only block barrier is one per panel.  The panel warps apply the
+// previous panel's update to their next panel themselves.  Panels travel through
+// the block's image in shared memory (row stride N + 4: rows are read 16 bytes a
+// lane without conflicts), G also with every value twice, as the packed FMAs
+// (two columns to an instruction) want it.
 //
-// What bounds it: the 8 N-long chains of dependent columns on warp 0 and the
-// 2 N^3 flop of one SM's FP32 pipe are about equal at N = 160 (a panel is 2,000
-// to 2,500 clocks on either side), which is why the panel is 8 wide: 16 makes
-// the chain longer than the updates, 4 doubles the updates' loads.
+// What bounds it: the chain of N dependent columns, then the issue slots of the
+// updates (2 N^3 flop on one SM's FP32 pipe).  The loop over a panel's columns is
+// rolled and no branch depends on where the pivot is: with a jump per pivot row
+// a column took 720 clocks, 300 of them there, and with all of the panel's rows
+// on one warp 400, most of them selects.  The panel is 8 wide because 16 doubles
+// the panel warps' work per column and 4 doubles the updates' loads and stores.
 // ---------------------------------------------------------------------------
 constexpr int kLeafPanel = 8;
-constexpr int kLeafTrail = 15;                                // warps of the trailing update
-constexpr int kLeafThreads = 32 * (kLeafTrail + 1);
-constexpr int leaf_cols(int N) { return (N + kLeafTrail - 1) / kLeafTrail; }
-constexpr int leaf_ucols(int N) { return (leaf_cols(N) + 3) / 4 * 4; }
-// the block (odd row stride), G and the raw panels (two buffers each), U per warp, the pivot rows
-// of warp 0's panel, two pivot-row broadcasts
-constexpr size_t leaf_smem(int N)
+constexpr int kLeafThreads = 512;
+constexpr int leaf_trail(int RG) { return kLeafThreads / 32 - RG; }                 // warps of the trailing update
+constexpr int leaf_quads(int RG) { return (8 * RG + leaf_trail(RG) - 1) / leaf_trail(RG); }   // of one warp, at most
+constexpr int kLeafGd = 20;                                  // row stride of the doubled G
+// the block (row stride N + 4) with room for the quads past its end, two panels' doubled G
+constexpr size_t leaf_smem(int RG)
 {
-    return sizeof(float) * ((size_t)N * (N + 1) + 4 * kLeafPanel * N + (size_t)kLeafTrail * kLeafPanel * leaf_ucols(N) +
-                            kLeafPanel * kLeafPanel + 2 * kLeafPanel);
+    return sizeof(float) * ((size_t)32 * RG * (32 * RG + 4) + 2 * 32 * RG * kLeafGd);
 }
 
-// Calls f(A) with the constant A equal to pa (< RG), so that arrays indexed by A stay in registers.
-template <int RG, typename F>
-__device__ __forceinline__ void leaf_with_group(int pa, F f)
+// A predicated store: which of a lane's rows is the pivot is known at run time only, and a branch
+// per candidate (or a jump table) costs a few hundred clocks each time.
+__device__ __forceinline__ void store4_if(bool p, float *dst, float4 v)
 {
-    switch (pa) {
-    case 0: f(std::integral_constant<int, 0>()); break;
-    case 1: if constexpr (RG > 1) f(std::integral_constant<int, 1>()); break;
-    case 2: if constexpr (RG > 2) f(std::integral_constant<int, 2>()); break;
-    case 3: if constexpr (RG > 3) f(std::integral_constant<int, 3>()); break;
-    default: if constexpr (RG > 4) f(std::integral_constant<int, 4>()); break;
-    }
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t}"
+                 ::"r"((int)p), "r"((uint32_t)__cvta_generic_to_shared(dst)), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
 }
 
-// Store the 8 values of one row (row group pa of this lane) and clear it.
-template <int RG>
-__device__ __forceinline__ void leaf_take_row(float (&x)[RG][kLeafPanel], int pa, float *dst)
+// Two FMAs (products) in one instruction, on both halves.
+__device__ __forceinline__ void fma2(float2 &d, float2 a, float2 b)
 {
-    leaf_with_group<RG>(pa, [&](auto A) {
-        constexpr int a = decltype(A)::value;
-        *(float4 *)dst = make_float4(x[a][0], x[a][1], x[a][2], x[a][3]);
-        *(float4 *)(dst + 4) = make_float4(x[a][4], x[a][5], x[a][6], x[a][7]);
-#pragma unroll
-        for (int j = 0; j < kLeafPanel; ++j) x[a][j] = 0.0f;
-    });
+    unsigned long long &dd = reinterpret_cast<unsigned long long &>(d);
+    asm("fma.rn.f32x2 %0, %1, %2, %0;"
+        : "+l"(dd)
+        : "l"(reinterpret_cast<unsigned long long &>(a)), "l"(reinterpret_cast<unsigned long long &>(b)));
 }
+__device__ __forceinline__ void mul2(float2 &d, float2 a)
+{
+    unsigned long long &dd = reinterpret_cast<unsigned long long &>(d);
+    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(dd) : "l"(reinterpret_cast<unsigned long long &>(a)));
+}
+
+// 1 / x to an FP32 unit: the hardware's approximation and one Newton-Raphson step.  The division's
+// sequence is on the chain of every column (68 us against 63 for a block of 160).
+__device__ __forceinline__ float reciprocal(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    const float z = fmaf(y, fmaf(-x, y, 1.0f), y);
+    return fabsf(z) <= 3.402823466e38f ? z : 1.0f / x;      // subnormal or huge x
+}
+
+struct __align__(16) LeafCand {
+    float row[kLeafPanel];        // 1 / pivot, then the rest of the row times it
+};
 
 template <int RG>
 __global__ void __launch_bounds__(kLeafThreads, 1) k_leaf_inverse(const BcrLeaf *tasks, const int *skip, const Ctl *ctl)
 {
-    constexpr int N = 32 * RG, NP = kLeafPanel, NPAN = N / NP, NC = leaf_cols(N), UC = leaf_ucols(N), LD = N + 1;
-    if (stop(skip, ctl)) return;
-    const BcrLeaf t = tasks[blockIdx.x];
+    constexpr int N = 32 * RG, NP = kLeafPanel, NPAN = N / NP, LD = N + 4, TW = leaf_trail(RG), NQ = leaf_quads(RG);
     extern __shared__ __align__(16) float sm[];
     float *tile = sm;                          // [N][LD]
-    float *G = tile + N * LD;                  // [2][NP][N]
-    float *raw = G + 2 * NP * N;               // [2][NP][N]: panel columns as the trailing warps left them
-    float *U = raw + 2 * NP * N;               // [kLeafTrail][NP][UC]
-    float *pu = U + kLeafTrail * NP * UC;      // [NP][NP]: the previous panel's pivot rows in this panel
-    float *rowb = pu + NP * NP;                // [2][NP]
+    float *Gd = tile + N * LD;                 // [2][N][kLeafGd]
+    __shared__ LeafCand cand[2][RG];
+    __shared__ __align__(16) unsigned keys[2][8];
     __shared__ int piv[2][NP], perm[N];
     const int ln = threadIdx.x & 31, wv = threadIdx.x >> 5;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const BcrLeaf t = tasks[blockIdx.x];
+    if (threadIdx.x < 16) keys[threadIdx.x >> 3][threadIdx.x & 7] = 0u;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (stop(skip, ctl)) return;
 #pragma unroll 10
     for (int e = threadIdx.x; e < N * N; e += kLeafThreads) {
         const int r = e / N, j = e - r * N;
         tile[r * LD + j] = t.in[(long long)r * t.ldin + j];
     }
     __syncthreads();
-    if (wv == 0) {
-        float g[RG][NP];                       // G of the previous panel, rows ln + 32 a
-        unsigned used = 0;
-        for (int p = 0; p <= NPAN; ++p) {
-            if (p < NPAN) {
-                float x[RG][NP];
-                if (p < 2) {
-#pragma unroll
-                    for (int a = 0; a < RG; ++a)
-#pragma unroll
-                        for (int j = 0; j < NP; ++j) x[a][j] = tile[(ln + 32 * a) * LD + p * NP + j];
-                } else {
-                    const float *src = raw + (p & 1) * NP * N + ln;
-#pragma unroll
-                    for (int a = 0; a < RG; ++a)
-#pragma unroll
-                        for (int j = 0; j < NP; ++j) x[a][j] = src[j * N + 32 * a];
-                }
+    if (wv < RG) {
+        const int me = 32 * wv + ln;                       // this lane's row
+        unsigned live = 0x7fffff00u, code = 255u - me;     // of the pivot search: zero once the row has been a pivot
+        bool last = false;                                 // a pivot of the previous panel
+        float2 g[NP];                                      // the row of the previous panel's G, doubled
+        for (int p = 0; p < NPAN; ++p) {
+            float *at = tile + me * LD + p * NP;
+            float x[NP];
+            {
+                const float4 v0 = *(const float4 *)at, v1 = *(const float4 *)(at + 4);
+                float2 xx[4] = {{v0.x, v0.y}, {v0.z, v0.w}, {v1.x, v1.y}, {v1.z, v1.w}};
                 if (p > 0) {
+                    if (last) xx[0] = xx[1] = xx[2] = xx[3] = float2{0.f, 0.f};
                     const int *pp = piv[(p - 1) & 1];
 #pragma unroll
                     for (int l = 0; l < NP; ++l) {
-                        const int row = pp[l];
-                        if (ln == (row & 31)) leaf_take_row<RG>(x, row >> 5, pu + l * NP);
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int l = 0; l < NP; ++l) {
-                        const float4 u0 = *(const float4 *)(pu + l * NP), u1 = *(const float4 *)(pu + l * NP + 4);
-                        const float u[NP] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-#pragma unroll
-                        for (int j = 0; j < NP; ++j)
-#pragma unroll
-                            for (int a = 0; a < RG; ++a) x[a][j] = fmaf(g[a][l], u[j], x[a][j]);
+                        const float *ur = tile + pp[l] * LD + p * NP;
+                        const float4 u0 = *(const float4 *)ur, u1 = *(const float4 *)(ur + 4);
+                        fma2(xx[0], g[l], float2{u0.x, u0.y});
+                        fma2(xx[1], g[l], float2{u0.z, u0.w});
+                        fma2(xx[2], g[l], float2{u1.x, u1.y});
+                        fma2(xx[3], g[l], float2{u1.z, u1.w});
                     }
                 }
 #pragma unroll
-                for (int c = 0; c < NP; ++c) {
-                    // pivot: the unused row of largest |value| (its float bits without the low eight, which
-                    // hold the row so that one reduction finds both; the lowest row among near-equals)
-                    unsigned key = 0u;
-#pragma unroll
-                    for (int a = 0; a < RG; ++a) {
-                        const unsigned m = __float_as_uint(x[a][c]) & 0x7fffffffu;
-                        const unsigned k = ((m > 0x7f800000u ? 0u : m) & 0xffffff00u) | (unsigned)(255 - (ln + 32 * a));
-                        if (!((used >> a) & 1u)) key = max(key, k);
-                    }
-                    key = __reduce_max_sync(0xffffffffu, key);
-                    const int row = 255 - (int)(key & 0xffu);
-                    const bool mine = ln == (row & 31);
-                    float *rb = rowb + (c & 1) * NP;
-                    if (mine) {
-                        used |= 1u << (row >> 5);
-                        leaf_take_row<RG>(x, row >> 5, rb);
-                    }
-                    __syncwarp();
-                    const float4 r0 = *(const float4 *)rb, r1 = *(const float4 *)(rb + 4);
-                    float pr[NP] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-                    // singular block: the FP64 Krylov solve sees a poor preconditioner
-                    const float inv = 1.0f / (pr[c] == 0.0f ? 1e-30f : pr[c]);
-#pragma unroll
-                    for (int j = 0; j < NP; ++j) pr[j] = j == c ? inv : pr[j] * inv;
-                    // the pivot row is now zero: a multiplier of -1 leaves it as the scaled row, exactly
-#pragma unroll
-                    for (int a = 0; a < RG; ++a) {
-                        const float f = mine && a == (row >> 5) ? -1.0f : x[a][c];
-#pragma unroll
-                        for (int q = 1; q < NP; ++q) {
-                            const int j = (c + q) % NP;
-                            x[a][j] = fmaf(-f, pr[j], x[a][j]);
-                        }
-                        x[a][c] = -f * inv;
-                    }
-                    if (ln == 0) {
-                        piv[p & 1][c] = row;
-                        perm[p * NP + c] = row;
-                    }
+                for (int j = 0; j < 4; ++j) {
+                    x[2 * j] = xx[j].x;
+                    x[2 * j + 1] = xx[j].y;
                 }
-                float *dst = G + (p & 1) * NP * N + ln;
-#pragma unroll
-                for (int a = 0; a < RG; ++a)
-#pragma unroll
-                    for (int j = 0; j < NP; ++j) {
-                        dst[j * N + 32 * a] = x[a][j];
-                        g[a][j] = x[a][j];
-                    }
             }
+            last = false;
+            // column c is always x[0]: each step shifts the others down one and puts the finished column
+            // last, so that after eight steps they are in their places again
+#pragma unroll 1
+            for (int c = 0; c < NP; ++c) {
+                // pivot: the unused row of largest |value| (its float bits without the low eight, which
+                // hold the row so that one reduction finds both; the lowest row among near-equals)
+                const unsigned k = (__float_as_uint(x[0]) & live) | code;
+                unsigned top = __reduce_max_sync(0xffffffffu, k);
+                // meanwhile this lane's own row, scaled (a singular block: the FP64 Krylov solve sees a
+                // poor preconditioner)
+                float s[NP];
+                s[0] = reciprocal(x[0] == 0.0f ? 1e-30f : x[0]);
+#pragma unroll
+                for (int j = 1; j < NP; ++j) s[j] = x[j] * s[0];
+                LeafCand *cb = cand[c & 1];
+                const bool best = k == top;
+                store4_if(best, cb[wv].row, make_float4(s[0], s[1], s[2], s[3]));
+                store4_if(best, cb[wv].row + 4, make_float4(s[4], s[5], s[6], s[7]));
+                if (RG > 1) {
+                    if (ln == 0) keys[c & 1][wv] = top;
+                    asm volatile("bar.sync 1, %0;" ::"n"(32 * RG) : "memory");
+                    const uint4 k0 = *(const uint4 *)keys[c & 1];
+                    top = max(max(k0.x, k0.y), max(k0.z, k0.w));
+                    if (RG > 4) top = max(top, keys[c & 1][4]);
+                } else {
+                    __syncwarp();
+                }
+                const int row = 255 - (int)(top & 0xffu);
+                const float4 r0 = *(const float4 *)cb[row >> 5].row, r1 = *(const float4 *)(cb[row >> 5].row + 4);
+                const float pr[NP] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+                const bool is = k == top;                  // the pivot row becomes the scaled row
+                const float f = x[0];
+#pragma unroll
+                for (int j = 1; j < NP; ++j) {
+                    const float v = fmaf(-f, pr[j], x[j]);
+                    x[j - 1] = is ? s[j] : v;
+                }
+                x[NP - 1] = is ? s[0] : -f * pr[0];
+                if (is) {
+                    live = code = 0u;
+                    last = true;
+                    piv[p & 1][c] = row;
+                    perm[p * NP + c] = row;
+                }
+            }
+            *(float4 *)at = make_float4(x[0], x[1], x[2], x[3]);
+            *(float4 *)(at + 4) = make_float4(x[4], x[5], x[6], x[7]);
+            float *gd = Gd + ((p & 1) * N + me) * kLeafGd;
+#pragma unroll
+            for (int j = 0; j < NP; j += 2) *(float4 *)(gd + 2 * j) = make_float4(x[j], x[j], x[j + 1], x[j + 1]);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) g[j] = float2{x[j], x[j]};
             __syncthreads();
         }
+        __syncthreads();
     } else {
-        const int tw = wv - 1, j0 = tw * NC;
-        float w[NC][RG];                       // w[b][a] = W[ln + 32 a][j0 + b]
+        const int tw = wv - RG;
+        float2 w[NQ][RG][2];                   // this warp's quads tw + TW i: rows ln + 32 a
 #pragma unroll
-        for (int b = 0; b < NC; ++b)
+        for (int i = 0; i < NQ; ++i) {
+            const int q = tw + TW * i;
 #pragma unroll
-            for (int a = 0; a < RG; ++a) w[b][a] = j0 + b < N ? tile[(ln + 32 * a) * LD + j0 + b] : 0.0f;
-        float *uw = U + tw * NP * UC;
-        for (int p = 0; p <= NPAN; ++p) {
-            if (p > 0) {
-                const float *gq = G + ((p - 1) & 1) * NP * N + ln;
-                const int *pp = piv[(p - 1) & 1];
-                // the pivot rows of panel p - 1 in this warp's columns; they start from zero in the update
+            for (int a = 0; a < RG; ++a) {
+                const float4 v = q < N / 4 ? *(const float4 *)(tile + (ln + 32 * a) * LD + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+                w[i][a][0] = float2{v.x, v.y};
+                w[i][a][1] = float2{v.z, v.w};
+            }
+        }
+        __syncthreads();
+        for (int p = 1; p <= NPAN; ++p) {      // panel p - 1 is done; the panel warps are at panel p
+            const int *pp = piv[(p - 1) & 1];
+            unsigned mine = 0;                 // bit a: row ln + 32 a is a pivot row of the panel
 #pragma unroll
-                for (int l = 0; l < NP; ++l) {
-                    const int row = pp[l];
-                    if (ln == (row & 31)) {
-                        leaf_with_group<RG>(row >> 5, [&](auto A) {
-                            constexpr int a = decltype(A)::value;
+            for (int l = 0; l < NP; ++l) mine |= ln == (pp[l] & 31) ? 1u << (pp[l] >> 5) : 0u;
+            // the pivot rows start from zero in the update
 #pragma unroll
-                            for (int b = 0; b < NC; ++b) {
-                                uw[l * UC + b] = w[b][a];
-                                w[b][a] = 0.0f;
-                            }
-                        });
+            for (int a = 0; a < RG; ++a) {
+                const float z = (mine >> a) & 1u ? 0.0f : 1.0f;
+#pragma unroll
+                for (int i = 0; i < NQ; ++i) {
+                    mul2(w[i][a][0], float2{z, z});
+                    mul2(w[i][a][1], float2{z, z});
+                }
+            }
+            const float *gp = Gd + (((p - 1) & 1) * N + ln) * kLeafGd;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {      // two of the panel's columns at a time
+                float4 g4[RG];
+#pragma unroll
+                for (int a = 0; a < RG; ++a) g4[a] = *(const float4 *)(gp + 32 * a * kLeafGd + 4 * h);
+#pragma unroll
+                for (int l = 0; l < 2; ++l) {
+                    const float *ur = tile + pp[2 * h + l] * LD + 4 * tw;      // the pivot row as it was
+#pragma unroll
+                    for (int i = 0; i < NQ; ++i) {
+                        const float4 u = *(const float4 *)(ur + 4 * TW * i);
+#pragma unroll
+                        for (int a = 0; a < RG; ++a) {
+                            const float2 gl = l == 0 ? float2{g4[a].x, g4[a].y} : float2{g4[a].z, g4[a].w};
+                            fma2(w[i][a][0], gl, float2{u.x, u.y});
+                            fma2(w[i][a][1], gl, float2{u.z, u.w});
+                        }
                     }
                 }
-                __syncwarp();
+            }
+            __syncwarp();                      // every lane has read the pivot rows
+            // the tile follows: the next panel's pivot rows are read there, and the panel warps read
+            // their panels there.  The quads of panel p - 1 are G already; those of panel p are theirs
 #pragma unroll
-                for (int l = 0; l < NP; ++l) {
-                    float gl[RG], ul[UC];
+            for (int i = 0; i < NQ; ++i) {
+                const int q = tw + TW * i, pq = q / (NP / 4);
+                float *at = tile + ln * LD + 4 * q;
+                if (q < N / 4 && pq == p - 1) {
 #pragma unroll
-                    for (int a = 0; a < RG; ++a) gl[a] = gq[l * N + 32 * a];
-#pragma unroll
-                    for (int b = 0; b < UC; b += 4) {
-                        const float4 v = *(const float4 *)(uw + l * UC + b);
-                        ul[b] = v.x; ul[b + 1] = v.y; ul[b + 2] = v.z; ul[b + 3] = v.w;
+                    for (int a = 0; a < RG; ++a) {
+                        const float4 v = *(const float4 *)(at + 32 * a * LD);
+                        w[i][a][0] = float2{v.x, v.y};
+                        w[i][a][1] = float2{v.z, v.w};
                     }
+                } else if (q < N / 4 && pq != p) {
 #pragma unroll
-                    for (int b = 0; b < NC; ++b)
-#pragma unroll
-                        for (int a = 0; a < RG; ++a) w[b][a] = fmaf(gl[a], ul[b], w[b][a]);
+                    for (int a = 0; a < RG; ++a)
+                        *(float4 *)(at + 32 * a * LD) = make_float4(w[i][a][0].x, w[i][a][0].y, w[i][a][1].x, w[i][a][1].y);
                 }
-                // panel p - 1's own columns are G; panel p + 1's go to warp 0
-#pragma unroll
-                for (int b = 0; b < NC; ++b) {
-                    const int j = j0 + b, pj = j / NP;
-                    if (j < N && pj == p - 1) {
-#pragma unroll
-                        for (int a = 0; a < RG; ++a) w[b][a] = gq[(j % NP) * N + 32 * a];
-                    } else if (j < N && pj == p + 1) {
-                        float *dst = raw + (pj & 1) * NP * N + (j % NP) * N + ln;
-#pragma unroll
-                        for (int a = 0; a < RG; ++a) dst[32 * a] = w[b][a];
-                    }
-                }
-                __syncwarp();
             }
             __syncthreads();
         }
         // M^-1[k][p(c)] = W[p(k)][c]: columns permuted here, rows on the way out
 #pragma unroll
-        for (int b = 0; b < NC; ++b)
-            if (j0 + b < N) {
-                const int c = perm[j0 + b];
+        for (int i = 0; i < NQ; ++i) {
+            const int q = tw + TW * i;
+            if (q < N / 4) {
+                const int c0 = perm[4 * q], c1 = perm[4 * q + 1], c2 = perm[4 * q + 2], c3 = perm[4 * q + 3];
 #pragma unroll
-                for (int a = 0; a < RG; ++a) tile[(ln + 32 * a) * LD + c] = w[b][a];
+                for (int a = 0; a < RG; ++a) {
+                    float *at = tile + (ln + 32 * a) * LD;
+                    at[c0] = w[i][a][0].x;
+                    at[c1] = w[i][a][0].y;
+                    at[c2] = w[i][a][1].x;
+                    at[c3] = w[i][a][1].y;
+                }
             }
+        }
     }
     __syncthreads();
 #pragma unroll 10
@@ -293,13 +329,12 @@ __global__ void __launch_bounds__(kLeafThreads, 1) k_leaf_inverse(const BcrLeaf 
 template <int RG>
 cudaError_t launch_leaf_rg(const BcrLeaf *tasks, int count, const int *skip, const Ctl *ctl, cudaStream_t st)
 {
-    constexpr size_t smem = leaf_smem(32 * RG);
+    constexpr size_t smem = leaf_smem(RG);
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_leaf_inverse<RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr != cudaSuccess) return attr;
     count_launches(1);
-    k_leaf_inverse<RG><<<count, kLeafThreads, smem, st>>>(tasks, skip, ctl);
-    return cudaGetLastError();
+    return launch_dependent(k_leaf_inverse<RG>, dim3(count), dim3(kLeafThreads), smem, st, tasks, skip, ctl);
 }
 
 // One CTA per block; every block of a launch has the same n, a multiple of 32 up to kBcrLeafMax.
@@ -420,7 +455,9 @@ struct Builder {
     void gemm_stage(std::vector<TcTask> &ts, int level)
     {
         if (ts.empty()) return;
-        BcrStage s{kBcrGemm, (int)p.gemm.size(), (int)ts.size(), tc_number_tiles(ts.data(), (int)ts.size()), level};
+        BcrStage s{kBcrGemm, (int)p.gemm.size(), (int)ts.size(), (int)p.tile_task.size(),
+                   tc_number_tiles(ts.data(), (int)ts.size()), level};
+        for (int q = 0; q < (int)ts.size(); ++q) p.tile_task.insert(p.tile_task.end(), ts[q].tiles, q);
         p.gemm.insert(p.gemm.end(), ts.begin(), ts.end());
         p.fac.push_back(s);
     }
@@ -439,7 +476,7 @@ struct Builder {
     {
         const int B = (int)zin.size();
         if (n <= kBcrLeafMax) {
-            BcrStage s{kBcrLeafStage, (int)p.leaf.size(), B, n, level};
+            BcrStage s{kBcrLeafStage, (int)p.leaf.size(), B, 0, n, level};
             for (int b = 0; b < B; ++b)
                 p.leaf.push_back(BcrLeaf{ptr(in.arr, zin[b], in.r0, in.c0), ptr(out.arr, zout[b], out.r0, out.c0),
                                          cols(in.arr), cols(out.arr), n});
@@ -501,7 +538,7 @@ struct Builder {
     void mv_stage(std::vector<BcrMv> &ts, int level)
     {
         if (ts.empty()) return;
-        BcrStage s{kBcrMv, (int)p.mv.size(), (int)ts.size(), 0, level};
+        BcrStage s{kBcrMv, (int)p.mv.size(), (int)ts.size(), 0, 0, level};
         p.mv.insert(p.mv.end(), ts.begin(), ts.end());
         p.sol.push_back(s);
     }
@@ -545,7 +582,7 @@ struct Builder {
             for (size_t q = 1; q < a.size(); q += 2) elim.push_back(a[q]);
             inverse(Sp, Dfull, elim, Ifull, elim, 0, l);
             if (l == 0) {
-                p.fac.push_back(BcrStage{kBcrLevel0, 0, (int)p.level0_kept.size(), 0, 0});
+                p.fac.push_back(BcrStage{kBcrLevel0, 0, (int)p.level0_kept.size(), 0, 0, 0});
                 continue;
             }
             std::vector<TcTask> ts;
@@ -678,6 +715,7 @@ BcrSizes bcr_sizes(int L, int S)
     z.Zt = p.Zt;
     z.Ncp = p.Ncp;
     z.ngemm = (int)p.gemm.size();
+    z.ntile = (int)p.tile_task.size();
     z.nleaf = (int)p.leaf.size();
     z.nmv = (int)p.mv.size();
     z.nsol = (int)p.sol.size();
@@ -696,7 +734,7 @@ int bcr_build(BcrPlan &p, int L, int S, cudaStream_t st)
     p.L = L;
     p.S = S;
     p.Sp = (S + 31) / 32 * 32;
-    p.gemm.clear(); p.leaf.clear(); p.mv.clear(); p.fac.clear(); p.sol.clear();
+    p.gemm.clear(); p.tile_task.clear(); p.leaf.clear(); p.mv.clear(); p.fac.clear(); p.sol.clear();
     Builder b{p, L, S, p.Sp, {}};
     b.build();
     // tensor maps of the five arrays
@@ -706,6 +744,9 @@ int bcr_build(BcrPlan &p, int L, int S, cudaStream_t st)
     for (int a = 0; a < kArrays; ++a)
         if (tc_make_maps(arrs[a], &p.maps[2 * a], &p.maps[2 * a + 1]) != 0) return -1;
     if (!p.gemm.empty() && cudaMemcpyAsync(p.gemm_d, p.gemm.data(), p.gemm.size() * sizeof(TcTask), cudaMemcpyHostToDevice, st))
+        return -1;
+    if (!p.tile_task.empty() &&
+        cudaMemcpyAsync(p.tile_task_d, p.tile_task.data(), p.tile_task.size() * sizeof(int), cudaMemcpyHostToDevice, st))
         return -1;
     if (!p.leaf.empty() && cudaMemcpyAsync(p.leaf_d, p.leaf.data(), p.leaf.size() * sizeof(BcrLeaf), cudaMemcpyHostToDevice, st))
         return -1;
@@ -755,7 +796,7 @@ cudaError_t bcr_factor(const BcrPlan &p, const int *skip, Ctl *ctl, cudaStream_t
         }
         case kBcrGemm: {
             if (timer) timer->begin(s.kind);
-            cudaError_t e = launch_tc_gemm(p.gemm_d + s.off, s.count, s.tiles, p.maps_d, skip, ctl, st);
+            cudaError_t e = launch_tc_gemm(p.gemm_d + s.off, p.tile_task_d + s.tile, s.tiles, p.maps_d, skip, ctl, st);
             if (timer) timer->end(s.kind);
             if (e != cudaSuccess) return e;
             break;

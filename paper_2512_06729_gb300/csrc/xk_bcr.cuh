@@ -34,6 +34,7 @@ struct BcrMv {
 struct BcrStage {
     int kind;          // BcrKind
     int off, count;    // range in the task list of that kind
+    int tile;          // GEMM: first entry of its tiles in the tile list
     int tiles;         // GEMM: output tiles of the launch; leaf inversions: the blocks' order n
     int level;         // the reduction level it belongs to
 };
@@ -49,11 +50,13 @@ struct BcrPlan {
     float *bw = nullptr, *tw = nullptr, *xw = nullptr;      // [L][Sp] vectors of the solve
     const float *lo = nullptr, *up = nullptr;                // level-0 couplings [L][S] (FP32)
     std::vector<TcTask> gemm;
+    std::vector<int> tile_task;    // per product stage: the stage's task of each output tile
     std::vector<BcrLeaf> leaf;
     std::vector<BcrMv> mv;
     std::vector<BcrStage> fac, sol;
     std::vector<int> level0_kept;                            // even layers kept at level 0
     TcTask *gemm_d = nullptr;
+    int *tile_task_d = nullptr;
     BcrLeaf *leaf_d = nullptr;
     BcrMv *mv_d = nullptr;
     CUtensorMap *maps_d = nullptr;
@@ -66,7 +69,7 @@ struct BcrPlan {
 
 // Sizes of the device arrays and task lists of an L-layer, S-species column (no pointers).
 struct BcrSizes {
-    int Sp, Wt, Zt, Ncp, ngemm, nleaf, nmv, nsol;
+    int Sp, Wt, Zt, Ncp, ngemm, ntile, nleaf, nmv, nsol;
     size_t floats_D, floats_INV, floats_TMP, floats_CP, floats_PQ, floats_vec;
 };
 BcrSizes bcr_sizes(int L, int S);

@@ -708,8 +708,10 @@ int factor_plan(int S, int precision_bytes, int nb_hint, int ctas_hint, FactorPl
     if (want < 1) want = 1;
     p.ctas = want;
     if (precision_bytes == 8) {
-        if (p.nb == 8) p.smem = factor_smem<double, 8>(S, p.ctas);
-        else if (p.nb == 16) p.smem = factor_smem<double, 16>(S, p.ctas);
+        if (p.nb == 8) {
+            p.smem = 0;
+            if (factor64_plan(S, want, &p) != 0) return -1;
+        } else if (p.nb == 16) p.smem = factor_smem<double, 16>(S, p.ctas);
         else if (p.nb == 32) p.smem = 0;
         else return -1;
         // the pivot choice: S x (nb + 1) doubles and S ints; the trailing update: nb x 8 doubles
@@ -773,7 +775,7 @@ cudaError_t launch_factor<double>(const BlockSys<double> &sys, const FactorPlan 
         if (plan.nb == 32) return launch_factor_pv_nb<32>(sys, plan, ctl, st, skip);
         return cudaErrorInvalidValue;
     }
-    if (plan.nb == 8) return launch_factor_nb<double, 8>(sys, plan, ctl, st, skip);
+    if (plan.nb == 8) return launch_factor64(sys, plan, ctl, st, skip);
     if (plan.nb == 16) return launch_factor_nb<double, 16>(sys, plan, ctl, st, skip);
     return cudaErrorInvalidValue;
 }

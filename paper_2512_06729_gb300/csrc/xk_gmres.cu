@@ -261,59 +261,94 @@ __global__ void k_gm_report(const GmState *gm, Ctl *ctl, const int *skip_solve, 
 
 }  // namespace
 
-void enqueue_fgmres(const GmArgs &a, cudaStream_t st)
+// Iteration slots that are always enqueued; most solves end within them, the others are one IF node of
+// a captured step.
+constexpr int kPlainSlots = 3;
+
+cudaError_t enqueue_fgmres(const GmArgs &a, cudaStream_t st0)
 {
     const long long N = a.N;
     const int m = a.m < kMaxBasis ? a.m : kMaxBasis;
     // iteration slots: the budget max_iter split into cycles of m, then a short spare cycle for a
     // restart after a cycle that ended on the recurrence estimate without true convergence;
-    // slots past convergence cost one early-exit launch per kernel
+    // slots past convergence cost one early-exit launch per kernel where they are enqueued
     const int full = (a.max_iter + m - 1) / m;
     const int spare = m < 8 ? m : 8;
     const int cycles = full + 1;
     int eb = (int)((N + kRedThreads - 1) / kRedThreads);
     if (eb > 4 * kRedBlocks) eb = 4 * kRedBlocks;
-    count_launches(1); k_gm_init<<<1, 1, 0, st>>>(a.gm, a.tol);
-    count_launches(1); k_gm_skip_if_finished<<<1, 1, 0, st>>>(a.gm, a.ctl, a.skip_solve);
-    count_launches(1); k_zero<<<eb, kRedThreads, 0, st>>>(a.x, N, a.gm);
-    for (int cyc = 0; cyc < cycles; ++cyc) {
-        double *r = a.V;                       // V_0 slot holds the residual before scaling
-        if (cyc == 0) {
-            count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, 0, a.b, N, a.partials, a.counter, a.red, a.gm, 1);
-            // red[0] = ||b||^2 (nv = 0: the norm lands in out[0])
-            count_launches(1); k_cycle_begin<<<1, 1, 0, st>>>(a.gm, a.red, 1, a.max_iter);
-            count_launches(1); k_scale<<<eb, kRedThreads, 0, st>>>(a.b, a.V, N, &a.gm->beta, a.gm);
-        } else {
-            a.matvec(a.x, a.w, &a.gm->done, st);
-            count_launches(1); k_sub<<<eb, kRedThreads, 0, st>>>(a.b, a.w, r, N, a.gm);
-            count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, 0, r, N, a.partials, a.counter, a.red, a.gm, 1);
-            count_launches(1); k_cycle_begin<<<1, 1, 0, st>>>(a.gm, a.red, 0, a.max_iter);
-            count_launches(1); k_scale<<<eb, kRedThreads, 0, st>>>(r, a.V, N, &a.gm->beta, a.gm);
+    cudaError_t err = cudaSuccess;
+    auto keep = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
+    // a device flag as the host sees it now
+    auto flag = [&](const int *f) {
+        if (!a.host) return false;
+        keep(cudaMemcpyAsync(a.host, f, sizeof(int), cudaMemcpyDeviceToHost, st0));
+        keep(cudaStreamSynchronize(st0));
+        return err != cudaSuccess || *a.host != 0;
+    };
+    auto slot = [&](int jj, int mc, cudaStream_t st) {
+        double *vj = a.V + (long long)jj * N;
+        double *zj = a.Z + (long long)jj * N;
+        a.precond(vj, zj, &a.gm->idle, st);
+        a.matvec(zj, a.w, &a.gm->idle, st);
+        count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, jj + 1, a.w, N, a.partials, a.counter, a.h1, a.gm, 0);
+        count_launches(1); k_axpy_basis<<<eb, kRedThreads, 0, st>>>(a.V, jj + 1, a.h1, a.w, N, a.gm);
+        count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, jj + 1, a.w, N, a.partials, a.counter, a.h2, a.gm, 0);
+        count_launches(1); k_axpy_basis<<<eb, kRedThreads, 0, st>>>(a.V, jj + 1, a.h2, a.w, N, a.gm);
+        // ||w||^2 into h2[jj + 1]
+        count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, 0, a.w, N, a.partials, a.counter, a.h2 + jj + 1, a.gm, 1);
+        count_launches(1); k_arnoldi_end<<<1, 1, 0, st>>>(a.gm, a.h1, a.h2, jj, mc, a.max_iter);
+        count_launches(1); k_scale<<<eb, kRedThreads, 0, st>>>(a.w, a.V + (long long)(jj + 1) * N, N, &a.gm->hnext, a.gm);
+    };
+    auto iterate = [&](int mc, cudaStream_t st) {
+        const int plain = mc < kPlainSlots ? mc : kPlainSlots;
+        bool over = false;
+        for (int jj = 0; jj < plain && !over; ++jj) {
+            slot(jj, mc, st);
+            over = flag(&a.gm->idle);
         }
-        const int mc = cyc < full ? (a.max_iter - cyc * m < m ? a.max_iter - cyc * m : m) : spare;
-        for (int jj = 0; jj < mc; ++jj) {
-            double *vj = a.V + (long long)jj * N;
-            double *zj = a.Z + (long long)jj * N;
-            a.precond(vj, zj, &a.gm->idle, st);
-            a.matvec(zj, a.w, &a.gm->idle, st);
-            count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, jj + 1, a.w, N, a.partials, a.counter, a.h1, a.gm, 0);
-            count_launches(1); k_axpy_basis<<<eb, kRedThreads, 0, st>>>(a.V, jj + 1, a.h1, a.w, N, a.gm);
-            count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, jj + 1, a.w, N, a.partials, a.counter, a.h2, a.gm, 0);
-            count_launches(1); k_axpy_basis<<<eb, kRedThreads, 0, st>>>(a.V, jj + 1, a.h2, a.w, N, a.gm);
-            // ||w||^2 into h2[jj + 1]
-            count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, 0, a.w, N, a.partials, a.counter, a.h2 + jj + 1, a.gm, 1);
-            count_launches(1); k_arnoldi_end<<<1, 1, 0, st>>>(a.gm, a.h1, a.h2, jj, mc, a.max_iter);
-            count_launches(1); k_scale<<<eb, kRedThreads, 0, st>>>(a.w, a.V + (long long)(jj + 1) * N, N, &a.gm->hnext, a.gm);
-        }
+        if (mc > plain && !over)
+            keep(enqueue_if(st, a.cond, &a.gm->idle, 0, [&](cudaStream_t s) {
+                for (int jj = plain; jj < mc && !over; ++jj) {
+                    slot(jj, mc, s);
+                    over = flag(&a.gm->idle);
+                }
+            }));
         count_launches(1); k_update<<<eb, kRedThreads, 0, st>>>(a.gm, a.Z, a.x, N, a.max_iter);
         count_launches(1); k_update_done<<<1, 1, 0, st>>>(a.gm, a.max_iter);
+    };
+    count_launches(1); k_gm_init<<<1, 1, 0, st0>>>(a.gm, a.tol);
+    count_launches(1); k_gm_skip_if_finished<<<1, 1, 0, st0>>>(a.gm, a.ctl, a.skip_solve);
+    count_launches(1); k_zero<<<eb, kRedThreads, 0, st0>>>(a.x, N, a.gm);
+    count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st0>>>(a.V, 0, a.b, N, a.partials, a.counter, a.red, a.gm, 1);
+    // red[0] = ||b||^2 (nv = 0: the norm lands in out[0])
+    count_launches(1); k_cycle_begin<<<1, 1, 0, st0>>>(a.gm, a.red, 1, a.max_iter);
+    count_launches(1); k_scale<<<eb, kRedThreads, 0, st0>>>(a.b, a.V, N, &a.gm->beta, a.gm);
+    iterate(a.max_iter < m ? a.max_iter : m, st0);
+    // later cycles, each behind a check of the true residual r = b - A x (V_0 holds r before scaling)
+    auto residual = [&](double *r, cudaStream_t st) {
+        a.matvec(a.x, a.w, &a.gm->done, st);
+        count_launches(1); k_sub<<<eb, kRedThreads, 0, st>>>(a.b, a.w, r, N, a.gm);
+        count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, 0, r, N, a.partials, a.counter, a.red, a.gm, 1);
+    };
+    for (int cyc = 1; cyc < cycles; ++cyc) {
+        const int mc = cyc < full ? (a.max_iter - cyc * m < m ? a.max_iter - cyc * m : m) : spare;
+        residual(a.V, st0);
+        count_launches(1); k_cycle_begin<<<1, 1, 0, st0>>>(a.gm, a.red, 0, a.max_iter);
+        if (flag(&a.gm->done)) break;
+        keep(enqueue_if(st0, a.cond, &a.gm->done, 0, [&](cudaStream_t st) {
+            count_launches(1); k_scale<<<eb, kRedThreads, 0, st>>>(a.V, a.V, N, &a.gm->beta, a.gm);
+            iterate(mc, st);
+        }));
     }
     // final check on the true residual (a cycle may have ended on the recurrence estimate)
-    a.matvec(a.x, a.w, &a.gm->done, st);
-    count_launches(1); k_sub<<<eb, kRedThreads, 0, st>>>(a.b, a.w, a.w, N, a.gm);
-    count_launches(1); k_dots<<<kRedBlocks, kRedThreads, 0, st>>>(a.V, 0, a.w, N, a.partials, a.counter, a.red, a.gm, 1);
-    count_launches(1); k_final<<<1, 1, 0, st>>>(a.gm, a.red);
-    count_launches(1); k_gm_report<<<1, 1, 0, st>>>(a.gm, a.ctl, a.skip_solve, a.role, a.reuse_max_iters);
+    if (!flag(&a.gm->done))
+        keep(enqueue_if(st0, a.cond, &a.gm->done, 0, [&](cudaStream_t st) {
+            residual(a.w, st);
+            count_launches(1); k_final<<<1, 1, 0, st>>>(a.gm, a.red);
+        }));
+    count_launches(1); k_gm_report<<<1, 1, 0, st0>>>(a.gm, a.ctl, a.skip_solve, a.role, a.reuse_max_iters);
+    return err;
 }
 
 }  // namespace xk

@@ -40,12 +40,15 @@ struct GmArgs {
     int role;                // 0: FP32-preconditioned attempt, 1: attempt with the reused FP64 factorization,
                              // 2: refinement around a fresh FP64 factorization (recorded, no routing)
     int reuse_max_iters;     // role 1: more iterations than this trigger a fresh factorization next step
+    CondStreams *cond = nullptr;   // captured steps: iterations past convergence in IF nodes
+    int *host = nullptr;           // pinned word: the host follows the iteration (launched, not captured) and
+                                   // stops enqueueing when it has converged; nullptr: every slot is enqueued
     VecOp matvec;        // y = A x (FP64); must return at once while *skip != 0
     VecOp precond;       // z ~ A^-1 v (low precision); same skip rule
 };
 
 constexpr int kGmPartialBlocks = 304;
 
-void enqueue_fgmres(const GmArgs &a, cudaStream_t st);
+cudaError_t enqueue_fgmres(const GmArgs &a, cudaStream_t st);
 
 }  // namespace xk

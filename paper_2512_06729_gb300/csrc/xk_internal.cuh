@@ -265,6 +265,57 @@ struct ParcelArgs {
 // One global iteration on one CTA (photolysis and rate coefficients already in c).
 cudaError_t launch_parcel_iteration(const Col &c, const ParcelArgs &a, cudaStream_t st);
 
+// Launch a kernel that may start while its predecessor on the stream drains (programmatic dependent
+// launch): it must execute griddepcontrol.wait before it touches anything an earlier launch writes.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
+// Conditional parts of a captured step (xk_cond.cu).  A part is captured on a stream of its own
+// nesting level into the body of an IF node that runs when (*flag != 0) == (when != 0), the flag read
+// where the node stands.
+struct CondStreams {
+    cudaStream_t inner[2] = {nullptr, nullptr};
+    int depth = 0;
+};
+bool capturing(cudaStream_t st);
+cudaError_t cond_open(cudaStream_t st, cudaStream_t inner, const int *flag, int when, cudaGraphNode_t *node);
+cudaError_t cond_close(cudaStream_t st, cudaStream_t inner, cudaGraphNode_t node);
+// body(stream) as such a part while st is being captured; otherwise body(st), whose kernels check the
+// flag themselves.  Kernels of a part are not counted as launches: it may not run.
+template <typename F>
+cudaError_t enqueue_if(cudaStream_t st, CondStreams *cs, const int *flag, int when, F body)
+{
+    if (!cs || cs->depth >= 2 || !capturing(st)) {
+        body(st);
+        return cudaSuccess;
+    }
+    cudaStream_t &in = cs->inner[cs->depth];
+    cudaError_t e = cudaSuccess;
+    if (!in) e = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking);
+    cudaGraphNode_t node;
+    if (e == cudaSuccess) e = cond_open(st, in, flag, when, &node);
+    if (e != cudaSuccess) return e;
+    const long long n0 = launches();
+    ++cs->depth;
+    body(in);
+    --cs->depth;
+    count_launches(n0 - launches());
+    return cond_close(st, in, node);
+}
+
 constexpr unsigned long long kSyncPolls = 1ull << 22;   // polls of GridSync, without a sleep: a second or two
 constexpr unsigned long long kSpinLimit = 1ull << 24;   // polls of a bounded wait: ~1-2 s with the sleep below
 
@@ -393,6 +444,8 @@ struct FactorPlan {
     int twisted = 0;           // k_factor: eliminate from both ends on the two halves of the grid
     int preview = 0;           // FP64: each panel's pivots chosen first on one CTA (k_factor_pv)
     double *dinv = nullptr;    // that path: nb x nb LU factors of the panel's pivot block (global)
+    int cs = 0, ctas64 = 0;    // FP64, panels of 8 (xk_factor64.cu): CTAs of the panel's cluster, CTAs of the launch
+    size_t smem64 = 0;
 };
 template <typename T>
 struct BlockSys {
@@ -401,10 +454,15 @@ struct BlockSys {
     int *perm;       // [L][S] pivot row of each column
     int *iperm;      // [L][S] column each row was pivot of
     int *pinfo;      // panel scratch: pivot rows of the current panel
-    unsigned *bar;   // grid barrier: [2]
+    unsigned *bar;   // barrier words: [8] (0-3 the grid barriers of up to two chains, 6-7 with xk_factor64.cu)
     int L, S, ld;
 };
 int factor_plan(int S, int precision_bytes, int nb_hint, int ctas_hint, FactorPlan *out);
+// FP64 in panels of 8 columns, the panel on a thread-block cluster (xk_factor64.cu): fills cs, ctas64
+// and smem64 for up to `want` CTAs (0, or -1 when S does not fit)
+int factor64_plan(int S, int want, FactorPlan *p);
+cudaError_t launch_factor64(const BlockSys<double> &sys, const FactorPlan &plan, Ctl *ctl, cudaStream_t st,
+                            const int *skip);
 template <typename T>
 cudaError_t launch_factor(const BlockSys<T> &sys, const FactorPlan &plan, Ctl *ctl, cudaStream_t st,
                           const int *skip = nullptr);

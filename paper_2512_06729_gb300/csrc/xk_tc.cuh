@@ -53,9 +53,10 @@ int tc_make_maps(const TcArray &a, CUtensorMap *amap, CUtensorMap *bmap);
 // Host: number the output tiles of a task list; returns the total.
 int tc_number_tiles(TcTask *tasks, int ntasks);
 // Launch one kernel over all tiles of the task list (tasks and maps in device memory, maps as
-// [array][role]).  Exits at once when *skip != 0 or the control block reports a finished step
-// or a timed-out wait; a wait of its own that gives up sets ctl->err_timeout.
-cudaError_t launch_tc_gemm(const TcTask *tasks, int ntasks, int total_tiles, const CUtensorMap *maps,
+// [array][role]; tile_task [total_tiles], device: the task of each tile, nullptr for a single task).
+// Exits at once when *skip != 0 or the control block reports a finished step or a timed-out wait; a
+// wait of its own that gives up sets ctl->err_timeout.
+cudaError_t launch_tc_gemm(const TcTask *tasks, const int *tile_task, int total_tiles, const CUtensorMap *maps,
                            const int *skip, Ctl *ctl, cudaStream_t st);
 
 }  // namespace xk
