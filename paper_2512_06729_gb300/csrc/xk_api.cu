@@ -595,7 +595,7 @@ size_t layout(xk_ctx *c, char *base)
     c->pinfo = b.take<int>(1 + 4 * 64);
     c->dinv = b.take<double>(32 * 32);
     c->ymid = b.take<double>(2 * (size_t)S);
-    c->bar = b.take<unsigned>(8);
+    c->bar = b.take<unsigned>(factor64_words());
     c->bcr.bar = c->bar ? c->bar + 4 : nullptr;      // words 4-5: the reduction's solve and FGMRES
     c->ctl = b.take<Ctl>(1);
     c->ctl_aux = b.take<Ctl>(1);
@@ -733,7 +733,7 @@ Ctl fresh_ctl(const xk_ctx *c)
 // (and the flag) before the context is used again.
 int timed_out(xk_ctx *c)
 {
-    cudaMemsetAsync(c->bar, 0, 8 * sizeof(unsigned), c->st);
+    cudaMemsetAsync(c->bar, 0, factor64_words() * sizeof(unsigned), c->st);
     cudaMemsetAsync(&c->ctl->err_timeout, 0, sizeof(int), c->st);
     cudaMemsetAsync(&c->ctl_aux->err_timeout, 0, sizeof(int), c->st);
     cudaError_t e = cudaStreamSynchronize(c->st);
@@ -1321,7 +1321,7 @@ int xk_set_workspace(xk_ctx *c, void *dptr, size_t bytes)
     up(c, k.abs_sp, c->abs_sp);
     up(c, k.sig_sca, c->sig_sca_c); up(c, k.sca_sp, c->sca_sp);
     up(c, k.P, c->P); up(c, k.T, c->T); up(c, k.Kzz, c->Kzz);
-    cudaMemsetAsync(c->bar, 0, 8 * sizeof(unsigned), c->st);
+    cudaMemsetAsync(c->bar, 0, factor64_words() * sizeof(unsigned), c->st);
     if (c->counter) cudaMemsetAsync(c->counter, 0, 8 * sizeof(unsigned), c->st);
     cudaMemsetAsync(c->col.n, 0, sizeof(double) * (size_t)c->L * c->S, c->st);
     Ctl init = fresh_ctl(c);

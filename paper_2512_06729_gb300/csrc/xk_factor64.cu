@@ -6,11 +6,18 @@
 // rows factored by one CTA, with a block barrier pair per column, is most of the time: 51 us per
 // panel at 594 species (of which the other 75 SMs idle through about 40), 22 us at 96.  Here
 //  - the panel belongs to a thread-block cluster, its rows spread over the cluster's CTAs, one row
-//    per thread in registers.  A column costs one cluster barrier: every warp pushes its best
-//    candidate row (value and the row's 8 panel entries) to all CTAs through distributed shared
-//    memory, and after the barrier each CTA picks the winner from its own copy;
-//  - the other CTAs apply the previous panel to their columns meanwhile (look-ahead): the cluster
-//    applies it to the next panel itself.  One grid barrier per panel instead of two.
+//    per thread in registers.  Per column every warp sends its best candidate row (the reciprocal of
+//    its pivot and the row's panel entries) to all CTAs as asynchronous stores that complete on the
+//    receiver's mbarrier, and each picks the winner from its own copy: no barrier of the cluster or
+//    the block.  The loop over the panel's columns is rolled (the finished column moves to the end):
+//    unrolled, its code ran out of the instruction cache and a column took 1,900 clocks;
+//  - the other CTAs apply the previous panels to their columns meanwhile.  k_factor64_flow: a CTA
+//    keeps its columns of the layer in shared memory, takes each panel as its flag appears and hands
+//    the columns of panel p + 2 over once panel p has been applied to them; grid barriers only at a
+//    layer's end.  k_factor64: columns too many for shared memory (a small share of the SMs in a
+//    batch) stay in global memory, with one grid barrier per panel.
+// Bound by the FP64 updates at 594 species (8 S^2 fused operations per panel over the chain's SMs,
+// 24,400 clocks), by the chain of columns below some 300.
 // The pivot is the unused row of largest magnitude to 20 bits (the high word of the double), the
 // lowest row among equals.
 //
@@ -34,7 +41,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kPS = kNB + 1;              // padded row of the panel in shared memory
 constexpr size_t kSmemMax = 227 * 1024;
 
-// A warp's best candidate for a pivot: the row's panel entries, the magnitude's high word, the row.
+// A warp's best candidate for a pivot: the reciprocal of the pivot and the rest of the row's panel
+// entries, the magnitude's high word, the row.
 struct __align__(16) Cand {
     double row[kNB];
     unsigned key;
@@ -56,15 +64,57 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank)
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_cluster(uint32_t addr, uint4 v)
-{
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-                 : "memory");
-}
 __device__ __forceinline__ void st_cluster(uint32_t addr, int v)
 {
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
+// Asynchronous store of 16 bytes into a CTA of the cluster, counted by that CTA's mbarrier.
+__device__ __forceinline__ void st_async(uint32_t addr, uint4 v, uint32_t mbar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(mbar)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Bounded wait for a phase.  Giving up is recorded, and the caller carries on (every index it takes
+// from what did not arrive is clamped) to the next grid barrier, where the cluster leaves together.
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, Ctl *ctl)
+{
+    for (unsigned long long i = 0; i < kSyncPolls; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return;
+        if ((i & 63) == 63 && *(volatile int *)&ctl->err_timeout) return;
+    }
+    atomicExch(&ctl->err_timeout, 1);
+}
+// Bounded wait for a counter that other CTAs raise; as above.
+__device__ __forceinline__ void wait_count(const unsigned *word, unsigned target, Ctl *ctl)
+{
+    const unsigned long long limit = ctl->wait_polls ? ctl->wait_polls : kSyncPolls;
+    for (unsigned long long i = 0; i < limit; ++i) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+        if ((int)(v - target) >= 0) return;
+        if ((i & 63) == 63 && *(volatile int *)&ctl->err_timeout) return;
+    }
+    atomicExch(&ctl->err_timeout, 1);
+}
+__device__ __forceinline__ void raise_count(unsigned *word)
+{
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word) : "memory");
+}
+
 __device__ __forceinline__ void cluster_sync(int cs)
 {
     if (cs == 1) {
@@ -138,6 +188,225 @@ struct ChainSync {
     }
 };
 
+// The panel's share of one CTA of its cluster.
+struct Panel {
+    int S, ld, cs, crank, rpc, r0, nr, nw, ncand;
+    double *P, *G;                // [rpc][kPS]: the panel's rows, the previous panel's result
+    double *us;                   // [kNB * kNB]: the previous panel's pivot rows in this panel
+    Cand *stage, *cand;           // [kWarps], [2][32]
+    int *piv;                     // [2][kNB]
+    uint32_t mbar;                // two mbarriers, one per candidate buffer
+    unsigned col;                 // columns done in this launch: buffer col & 1, phase (col / 2) & 1
+    Ctl *ctl;
+};
+
+// Panel p of layer block D: takes its columns from D (the panels before p - 1 are applied), applies
+// panel p - 1, factors it and leaves G in D's panel columns and in G.
+template <int RPT>
+__device__ __forceinline__ void panel_step(Panel &q, double *D, int *perm, int *iperm, int p, unsigned &used)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int c0 = p * kNB, nb = min(kNB, q.S - c0);
+    const int *pp = q.piv + ((p + 1) & 1) * kNB;   // the previous panel's pivot rows
+    int *pc = q.piv + (p & 1) * kNB;
+    for (int e = tid; e < q.nr * kNB; e += kThreads) {
+        const int r = e / kNB, j = e % kNB;
+        q.P[r * kPS + j] = j < nb ? __ldcg(D + (size_t)(q.r0 + r) * q.ld + c0 + j) : 0.0;
+    }
+    if (p > 0 && tid < kNB * kNB) {
+        const int l = tid / kNB, j = tid % kNB;
+        q.us[tid] = j < nb ? __ldcg(D + (size_t)pp[l] * q.ld + c0 + j) : 0.0;
+    }
+    __syncthreads();
+    if (p > 0) {
+        for (int e = tid; e < q.nr * kNB; e += kThreads) {
+            const int r = e / kNB, j = e % kNB;
+            bool piv = false;
+#pragma unroll
+            for (int l = 0; l < kNB; ++l) piv |= pp[l] == q.r0 + r;
+            double acc = piv ? 0.0 : q.P[r * kPS + j];
+#pragma unroll
+            for (int l = 0; l < kNB; ++l) acc = fma(q.G[r * kPS + l], q.us[l * kNB + j], acc);
+            q.P[r * kPS + j] = acc;
+        }
+        __syncthreads();
+    }
+    if (warp < q.nw) {
+        double x[RPT][kNB];
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int r = tid + i * kThreads;
+#pragma unroll
+            for (int j = 0; j < kNB; ++j) x[i][j] = r < q.nr ? q.P[r * kPS + j] : 0.0;
+        }
+        // column c is always x[.][0]: each step shifts the others down one and puts the finished column
+        // last, so that after eight steps they are in their places again
+#pragma unroll 1
+        for (int c = 0; c < kNB; ++c) {
+            if (c >= nb) {                      // a ragged panel's missing columns
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    const double t = x[i][0];
+#pragma unroll
+                    for (int j = 1; j < kNB; ++j) x[i][j - 1] = x[i][j];
+                    x[i][kNB - 1] = t;
+                }
+                continue;
+            }
+            const int par = q.col & 1;
+            const uint32_t bar = q.mbar + 8u * par, phase = (q.col >> 1) & 1u;
+            ++q.col;
+            Cand *cb = q.cand + 32 * par;
+            if (tid == 0) mbar_expect(bar, (uint32_t)(q.ncand * sizeof(Cand)));
+            // this warp's best unused row (and its reciprocal, while the reduction runs)
+            unsigned key = 0u;
+            int bi = -1;
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const unsigned m = (unsigned)__double2hiint(x[i][0]) & 0x7fffffffu;
+                if (!((used >> i) & 1u) && (bi < 0 || m > key)) { key = m; bi = i; }
+            }
+            double mine_row[kNB];
+#pragma unroll
+            for (int j = 0; j < kNB; ++j) mine_row[j] = RPT > 1 && bi == RPT - 1 ? x[RPT - 1][j] : x[0][j];
+            // (a column without a nonzero candidate is singular: the bookkeeping goes on)
+            mine_row[0] = key == 0u ? 0.0 : reciprocal(mine_row[0]);
+            const unsigned best = __reduce_max_sync(0xffffffffu, bi >= 0 ? key + 1u : 0u);
+            const unsigned who = __ballot_sync(0xffffffffu, bi >= 0 && key + 1u == best);
+            const int src = who ? __ffs(who) - 1 : 0;
+            if (lane == src) {
+                Cand &o = q.stage[warp];
+#pragma unroll
+                for (int j = 0; j < kNB; j += 2) *(double2 *)&o.row[j] = make_double2(mine_row[j], mine_row[j + 1]);
+                o.key = key;
+                o.idx = who ? q.r0 + tid + bi * kThreads : -1;
+            }
+            __syncwarp();
+            for (int it = lane; it < q.cs * kCandParts; it += 32) {
+                const int dst = it / kCandParts, part = it % kCandParts;
+                st_async(map_rank(smem_u32(&cb[q.crank * q.nw + warp]) + 16u * part, dst), ((const uint4 *)&q.stage[warp])[part],
+                         map_rank(bar, dst));
+            }
+            mbar_wait(bar, phase, q.ctl);
+            __syncwarp();
+            const bool have = lane < q.ncand && cb[lane].idx >= 0;
+            const unsigned ck = have ? cb[lane].key : 0u;
+            const unsigned top = __reduce_max_sync(0xffffffffu, have ? ck + 1u : 0u);
+            const unsigned win = __ballot_sync(0xffffffffu, have && ck + 1u == top);
+            const Cand &w = cb[win ? __ffs(win) - 1 : 0];
+            const int row = min(max(w.idx, 0), q.S - 1);
+            double pr[kNB];
+#pragma unroll
+            for (int j = 0; j < kNB; j += 2) {
+                const double2 v = *(const double2 *)&w.row[j];
+                pr[j] = v.x;
+                pr[j + 1] = v.y;
+            }
+            if (tid == 0) {
+                pc[c] = row;
+                if (q.crank == 0 && top <= 1u) atomicExch(&q.ctl->err_singular, 1);
+            }
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const bool mine = q.r0 + tid + i * kThreads == row && tid + i * kThreads < q.nr;
+                if (mine) {
+                    used |= 1u << i;
+                    perm[c0 + c] = row;
+                    iperm[row] = c0 + c;
+                }
+                // the pivot row starts from zero and takes the multiplier that leaves it scaled
+                const double f = mine ? -pr[0] : x[i][0] * pr[0];
+#pragma unroll
+                for (int j = 1; j < kNB; ++j) x[i][j - 1] = fma(-f, pr[j], mine ? 0.0 : x[i][j]);
+                x[i][kNB - 1] = -f;
+            }
+        }
+        // the panel's columns become G
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int r = tid + i * kThreads;
+            if (r >= q.nr) continue;
+            double *Dr = D + (size_t)(q.r0 + r) * q.ld + c0;
+#pragma unroll
+            for (int j = 0; j < kNB; ++j) {
+                q.G[r * kPS + j] = j < nb ? x[i][j] : 0.0;
+                if (j < nb) __stcg(Dr + j, x[i][j]);
+            }
+        }
+    }
+}
+
+// Which layers a chain takes, and in which order.
+struct Order {
+    int nsteps, k0, dk;
+};
+__device__ __forceinline__ Order order_of(int mode, int half, int L, int mid)
+{
+    if (mode == 1) return half == 0 ? Order{mid, 0, 1} : Order{L - 1 - mid, L - 1, -1};
+    if (mode == 2) return Order{1, mid, 0};
+    return Order{L, 0, 1};
+}
+
+// Schur terms of layer k: f(n, rowc, colc) for each neighbour n already eliminated,
+// D_k -= diag(rowc) D'^-1_n diag(colc).
+template <typename F>
+__device__ __forceinline__ bool schur_terms(const BlockSys<double> &a, int mode, int step, int dk, int k, F f)
+{
+    const size_t S = a.S;
+    const bool below = mode == 2 ? k > 0 : step > 0 && dk > 0;
+    const bool above = mode == 2 ? k + 1 < a.L : step > 0 && dk < 0;
+    if (below) f(k - 1, a.lo + k * S, a.up + (k - 1) * S);
+    if (above) f(k + 1, a.up + k * S, a.lo + (k + 1) * S);
+    return below || above;
+}
+
+struct PanelShared {
+    Cand stage[kWarps], cand[2][32];
+    double us[kNB * kNB];
+    int piv[2][kNB], go;
+    unsigned long long mbar[2];
+};
+
+__device__ __forceinline__ Panel make_panel(PanelShared &sh, double *dyn, const BlockSys<double> &a, Ctl *ctl, int cs, int crank)
+{
+    Panel q;
+    q.S = a.S;
+    q.ld = a.ld;
+    q.cs = cs;
+    q.crank = crank;
+    q.rpc = (a.S + cs - 1) / cs;
+    q.r0 = crank * q.rpc;
+    q.nr = max(0, min(a.S, q.r0 + q.rpc) - q.r0);
+    q.nw = min(kWarps, (q.rpc + 31) / 32);
+    q.ncand = cs * q.nw;
+    q.P = dyn;
+    q.G = q.P + (size_t)q.rpc * kPS;
+    q.us = sh.us;
+    q.stage = sh.stage;
+    q.cand = sh.cand[0];
+    q.piv = sh.piv[0];
+    q.mbar = smem_u32(sh.mbar);
+    q.col = 0;
+    q.ctl = ctl;
+    // every CTA's mbarriers stand before another CTA sends to them
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(q.mbar + 8u * i) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cluster_sync(cs);
+    return q;
+}
+
+template <int RPT>
+__device__ __forceinline__ unsigned unused_rows(const Panel &q)
+{
+    unsigned used = 0;                           // bit i: this thread's row i has been a pivot, or is none
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+        if ((int)threadIdx.x + i * kThreads >= q.nr) used |= 1u << i;
+    return used;
+}
+
 // mode 0: all layers top-down on the whole grid.  mode 1 (twisted): two chains on the two halves of
 // the grid, layers 0 .. mid-1 top-down and L-1 .. mid+1 bottom-up.  mode 2: the middle layer on the
 // whole grid, with both Schur terms.  RPT: panel rows per thread.
@@ -147,48 +416,27 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
 {
     if (ctl->finished || ctl->err_timeout || (skip && *skip)) return;
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ Cand stage[kWarps];
-    __shared__ Cand cand[2][32];
-    __shared__ double us[kNB * kNB];
-    __shared__ int s_piv[2][kNB], s_go;
-    const int S = a.S, ld = a.ld, L = a.L;
+    __shared__ PanelShared sh;
+    const int S = a.S, ld = a.ld;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = mode == 1 ? (int)(blockIdx.x >= gridDim.x / 2) : 0;
     const int nblk = mode == 1 ? (int)gridDim.x / 2 : (int)gridDim.x;
     const int bid = (int)blockIdx.x - half * nblk;
     const int crank = (int)cluster_rank(), cidx = bid / cs, nclus = nblk / cs;
-    const bool panel_cta = cidx == 0;
     // trailing updates: the CTAs of the other clusters, or everyone where there is only one
     const int ntrail = nclus > 1 ? nblk - cs : nblk, tq = nclus > 1 ? bid - cs : bid;
-    int *pinfo = a.pinfo + 64 * half;
-    ChainSync chain{a.bar + 2 * half, a.bar + 6 + half, ctl, cs, nclus, crank, &s_go, 0u};
-
-    const int rpc = (S + cs - 1) / cs, r0 = crank * rpc, nr = max(0, min(S, r0 + rpc) - r0);
-    const int nw = min(kWarps, (rpc + 31) / 32), ncand = cs * nw;     // warps with panel rows, per CTA and in all
-    double *P = (double *)dyn;                       // [rpc][kPS]: the panel's rows of this CTA
-    double *G = P + (size_t)rpc * kPS;               // [rpc][kPS]: the previous panel's
-    double *U = G + (size_t)rpc * kPS;               // [kNB][cw]: pivot rows in this CTA's columns
+    ChainSync chain{a.bar + 2 * half, a.bar + 6 + half, ctl, cs, nclus, crank, &sh.go, 0u};
+    Panel q = make_panel(sh, (double *)dyn, a, ctl, cs, crank);
+    double *U = q.G + (size_t)q.rpc * kPS;                // [kNB][cw]: pivot rows in this CTA's columns
     double *rowbuf = (double *)dyn + (size_t)warp * S;    // Schur term: a source row per warp
-
-    int nsteps = L, k0 = 0, dk = 1;
-    if (mode == 1) {
-        nsteps = half == 0 ? mid : L - 1 - mid;
-        k0 = half == 0 ? 0 : L - 1;
-        dk = half == 0 ? 1 : -1;
-    } else if (mode == 2) {
-        nsteps = 1;
-        k0 = mid;
-        dk = 0;
-    }
+    const Order o = order_of(mode, half, a.L, mid);
     const int npan = (S + kNB - 1) / kNB;
-    int par = 0;                                     // candidate buffer of the next column
-    for (int step = 0; step < nsteps; ++step) {
-        const int k = k0 + step * dk;
+    for (int step = 0; step < o.nsteps; ++step) {
+        const int k = o.k0 + step * o.dk;
         double *D = a.D + (size_t)k * S * ld;
         int *perm = a.perm + (size_t)k * S, *iperm = a.iperm + (size_t)k * S;
-        // D_k -= diag(rowc) D'^-1_n diag(colc), D'^-1_n[i][j] = B_n[perm_n(i)][iperm_n(j)]: a warp per
-        // row, the source row through shared memory
-        auto schur = [&](int nbr, const double *rowc, const double *colc) {
+        // D'^-1_n[i][j] = B_n[perm_n(i)][iperm_n(j)]: a warp per row, the source row through shared memory
+        const bool touched = schur_terms(a, mode, step, o.dk, k, [&](int nbr, const double *rowc, const double *colc) {
             const double *Bn = a.D + (size_t)nbr * S * ld;
             const int *pn = a.perm + (size_t)nbr * S, *ipn = a.iperm + (size_t)nbr * S;
             for (int i = bid * kWarps + warp; i < S; i += nblk * kWarps) {
@@ -200,151 +448,11 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
                 double *Di = D + (size_t)i * ld;
                 for (int j = lane; j < S; j += 32) Di[j] -= rc * rowbuf[__ldcg(ipn + j)] * colc[j];
             }
-        };
-        bool touched = true;
-        if (mode == 2) {
-            if (k > 0) schur(k - 1, a.lo + (size_t)k * S, a.up + (size_t)(k - 1) * S);
-            if (k + 1 < L) schur(k + 1, a.up + (size_t)k * S, a.lo + (size_t)(k + 1) * S);
-        } else if (step > 0) {
-            if (dk > 0) schur(k - 1, a.lo + (size_t)k * S, a.up + (size_t)(k - 1) * S);
-            else schur(k + 1, a.up + (size_t)k * S, a.lo + (size_t)(k + 1) * S);
-        } else {
-            touched = false;
-        }
+        });
         if (touched && !chain.sync()) return;
-
-        unsigned used = 0;                           // bit i: this thread's row i has been a pivot
-#pragma unroll
-        for (int i = 0; i < RPT; ++i)
-            if (tid + i * kThreads >= nr) used |= 1u << i;
+        unsigned used = unused_rows<RPT>(q);
         for (int p = 0; p <= npan; ++p) {
-            if (panel_cta && p < npan) {
-                const int c0 = p * kNB, nb = min(kNB, S - c0);
-                const int *pp = s_piv[(p + 1) & 1];  // the previous panel's pivot rows
-                int *pc = s_piv[p & 1];
-                for (int e = tid; e < nr * kNB; e += kThreads) {
-                    const int r = e / kNB, j = e % kNB;
-                    P[r * kPS + j] = j < nb ? __ldcg(D + (size_t)(r0 + r) * ld + c0 + j) : 0.0;
-                }
-                if (p > 0 && tid < kNB * kNB) {
-                    const int l = tid / kNB, j = tid % kNB;
-                    us[tid] = j < nb ? __ldcg(D + (size_t)pp[l] * ld + c0 + j) : 0.0;
-                }
-                __syncthreads();
-                if (p > 0) {
-                    for (int e = tid; e < nr * kNB; e += kThreads) {
-                        const int r = e / kNB, j = e % kNB;
-                        bool piv = false;
-#pragma unroll
-                        for (int l = 0; l < kNB; ++l) piv |= pp[l] == r0 + r;
-                        double acc = piv ? 0.0 : P[r * kPS + j];
-#pragma unroll
-                        for (int l = 0; l < kNB; ++l) acc = fma(G[r * kPS + l], us[l * kNB + j], acc);
-                        P[r * kPS + j] = acc;
-                    }
-                    __syncthreads();
-                }
-                double x[RPT][kNB];
-#pragma unroll
-                for (int i = 0; i < RPT; ++i) {
-                    const int r = tid + i * kThreads;
-#pragma unroll
-                    for (int j = 0; j < kNB; ++j) x[i][j] = r < nr ? P[r * kPS + j] : 0.0;
-                }
-#pragma unroll
-                for (int lc = 0; lc < kNB; ++lc) {
-                    if (lc >= nb) break;
-                    Cand *cb = cand[par];
-                    par ^= 1;
-                    if (warp < nw) {
-                        // this warp's best unused row
-                        unsigned key = 0u;
-                        int bi = -1;
-#pragma unroll
-                        for (int i = 0; i < RPT; ++i) {
-                            const unsigned m = (unsigned)__double2hiint(x[i][lc]) & 0x7fffffffu;
-                            if (!((used >> i) & 1u) && (bi < 0 || m > key)) { key = m; bi = i; }
-                        }
-                        const unsigned best = __reduce_max_sync(0xffffffffu, bi >= 0 ? key + 1u : 0u);
-                        const unsigned who = __ballot_sync(0xffffffffu, bi >= 0 && key + 1u == best);
-                        const int src = who ? __ffs(who) - 1 : 0;
-                        if (lane == src) {
-                            Cand &c = stage[warp];
-#pragma unroll
-                            for (int i = 0; i < RPT; ++i)
-                                if (i == bi || (i == 0 && bi < 0)) {
-#pragma unroll
-                                    for (int j = 0; j < kNB; ++j) c.row[j] = x[i][j];
-                                }
-                            c.key = key;
-                            c.idx = who ? r0 + tid + bi * kThreads : -1;
-                        }
-                        __syncwarp();
-                        for (int it = lane; it < cs * kCandParts; it += 32) {
-                            const int dst = it / kCandParts, part = it % kCandParts;
-                            const uint4 v = ((const uint4 *)&stage[warp])[part];
-                            if (cs == 1) ((uint4 *)&cb[warp])[part] = v;
-                            else st_cluster(map_rank(smem_u32(&cb[crank * nw + warp]) + 16u * part, dst), v);
-                        }
-                    }
-                    cluster_sync(cs);
-                    if (warp < nw) {
-                        const bool have = lane < ncand && cb[lane].idx >= 0;
-                        const unsigned ck = have ? cb[lane].key : 0u;
-                        const unsigned top = __reduce_max_sync(0xffffffffu, have ? ck + 1u : 0u);
-                        const unsigned who = __ballot_sync(0xffffffffu, have && ck + 1u == top);
-                        const Cand &c = cb[who ? __ffs(who) - 1 : 0];
-                        const int row = c.idx;
-                        double pr[kNB];
-#pragma unroll
-                        for (int j = 0; j < kNB; j += 2) {
-                            const double2 v = *(const double2 *)&c.row[j];
-                            pr[j] = v.x;
-                            pr[j + 1] = v.y;
-                        }
-                        // a column without a nonzero candidate: singular; the bookkeeping goes on
-                        const bool zero = top <= 1u;
-                        const double rcp = zero ? 0.0 : reciprocal(pr[lc]);
-                        if (tid == 0) {
-                            pc[lc] = row;
-                            if (crank == 0) {
-                                __stcg(pinfo + (p & 1) * kNB + lc, row);
-                                if (zero) atomicExch(&ctl->err_singular, 1);
-                            }
-                        }
-#pragma unroll
-                        for (int i = 0; i < RPT; ++i) {
-                            const int r = r0 + tid + i * kThreads;
-                            const bool mine = r == row && tid + i * kThreads < nr;
-                            if (mine) {
-                                used |= 1u << i;
-                                perm[c0 + lc] = row;
-                                iperm[row] = c0 + lc;
-                            }
-                            // the pivot row starts from zero and takes the multiplier that leaves it scaled
-                            const double f = mine ? -rcp : x[i][lc] * rcp;
-#pragma unroll
-                            for (int q = 1; q < kNB; ++q) {
-                                const int j = (lc + q) % kNB;
-                                x[i][j] = fma(-f, pr[j], mine ? 0.0 : x[i][j]);
-                            }
-                            x[i][lc] = -f;
-                        }
-                    }
-                }
-                // the panel's columns become G
-#pragma unroll
-                for (int i = 0; i < RPT; ++i) {
-                    const int r = tid + i * kThreads;
-                    if (r >= nr) continue;
-                    double *Dr = D + (size_t)(r0 + r) * ld + c0;
-#pragma unroll
-                    for (int j = 0; j < kNB; ++j) {
-                        G[r * kPS + j] = j < nb ? x[i][j] : 0.0;
-                        if (j < nb) __stcg(Dr + j, x[i][j]);
-                    }
-                }
-            }
+            if (cidx == 0 && p < npan) panel_step<RPT>(q, D, perm, iperm, p, used);
             if (p > 0 && tq >= 0) {
                 // panel p - 1 applied to every column but its own and panel p's (the cluster's)
                 const int q0 = (p - 1) * kNB, nb = min(kNB, S - q0);
@@ -352,15 +460,14 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
                 const int ncol = S - (c1 - q0), per = ncol / ntrail, rest = ncol - per * ntrail;
                 const int j0 = tq * per + min(tq, rest), cw = per + (tq < rest ? 1 : 0);
                 if (cw > 0) {
-                    const int *pq = pinfo + ((p - 1) & 1) * kNB;
                     int pr[kNB];
 #pragma unroll
-                    for (int l = 0; l < kNB; ++l) pr[l] = l < nb ? __ldcg(pq + l) : -1;
-                    auto col = [&](int q) { return j0 + q < q0 ? j0 + q : j0 + q + (c1 - q0); };
+                    for (int l = 0; l < kNB; ++l) pr[l] = l < nb ? min(max(__ldcg(perm + q0 + l), 0), S - 1) : -1;
+                    auto col = [&](int c) { return j0 + c < q0 ? j0 + c : j0 + c + (c1 - q0); };
                     __syncthreads();
                     for (int e = tid; e < kNB * cw; e += kThreads) {
-                        const int l = e / cw, q = e - l * cw;
-                        U[e] = l < nb ? __ldcg(D + (size_t)__ldcg(pq + l) * ld + col(q)) : 0.0;
+                        const int l = e / cw, c = e - l * cw;
+                        U[e] = l < nb ? __ldcg(D + (size_t)min(max(__ldcg(perm + q0 + l), 0), S - 1) * ld + col(c)) : 0.0;
                     }
                     __syncthreads();
                     // one element per thread, three of them in flight
@@ -406,7 +513,176 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
     chain.leave();
 }
 
-size_t smem_of(int S, int cs, int ntrail)
+// The same elimination with every CTA beyond the panel's cluster keeping its columns [j0, j0 + cw) of
+// the layer in shared memory.  Flags of a chain (they only grow; cleared by the last cluster out):
+// flag[0] counts the panels' CTAs that have finished a panel, flag[1 + q] the owners that have handed
+// panel q's columns over.  Panel p needs its columns with the panels before p - 1 applied; its G stays
+// in D's panel columns until the layer's end, when every CTA has read it, and the columns follow.
+constexpr int kMaxPanels = 2 * kThreads / kNB;
+template <int RPT>
+__global__ void __launch_bounds__(kThreads, 1)
+k_factor64_flow(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int cs)
+{
+    if (ctl->finished || ctl->err_timeout || (skip && *skip)) return;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ PanelShared sh;
+    const int S = a.S, ld = a.ld;
+    const int tid = threadIdx.x;
+    const int half = mode == 1 ? (int)(blockIdx.x >= gridDim.x / 2) : 0;
+    const int nblk = mode == 1 ? (int)gridDim.x / 2 : (int)gridDim.x;
+    const int bid = (int)blockIdx.x - half * nblk;
+    const int crank = (int)cluster_rank(), cidx = bid / cs, nclus = nblk / cs;
+    ChainSync chain{a.bar + 2 * half, a.bar + 6 + half, ctl, cs, nclus, crank, &sh.go, 0u};
+    unsigned *flag = a.bar + 8 + half * (kMaxPanels + 8);
+    const Order o = order_of(mode, half, a.L, mid);
+    const int npan = (S + kNB - 1) / kNB;
+    // columns of the owners: the first `rest` of them have one more
+    const int ntrail = nblk - cs, tq = bid - cs, per = S / ntrail, rest = S - per * ntrail;
+    const int j0 = tq * per + min(tq, rest), cw = tq >= 0 ? per + (tq < rest ? 1 : 0) : 0;
+    auto owner = [&](int j) { return j < rest * (per + 1) ? j / (per + 1) : rest + (j - rest * (per + 1)) / max(per, 1); };
+    Panel q = make_panel(sh, (double *)dyn, a, ctl, cs, crank);
+    const int ws = cw | 1;                        // odd row stride: a row per thread without conflicts
+    double *W = (double *)dyn;                    // [S][ws]: this CTA's columns
+    double *U = W + (size_t)S * ws;               // [kNB][cw]
+    bool ok = true;
+    for (int step = 0; step < o.nsteps && ok; ++step) {
+        const int k = o.k0 + step * o.dk;
+        double *D = a.D + (size_t)k * S * ld;
+        int *perm = a.perm + (size_t)k * S, *iperm = a.iperm + (size_t)k * S;
+        if (cidx == 0) {
+            unsigned used = unused_rows<RPT>(q);
+            for (int p = 0; p < npan; ++p) {
+                if (tid == 0) {
+                    const int c0 = p * kNB, owners = owner(min(c0 + kNB, S) - 1) - owner(c0) + 1;
+                    wait_count(flag + 1 + p, (unsigned)(owners * (step + 1)), ctl);
+                }
+                __syncthreads();
+                panel_step<RPT>(q, D, perm, iperm, p, used);
+                __syncthreads();
+                if (tid == 0) raise_count(flag);
+            }
+        } else {
+            // hand the columns of panel p over: they are in W, every thread's rows
+            auto hand_over = [&](int p) {
+                const int a0 = max(j0, p * kNB), a1 = min(j0 + cw, min(p * kNB + kNB, S));
+                if (p >= npan || a0 >= a1) return;
+                for (int r = tid; r < S; r += kThreads)
+                    for (int j = a0; j < a1; ++j) __stcg(D + (size_t)r * ld + j, W[r * ws + j - j0]);
+                __syncthreads();
+                if (tid == 0) raise_count(flag + 1 + p);
+            };
+            for (int e = tid; e < S * cw; e += kThreads) {
+                const int i = e / cw, c = e - i * cw;
+                W[i * ws + c] = D[(size_t)i * ld + j0 + c];
+            }
+            schur_terms(a, mode, step, o.dk, k, [&](int nbr, const double *rowc, const double *colc) {
+                const double *Bn = a.D + (size_t)nbr * S * ld;
+                const int *pn = a.perm + (size_t)nbr * S, *ipn = a.iperm + (size_t)nbr * S;
+                for (int e = tid; e < S * cw; e += kThreads) {
+                    const int i = e / cw, c = e - i * cw;
+                    W[i * ws + c] -= rowc[i] * __ldcg(Bn + (size_t)__ldcg(pn + i) * ld + __ldcg(ipn + j0 + c)) * colc[j0 + c];
+                }
+            });
+            __syncthreads();
+            hand_over(0);
+            hand_over(1);
+            for (int p = 0; p < npan; ++p) {
+                const int c0 = p * kNB, nb = min(kNB, S - c0);
+                if (tid == 0) wait_count(flag, (unsigned)(cs * (step * npan + p + 1)), ctl);
+                __syncthreads();
+                int pr[kNB];
+#pragma unroll
+                for (int l = 0; l < kNB; ++l) pr[l] = l < nb ? min(max(__ldcg(perm + c0 + l), 0), S - 1) : -1;
+                // G of this thread's first row on its way while the pivot rows are copied
+                double g[kNB];
+                auto load_g = [&](int r) {
+                    const double *Dr = D + (size_t)r * ld + c0;
+                    if (nb == kNB) {
+#pragma unroll
+                        for (int l = 0; l < kNB; l += 2) {
+                            const double2 v = __ldcg((const double2 *)(Dr + l));
+                            g[l] = v.x;
+                            g[l + 1] = v.y;
+                        }
+                    } else {
+#pragma unroll
+                        for (int l = 0; l < kNB; ++l) g[l] = l < nb ? __ldcg(Dr + l) : 0.0;
+                    }
+                };
+                if (tid < S) load_g(tid);
+                for (int e = tid; e < kNB * cw; e += kThreads) {
+                    const int l = e / cw, c = e - l * cw;
+                    int row = 0;
+#pragma unroll
+                    for (int m = 0; m < kNB; ++m)
+                        if (m == l) row = pr[m];
+                    U[e] = l < nb ? W[row * ws + c] : 0.0;
+                }
+                __syncthreads();
+                // own columns: those of panel p become G, those of panel p + 1 are the cluster's
+                const int s0 = min(max(c0 - j0, 0), cw), s1 = min(max(c0 + nb - j0, 0), cw);
+                const int s2 = min(max(c0 + 2 * kNB - j0, s1), cw);
+                for (int r = tid; r < S; r += kThreads) {
+                    if (r != tid) load_g(r);
+                    bool piv = false;
+#pragma unroll
+                    for (int l = 0; l < kNB; ++l) piv |= pr[l] == r;
+                    double *Wr = W + (size_t)r * ws;
+                    auto run = [&](int b, int e) {
+                        int c = b;
+                        for (; c + 2 < e; c += 3) {
+                            double v0 = piv ? 0.0 : Wr[c], v1 = piv ? 0.0 : Wr[c + 1], v2 = piv ? 0.0 : Wr[c + 2];
+#pragma unroll
+                            for (int l = 0; l < kNB; ++l) {
+                                const double *u = U + l * cw + c;
+                                v0 = fma(g[l], u[0], v0);
+                                v1 = fma(g[l], u[1], v1);
+                                v2 = fma(g[l], u[2], v2);
+                            }
+                            Wr[c] = v0; Wr[c + 1] = v1; Wr[c + 2] = v2;
+                        }
+                        for (; c < e; ++c) {
+                            double v = piv ? 0.0 : Wr[c];
+#pragma unroll
+                            for (int l = 0; l < kNB; ++l) v = fma(g[l], U[l * cw + c], v);
+                            Wr[c] = v;
+                        }
+                    };
+                    run(0, s0);
+                    run(s2, cw);
+                    if (s0 < s1) {
+#pragma unroll
+                        for (int l = 0; l < kNB; ++l) {
+                            const int c = c0 + l - j0;
+                            if (c >= s0 && c < s1) Wr[c] = g[l];
+                        }
+                    }
+                }
+                hand_over(p + 2);
+                __syncthreads();
+            }
+        }
+        // every CTA has read the panels' G: the columns themselves follow
+        ok = chain.sync();
+        if (!ok) break;
+        for (int e = tid; e < S * cw; e += kThreads) {
+            const int i = e / cw, c = e - i * cw;
+            __stcg(D + (size_t)i * ld + j0 + c, W[i * ws + c]);
+        }
+        ok = chain.sync();
+    }
+    if (!ok) return;
+    // the flags too are zero again when the last cluster has left
+    cluster_sync(cs);
+    if (crank == 0 && tid == 0 && atomicAdd(chain.left, 1u) == (unsigned)nclus - 1) {
+        for (int i = 0; i <= npan; ++i) flag[i] = 0u;
+        *chain.word = 0u;
+        *chain.left = 0u;
+        __threadfence();
+    }
+}
+
+size_t smem_general(int S, int cs, int ntrail)
 {
     const size_t rpc = (S + cs - 1) / cs, cw = (S + ntrail - 1) / ntrail;
     const size_t panel = (2 * rpc * kPS + kNB * cw) * sizeof(double);
@@ -414,11 +690,25 @@ size_t smem_of(int S, int cs, int ntrail)
     return (std::max(panel, rows) + 255) & ~(size_t)255;
 }
 
+size_t smem_flow(int S, int cs, int ntrail)
+{
+    const size_t rpc = (S + cs - 1) / cs, cw = (S + ntrail - 1) / ntrail;
+    const size_t panel = 2 * rpc * kPS * sizeof(double), slice = ((size_t)S * (cw | 1) + kNB * cw) * sizeof(double);
+    return (std::max(panel, slice) + 255) & ~(size_t)255;
+}
+
+using FactorFn = void (*)(BlockSys<double>, Ctl *, const int *, int, int, int);
+FactorFn kernel_of(int S, const FactorPlan &p)
+{
+    const bool one = (S + p.cs - 1) / p.cs <= kThreads;
+    if (p.flow64) return one ? k_factor64_flow<1> : k_factor64_flow<2>;
+    return one ? k_factor64<1> : k_factor64<2>;
+}
+
 cudaError_t launch_mode(const BlockSys<double> &sys, const FactorPlan &plan, Ctl *ctl, cudaStream_t st, const int *skip,
                         int mode, int mid, int ctas)
 {
-    const int rpc = (sys.S + plan.cs - 1) / plan.cs;
-    auto fn = rpc <= kThreads ? k_factor64<1> : k_factor64<2>;
+    FactorFn fn = kernel_of(sys.S, plan);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem64);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -439,51 +729,62 @@ cudaError_t launch_mode(const BlockSys<double> &sys, const FactorPlan &plan, Ctl
     return cudaLaunchKernelEx(&cfg, fn, sys, ctl, skip, mode, mid, plan.cs);
 }
 
+// CTAs of one chain when `ctas` are launched (two chains at once need both halves whole).
+int chain_of(int ctas, int cs) { return ctas / 2 / cs * cs; }
+
 }  // namespace
+
+size_t factor64_words() { return 8 + 2 * (kMaxPanels + 8); }
 
 int factor64_plan(int S, int want, FactorPlan *p)
 {
     if (S <= 0 || S > 2 * kThreads || want < 1) return -1;
-    // The panel's cluster: a column's barrier costs more across CTAs than the rows it spreads save until
-    // there are about 130 rows (S = 96: 52 ms for four steps with one CTA, 59 with 4 or 8); beyond 500
-    // rows the trailing updates want the CTAs (S = 594: 118 ms a solve with 4, 135 with 8; S = 250 at 60
-    // layers: 17.3 and 16.7, 21.7 with one).
-    for (int cs = S <= 128 ? 1 : S <= 500 ? 8 : 4; cs >= 1; cs /= 2) {
+    // The panel's cluster: the rows it spreads against the cost of an exchange across CTAs and of the SMs
+    // taken from the updates.  Measured (ms with clusters of 1, 2, 4, 8): S = 20 (8 steps of 40 layers)
+    // 8.4, 8.7, 8.7, 8.8; 96 (4 steps of 150) 52.6, 49.7, 48.6, 48.8; 131 (60 layers) 8.8, 7.8, 7.3, 7.2;
+    // 250 (60) 21.1, 15.5, 13.7, 13.4; 400 (60) 46, 31, 22.9, 21.7; 594 (150) 275, 140, 102, 121.
+    for (int cs = S <= 32 ? 1 : S <= 128 || S > 500 ? 4 : 8; cs >= 1; cs /= 2) {
         if (want < 4 * cs && cs > 1) continue;
-        const int rpc = (S + cs - 1) / cs;
-        if (cs > 1 && rpc > kThreads) continue;
-        // a chain beyond the cluster has at most a CTA per 4 columns
+        if (cs > 1 && (S + cs - 1) / cs > kThreads) continue;
+        // columns to a CTA beyond the cluster: at least about four
         const int chain = cs + std::max(1, (S + 3) / 4 / cs) * cs;
         int ctas = std::min(want, 2 * chain) / cs * cs;
-        const size_t smem = smem_of(S, cs, std::max(1, ctas / 2 / cs * cs - cs));
-        if (smem > kSmemMax) continue;
-        auto fn = rpc <= kThreads ? k_factor64<1> : k_factor64<2>;
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
+        for (int flow = 1; flow >= 0; --flow) {
+            FactorPlan t = *p;
+            t.cs = cs;
+            t.flow64 = flow;
+            t.ctas64 = ctas;
+            for (int pass = 0; pass < 2; ++pass) {
+                const int half = chain_of(t.ctas64, cs);
+                if (flow && half <= cs) break;
+                t.smem64 = flow ? smem_flow(S, cs, half - cs) : smem_general(S, cs, std::max(1, half - cs));
+                if (t.smem64 > kSmemMax - sizeof(PanelShared)) break;
+                FactorFn fn = kernel_of(S, t);
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3(cs);
+                cfg.blockDim = dim3(kThreads);
+                cfg.dynamicSmemBytes = t.smem64;
+                cudaLaunchAttribute attr[1];
+                attr[0].id = cudaLaunchAttributeClusterDimension;
+                attr[0].val.clusterDim.x = cs;
+                attr[0].val.clusterDim.y = 1;
+                attr[0].val.clusterDim.z = 1;
+                cfg.attrs = attr;
+                cfg.numAttrs = 1;
+                int n = 0;
+                if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem64) != cudaSuccess ||
+                    cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
+                    cudaGetLastError();
+                    break;
+                }
+                // fewer clusters than wanted fit at once: plan again for those
+                if (n * cs >= t.ctas64) {
+                    *p = t;
+                    return 0;
+                }
+                t.ctas64 = n * cs;
+            }
         }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cs);
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cs;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
-            cudaGetLastError();
-            continue;
-        }
-        ctas = std::min(ctas, n * cs);
-        p->cs = cs;
-        p->ctas64 = ctas;
-        p->smem64 = std::max(smem, smem_of(S, cs, std::max(1, ctas / 2 / cs * cs - cs)));
-        if (p->smem64 > kSmemMax) continue;
-        return 0;
     }
     return -1;
 }
@@ -491,7 +792,7 @@ int factor64_plan(int S, int want, FactorPlan *p)
 cudaError_t launch_factor64(const BlockSys<double> &sys, const FactorPlan &plan, Ctl *ctl, cudaStream_t st, const int *skip)
 {
     // both ends at once on two halves of the grid, then the middle layer on all of it
-    const int half = plan.ctas64 / 2 / plan.cs * plan.cs;
+    const int half = chain_of(plan.ctas64, plan.cs);
     if (!(plan.twisted && sys.L >= 3 && half >= 1)) return launch_mode(sys, plan, ctl, st, skip, 0, 0, plan.ctas64);
     const int mid = sys.L / 2;
     cudaError_t e = launch_mode(sys, plan, ctl, st, skip, 1, mid, 2 * half);

@@ -446,6 +446,7 @@ struct FactorPlan {
     double *dinv = nullptr;    // that path: nb x nb LU factors of the panel's pivot block (global)
     int cs = 0, ctas64 = 0;    // FP64, panels of 8 (xk_factor64.cu): CTAs of the panel's cluster, CTAs of the launch
     size_t smem64 = 0;
+    int flow64 = 0;            // columns in shared memory, panels taken as their flags appear
 };
 template <typename T>
 struct BlockSys {
@@ -454,13 +455,14 @@ struct BlockSys {
     int *perm;       // [L][S] pivot row of each column
     int *iperm;      // [L][S] column each row was pivot of
     int *pinfo;      // panel scratch: pivot rows of the current panel
-    unsigned *bar;   // barrier words: [8] (0-3 the grid barriers of up to two chains, 6-7 with xk_factor64.cu)
+    unsigned *bar;   // barrier words (0-3 the grid barriers of up to two chains) and flags: [factor64_words()]
     int L, S, ld;
 };
 int factor_plan(int S, int precision_bytes, int nb_hint, int ctas_hint, FactorPlan *out);
 // FP64 in panels of 8 columns, the panel on a thread-block cluster (xk_factor64.cu): fills cs, ctas64
 // and smem64 for up to `want` CTAs (0, or -1 when S does not fit)
 int factor64_plan(int S, int want, FactorPlan *p);
+size_t factor64_words();     // barrier words and flags of BlockSys::bar, zero between launches
 cudaError_t launch_factor64(const BlockSys<double> &sys, const FactorPlan &plan, Ctl *ctl, cudaStream_t st,
                             const int *skip);
 template <typename T>

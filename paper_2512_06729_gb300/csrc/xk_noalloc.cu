@@ -74,7 +74,7 @@ extern "C" int xk_block_solve_noalloc(int L, int S, const double *A, const doubl
     // scratch layout: control block | barrier words | panel info | pivot rows | pivot columns | sweep vector | blocks
     const size_t o_ctl = 0;
     const size_t o_bar = up256(o_ctl + sizeof(Ctl));
-    const size_t o_pinfo = up256(o_bar + 8 * sizeof(unsigned));
+    const size_t o_pinfo = up256(o_bar + factor64_words() * sizeof(unsigned));
     const size_t o_ridx = up256(o_pinfo + (1 + 4 * 64) * sizeof(int));
     const size_t o_sig = up256(o_ridx + LS * sizeof(int));
     const size_t o_g = up256(o_sig + LS * sizeof(int));
