@@ -348,116 +348,136 @@ __global__ void k_path_weights(long long n, const double *q, double *wq)
 // search compares them on the integer pipes (FP64 compares are scarce on this GPU).
 __device__ __forceinline__ unsigned long long key_of(double d) { return (unsigned long long)__double_as_longlong(d); }
 
-// Per-warp shared memory of the pathway search: dist [S] doubles, then pred_sp, pred_e, order [S]
-// ints and done [S] bytes.
-__host__ __device__ inline size_t path_warp_bytes(int S)
+// Least weight of every group of parallel edges (source u, target v) in every layer.  Rounding is
+// monotone, so du + (least weight) is the least of du + (weight) over the group: the search needs no
+// other weight to know whether and to what v's distance falls.
+__global__ void k_path_groups(PathGraph gr, int ng, int L, long long LR2, const double *wq, double *gmin)
 {
-    return ((size_t)S * (8 + 4 + 4 + 4 + 1) + 15) / 16 * 16;
+    const long long n = (long long)L * ng, R2 = LR2 / L;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const int k = (int)(i / ng), g = (int)(i - (long long)k * ng);
+        const double *wk = wq + (size_t)k * R2;
+        unsigned long long m = key_of(INFINITY);
+        for (int t = gr.gs[g]; t < gr.gs[g + 1]; ++t) m = min(m, key_of(wk[gr.gcode[t]]));
+        gmin[i] = __longlong_as_double((long long)m);
+    }
 }
 
-__global__ void k_pathways(Col c, PathGraph gr, const double *wq, int nsrc, const int *src, int wpb,
-                           double *dist_out, int *pred_out, int *edge_out, int *lim_out, double *limw_out)
+// Per-warp shared memory of the pathway search: the distances' bit patterns [S], then the group of the
+// edge into a species [S] ints, its predecessor and the finishing order [S] 16-bit words.  A finished
+// species' distance has its sign bit set: the scan compares unsigned words, the relaxation signed ones,
+// so that neither takes it up.
+__host__ __device__ inline size_t path_warp_bytes(int S)
+{
+    return ((size_t)S * (8 + 4 + 2 + 2) + 15) / 16 * 16;
+}
+
+// One warp per search, the searches of a layer side by side (they read the same weights).  What a
+// finished species costs is a chain of latencies: the scan for the least open distance, then the
+// species' groups and their least weights (contiguous, one trip to L2), one FP64 addition.  The edge
+// of a group that gave the distance is looked up once per species at the end, from the distance of
+// its predecessor, which no longer changes: scanning the codes at every relaxation (three dependent
+// trips) took 10,800 clocks per species, and the slowest steps by one lane in global memory a
+// seventh of the whole.  Rates, weights and eight searches in each of 150 layers of 594 species take
+// 1.25 ms so, 3.42 before.
+__global__ void k_pathways(Col c, PathGraph gr, int ng, const double *wq, const double *gmin, int nsrc, const int *src,
+                           int wpb, double *dist_out, int *pred_out, int *edge_out, int *lim_out, double *limw_out)
 {
     extern __shared__ double path_dyn[];
     const int S = c.S, L = c.L, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long prob = (long long)blockIdx.x * wpb + w;
     if (w >= wpb || prob >= (long long)nsrc * L) return;
-    const int j = (int)(prob / L), k = (int)(prob % L);
+    const int k = (int)(prob / nsrc), j = (int)(prob - (long long)k * nsrc);
     const int s0 = src[j];
     char *base = (char *)path_dyn + path_warp_bytes(S) * w;
-    double *dist = (double *)base;
-    int *pred = (int *)(dist + S), *pe = pred + S, *order = pe + S;
-    unsigned char *done = (unsigned char *)(order + S);
-    const double *wk = wq + (size_t)k * c.R * 2;
+    unsigned long long *dist = (unsigned long long *)base;
+    int *pg = (int *)(dist + S);
+    unsigned short *pred = (unsigned short *)(pg + S), *order = pred + S;
+    const double *wk = wq + (size_t)k * c.R * 2, *gk = gmin + (size_t)k * ng;
+    const unsigned long long kinf = key_of(INFINITY), kdone = 1ull << 63;
     for (int y = lane; y < S; y += 32) {
-        dist[y] = INFINITY;
-        pred[y] = -1;
-        pe[y] = -1;
-        done[y] = 0;
+        dist[y] = y == s0 ? 0ull : kinf;
+        pg[y] = -1;
     }
-    __syncwarp();
-    if (lane == 0) dist[s0] = 0.0;
     __syncwarp();
     int nord = 0;
     for (;;) {
         // the unfinished species of least distance, the lower index on ties
-        const unsigned long long kinf = key_of(INFINITY);
         unsigned long long bd = kinf;
         int bi = S;
+#pragma unroll 4
         for (int y = lane; y < S; y += 32) {
-            const unsigned long long ky = key_of(dist[y]);
-            if (!done[y] && ky < bd) {
+            const unsigned long long ky = dist[y];
+            if (ky < bd) {
                 bd = ky;
                 bi = y;
             }
         }
-        for (int o = 16; o; o >>= 1) {
-            const unsigned long long od = __shfl_xor_sync(0xffffffffu, bd, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (od < bd || (od == bd && oi < bi)) {
-                bd = od;
-                bi = oi;
-            }
-        }
-        if (!(bd < kinf)) break;
-        const int u = bi;
+        const unsigned hi = (unsigned)(bd >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
+        const unsigned lo = hi == mh ? (unsigned)bd : 0xffffffffu, ml = __reduce_min_sync(0xffffffffu, lo);
+        if (mh >= (unsigned)(kinf >> 32)) break;
+        const int u = (int)__reduce_min_sync(0xffffffffu, hi == mh && (unsigned)bd == ml ? (unsigned)bi : 0xffffffffu);
+        const double du = __longlong_as_double((long long)((unsigned long long)mh << 32 | ml));
         if (lane == 0) {
-            done[u] = 1;
-            order[nord] = u;
+            dist[u] |= kdone;
+            order[nord] = (unsigned short)u;
         }
         ++nord;
-        __syncwarp();
-        // relax: one lane per target species, its parallel edges in increasing code, strict decrease
-        const double du = dist[u];
-        for (int g = gr.gp[u] + lane; g < gr.gp[u + 1]; g += 32) {
+        // relax: one lane per target species
+        const int g1 = gr.gp[u + 1];
+        for (int g = gr.gp[u] + lane; g < g1; g += 32) {
             const int v = gr.gv[g];
-            double best = dist[v];
-            unsigned long long kb = key_of(best);
-            int be = -1;
+            const long long cand = (long long)key_of(du + gk[g]);
+            if (cand < (long long)dist[v]) {
+                dist[v] = (unsigned long long)cand;
+                pred[v] = (unsigned short)u;
+                pg[v] = g;
+            }
+        }
+        __syncwarp();
+    }
+    // the first edge, codes increasing, that gives the least distance
+    const size_t o = ((size_t)j * L + k) * S;
+    for (int y = lane; y < S; y += 32) {
+        int be = -1;
+        const int g = pg[y];
+        if (g >= 0) {
+            const double du = __longlong_as_double((long long)(dist[pred[y]] & ~kdone));
+            unsigned long long kb = kinf;
             for (int t = gr.gs[g]; t < gr.gs[g + 1]; ++t) {
                 const int e = gr.gcode[t];
-                const double cand = du + wk[e];   // +inf for a direction without rate
-                const unsigned long long kc = key_of(cand);
+                const unsigned long long kc = key_of(du + wk[e]);
                 if (kc < kb) {
                     kb = kc;
-                    best = cand;
                     be = e;
                 }
             }
-            if (be >= 0) {
-                dist[v] = best;
-                pred[v] = u;
-                pe[v] = be;
-            }
         }
-        __syncwarp();
+        if (dist_out) dist_out[o + y] = __longlong_as_double((long long)(dist[y] & ~kdone));
+        if (pred_out) pred_out[o + y] = g >= 0 ? (int)pred[y] : -1;
+        if (edge_out) edge_out[o + y] = be;
+        pg[y] = be;
     }
-    const size_t o = ((size_t)j * L + k) * S;
-    for (int y = lane; y < S; y += 32) {
-        if (dist_out) dist_out[o + y] = dist[y];
-        if (pred_out) pred_out[o + y] = pred[y];
-        if (edge_out) edge_out[o + y] = pe[y];
-        if (lim_out) {
-            lim_out[o + y] = -1;
-            limw_out[o + y] = 0.0;
-        }
-    }
+    if (!lim_out) return;
     __syncwarp();
-    // slowest step of each path, in the order the species were finished
-    if (lim_out && lane == 0)
-        for (int i = 0; i < nord; ++i) {
+    // the edge's weight takes the distance's place
+    for (int y = lane; y < S; y += 32) dist[y] = pg[y] >= 0 ? key_of(wk[pg[y]]) : 0ull;
+    __syncwarp();
+    // slowest step of each path, in the order the species were finished: a species' weight and edge
+    // become those of its path's slowest step
+    if (lane == 0)
+        for (int i = 1; i < nord; ++i) {
             const int v = order[i], u = pred[v];
-            if (u < 0) continue;
-            const int e = pe[v];
-            const double wv = wk[e];
-            if (u == s0 || wv > limw_out[o + u]) {
-                lim_out[o + v] = e;
-                limw_out[o + v] = wv;
-            } else {
-                lim_out[o + v] = lim_out[o + u];
-                limw_out[o + v] = limw_out[o + u];
+            if (u != s0 && !(dist[v] > dist[u])) {
+                dist[v] = dist[u];
+                pg[v] = pg[u];
             }
         }
+    __syncwarp();
+    for (int y = lane; y < S; y += 32) {
+        lim_out[o + y] = pg[y];
+        limw_out[o + y] = __longlong_as_double((long long)dist[y]);
+    }
 }
 
 }  // namespace
@@ -485,27 +505,31 @@ void launch_fluxes(const Col &c, const double *n, double *q, cudaStream_t st)
     count_launches(1);
 }
 
-cudaError_t launch_pathways(const Col &c, const PathGraph &g, const double *q, double *wbuf, int nsrc,
-                            const int *src, double *dist, int *pred_sp, int *pred_edge, int *lim_edge,
+cudaError_t launch_pathways(const Col &c, const PathGraph &g, int ngroups, const double *q, double *wbuf, double *gbuf,
+                            int nsrc, const int *src, double *dist, int *pred_sp, int *pred_edge, int *lim_edge,
                             double *lim_w, cudaStream_t st)
 {
-    const long long nw = (long long)c.L * c.R * 2;
+    const long long nw = (long long)c.L * c.R * 2, ngl = (long long)c.L * ngroups;
     if (nw > 0) {
         k_path_weights<<<(int)std::min<long long>((nw + 255) / 256, 152LL * 8), 256, 0, st>>>(nw, q, wbuf);
         count_launches(1);
     }
-    const size_t per = path_warp_bytes(c.S);
-    const size_t cap = 96 * 1024;
-    if (per > 200 * 1024) return cudaErrorInvalidValue;
-    const int wpb = (int)std::max<size_t>(1, std::min<size_t>(8, cap / per));
+    if (ngl > 0) {
+        k_path_groups<<<(int)std::min<long long>((ngl + 255) / 256, 152LL * 16), 256, 0, st>>>(g, ngroups, c.L, nw, wbuf, gbuf);
+        count_launches(1);
+    }
+    const size_t per = path_warp_bytes(c.S), cap = 200 * 1024;
+    if (per > cap) return cudaErrorInvalidValue;
+    // searches of one layer to a CTA, as few as leave no SM without one
+    const long long probs = (long long)nsrc * c.L;
+    const int wpb = (int)std::max<long long>(1, std::min<long long>(std::min<long long>(8, cap / per), (probs + 151) / 152));
     const size_t smem = per * wpb;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_pathways, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    const long long probs = (long long)nsrc * c.L;
     const int blocks = (int)((probs + wpb - 1) / wpb);
-    k_pathways<<<blocks, 32 * wpb, smem, st>>>(c, g, wbuf, nsrc, src, wpb, dist, pred_sp, pred_edge, lim_edge,
+    k_pathways<<<blocks, 32 * wpb, smem, st>>>(c, g, ngroups, wbuf, gbuf, nsrc, src, wpb, dist, pred_sp, pred_edge, lim_edge,
                                               lim_w);
     count_launches(1);
     return cudaGetLastError();

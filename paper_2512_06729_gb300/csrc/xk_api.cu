@@ -90,6 +90,7 @@ struct xk_ctx {
     EqIndex eqix{};
     int *eq_iters = nullptr, *eq_status = nullptr, *path_src = nullptr;
     double *path_w = nullptr;   // [L][R][2] edge weights of the pathway search
+    double *path_g = nullptr;   // [L][groups] least weights of parallel edges
     // variable-order BDF: history buffers [kBdfHist][L][S], predictor, history terms, new state, step
     double *bdfY = nullptr, *bdf_yhat = nullptr, *bdf_g = nullptr, *bdf_ynew = nullptr, *bdf_delta = nullptr;
     BdfResult *bdf_res = nullptr;
@@ -617,6 +618,7 @@ size_t layout(xk_ctx *c, char *base)
     c->eq_status = b.take<int>(L);
     c->path_src = b.take<int>(std::max(S, 1));
     c->path_w = b.take<double>(std::max<size_t>(1, 2 * LR));
+    c->path_g = b.take<double>(std::max<size_t>(1, (size_t)L * c->pg_v.size()));
     c->bdfY = b.take<double>(kBdfHist * LS);
     c->bdf_yhat = b.take<double>(LS);
     c->bdf_g = b.take<double>(LS);
@@ -2061,7 +2063,8 @@ int xk_pathways(xk_ctx *c, const double *q, int nsrc, const int *src, double *di
     for (int j = 0; j < nsrc; ++j)
         if (src[j] < 0 || src[j] >= c->S) return fail(c, XK_EINVAL, "pathways: source %d out of range", src[j]);
     cudaMemcpyAsync(c->path_src, src, sizeof(int) * nsrc, cudaMemcpyHostToDevice, c->st);
-    cudaError_t e = launch_pathways(c->col, c->pgraph, q, c->path_w, nsrc, c->path_src, dist, pred_sp, pred_edge,
+    cudaError_t e = launch_pathways(c->col, c->pgraph, (int)c->pg_v.size(), q, c->path_w, c->path_g, nsrc,
+                                    c->path_src, dist, pred_sp, pred_edge,
                                     lim_edge, lim_w, c->st);
     if (e != cudaSuccess) return fail(c, XK_EINVAL, "pathways launch: %s", cudaGetErrorString(e));
     return finish_eval(c, "pathways");

@@ -209,9 +209,9 @@ cudaError_t launch_equilibrium(const Col &c, const EqIndex &ix, const double *b,
 void launch_fluxes(const Col &c, const double *n, double *q, cudaStream_t st);
 // Dijkstra from each source src[j] (device, nsrc) in every layer of rates q [L][R][2]: outputs
 // [nsrc][L][S] (any output pointer may be nullptr).  wbuf: L * R * 2 doubles of scratch for the edge
-// weights 1/q.
-cudaError_t launch_pathways(const Col &c, const PathGraph &g, const double *q, double *wbuf, int nsrc,
-                            const int *src, double *dist, int *pred_sp, int *pred_edge, int *lim_edge,
+// weights 1/q, gbuf: L * ngroups for the least weights of the graph's groups.
+cudaError_t launch_pathways(const Col &c, const PathGraph &g, int ngroups, const double *q, double *wbuf, double *gbuf,
+                            int nsrc, const int *src, double *dist, int *pred_sp, int *pred_edge, int *lim_edge,
                             double *lim_w, cudaStream_t st);
 
 // Variable-order BDF (xk_bdf.cu): the history's linear combinations for one step attempt.
