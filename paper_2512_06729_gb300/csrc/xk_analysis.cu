@@ -5,9 +5,9 @@
 // T and P for given element totals.  The unknowns are ln N_y of every species, the total ln N and
 // one potential pi_e per element; each Newton iteration reduces to an (E+1) x (E+1) system (the
 // reduced Gibbs iteration of the NASA equilibrium program, Gordon & McBride 1994).  The species
-// loop (exp, chemical potentials, the update) is spread over the CTA's threads, each of the
-// system's sums over species is taken by one thread in species order, and one warp solves the
-// small system with partial pivoting.  At convergence the mole fractions are rebuilt from the
+// loop (exp, chemical potentials, the update) is spread over the CTA's threads, the system's sums
+// over species over its lanes in sublists of fixed order, and one warp solves the small system with
+// partial pivoting.  At convergence the mole fractions are rebuilt from the
 // potentials, x_y = exp(sum_e pi_e a_ey - G_y/RT - ln P), so trace species keep full relative
 // accuracy however small.
 //
@@ -31,60 +31,39 @@ constexpr int kEqMaxE = 31;              // E + 1 rows of the Newton system fit 
 constexpr double kLnMajor = -18.420680743952367;   // ln 1e-8: species above this fraction are "major"
 constexpr double kTraceCap = 9.2103;               // a trace species may rise to about 1e-4 of N per step
 
+constexpr int kEqWarps = kEqThreads / 32;
+
 struct EqShared {
     double A[kEqMaxE + 1][kEqMaxE + 2];  // the (E+1) x (E+1) system with its right-hand side
     double sol[kEqMaxE + 1];
     double bk[kEqMaxE];
-    double red[3][kEqThreads / 32];
-    double lntot, bsum, sn, snm;
-    int eact[kEqMaxE];
-    int done, singular, nact;
+    double red[2][kEqWarps];
+    unsigned long long kred[2][kEqWarps];
+    double lntot, bsum;
+    int eact[kEqMaxE], ired[kEqWarps];
+    int singular;
 };
 
-__device__ __forceinline__ double warp_max(double v)
-{
-    for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ double warp_min(double v)
-{
-    for (int o = 16; o; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
 __device__ __forceinline__ double warp_sum(double v)
 {
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-// Block-wide reduction of three values (max, min, sum) with one barrier pair; every thread gets them.
-__device__ void block_reduce3(EqShared &sh, double &mx, double &mn, double &sm)
+// Largest (least) bit pattern of the warp: non-negative doubles order like them, and two integer
+// reductions take a tenth of an FP64 comparison tree.
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    mx = warp_max(mx);
-    mn = warp_min(mn);
-    sm = warp_sum(sm);
-    if (lane == 0) {
-        sh.red[0][w] = mx;
-        sh.red[1][w] = mn;
-        sh.red[2][w] = sm;
-    }
-    __syncthreads();
-    mx = -INFINITY;
-    mn = INFINITY;
-    sm = 0.0;
-    for (int i = 0; i < nw; ++i) {   // same order in every thread: identical results everywhere
-        mx = fmax(mx, sh.red[0][i]);
-        mn = fmin(mn, sh.red[1][i]);
-        sm += sh.red[2][i];
-    }
-    __syncthreads();
+    const unsigned h = (unsigned)(k >> 32), mh = __reduce_max_sync(0xffffffffu, h);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, h == mh ? (unsigned)k : 0u);
+    return (unsigned long long)mh << 32 | ml;
 }
+__device__ __forceinline__ unsigned long long key_of(double d) { return (unsigned long long)__double_as_longlong(d); }
 
 // Block-wide sums of two values, the same in every thread.
 __device__ void block_sum2(EqShared &sh, double &a, double &b)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     a = warp_sum(a);
     b = warp_sum(b);
     if (lane == 0) {
@@ -92,77 +71,81 @@ __device__ void block_sum2(EqShared &sh, double &a, double &b)
         sh.red[1][w] = b;
     }
     __syncthreads();
-    a = 0.0;
-    b = 0.0;
-    for (int i = 0; i < nw; ++i) {
-        a += sh.red[0][i];
-        b += sh.red[1][i];
-    }
+    // both sums in one tree: lanes 0 .. 7 the first, 8 .. 15 the second
+    double v = lane < 2 * kEqWarps ? sh.red[lane / kEqWarps][lane % kEqWarps] : 0.0;
+    for (int o = kEqWarps / 2; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    a = __shfl_sync(0xffffffffu, v, 0);
+    b = __shfl_sync(0xffffffffu, v, kEqWarps);
     __syncthreads();
 }
 
-// Gaussian elimination with partial pivoting of the M x (M+1) augmented system on warp 0: lane r
-// owns row r; the pivot is the first row of largest magnitude in the column.
-__device__ void warp_solve(EqShared &sh, int M)
+// Gauss-Jordan with implicit partial pivoting of the M x (M+1) augmented system on the first four
+// warps, one to each FP64 unit of the SM: lane r stands for row r, warp w updates the columns j = w
+// (mod 4), pivot and multipliers are found by all four alike.  Eliminating above the pivot costs no
+// more instructions than below and leaves no back substitution (M (M+1) / 2 dependent results on one
+// lane before).  The pivot is the unused row of largest magnitude by its high word, the first among
+// equals.  Column c is only read in step c, so one barrier per step does.
+constexpr int kSolveWarps = 4;
+__device__ void warps_solve(EqShared &sh, int M)
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, wrp = threadIdx.x >> 5;
+    bool used = lane >= M;
+    int mycol = 0;
+    double myrcp = 0.0;
     for (int c = 0; c < M; ++c) {
-        double v = (lane >= c && lane < M) ? fabs(sh.A[lane][c]) : -1.0;
-        int idx = lane;
-        for (int o = 16; o; o >>= 1) {
-            const double ov = __shfl_xor_sync(0xffffffffu, v, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-            if (ov > v || (ov == v && oi < idx)) {
-                v = ov;
-                idx = oi;
-            }
-        }
-        if (!(v > 0.0)) {
+        const double v = lane < M ? sh.A[lane][c] : 0.0;
+        const unsigned key = used ? 0u : (unsigned)__double2hiint(v) & 0x7fffffffu;
+        const unsigned top = __reduce_max_sync(0xffffffffu, key);
+        if (top == 0u || top > 0x7ff00000u) {          // nothing left, or not a number: in all four warps
             if (lane == 0) sh.singular = 1;
-            __syncwarp();
             return;
         }
-        if (idx != c && lane <= M) {
-            const double t = sh.A[c][lane];
-            sh.A[c][lane] = sh.A[idx][lane];
-            sh.A[idx][lane] = t;
+        const int p = __ffs(__ballot_sync(0xffffffffu, !used && key == top)) - 1;
+        const double rcp = reciprocal64(sh.A[p][c]);
+        if (lane == p) {
+            used = true;
+            mycol = c;
+            myrcp = rcp;
         }
-        __syncwarp();
-        if (lane > c && lane < M) {
-            const double l = sh.A[lane][c] / sh.A[c][c];
-            for (int j = c; j <= M; ++j) sh.A[lane][j] -= l * sh.A[c][j];
+        if (lane < M && lane != p) {
+            const double l = -(v * rcp);
+            for (int j = c + 1 + ((wrp - c - 1) & (kSolveWarps - 1)); j <= M; j += kSolveWarps)
+                sh.A[lane][j] = fma(l, sh.A[p][j], sh.A[lane][j]);
         }
-        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kSolveWarps) : "memory");
     }
-    if (lane == 0)
-        for (int i = M - 1; i >= 0; --i) {
-            double s = sh.A[i][M];
-            for (int j = i + 1; j < M; ++j) s -= sh.A[i][j] * sh.sol[j];
-            sh.sol[i] = s / sh.A[i][i];
-        }
-    __syncwarp();
+    if (wrp == 0 && lane < M) sh.sol[mycol] = sh.A[lane][M] * myrcp;
 }
 
-// Dynamic shared memory: lnN, nj, mu [S] doubles, then the activity flags [S] as bytes.
+// Dynamic shared memory: lnN, nj, mu [S] doubles, the entries' parts [2 nsub] doubles (sums of nj and
+// of nj mu), then the activity flags [S] as bytes.  Bound by FP64 latency and issue (a warp instruction
+// holds its unit some 75 clocks, a dependent one waits some 180): per iteration the exponentials, then
+// the system's chain of M pivots.  At 594 species x 150 layers an iteration takes 25 us; with one thread
+// to an entry (the longest some 550 terms), divisions and a back substitution on one lane it took 110.
 __global__ void __launch_bounds__(kEqThreads) k_equilibrium(Col c, EqIndex ix, const double *b, double *x,
                                                              double *nout, int max_iter, double tol, int *iters,
                                                              int *status)
 {
     __shared__ EqShared sh;
     extern __shared__ double eq_dyn[];
-    const int S = c.S, E = c.E, M = c.E + 1, k = blockIdx.x, tid = threadIdx.x;
-    double *lnN = eq_dyn, *nj = lnN + S, *mu = nj + S;
-    unsigned char *act = (unsigned char *)(mu + S);
+    const int S = c.S, E = c.E, M = c.E + 1, k = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wrp = tid >> 5;
+    double *lnN = eq_dyn, *nj = lnN + S, *mu = nj + S, *part = mu + S;
+    unsigned char *act = (unsigned char *)(part + 2 * ix.nsub);
     const double *g = c.grt + (size_t)k * S;
     const double lnP = log(c.P[k]);
 
-    if (tid < E) {
+    // element totals: a warp per element
+    for (int e = wrp; e < E; e += kEqWarps) {
         double v = 0.0;
-        if (b) v = b[(size_t)k * E + tid];
-        else
-            for (int y = 0; y < S; ++y) v += (double)c.elem[y * E + tid] * c.n[(size_t)k * S + y];
-        sh.bk[tid] = v;
-        sh.eact[tid] = v > 0.0;
+        if (b) v = b[(size_t)k * E + e];
+        else {
+            for (int y = lane; y < S; y += 32) v += (double)c.elem[y * E + e] * c.n[(size_t)k * S + y];
+            v = warp_sum(v);
+        }
+        if (lane == 0) {
+            sh.bk[e] = v;
+            sh.eact[e] = v > 0.0;
+        }
     }
     __syncthreads();
     if (tid == 0) {
@@ -171,20 +154,21 @@ __global__ void __launch_bounds__(kEqThreads) k_equilibrium(Col c, EqIndex ix, c
             if (sh.eact[e]) s += sh.bk[e];
         sh.bsum = s;
         sh.lntot = 0.0;
-        sh.done = 0;
         sh.singular = 0;
     }
     int cnt = 0;
-    for (int y = tid; y < S; y += blockDim.x) {
+    for (int y = tid; y < S; y += kEqThreads) {
         int on = 1;
         for (int q = ix.sp[y]; q < ix.sp[y + 1]; ++q)
             if (!sh.eact[ix.se[q]]) on = 0;
         act[y] = (unsigned char)on;
         cnt += on;
     }
-    double d0 = -INFINITY, d1 = INFINITY, d2 = cnt;
-    block_reduce3(sh, d0, d1, d2);
-    const int nact = (int)d2;
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) sh.ired[wrp] = cnt;
+    __syncthreads();
+    int nact = 0;
+    for (int i = 0; i < kEqWarps; ++i) nact += sh.ired[i];
     if (nact == 0 || !(sh.bsum > 0.0)) {
         if (tid == 0) {
             iters[k] = 0;
@@ -192,36 +176,52 @@ __global__ void __launch_bounds__(kEqThreads) k_equilibrium(Col c, EqIndex ix, c
         }
         return;
     }
-    for (int y = tid; y < S; y += blockDim.x) lnN[y] = act[y] ? log(1.0 / nact) : 0.0;
+    for (int y = tid; y < S; y += kEqThreads) {
+        lnN[y] = act[y] ? log(1.0 / nact) : 0.0;
+        if (!act[y]) nj[y] = mu[y] = 0.0;
+    }
     __syncthreads();
 
-    int it = 0;
+    int it = 0, done = 0;
     for (; it < max_iter; ++it) {
-        const double lntot = sh.lntot, ntot = exp(lntot);
+        const double lntot = sh.lntot, ntot = exp(lntot), shift = lnP - lntot;
         double sn = 0.0, snm = 0.0;
-        for (int y = tid; y < S; y += blockDim.x) {
-            if (act[y]) {
-                nj[y] = exp(lnN[y]);
-                mu[y] = g[y] + lnP + lnN[y] - lntot;
-            } else {
-                nj[y] = 0.0;
-                mu[y] = 0.0;
-            }
-            sn += nj[y];
-            snm += nj[y] * mu[y];
+        for (int y = tid; y < S; y += kEqThreads) {
+            if (!act[y]) continue;
+            const double n = exp(lnN[y]), m = g[y] + lnN[y] + shift;
+            const double nm = n * m;
+            nj[y] = n;
+            mu[y] = nm;
+            sn += n;
+            snm += nm;
         }
         // the system starts from zero (pairs of elements no species shares stay zero)
-        for (int t = tid; t < M * (M + 1); t += blockDim.x) sh.A[t / (M + 1)][t % (M + 1)] = 0.0;
+        for (int t = tid; t < M * (M + 1); t += kEqThreads) sh.A[t / (M + 1)][t % (M + 1)] = 0.0;
         block_sum2(sh, sn, snm);
-        // each entry's sparse sum over the species holding its elements, in species order
-        for (int t = tid; t < ix.nent; t += blockDim.x) {
+        // each entry's sublists, a lane each; element sums take nj mu along
+        for (int q = wrp; q < ix.ngrp; q += kEqWarps) {
+            double sv = 0.0, dv = 0.0;
+            for (int r = ix.gp[q]; r < ix.gp[q + 1]; ++r) {
+                const int y = ix.ent[32 * r + lane];
+                if (y >= 0) {
+                    const double a = ix.ec[32 * r + lane];
+                    sv = fma(a, nj[y], sv);
+                    dv = fma(a, mu[y], dv);
+                }
+            }
+            const int to = ix.part[32 * q + lane];
+            if (to >= 0) {
+                part[to] = sv;
+                part[ix.nsub + to] = dv;
+            }
+        }
+        __syncthreads();
+        for (int t = tid; t < ix.nent; t += kEqThreads) {
             const int code = ix.eij[t];
             double sv = 0.0, dv = 0.0;
             for (int q = ix.ep[t]; q < ix.ep[t + 1]; ++q) {
-                const int y = ix.ey[q];
-                const double v = ix.ec[q] * nj[y];
-                sv += v;
-                if (code < 0) dv += v * mu[y];
+                sv += part[q];
+                if (code < 0) dv += part[ix.nsub + q];
             }
             if (code >= 0) {
                 const int i = code >> 5, j = code & 31;
@@ -240,40 +240,56 @@ __global__ void __launch_bounds__(kEqThreads) k_equilibrium(Col c, EqIndex ix, c
         }
         if (tid == 0) {
             sh.A[E][E] = sn - ntot;
-            sh.sn = sn;
-            sh.snm = snm;
+            sh.A[E][M] = ntot - sn + snm;
         }
         __syncthreads();
         if (tid < E && !sh.eact[tid]) sh.A[tid][tid] = 1.0;
-        if (tid == 0) sh.A[E][M] = ntot - sh.sn + sh.snm;
         __syncthreads();
-        if (tid < 32) warp_solve(sh, M);
+        if (wrp < kSolveWarps) warps_solve(sh, M);
         __syncthreads();
         if (sh.singular) break;
         const double dlntot = sh.sol[E];
-        // step limit and convergence measure
-        double big = 5.0 * fabs(dlntot), lam2 = 1.0, conv = 0.0;
-        for (int y = tid; y < S; y += blockDim.x) {
+        // step limit (the largest of non-negative values by their bit patterns) and convergence measure
+        unsigned long long big = key_of(5.0 * fabs(dlntot)), rise = 0ull;
+        double conv = 0.0;
+        for (int y = tid; y < S; y += kEqThreads) {
             if (!act[y]) continue;
-            double d = -mu[y] + dlntot;
-            for (int q = ix.sp[y]; q < ix.sp[y + 1]; ++q) d += sh.sol[ix.se[q]] * ix.sc[q];
+            double d = dlntot - (g[y] + lnN[y] + shift);
+            for (int q = ix.sp[y]; q < ix.sp[y + 1]; ++q) d = fma(sh.sol[ix.se[q]], ix.sc[q], d);
             mu[y] = d;
             const double lx = lnN[y] - lntot;
-            if (lx > kLnMajor) big = fmax(big, fabs(d));
-            else if (d - dlntot > 0.0) lam2 = fmin(lam2, fabs((-lx - kTraceCap) / (d - dlntot)));
-            conv += nj[y] * fabs(d);
+            const unsigned long long kd = key_of(d) & 0x7fffffffffffffffull;
+            // ln x is negative at these magnitudes: above ln 1e-8 means a smaller bit pattern
+            if (!(lx < 0.0) || key_of(lx) < key_of(kLnMajor)) big = max(big, kd);
+            else if (d - dlntot > 0.0)
+                rise = max(rise, key_of((d - dlntot) * reciprocal64(-lx - kTraceCap)) & 0x7fffffffffffffffull);
+            conv = fma(nj[y], __longlong_as_double((long long)kd), conv);
         }
-        block_reduce3(sh, big, lam2, conv);
-        conv /= sh.sn;
-        double lam = big > 2.0 ? 2.0 / big : 1.0;
-        lam = fmin(lam, lam2);
-        for (int y = tid; y < S; y += blockDim.x)
-            if (act[y]) lnN[y] += lam * mu[y];
+        big = warp_max_key(big);
+        rise = warp_max_key(rise);
+        conv = warp_sum(conv);
+        if (lane == 0) {
+            sh.kred[0][wrp] = big;
+            sh.kred[1][wrp] = rise;
+            sh.red[0][wrp] = conv;
+        }
+        __syncthreads();
+        conv = 0.0;
+        for (int i = 0; i < kEqWarps; ++i) {   // same order in every thread: identical results everywhere
+            big = max(big, sh.kred[0][i]);
+            rise = max(rise, sh.kred[1][i]);
+            conv += sh.red[0][i];
+        }
+        const double bigd = __longlong_as_double((long long)big), rised = __longlong_as_double((long long)rise);
+        double lam = bigd > 2.0 ? 2.0 / bigd : 1.0;
+        if (rised > 1.0) lam = fmin(lam, 1.0 / rised);
+        for (int y = tid; y < S; y += kEqThreads)
+            if (act[y]) lnN[y] = fma(lam, mu[y], lnN[y]);
         __syncthreads();
         if (tid == 0) sh.lntot = lntot + lam * dlntot;
-        if (conv < tol && fabs(dlntot) < tol) {
+        if (conv / sn < tol && fabs(dlntot) < tol) {
             ++it;
-            sh.done = 1;   // same decision in every thread (block-reduced values)
+            done = 1;   // same decision in every thread (block-reduced values)
             break;
         }
         __syncthreads();
@@ -281,28 +297,30 @@ __global__ void __launch_bounds__(kEqThreads) k_equilibrium(Col c, EqIndex ix, c
     __syncthreads();
     if (tid == 0) {
         iters[k] = it;
-        status[k] = sh.singular ? -1 : (sh.done ? 0 : 1);
+        status[k] = sh.singular ? -1 : (done ? 0 : 1);
     }
     if (sh.singular) return;
     // mole fractions from the potentials of the last solve, normalised
     double amax = -INFINITY;
-    for (int y = tid; y < S; y += blockDim.x) {
+    for (int y = tid; y < S; y += kEqThreads) {
         if (!act[y]) continue;
         double v = -g[y] - lnP;
         for (int q = ix.sp[y]; q < ix.sp[y + 1]; ++q) v += sh.sol[ix.se[q]] * ix.sc[q];
         mu[y] = v;
         amax = fmax(amax, v);
     }
-    double dummy = INFINITY, zero = 0.0;
-    block_reduce3(sh, amax, dummy, zero);
-    double z = 0.0;
-    for (int y = tid; y < S; y += blockDim.x)
+    for (int o = 16; o; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    if (lane == 0) sh.red[0][wrp] = amax;
+    __syncthreads();
+    for (int i = 0; i < kEqWarps; ++i) amax = fmax(amax, sh.red[0][i]);
+    __syncthreads();
+    double z = 0.0, zero = 0.0;
+    for (int y = tid; y < S; y += kEqThreads)
         if (act[y]) z += exp(mu[y] - amax);
-    double mx2 = -INFINITY, mn2 = INFINITY;
-    block_reduce3(sh, mx2, mn2, z);
+    block_sum2(sh, z, zero);
     const double lz = log(z);
     const double ng = c.ngas[k];
-    for (int y = tid; y < S; y += blockDim.x) {
+    for (int y = tid; y < S; y += kEqThreads) {
         const double v = act[y] ? exp(mu[y] - amax - lz) : 0.0;
         if (x) x[(size_t)k * S + y] = v;
         if (nout) nout[(size_t)k * S + y] = v * ng;
@@ -345,8 +363,7 @@ __global__ void k_path_weights(long long n, const double *q, double *wq)
 }
 
 // Distances are non-negative doubles (or +inf): their bit patterns order like the values, so the
-// search compares them on the integer pipes (FP64 compares are scarce on this GPU).
-__device__ __forceinline__ unsigned long long key_of(double d) { return (unsigned long long)__double_as_longlong(d); }
+// search compares them (key_of) on the integer pipes: FP64 compares are scarce on this GPU.
 
 // Least weight of every group of parallel edges (source u, target v) in every layer.  Rounding is
 // monotone, so du + (least weight) is the least of du + (weight) over the group: the search needs no
@@ -486,8 +503,8 @@ cudaError_t launch_equilibrium(const Col &c, const EqIndex &ix, const double *b,
                                int max_iter, double tol, int *iters, int *status, cudaStream_t st)
 {
     if (c.E + 1 > kEqMaxE) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)c.S * 3 * sizeof(double) + (size_t)c.S;
-    if (smem > 200 * 1024) return cudaErrorInvalidValue;
+    const size_t species = (size_t)c.S * (3 * sizeof(double) + 1), smem = species + 2 * (size_t)ix.nsub * sizeof(double);
+    if (species > 200 * 1024) return cudaErrorInvalidValue;   // with the parts (kEqMaxSub) and EqShared: 227 KB
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_equilibrium, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

@@ -48,7 +48,8 @@ struct xk_ctx {
     std::vector<uint4> rx;
     std::vector<int> yp, yent, jp, jcol, jtp, jrs, jdq, abs_sp;
     std::vector<int> pg_p, pg_v, pg_s, pg_code;   // reaction graph of the pathway analyser
-    std::vector<int> eq_sp, eq_se, eq_ep, eq_ey, eq_eij;   // sparse element structure (equilibrium)
+    std::vector<int> eq_sp, eq_se, eq_gp, eq_ent, eq_part, eq_ep, eq_eij;   // sparse element structure (equilibrium)
+    int eq_nsub = 0;
     std::vector<double> eq_sc, eq_ec;
     std::vector<double> sig_abs_c;
     std::vector<int> sca_sp;           // species with a non-zero scattering cross section
@@ -189,7 +190,7 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 // Lists cut into sublists of nearly equal length, one lane each, 32 of similar length to a group (see
 // Col::sgp); returns the number of sublists.
 int build_sublists(const std::vector<std::vector<int>> &lists, std::vector<int> &gp, std::vector<int> &ent,
-                   std::vector<int> &part, std::vector<int> &sp)
+                   std::vector<int> &part, std::vector<int> &sp, size_t longest = kSubMax, size_t most = 8192)
 {
     struct Sub {
         int list, e0, n, part;
@@ -197,8 +198,8 @@ int build_sublists(const std::vector<std::vector<int>> &lists, std::vector<int> 
     std::vector<Sub> subs;
     size_t total = 0;
     for (const auto &l : lists) total += l.size();
-    // at most about 8192 besides one per list
-    const size_t sub_max = kSubMax * std::max<size_t>(1, (total + kSubMax * 8192 - 1) / (kSubMax * 8192));
+    // of `longest` entries unless that would be more than `most` besides one per list
+    const size_t sub_max = longest * std::max<size_t>(1, (total + longest * most - 1) / (longest * most));
     sp.assign(lists.size() + 1, 0);
     for (size_t y = 0; y < lists.size(); ++y) {
         const size_t n = lists[y].size(), m = (n + sub_max - 1) / sub_max;
@@ -400,26 +401,36 @@ void build_indices(xk_ctx *c)
             }
         c->eq_sp[y + 1] = (int)c->eq_se.size();
     }
-    c->eq_ep.assign(1, 0);
-    c->eq_ey.clear();
-    c->eq_ec.clear();
+    // each entry of the Newton system is a sum over the species that hold its element(s); the terms as
+    // sublists (Col::sgp), coefficients beside them
+    std::vector<std::vector<int>> eterms;
+    std::vector<int> term_y;
+    std::vector<double> term_c;
     c->eq_eij.clear();
     auto add_entry = [&](int code, int i, int j) {
+        eterms.emplace_back();
         for (int y = 0; y < S; ++y) {
             const double ai = c->elem[(size_t)y * E + i], aj = j >= 0 ? c->elem[(size_t)y * E + j] : 1.0;
             if (ai != 0.0 && aj != 0.0) {
-                c->eq_ey.push_back(y);
-                c->eq_ec.push_back(ai * aj);
+                eterms.back().push_back((int)term_y.size());
+                term_y.push_back(y);
+                term_c.push_back(ai * aj);
             }
         }
         c->eq_eij.push_back(code);
-        c->eq_ep.push_back((int)c->eq_ey.size());
     };
     if (E <= 30) {
         for (int i = 0; i < E; ++i)
             for (int j = i; j < E; ++j) add_entry(i * 32 + j, i, j);
         for (int i = 0; i < E; ++i) add_entry(-1 - i, i, -1);
     }
+    c->eq_nsub = build_sublists(eterms, c->eq_gp, c->eq_ent, c->eq_part, c->eq_ep, kEqSub, kEqMaxSub);
+    c->eq_ec.assign(c->eq_ent.size(), 0.0);
+    for (size_t q = 0; q < c->eq_ent.size(); ++q)
+        if (c->eq_ent[q] >= 0) {
+            c->eq_ec[q] = term_c[c->eq_ent[q]];
+            c->eq_ent[q] = term_y[c->eq_ent[q]];
+        }
     // pathway graph: each reaction direction gives an edge from every species it consumes to every
     // species it produces (itself excepted), grouped by source, then target, codes increasing
     std::vector<std::vector<std::pair<int, int>>> out(S);   // (target, code) per source
@@ -629,9 +640,13 @@ size_t layout(xk_ctx *c, char *base)
     ei.sp = b.take<int>(S + 1);
     ei.se = b.take<int>(std::max<size_t>(1, c->eq_se.size()));
     ei.sc = b.take<double>(std::max<size_t>(1, c->eq_sc.size()));
-    ei.ep = b.take<int>(c->eq_ep.size());
-    ei.ey = b.take<int>(std::max<size_t>(1, c->eq_ey.size()));
+    ei.gp = b.take<int>(std::max<size_t>(1, c->eq_gp.size()));
+    ei.ent = b.take<int>(std::max<size_t>(1, c->eq_ent.size()));
     ei.ec = b.take<double>(std::max<size_t>(1, c->eq_ec.size()));
+    ei.part = b.take<int>(std::max<size_t>(1, c->eq_part.size()));
+    ei.ep = b.take<int>(std::max<size_t>(1, c->eq_ep.size()));
+    ei.ngrp = (int)c->eq_gp.size() - 1;
+    ei.nsub = c->eq_nsub;
     ei.eij = b.take<int>(std::max<size_t>(1, c->eq_eij.size()));
     ei.nent = (int)c->eq_eij.size();
     c->pgraph.gp = b.take<int>(S + 1);
@@ -1307,7 +1322,8 @@ int xk_set_workspace(xk_ctx *c, void *dptr, size_t bytes)
     up(c, c->pgraph.gp, c->pg_p); up(c, c->pgraph.gv, c->pg_v); up(c, c->pgraph.gs, c->pg_s);
     up(c, c->pgraph.gcode, c->pg_code);
     up(c, c->eqix.sp, c->eq_sp); up(c, c->eqix.se, c->eq_se); up(c, c->eqix.sc, c->eq_sc);
-    up(c, c->eqix.ep, c->eq_ep); up(c, c->eqix.ey, c->eq_ey); up(c, c->eqix.ec, c->eq_ec);
+    up(c, c->eqix.gp, c->eq_gp); up(c, c->eqix.ent, c->eq_ent); up(c, c->eqix.ec, c->eq_ec);
+    up(c, c->eqix.part, c->eq_part); up(c, c->eqix.ep, c->eq_ep);
     up(c, c->eqix.eij, c->eq_eij);
     up(c, k.mass, c->mass); up(c, k.nasa, c->nasa); up(c, k.dcoef, c->dcoef);
     up(c, k.arr, c->arr); up(c, k.troe, c->troe); up(c, k.rtype, c->rtype); up(c, k.reac, c->reac);

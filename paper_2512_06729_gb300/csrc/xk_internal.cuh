@@ -114,6 +114,9 @@ struct Ctl {
 };
 
 constexpr int kJacWarps = 8, kJacOcc = 128, kJacHeavyOcc = kJacWarps * kJacOcc;
+constexpr int kEqSub = 24;      // terms of an equilibrium entry summed by one lane: the longest entry has some
+                                // 24 x 24 (hydrogen with itself), the two chains of FP64 additions are even
+constexpr int kEqMaxSub = 512;  // places of such sums besides one per entry (shared memory)
 constexpr int kSubMax = 48;     // entries of a species list summed by one lane
 
 struct Policy {
@@ -170,6 +173,20 @@ __device__ __forceinline__ void reaction_terms_at(const Col &c, int k, int r, co
     }
 }
 
+// 1 / x from the hardware's approximation (some 20 bits) by one third-order step, y (1 + e + e^2) with
+// e = 1 - x y: the series of 1 / (1 - e).  Three dependent FP64 operations; an FP64 result takes some
+// 180 clocks on this part, a division about ten of them.  The division where the approximation's range
+// ends (the exponent looked at as an integer).
+__device__ __forceinline__ double reciprocal64(double x)
+{
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    if (ex - 32u > 1984u) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
 // Entry q of the Jacobian pattern (row-grouped): sum of its terms, -dF_i/dn_j of one layer, in a
 // fixed order (dk: that layer's reaction derivatives [R][6]).
 __device__ __forceinline__ double jac_entry(const Col &c, int q, const double *dk)
@@ -192,12 +209,14 @@ struct PathGraph {
 };
 // Sparse element structure for the equilibrium solve, built on the host: species y holds elements
 // se[sp[y] .. sp[y+1]) with counts sc[..]; entry t of the Newton system (eij[t] = i * 32 + j for the
-// element pair i <= j, -1 - i for element i's own sums) is a sum over the species ey[ep[t] ..
-// ep[t+1]) (increasing) with coefficients ec[..] (a_iy a_jy, or a_iy).
+// element pair i <= j, -1 - i for element i's own sums) is a sum over the species that hold them with
+// coefficients a_iy a_jy (a_iy), cut into sublists as Col::sgp: group g's terms are species ent[32 q +
+// lane] (-1: none) with ec[..], q = gp[g] .. gp[g+1), part[32 g + lane] the sublist's place, entry t's
+// places ep[t] .. ep[t+1); ngrp groups, nsub places.
 struct EqIndex {
-    const int *sp, *se, *ep, *ey, *eij;
+    const int *sp, *se, *gp, *ent, *part, *ep, *eij;
     const double *sc, *ec;
-    int nent;
+    int nent, ngrp, nsub;
 };
 // Equilibrium composition per layer (xk_analysis.cu): element totals b [L][E] (nullptr: from the
 // state c.n); mole fractions into x [L][S] (may be nullptr) and, when nout is set, number densities
