@@ -187,6 +187,17 @@ __device__ __forceinline__ double reciprocal64(double x)
     return fma(y, fma(e, e, e), y);
 }
 
+// 1 / x correctly rounded, without the division's length: reciprocal64 is within one unit in the last
+// place, and from there y + y (1 - x y) rounds correctly (Markstein 1990) unless x's fraction is all
+// ones.  That case, and exponents at which the residual may not be exact, take the division.
+__device__ __forceinline__ double reciprocal_rn(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), ex = (hi >> 20) & 0x7ffu;
+    if (ex - 64u > 1900u || ((hi & 0xfffffu) == 0xfffffu && __double2loint(x) == -1)) return 1.0 / x;
+    const double y = reciprocal64(x);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
 // Entry q of the Jacobian pattern (row-grouped): sum of its terms, -dF_i/dn_j of one layer, in a
 // fixed order (dk: that layer's reaction derivatives [R][6]).
 __device__ __forceinline__ double jac_entry(const Col &c, int q, const double *dk)

@@ -10,12 +10,13 @@
 // layer's.
 //
 // The sweep is sequential in the layers, so one CTA runs a whole iteration: every reduction,
-// pivot search and elimination step stays inside the block (no grid-wide wait).  The step's
-// vectors live in shared memory, and so do its two S x S matrices (the system and its factors)
-// when they fit (S up to 111); larger systems keep them in global memory, where they stay in L2.
+// pivot search and elimination step stays inside the block (no grid-wide wait).  Systems whose two
+// S x S matrices (the system and its factors) fit in shared memory (S up to 111) have a kernel of
+// their own; larger ones keep them in global memory, where they stay in L2.
 #include <cfloat>
 
 #include "xk_internal.cuh"
+#include "xk_layer.cuh"
 
 namespace xk {
 
@@ -166,7 +167,35 @@ __device__ int dense_solve(const double *A0, double *A, int *piv, const double *
     return 0;
 }
 
-__global__ void __launch_bounds__(1024, 1) k_parcel_iteration(Col c, ParcelArgs a, int mats_in_smem)
+// The step size and what the controller says of a step with largest relative change mr (thread 0).
+__device__ void step_size(Shared &sh, const Policy &pol, double tau)
+{
+    const double rest = tau - sh.t;
+    double hs = sh.h < rest ? sh.h : rest;
+    if (hs > pol.dt_max) hs = pol.dt_max;
+    sh.hs = hs;
+    sh.last = hs >= rest;
+}
+__device__ void step_control(Shared &sh, const Policy &pol, double tau, double hs, double mr, bool ok, int visit_steps,
+                             int max_visit_steps)
+{
+    if (ok) {
+        sh.t = sh.last ? tau : sh.t + hs;
+        double fac = mr > 0.0 ? pol.rel_target / mr : pol.grow_max;
+        if (fac > pol.grow_max) fac = pol.grow_max;
+        if (fac < pol.shrink_min) fac = pol.shrink_min;
+        double next = hs * fac;
+        if (hs < sh.h && fac >= 1.0 && next < sh.h) next = sh.h;   // cut short by the visit's end
+        sh.h = next;
+        sh.done = 0;
+    } else {
+        sh.h = 0.5 * hs;
+        sh.done = sh.h < pol.dt_min ? XK_ENEG : 0;
+    }
+    if (visit_steps > max_visit_steps && !sh.done) sh.done = XK_ENOCONV;
+}
+
+__global__ void __launch_bounds__(1024, 1) k_parcel_iteration(Col c, ParcelArgs a)
 {
     __shared__ Shared sh;
     extern __shared__ double dyn[];
@@ -175,12 +204,9 @@ __global__ void __launch_bounds__(1024, 1) k_parcel_iteration(Col c, ParcelArgs 
     const int warp = tid >> 5, lane = tid & 31, nw = nwarps();
     const Policy &pol = a.pol;
     ParcelState *st = a.st;
-    // vectors always in shared memory; the two S x S matrices there too when they fit
     double *x = dyn, *F = x + S, *d = F + S, *r = d + S;
     int *piv = (int *)(r + S);
-    double *mats = (double *)(piv + ((S + 1) & ~1));
-    double *A0 = mats_in_smem ? mats : a.A;
-    double *A = mats_in_smem ? mats + (long long)S * S : a.A + (long long)S * S;
+    double *A0 = a.A, *A = a.A + (long long)S * S;
     for (long long i = tid; i < (long long)L * S; i += nt) a.Nold[i] = a.N[i];
     for (int y = tid; y < S; y += nt) a.vmr[y] = a.N[y] / c.ngas[0];
     if (tid == 0) sh.h = st->h;
@@ -195,13 +221,7 @@ __global__ void __launch_bounds__(1024, 1) k_parcel_iteration(Col c, ParcelArgs 
         __syncthreads();
         int visit_steps = 0;
         while (sh.t < tau) {
-            if (tid == 0) {
-                const double rest = tau - sh.t;
-                double hs = sh.h < rest ? sh.h : rest;
-                if (hs > pol.dt_max) hs = pol.dt_max;
-                sh.hs = hs;
-                sh.last = hs >= rest;
-            }
+            if (tid == 0) step_size(sh, pol, tau);
             __syncthreads();
             const double hs = sh.hs;
             // reaction terms at the parcel's densities (Sec. 2.3)
@@ -262,22 +282,8 @@ __global__ void __launch_bounds__(1024, 1) k_parcel_iteration(Col c, ParcelArgs 
                     x[y] = nn < 0.0 ? 0.0 : nn;
                 }
             __syncthreads();
-            if (tid == 0) {
-                if (ok) {
-                    sh.t = sh.last ? tau : sh.t + hs;
-                    double fac = mr > 0.0 ? pol.rel_target / mr : pol.grow_max;
-                    if (fac > pol.grow_max) fac = pol.grow_max;
-                    if (fac < pol.shrink_min) fac = pol.shrink_min;
-                    double next = hs * fac;
-                    if (hs < sh.h && fac >= 1.0 && next < sh.h) next = sh.h;   // cut short by the visit's end
-                    sh.h = next;
-                    sh.done = 0;
-                } else {
-                    sh.h = 0.5 * hs;
-                    sh.done = sh.h < pol.dt_min ? XK_ENEG : 0;
-                }
-                if (++visit_steps > a.max_visit_steps && !sh.done) sh.done = XK_ENOCONV;
-            }
+            ++visit_steps;
+            if (tid == 0) step_control(sh, pol, tau, hs, mr, ok, visit_steps, a.max_visit_steps);
             if (ok) ++steps;
             else ++rejected;
             __syncthreads();
@@ -308,26 +314,385 @@ __global__ void __launch_bounds__(1024, 1) k_parcel_iteration(Col c, ParcelArgs 
     }
 }
 
-}  // namespace
+// ---------------------------------------------------------------------------
+// systems of at most kSmallS species: matrices in shared memory
+// ---------------------------------------------------------------------------
+// A step is a chain of small dependent operations, and what it costs is their latency: an FP64 result
+// takes some 180 clocks, a division ten of them, a comparison as much as a product, a barrier thirty.
+// So pivots are compared as bit patterns, by every warp for itself; a column of the elimination has one
+// barrier; its reciprocals are kept for the triangular solves, which one warp does with the vector in
+// registers; and every sum is formed in the order of the general kernel, whose results these are bit
+// for bit (a parcel carries a rounding through hundreds of steps, grown many orders of magnitude).
+// A step of 40 species takes 71 us, on the general kernel (matrices in shared memory too) 185.
+constexpr int kSmallS = 128;
+constexpr int kSmallThreads = 256;
+constexpr int kSmallWarps = kSmallThreads / 32;
 
-size_t parcel_vector_bytes(int S) { return sizeof(double) * 4 * (size_t)S + sizeof(int) * (size_t)((S + 1) & ~1); }
-
-bool parcel_mats_in_smem(int S)
+// Order of |v| among pivot candidates as a bit pattern; 0 for zero and for what is not a number, which
+// no pivot search takes.
+__device__ __forceinline__ unsigned long long pivot_key(double v)
 {
-    return parcel_vector_bytes(S) + 2 * sizeof(double) * (size_t)S * S <= kSmemLimit;
+    const unsigned long long k = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return k > 0x7ff0000000000000ull ? 0ull : k;
 }
+
+// Shared-memory layout of the small kernel (doubles): the matrices' rows are an odd number of words
+// apart, so that 32 rows of a column lie in 32 banks.
+struct SmallLayout {
+    int ld;
+    size_t vec, mats, rates, bytes;
+};
+__host__ __device__ inline SmallLayout small_layout(int S, int R, bool rates_in_smem)
+{
+    SmallLayout l;
+    l.ld = S | 1;
+    l.vec = 0;                                     // x, F, d, r, gain, loss, loss / dz, 1 / pivots; then the row order
+    l.mats = 8 * (size_t)S + (size_t)(S + 1) / 2;
+    l.rates = l.mats + 2 * (size_t)S * l.ld;
+    l.bytes = (l.rates + (rates_in_smem ? 7 * (size_t)R : 0)) * sizeof(double);
+    return l;
+}
+
+// A <- its LU factors, order[i] the original row at place i, inv the pivots' reciprocals.  Every warp
+// finds the pivot and the multipliers of column c for itself and updates its own columns j > c, rows
+// along the lanes, reading the rows where they were and writing them where the exchange puts them; the
+// last warp keeps the columns up to c (a column's multipliers wait in its registers until all have read
+// it).  0, or -1 on a zero pivot column, in every thread.
+__device__ int small_factor(double *A, int ld, int *order, double *inv, int S)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kC = kSmallS / 32;
+    double held[kC];                               // multipliers of the column before (last warp)
+    for (int c = 0; c <= S; ++c) {
+        if (c && warp == kSmallWarps - 1) {
+#pragma unroll
+            for (int t = 0; t < kC; ++t) {
+                const int i = c + t * 32 + lane;
+                if (i < S) A[i * ld + c - 1] = held[t];
+            }
+            __syncwarp();
+        }
+        if (c == S) break;
+        // the first row of largest magnitude
+        unsigned long long best = 0ull;
+        int bi = S;
+#pragma unroll
+        for (int t = 0; t < kC; ++t) {
+            const int i = c + t * 32 + lane;
+            if (i < S) {
+                const unsigned long long k = pivot_key(A[i * ld + c]);
+                if (k > best) {
+                    best = k;
+                    bi = i;
+                }
+            }
+        }
+        const unsigned hi = (unsigned)(best >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned lo = hi == mh ? (unsigned)best : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+        if ((mh | ml) == 0u) return -1;
+        const int p = (int)__reduce_min_sync(0xffffffffu, hi == mh && (unsigned)best == ml ? (unsigned)bi : 0xffffffffu);
+        const double ipv = reciprocal_rn(A[p * ld + c]);
+        if (warp == kSmallWarps - 1) {
+            if (lane == 0) {
+                inv[c] = ipv;
+                const int o = order[c];
+                order[c] = order[p];
+                order[p] = o;
+            }
+            if (p != c)
+                for (int j = lane; j < c; j += 32) {
+                    const double t = A[c * ld + j];
+                    A[c * ld + j] = A[p * ld + j];
+                    A[p * ld + j] = t;
+                }
+        }
+        // multipliers of the rows c + 1 .. S - 1 as they will stand: row p's place takes row c
+        const double vc = A[c * ld + c], vp = A[p * ld + c];
+        double l[kC];
+#pragma unroll
+        for (int t = 0; t < kC; ++t) {
+            const int i = c + 1 + t * 32 + lane;
+            l[t] = 0.0;
+            if (c + 1 + t * 32 < S && i < S) l[t] = (i == p ? vc : A[i * ld + c]) * ipv;
+        }
+        for (int j = c + 1 + warp; j < S; j += kSmallWarps) {
+            const double ap = A[p * ld + j], ac = A[c * ld + j];
+            __syncwarp();
+            if (lane == 0) A[c * ld + j] = ap;
+#pragma unroll
+            for (int t = 0; t < kC; ++t) {
+                if (c + 1 + t * 32 >= S) break;
+                const int i = c + 1 + t * 32 + lane;
+                if (i < S) A[i * ld + j] = fma(-l[t], ap, i == p ? ac : A[i * ld + j]);
+            }
+        }
+        __syncthreads();
+        // all have read column c: the last warp writes it (with the next column's start)
+        if (warp == kSmallWarps - 1) {
+#pragma unroll
+            for (int t = 0; t < kC; ++t) held[t] = l[t];
+            if (lane == 0) A[c * ld + c] = vp;
+        }
+    }
+    __syncthreads();
+    return 0;
+}
+
+// x <- (LU)^-1 P f on one warp, T words of the vector to a lane.
+template <int T>
+__device__ void warp_lu_solve(const double *A, int ld, const int *order, const double *inv, const double *f, double *x,
+                              int S)
+{
+    const int lane = threadIdx.x & 31;
+    double v[T], iv[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        const int i = t * 32 + lane;
+        v[t] = i < S ? f[order[i]] : 0.0;
+        iv[t] = i < S ? inv[i] : 0.0;
+    }
+#pragma unroll
+    for (int t = 0; t < T; ++t) {                  // unit lower triangle, column by column
+        const int n = min(32, S - 32 * t);
+        for (int q = 0; q < n; ++q) {
+            const int c = 32 * t + q;
+            double m[T];
+#pragma unroll
+            for (int u = t; u < T; ++u) {
+                const int i = u * 32 + lane;
+                m[u] = i > c && i < S ? A[i * ld + c] : 0.0;
+            }
+            const double xc = __shfl_sync(0xffffffffu, v[t], q);
+#pragma unroll
+            for (int u = t; u < T; ++u)
+                if (u * 32 + lane > c) v[u] = fma(-m[u], xc, v[u]);
+        }
+    }
+#pragma unroll
+    for (int t = T - 1; t >= 0; --t) {             // upper triangle
+        const int n = min(32, S - 32 * t);
+        for (int q = n - 1; q >= 0; --q) {
+            const int c = 32 * t + q;
+            double m[T];
+#pragma unroll
+            for (int u = 0; u <= t; ++u) m[u] = u * 32 + lane < c ? A[(u * 32 + lane) * ld + c] : 0.0;
+            const double own = v[t] * iv[t];
+            const double xc = __shfl_sync(0xffffffffu, own, q);
+            if (lane == q) v[t] = xc;
+#pragma unroll
+            for (int u = 0; u <= t; ++u)
+                if (u * 32 + lane < c) v[u] = fma(-m[u], xc, v[u]);
+        }
+    }
+    __syncwarp();                                  // f may be x
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+        if (t * 32 + lane < S) x[t * 32 + lane] = v[t];
+    __syncwarp();
+}
+
+__device__ void small_solve(const double *A, int ld, const int *order, const double *inv, const double *f, double *x, int S)
+{
+    if (S <= 32) warp_lu_solve<1>(A, ld, order, inv, f, x, S);
+    else if (S <= 64) warp_lu_solve<2>(A, ld, order, inv, f, x, S);
+    else warp_lu_solve<4>(A, ld, order, inv, f, x, S);
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_parcel_small(Col c, ParcelArgs a, int rates_in_smem)
+{
+    __shared__ Shared sh;
+    __shared__ double rh;                          // 1 / (step size)
+    extern __shared__ double dyn[];
+    const int S = c.S, L = c.L, R = c.R;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const Policy &pol = a.pol;
+    ParcelState *st = a.st;
+    const SmallLayout lay = small_layout(S, R, rates_in_smem);
+    const int ld = lay.ld;
+    double *x = dyn, *F = x + S, *d = F + S, *r = d + S, *gain = r + S, *loss = gain + S, *ldz = loss + S, *inv = ldz + S;
+    int *order = (int *)(inv + S);
+    double *A0 = dyn + lay.mats, *A = A0 + (size_t)S * ld;
+    double *w = rates_in_smem ? dyn + lay.rates : a.w, *dd = rates_in_smem ? w + R : a.dd;
+    // places of the pattern's entries in the matrices (-1 - place: on the diagonal); the general
+    // kernel's matrices hold them
+    int *place = (int *)a.A;
+    for (int i = warp; i < S; i += kSmallWarps)
+        for (int q = c.jp[i] + lane; q < c.jp[i + 1]; q += 32) {
+            const int j = c.jcol[q], e = i * ld + j;
+            place[q] = i == j ? -1 - e : e;
+        }
+    const int nnz = c.jp[S];
+    for (long long i = tid; i < (long long)L * S; i += kSmallThreads) a.Nold[i] = a.N[i];
+    for (int y = tid; y < S; y += kSmallThreads) a.vmr[y] = a.N[y] / c.ngas[0];
+    if (tid == 0) sh.h = st->h;
+    long long steps = 0, rejected = 0;
+    // the species' sums go to the first warps, the matrix to the others
+    const int fw = min((S + 31) / 32, kSmallWarps / 2);
+    __syncthreads();
+    for (int v = 0; v < 2 * L - 1; ++v) {
+        const int k = v < L ? v : 2 * L - 2 - v;
+        const double nk = c.ngas[k], dzk = c.dz[k];
+        const double tau = dzk * dzk / c.Kzz[k];
+        for (int y = tid; y < S; y += kSmallThreads) {
+            x[y] = a.vmr[y] * nk;
+            // the molecular-diffusion pair: the neighbours' densities stay during a visit
+            double ls = 0.0, gn = 0.0;
+            if (k + 1 < L) {
+                ls += a.um[(long long)k * S + y];
+                gn += a.vm[(long long)k * S + y] * a.N[(long long)(k + 1) * S + y];
+            }
+            if (k > 0) {
+                ls += a.vm[(long long)(k - 1) * S + y];
+                gn += a.um[(long long)(k - 1) * S + y] * a.N[(long long)(k - 1) * S + y];
+            }
+            gain[y] = gn;
+            loss[y] = ls;
+            ldz[y] = ls / dzk;
+        }
+        if (tid == 0) {
+            sh.t = 0.0;
+            step_size(sh, pol, tau);
+        }
+        __syncthreads();
+        int visit_steps = 0;
+        while (sh.t < tau) {
+            const double hs = sh.hs;
+            // reaction terms at the parcel's densities (Sec. 2.3)
+            for (int rr = tid; rr < R; rr += kSmallThreads) reaction_terms_at(c, k, rr, x, w + rr, dd + (long long)rr * 6);
+            if (tid == kSmallThreads - 1) rh = 1.0 / hs;
+            for (int e = tid; e < 2 * S * ld; e += kSmallThreads) A0[e] = 0.0;      // A follows A0
+            for (int y = tid; y < S; y += kSmallThreads) order[y] = y;
+            __syncthreads();
+            if (warp < fw) {
+                for (int y = tid; y < S; y += 32 * fw) {
+                    double f = 0.0;
+                    const int e1 = c.yp[y + 1];
+#pragma unroll 4
+                    for (int e = c.yp[y]; e < e1; ++e) {
+                        const int code = c.yent[e];
+                        f += signed_by(w[code >> 4], (code & 15) >= 8);
+                    }
+                    F[y] = f + (gain[y] - loss[y] * x[y]) / dzk;
+                    if (c.jdq[y] < 0) A0[y * ld + y] = A[y * ld + y] = rh + ldz[y];
+                }
+            } else {
+                // matrix I/h - dF/dx, entries of the pattern summed in a fixed order
+                for (int q = tid - 32 * fw; q < nnz; q += kSmallThreads - 32 * fw) {
+                    double acc = 0.0;
+                    const int t1 = c.jtp[q + 1];
+#pragma unroll 4
+                    for (int t = c.jtp[q]; t < t1; ++t) {
+                        const int code = c.jrs[t], rs = code >> 1;
+                        acc += signed_by(dd[(rs >> 3) * 6 + (rs & 7)], code & 1);
+                    }
+                    int e = place[q];
+                    if (e < 0) {
+                        e = -1 - e;
+                        acc += rh + ldz[e / (ld + 1)];
+                    }
+                    A0[e] = acc;
+                    A[e] = acc;
+                }
+            }
+            __syncthreads();
+            if (small_factor(A, ld, order, inv, S) != 0) {
+                if (tid == 0) { st->status = XK_ESINGULAR; st->visit = v; }
+                return;
+            }
+            if (warp == 0) small_solve(A, ld, order, inv, F, d, S);
+            for (int sweep = 0; sweep < kRefineSweeps; ++sweep) {
+                __syncthreads();
+                for (int i = warp; i < S; i += kSmallWarps) {
+                    const double *Ai = A0 + i * ld;
+                    double acc = 0.0;
+                    for (int j = lane; j < S; j += 32) acc += Ai[j] * d[j];
+                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                    if (lane == 0) r[i] = F[i] - acc;
+                }
+                __syncthreads();
+                if (warp == 0) {
+                    small_solve(A, ld, order, inv, r, r, S);
+                    for (int y = lane; y < S; y += 32) d[y] += r[y];
+                    __syncwarp();
+                }
+            }
+            // the Eulerian step controller: reject on a negative or a too large relative change
+            if (warp == 0) {
+                unsigned long long mk = 0ull;
+                int bad = 0;
+                for (int y = lane; y < S; y += 32) {
+                    const double xv = x[y], dv = d[y], nn = xv + dv;
+                    if (!isfinite(nn) || nn < -pol.neg_tol * nk) bad = 1;
+                    if (xv > pol.f_floor * nk) mk = max(mk, pivot_key(fabs(dv) / xv));
+                }
+                bad = __any_sync(0xffffffffu, bad);
+                const unsigned hi = (unsigned)(mk >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+                const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)mk : 0u);
+                const double mr = __longlong_as_double((long long)((unsigned long long)mh << 32 | ml));
+                const bool ok = !bad && !(mr > pol.rel_reject);
+                if (ok)
+                    for (int y = lane; y < S; y += 32) {
+                        const double nn = x[y] + d[y];
+                        x[y] = nn < 0.0 ? 0.0 : nn;
+                    }
+                if (ok) ++steps;
+                else ++rejected;
+                ++visit_steps;
+                if (lane == 0) {
+                    step_control(sh, pol, tau, hs, mr, ok, visit_steps, a.max_visit_steps);
+                    if (sh.t < tau) step_size(sh, pol, tau);
+                }
+            }
+            __syncthreads();
+            if (sh.done) {
+                if (tid == 0) { st->status = sh.done; st->visit = v; st->steps += steps; st->rejected += rejected; }
+                return;
+            }
+        }
+        for (int y = tid; y < S; y += kSmallThreads) {
+            a.N[(long long)k * S + y] = x[y];
+            a.vmr[y] = x[y] / nk;
+        }
+        __syncthreads();
+    }
+    double ch = 0.0;
+    for (long long i = tid; i < (long long)L * S; i += kSmallThreads) {
+        const int k = (int)(i / S);
+        const double nv = a.N[i];
+        if (nv > pol.f_floor * c.ngas[k]) ch = fmax(ch, fabs(nv - a.Nold[i]) / nv);
+    }
+    ch = block_max(ch, sh);
+    if (tid == 0) {
+        st->max_change = ch;
+        st->h = sh.h;
+        st->steps += steps;
+        st->rejected += rejected;
+        st->status = 0;
+    }
+}
+
+}  // namespace
 
 cudaError_t launch_parcel_iteration(const Col &c, const ParcelArgs &a, cudaStream_t st)
 {
     const int S = c.S;
-    const bool in_smem = parcel_mats_in_smem(S);
-    const size_t smem = parcel_vector_bytes(S) + (in_smem ? 2 * sizeof(double) * (size_t)S * S : 0);
-    // small systems: fewer warps, so that each barrier waits on less; large ones: the whole SM
+    SmallLayout small = small_layout(S, c.R, true);
+    const bool rates = small.bytes <= kSmemLimit;
+    if (!rates) small = small_layout(S, c.R, false);
+    count_launches(1);
+    if (S <= kSmallS && small.bytes <= kSmemLimit) {
+        // eight warps: what a barrier waits for, and two to each FP64 unit
+        cudaError_t e = cudaFuncSetAttribute(k_parcel_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small.bytes);
+        if (e != cudaSuccess) return e;
+        k_parcel_small<<<1, kSmallThreads, small.bytes, st>>>(c, a, rates ? 1 : 0);
+        return cudaGetLastError();
+    }
+    const size_t smem = sizeof(double) * 4 * (size_t)S + sizeof(int) * (size_t)((S + 1) & ~1);
+    // fewer warps while the system is small, so that each barrier waits on less; then the whole SM
     const int threads = S <= 160 ? 256 : 1024;
     cudaError_t e = cudaFuncSetAttribute(k_parcel_iteration, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    count_launches(1);
-    k_parcel_iteration<<<1, threads, smem, st>>>(c, a, in_smem ? 1 : 0);
+    k_parcel_iteration<<<1, threads, smem, st>>>(c, a);
     return cudaGetLastError();
 }
 
