@@ -538,6 +538,7 @@ size_t layout(xk_ctx *c, char *base)
     t.kf = b.take<double>(LR); t.kr = b.take<double>(LR);
     t.kph = b.take<double>((size_t)L * std::max(Rph, 1));
     t.alpha = b.take<double>((size_t)L * std::max(W, 1)); t.Jw = b.take<double>((size_t)L * std::max(W, 1));
+    t.Jd = b.take<double>((size_t)L * std::max(W, 1));
     t.w = b.take<double>(LR); t.d = b.take<double>(6 * LR); t.dw = b.take<double>(LR);
     t.n = b.take<double>(LS); t.F = b.take<double>(LS); t.s = b.take<double>(LS); t.b = b.take<double>(LS);
     t.x = b.take<double>(LS); t.delta = b.take<double>(LS); t.tmp = b.take<double>(LS);
@@ -2304,7 +2305,7 @@ int xk_parcel_begin(xk_ctx *c, int max_visit_steps, double h)
         if (!(c->Kzz[k] > 0.0)) return fail(c, XK_EINVAL, "parcel: K_zz must be positive (residence time dz^2 / K_zz)");
     ensure_rates(c);
     // photolysis from the stored profile at the start of the iteration; molecular-only u, v
-    launch_photolysis(c->col, c->col.n, c->st);
+    launch_photolysis(c->col, c->col.n, c->st, true);
     cudaMemsetAsync(c->parcel_kzz0, 0, sizeof(double) * c->L, c->st);
     launch_transport_coeffs(c->col, c->parcel_kzz0, const_cast<double *>(c->parcel.um),
                             const_cast<double *>(c->parcel.vm), c->st);

@@ -152,95 +152,180 @@ __global__ void k_rates(Col c)
 // photolysis (Sec. 2.3.3): extinction by absorption and Rayleigh scattering, direct beam with the
 // optical depth to the layer midpoint, and optionally the diffuse field J_diff = (J_up + J_down) / 2
 // ---------------------------------------------------------------------------
-constexpr int kExtLayers = 4;   // layers per thread of the extinction sums (sigma loaded once for them)
+constexpr int kExtLayers = 4;    // layers per thread of the extinction sums (sigma loaded once for them)
+constexpr int kExtChunk = 128;   // species whose densities are staged at a time
 
 // alpha (absorption) and alpha_s (scattering) per (layer, wavelength): one thread per wavelength and
-// kExtLayers consecutive layers, reading each cross section once for all of them (coalesced in w)
-__global__ void k_photo_alpha(Col c, const double *n)
+// kExtLayers consecutive layers, reading each cross section once for all of them (coalesced in w).
+// The densities come from shared memory: fetched through the species' index in the loop, they were
+// its latency.  Bound by FP64 issue (one multiply-add per species, layer and wavelength): 57 us at 154
+// species, 1,000 wavelengths and 150 layers (97 before, some 45 at the rate k_photo_k reaches).
+__global__ void __launch_bounds__(128) k_photo_alpha(Col c, const double *n)
 {
+    __shared__ __align__(16) double sn[kExtChunk][kExtLayers];
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     const int k0 = blockIdx.y * kExtLayers;
-    if (w >= c.W) return;
     const int nk = min(kExtLayers, c.L - k0);
-    double sa[kExtLayers], ss[kExtLayers];
+    for (int scatter = 0; scatter < 2; ++scatter) {
+        const int cnt = scatter ? c.Ssca : c.Sabs;
+        const int *sp = scatter ? c.sca_sp : c.abs_sp;
+        const double *sig = (scatter ? c.sig_sca : c.sig_abs) + w;
+        double *out = (scatter ? c.alpha_s : c.alpha) + (long long)k0 * c.W + w;
+        double s[kExtLayers];
 #pragma unroll
-    for (int j = 0; j < kExtLayers; ++j) sa[j] = ss[j] = 0.0;
-    for (int i = 0; i < c.Sabs; ++i) {
-        const double sg = c.sig_abs[(long long)i * c.W + w];
-        const int y = c.abs_sp[i];
+        for (int j = 0; j < kExtLayers; ++j) s[j] = 0.0;
+        for (int i0 = 0; i0 < cnt; i0 += kExtChunk) {
+            const int m = min(kExtChunk, cnt - i0);
+            __syncthreads();
+            for (int t = threadIdx.x; t < m * kExtLayers; t += blockDim.x) {
+                const int i = t / kExtLayers, j = t % kExtLayers;
+                sn[i][j] = j < nk ? n[(long long)(k0 + j) * c.S + sp[i0 + i]] : 0.0;
+            }
+            __syncthreads();
+            if (w < c.W) {
+                const double *sg = sig + (long long)i0 * c.W;
+#pragma unroll 4
+                for (int i = 0; i < m; ++i) {
+                    const double v = sg[(long long)i * c.W];
 #pragma unroll
-        for (int j = 0; j < kExtLayers; ++j)
-            if (j < nk) sa[j] += sg * n[(long long)(k0 + j) * c.S + y];
-    }
-    for (int i = 0; i < c.Ssca; ++i) {
-        const double sg = c.sig_sca[(long long)i * c.W + w];
-        const int y = c.sca_sp[i];
-#pragma unroll
-        for (int j = 0; j < kExtLayers; ++j)
-            if (j < nk) ss[j] += sg * n[(long long)(k0 + j) * c.S + y];
-    }
-#pragma unroll
-    for (int j = 0; j < kExtLayers; ++j)
-        if (j < nk) {
-            c.alpha[(long long)(k0 + j) * c.W + w] = sa[j];
-            c.alpha_s[(long long)(k0 + j) * c.W + w] = ss[j];
+                    for (int j = 0; j < kExtLayers; ++j) s[j] += v * sn[i][j];
+                }
+            }
         }
+#pragma unroll
+        for (int j = 0; j < kExtLayers; ++j)
+            if (w < c.W && j < nk) out[(long long)j * c.W] = s[j];
+    }
 }
 
-// One thread per wavelength.  Top-down: optical depth, direct beam into Jw and, with the diffuse
-// field, the two-stream recursion.  In layer k the diffuse fluxes leaving it, D_k down through its
-// bottom and U_k up through its top, obey
+// x / d by the (correctly rounded) reciprocal of d and one correction: a division takes some ten
+// dependent FP64 operations, this three, with the same result
+__device__ __forceinline__ double over(double x, double d, double rd)
+{
+    const double q = x * rd;
+    if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return q;   // the correction would be inf - inf
+    return fma(fma(-q, d, x), rd, q);
+}
+
+// The diffuse field.  In layer k the diffuse fluxes leaving it, D_k down through its bottom and U_k up
+// through its top, obey
 //     D_k = T_k D_{k+1} + r_k U_{k-1} + P_k / 2,   U_k = T_k U_{k-1} + r_k D_{k+1} + P_k / 2,
 // with D_L = 0 and U_{-1} = albedo (D_0 + beam at the bottom); r_k = (1 - t) omega / 2,
 // T_k = t + (1 - t) omega / 2, t = exp(-2 dtau_k), omega_k = dtau_s / dtau, and P_k = omega_k mu J0
-// (e^{-tau_top/mu} - e^{-tau_bot/mu}) the beam photons the layer scatters.  Going down, each layer's
-// fluxes are written in terms of the flux entering from below: D_k = p_k U_{k-1} + h0_k,
-// U_k = q_k U_{k-1} + h1_k (p_k is the reflectance of the layers from k up, as in the adding
-// method); going up, U_{-1} is found from the boundary and the fluxes follow layer by layer.
-__global__ void k_photo_J(Col c)
+// (e^{-tau_top/mu} - e^{-tau_bot/mu}) the beam photons the layer scatters.
+//
+// First kernel: the direct beam into Jw and r, T, P / 2 of every layer, which depend on the layers
+// above only through the optical depth.  A CTA takes 32 wavelengths, a warp a run of layers counted
+// from the top.  Bound by the FP64 issue of three exponentials a layer (a layer's bottom is the next
+// one's top).  Both kernels in one, a thread per wavelength, left half of the SMs' schedulers without
+// a warp and the rest waiting for one exponential after the other.  314 us at 10,000 wavelengths and
+// 150 layers, and 176 for the second.
+constexpr int kPhotoRuns = 16;
+__global__ void __launch_bounds__(32 * kPhotoRuns) k_photo_layers(Col c)
 {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= c.W) return;
+    __shared__ double runs[kPhotoRuns][33];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, w = blockIdx.x * 32 + lane;
+    const bool on = w < c.W;
+    const int per = (c.L + kPhotoRuns - 1) / kPhotoRuns;
+    const int i0 = min(c.L, g * per), i1 = min(c.L, i0 + per);   // positions from the top: layer L-1-i
     const long long LW = (long long)c.L * c.W;
-    const double J0 = c.J0[w], mu = c.mu;
-    double above = 0.0, pn = 0.0, h0n = 0.0;
-    for (int k = c.L - 1; k >= 0; --k) {
-        const long long i = (long long)k * c.W + w;
-        const double ta = c.alpha[i] * c.dz[k], ts = c.alpha_s[i] * c.dz[k];
-        const double dt = ta + ts;
-        c.Jw[i] = J0 * exp(-(above + 0.5 * dt) / mu);
-        if (c.diffuse) {
-            const double om = dt > 0.0 ? ts / dt : 0.0;
-            const double t = exp(-dt / 0.5);
-            const double r = (1.0 - t) * om / 2.0, T = t + (1.0 - t) * om / 2.0;
-            const double P = om * mu * J0 * (exp(-above / mu) - exp(-(above + dt) / mu));
-            const double den = 1.0 - r * pn;
-            const double q = T / den, h1 = (r * h0n + P / 2.0) / den;
-            const double p = r + T * pn * q;
-            const double h0 = T * pn * h1 + T * h0n + P / 2.0;
-            c.rt[i] = p;
-            c.rt[LW + i] = q;
-            c.rt[2 * LW + i] = h0;
-            c.rt[3 * LW + i] = h1;
-            pn = p;
-            h0n = h0;
+    double run = 0.0;
+    if (on)
+        for (int i = i0; i < i1; ++i) {
+            const int k = c.L - 1 - i;
+            const long long idx = (long long)k * c.W + w;
+            run += (c.alpha[idx] + c.alpha_s[idx]) * c.dz[k];
         }
+    runs[g][lane] = run;
+    __syncthreads();
+    double above = 0.0;
+    for (int h = 0; h < g; ++h) above += runs[h][lane];
+    if (!on || i0 >= i1) return;
+    const double J0 = c.J0[w], mu = c.mu, rmu = reciprocal_rn(mu);
+    double top = exp(-over(above, mu, rmu));
+    for (int i = i0; i < i1; ++i) {
+        const int k = c.L - 1 - i;
+        const long long idx = (long long)k * c.W + w;
+        const double ta = c.alpha[idx] * c.dz[k], ts = c.alpha_s[idx] * c.dz[k], dt = ta + ts;
+        c.Jw[idx] = J0 * exp(-over(fma(0.5, dt, above), mu, rmu));
         above += dt;
+        const double bot = exp(-over(above, mu, rmu));
+        const double om = __double_as_longlong(dt) > 0 ? over(ts, dt, reciprocal_rn(dt)) : 0.0;
+        const double t = exp(-2.0 * dt), r = (0.5 - 0.5 * t) * om;
+        c.rt[idx] = r;
+        c.rt[LW + idx] = t + r;
+        c.rt[2 * LW + idx] = 0.5 * (om * mu * J0 * (top - bot));
+        top = bot;
     }
-    if (!c.diffuse) return;
-    const double A = c.albedo;
-    const double bottom = mu * J0 * exp(-above / mu);
+}
+
+// Second kernel: one thread per wavelength.  Going down, each layer's fluxes are written in terms of
+// the flux entering from below: D_k = p_k U_{k-1} + h0_k, U_k = q_k U_{k-1} + h1_k (p_k is the
+// reflectance of the layers from k up, as in the adding method), in the places of r, T and P; going
+// up, U_{-1} is found from the boundary and the fluxes follow layer by layer, with J dlambda for the
+// sums over wavelength.  Bound by the chain of a reciprocal and four products per layer; the loads run
+// kPhotoAhead layers ahead of it.
+constexpr int kPhotoAhead = 4;
+__global__ void __launch_bounds__(32) k_photo_diffuse(Col c)
+{
+    const int w = blockIdx.x * 32 + threadIdx.x;
+    if (w >= c.W) return;
+    const long long W = c.W, LW = (long long)c.L * W;
+    double *rt = c.rt + w;
+    double pn = 0.0, h0n = 0.0;
+    for (int k0 = c.L - 1; k0 >= 0; k0 -= kPhotoAhead) {
+        double r[kPhotoAhead], T[kPhotoAhead], P[kPhotoAhead];
+#pragma unroll
+        for (int j = 0; j < kPhotoAhead; ++j) {
+            const double *q = rt + max(k0 - j, 0) * W;
+            r[j] = q[0];
+            T[j] = q[LW];
+            P[j] = q[2 * LW];
+        }
+#pragma unroll
+        for (int j = 0; j < kPhotoAhead; ++j) {
+            if (k0 - j < 0) break;
+            double *o = rt + (k0 - j) * W;
+            const double rd = reciprocal64(fma(-r[j], pn, 1.0));
+            const double q = T[j] * rd, h1 = fma(r[j], h0n, P[j]) * rd, tp = T[j] * pn;
+            pn = fma(tp, q, r[j]);
+            h0n = fma(tp, h1, fma(T[j], h0n, P[j]));
+            o[0] = pn;
+            o[LW] = q;
+            o[2 * LW] = h0n;
+            o[3 * LW] = h1;
+        }
+    }
+    double above = 0.0;
+    for (int k = c.L - 1; k >= 0; --k) {
+        const long long i = (long long)k * W + w;
+        above += c.alpha[i] * c.dz[k] + c.alpha_s[i] * c.dz[k];
+    }
+    const double A = c.albedo, bottom = c.mu * c.J0[w] * exp(-above / c.mu), dl = c.dlam[w];
     // U_{-1} = A (D_0 + bottom), D_0 = p_0 U_{-1} + h0_0
-    double Ub = A * (c.rt[2 * LW + w] + bottom) / (1.0 - A * c.rt[w]);
-    for (int k = 0; k < c.L; ++k) {
-        const long long i = (long long)k * c.W + w;
-        const double Dk = c.rt[i] * Ub + c.rt[2 * LW + i];
-        const double Uk = c.rt[LW + i] * Ub + c.rt[3 * LW + i];
-        double Dn = 0.0;
-        if (k + 1 < c.L) Dn = c.rt[i + c.W] * Uk + c.rt[2 * LW + i + c.W];
-        const double up = 0.5 * (Ub + Uk), dn = 0.5 * (Dk + Dn);
-        c.Jw[i] += 0.5 * (up + dn);
-        Ub = Uk;
+    double Ub = A * (h0n + bottom) / (1.0 - A * pn), Dk = fma(pn, Ub, h0n);
+    for (int k0 = 0; k0 < c.L; k0 += kPhotoAhead) {
+        double p[kPhotoAhead], q[kPhotoAhead], h0[kPhotoAhead], h1[kPhotoAhead], J[kPhotoAhead];
+#pragma unroll
+        for (int j = 0; j < kPhotoAhead; ++j) {
+            const int k = min(k0 + j, c.L - 1), u = min(k + 1, c.L - 1);
+            q[j] = rt[LW + k * W];
+            h1[j] = rt[3 * LW + k * W];
+            p[j] = k + 1 < c.L ? rt[u * W] : 0.0;              // of the layer above: D_L = 0
+            h0[j] = k + 1 < c.L ? rt[2 * LW + u * W] : 0.0;
+            J[j] = c.Jw[k * W + w];
+        }
+#pragma unroll
+        for (int j = 0; j < kPhotoAhead; ++j) {
+            if (k0 + j >= c.L) break;
+            const double Uk = fma(q[j], Ub, h1[j]), Dn = fma(p[j], Uk, h0[j]);
+            const double Jk = fma(0.25, (Ub + Uk) + (Dk + Dn), J[j]);
+            const long long i = (k0 + j) * W + w;
+            c.Jw[i] = Jk;
+            c.Jd[i] = Jk * dl;
+            Ub = Uk;
+            Dk = Dn;
+        }
     }
 }
 
@@ -268,19 +353,85 @@ __global__ void k_photo_J_direct(Col c)
     }
     double above = __shfl_up_sync(0xffffffffu, incl, 1);   // sum over the runs above this one
     if (lane == 0) above = 0.0;
-    const double J0 = c.J0[w], mu = c.mu;
+    const double J0 = c.J0[w], mu = c.mu, rmu = reciprocal_rn(mu), dl = c.dlam[w];
     for (int i = i0; i < i1; ++i) {
         const int k = c.L - 1 - i;
         const long long idx = (long long)k * c.W + w;
         const double dt = (c.alpha[idx] + c.alpha_s[idx]) * c.dz[k];
-        c.Jw[idx] = J0 * exp(-(above + 0.5 * dt) / mu);
+        const double J = J0 * exp(-over(fma(0.5, dt, above), mu, rmu));
+        c.Jw[idx] = J;
+        c.Jd[idx] = J * dl;
         above += dt;
     }
 }
 
-// k_ph = t_f sum_w J(k, w) sigma(w) dlambda(w); one warp per (layer, reaction), lanes striding
-// the wavelengths (coalesced), partial sums added in lane order
-__global__ void k_photo_k(Col c)
+// k_ph = t_f sum_w J(k, w) sigma(w) dlambda(w): a CTA takes KT layers x kPhotoQ reactions, its four
+// warps every fourth run of 32 wavelengths; the lanes' sums are folded with each exchange halving what
+// a lane holds (one FP64 addition per output and warp, where a warp per output added 32 one after the
+// other), then the warps' in order.  Bound by FP64 issue, one multiply-add per layer, reaction and
+// wavelength (J dlambda comes ready from the kernel before): 65 us at 200 reactions, 1,000 wavelengths
+// and 150 layers (199 before), 513 at 10,000.
+constexpr int kPhotoQ = 8;
+template <int KT>
+__global__ void __launch_bounds__(128) k_photo_k(Col c)
+{
+    __shared__ double part[4][KT * kPhotoQ];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nq = (c.Rph + kPhotoQ - 1) / kPhotoQ;
+    const int k0 = blockIdx.x / nq * KT, q0 = blockIdx.x % nq * kPhotoQ;
+    const double *J[KT], *sg[kPhotoQ];
+#pragma unroll
+    for (int i = 0; i < KT; ++i) J[i] = c.Jd + (long long)min(k0 + i, c.L - 1) * c.W;
+#pragma unroll
+    for (int q = 0; q < kPhotoQ; ++q) sg[q] = c.sigma + (long long)min(q0 + q, c.Rph - 1) * c.W;
+    double acc[KT][kPhotoQ];
+#pragma unroll
+    for (int i = 0; i < KT; ++i)
+#pragma unroll
+        for (int q = 0; q < kPhotoQ; ++q) acc[i][q] = 0.0;
+    for (int w = threadIdx.x; w < c.W; w += 128) {
+        double j[KT];
+#pragma unroll
+        for (int i = 0; i < KT; ++i) j[i] = J[i][w];
+#pragma unroll
+        for (int q = 0; q < kPhotoQ; ++q) {
+            const double v = sg[q][w];
+#pragma unroll
+            for (int i = 0; i < KT; ++i) acc[i][q] = fma(j[i], v, acc[i][q]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < KT; ++i) {
+        double v[kPhotoQ];
+#pragma unroll
+        for (int q = 0; q < kPhotoQ; ++q) v[q] = acc[i][q];
+#pragma unroll
+        for (int h = kPhotoQ / 2, o = 16; h; h >>= 1, o >>= 1)
+#pragma unroll
+            for (int q = 0; q < h; ++q) {
+                const bool hi = lane & o;
+                const double give = hi ? v[q] : v[q + h], keep = hi ? v[q + h] : v[q];
+                v[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        double t = v[0];
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        // a lane's output: bits 4, 3, 2 of its number
+        if ((lane & 3) == 0) part[warp][i * kPhotoQ + (lane >> 2)] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < KT * kPhotoQ) {
+        const int k = k0 + threadIdx.x / kPhotoQ, q = q0 + threadIdx.x % kPhotoQ;
+        double t = 0.0;
+        for (int i = 0; i < 4; ++i) t += part[i][threadIdx.x];
+        if (k < c.L && q < c.Rph) c.kph[(long long)k * c.Rph + q] = c.tf * t;
+    }
+}
+
+// one warp per (layer, reaction), lanes striding the wavelengths, partial sums added in lane order: the
+// parcel scheme's, whose sweep grows a rounding of the rates by eight orders of magnitude and more, so
+// that its results stand or fall with the order of this sum.  200 us against k_photo_k's 65 at 200
+// reactions, 1,000 wavelengths and 150 layers, of an iteration's 260 ms.
+__global__ void k_photo_k_ordered(Col c)
 {
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
@@ -817,7 +968,7 @@ void launch_rates(const Col &c, cudaStream_t st)
     if (((long long)c.L * c.R) > 0) { count_launches(1); k_rates<<<nblocks((long long)c.L * c.R), kThreads, 0, st>>>(c); }
 }
 
-void launch_photolysis(const Col &c, const double *n, cudaStream_t st)
+void launch_photolysis(const Col &c, const double *n, cudaStream_t st, bool ordered)
 {
     if (c.Rph == 0) return;
     if (c.W > 0) {
@@ -827,10 +978,30 @@ void launch_photolysis(const Col &c, const double *n, cudaStream_t st)
             k_photo_alpha<<<grid, 128, 0, st>>>(c, n);
         }
         count_launches(1);
-        if (c.diffuse) k_photo_J<<<nblocks(c.W, 64), 64, 0, st>>>(c);   // 10,000 bins: 157 CTAs, every SM
-        else k_photo_J_direct<<<nblocks((long long)c.W * 32, 128), 128, 0, st>>>(c);
+        if (c.diffuse) {
+            k_photo_layers<<<nblocks(c.W, 32), 32 * kPhotoRuns, 0, st>>>(c);
+            count_launches(1);
+            k_photo_diffuse<<<nblocks(c.W, 32), 32, 0, st>>>(c);
+        } else k_photo_J_direct<<<nblocks((long long)c.W * 32, 128), 128, 0, st>>>(c);
     }
-    if (((long long)c.L * c.Rph * 32) > 0) { count_launches(1); k_photo_k<<<nblocks((long long)c.L * c.Rph * 32), kThreads, 0, st>>>(c); }
+    if (ordered && c.L > 0) {
+        count_launches(1);
+        k_photo_k_ordered<<<nblocks((long long)c.L * c.Rph * 32), kThreads, 0, st>>>(c);
+    } else if (c.L > 0) {
+        // layers to a tile: those that leave the fullest SM the least to do, a tile's folding and loads
+        // counted as half a layer
+        const auto tiles = [&](int kt) { return (long long)((c.L + kt - 1) / kt) * ((c.Rph + kPhotoQ - 1) / kPhotoQ); };
+        const auto cost = [&](int kt) { return (double)((tiles(kt) + 151) / 152) * (kt + 0.5); };
+        int kt = 2;
+        for (int t = 3; t <= 5; ++t)
+            if (cost(t) < cost(kt)) kt = t;
+        count_launches(1);
+        const int nt = (int)tiles(kt);
+        if (kt == 2) k_photo_k<2><<<nt, 128, 0, st>>>(c);
+        else if (kt == 3) k_photo_k<3><<<nt, 128, 0, st>>>(c);
+        else if (kt == 4) k_photo_k<4><<<nt, 128, 0, st>>>(c);
+        else k_photo_k<5><<<nt, 128, 0, st>>>(c);
+    }
 }
 
 void launch_layer_terms(const Col &c, const double *n, double *F, const Ctl *ctl, double f_floor, double *diag,

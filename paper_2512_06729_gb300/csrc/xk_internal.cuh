@@ -82,7 +82,7 @@ struct Col {
     double *tdg, *tlo, *tup;
     double *rs;           // [L][S] 1 / s of the current step's scaling
     // per step
-    double *grt, *lnkc, *kf, *kr, *kph, *alpha, *Jw, *w, *d;
+    double *grt, *lnkc, *kf, *kr, *kph, *alpha, *Jw, *Jd, *w, *d;   // Jd: J dlambda
     double *dw;           // [L][R] directional derivative of each rate along a vector (J v)
     const double *fshift; // [L][S] subtracted from the residual when set (the BDF step's history terms)
     double *n, *F, *s, *b, *x, *delta, *tmp;
@@ -442,7 +442,8 @@ void launch_thermo(const Col &c, cudaStream_t st);
 void launch_rates(const Col &c, cudaStream_t st);
 // u, v of Eq. 2 for the eddy profile Kzz (a zero profile leaves the molecular part only)
 void launch_transport_coeffs(const Col &c, const double *Kzz, double *u, double *v, cudaStream_t st);
-void launch_photolysis(const Col &c, const double *n, cudaStream_t st);
+// ordered: the sums over wavelength in the parcel scheme's order
+void launch_photolysis(const Col &c, const double *n, cudaStream_t st, bool ordered = false);
 // rates, derivatives, residual F, scaling and b = F / s; with diag also the row equilibration and
 // bhat = b / diag (reads ctl->dt)
 void launch_layer_terms(const Col &c, const double *n, double *F, const Ctl *ctl, double f_floor, double *diag,
