@@ -85,6 +85,8 @@ struct xk_ctx {
     bool use_cluster_solve64 = false;
     BcrPlan bcr;           // block cyclic reduction on the tensor cores (mixed path, fp32_bcr)
     bool use_bcr = false;
+    Bcr64Plan bcr64;       // the same in FP64 (plain FP64 path, small blocks)
+    bool use_bcr64 = false;
     bool ready = false;
     // equilibrium initial state and pathway analyser
     PathGraph pgraph{};
@@ -477,6 +479,17 @@ int basis_size(const xk_ctx *c)
     return m;
 }
 
+// Whether the plain FP64 path factors by the reduction: blocks it was made for, a refinement around it,
+// and no setting that asks for a particular elimination.  Below kBcr64MinLayers the elimination's chain
+// is as short as the reduction's.
+constexpr int kBcr64MinLayers = 8;
+bool bcr64_wanted(const xk_ctx *c)
+{
+    const xk_config &g = c->cfg;
+    return g.precision == XK_PREC_FP64 && g.refine_max_iter > 0 && !g.fp64_panel && (g.panel_width == 0 || g.panel_width == 8) &&
+           g.factor_ctas == 0 && g.cluster_size == 0 && g.twisted == 1 && c->S <= kBcr64Max && c->L >= kBcr64MinLayers;
+}
+
 // Lay out the workspace; with base == nullptr only the size is computed.
 size_t layout(xk_ctx *c, char *base)
 {
@@ -564,6 +577,21 @@ size_t layout(xk_ctx *c, char *base)
     c->gm = b.take<GmState>(1);
     if (c->cfg.precision == XK_PREC_FP64) {
         c->A32 = nullptr; c->lo32 = nullptr; c->up32 = nullptr;
+        if (bcr64_wanted(c)) {
+            const Bcr64Sizes z = bcr64_sizes(L, S);
+            Bcr64Plan &q = c->bcr64;
+            q.D = c->A64; q.lo = c->lo64; q.up = c->up64;
+            q.INV = b.take<double>(z.inv);
+            q.CP = b.take<double>(z.cp);
+            q.PQ = b.take<double>(z.pq);
+            q.bw = b.take<double>(z.vec);
+            q.tw = b.take<double>(z.vec);
+            q.xw = b.take<double>(z.vec);
+            q.inv_d = b.take<Bcr64Inv>(z.ninv);
+            q.gemm_d = b.take<Bcr64Gemm>(std::max(z.ngemm, 1));
+            q.mv_d = b.take<BcrMvT<double>>(z.nmv);
+            q.sol_d = b.take<BcrStage>(z.nsol);
+        }
     } else if (c->cfg.fp32_bcr) {
         // FP32 blocks padded to Sp x Sp per layer (identity in the padding), and the reduction's arrays
         const BcrSizes z = bcr_sizes(L, S);
@@ -609,7 +637,7 @@ size_t layout(xk_ctx *c, char *base)
     c->dinv = b.take<double>(32 * 32);
     c->ymid = b.take<double>(2 * (size_t)S);
     c->bar = b.take<unsigned>(factor64_words());
-    c->bcr.bar = c->bar ? c->bar + 4 : nullptr;      // words 4-5: the reduction's solve and FGMRES
+    c->bcr.bar = c->bcr64.bar = c->bar ? c->bar + 4 : nullptr;      // words 4-5: the reduction's solve and FGMRES
     c->ctl = b.take<Ctl>(1);
     c->ctl_aux = b.take<Ctl>(1);
     // Lagrangian parcel scheme
@@ -709,7 +737,7 @@ cudaError_t factor32(xk_ctx *c, Ctl *ctl, const int *skip)
 cudaError_t solve32(xk_ctx *c, const double *b, double *x, Ctl *ctl, cudaStream_t st, const double *bscale,
                     const int *skip)
 {
-    if (c->use_bcr) return bcr_solve(c->bcr, b, x, bscale, nullptr, skip, ctl, st);
+    if (c->use_bcr) return bcr_solve(solve_of(c->bcr), b, x, bscale, nullptr, skip, ctl, st);
     if (c->use_cluster_solve && c->use_cluster && cluster_twisted(c->cplan, c->L) && c->splan.twisted)
         return launch_solve_twisted<float>(sys32(c), c->splan, false, b, x, c->gsol, c->ymid, ctl, st, bscale, skip);
     if (c->use_cluster_solve && !(c->use_cluster && cluster_twisted(c->cplan, c->L)))
@@ -788,8 +816,11 @@ cudaError_t enqueue_refine64(xk_ctx *c, const Col &col, Ctl *ctl, const FactorPl
     a.matvec = [col, ctl, rowd](const double *x, double *y, const int *sk, cudaStream_t s) {
         launch_jv(col, ctl, x, y, rowd, sk, s);
     };
-    a.precond = [c, plan, ctl, rowd](const double *v, double *z, const int *sk, cudaStream_t s) {
-        solve64(c, plan, v, z, ctl, s, rowd, sk, nullptr);
+    const bool reduced = c->use_bcr64 && !skip;
+    if (reduced && !col.photo_jac) return bcr_fgmres(solve_of(c->bcr64), col, a, rowd, c->st);
+    a.precond = [c, plan, ctl, rowd, reduced](const double *v, double *z, const int *sk, cudaStream_t s) {
+        if (reduced) bcr_solve(solve_of(c->bcr64), v, z, rowd, nullptr, sk, ctl, s);
+        else solve64(c, plan, v, z, ctl, s, rowd, sk, nullptr);
     };
     return enqueue_fgmres(a, c->st);
 }
@@ -822,7 +853,10 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
             PhaseMark m(c, XK_PH_JACOBIAN);
             launch_jacobian64(col, ctl, dt_override, 1, c->A64, c->lo64, c->up64, st);
         }
-        { PhaseMark m(c, XK_PH_FACTOR); e = launch_factor<double>(sys64(c), c->plan, ctl, st); }
+        {
+            PhaseMark m(c, XK_PH_FACTOR);
+            e = c->use_bcr64 ? bcr64_factor(c->bcr64, ctl, st) : launch_factor<double>(sys64(c), c->plan, ctl, st);
+        }
         if (e != cudaSuccess) return fail(c, XK_ECUDA, "factor launch: %s", cudaGetErrorString(e));
         PhaseMark m(c, XK_PH_SOLVE);
         if (refine > 0)
@@ -867,7 +901,7 @@ int enqueue_linear_step(xk_ctx *c, const double *n, double dt_override, double *
         };
         if (c->use_bcr && !col.photo_jac) {
             PhaseMark m(c, XK_PH_SOLVE);
-            e = bcr_fgmres(c->bcr, col, a, rowd, st);
+            e = bcr_fgmres(solve_of(c->bcr), col, a, rowd, st);
             if (e != cudaSuccess) return fail(c, XK_ECUDA, "solve launch: %s", cudaGetErrorString(e));
         } else {
             PhaseMark m(c, XK_PH_SOLVE);
@@ -1295,6 +1329,11 @@ int xk_set_workspace(xk_ctx *c, void *dptr, size_t bytes)
     c->use_cluster = false;
     c->use_cluster_solve = false;
     c->use_bcr = sz == 4 && c->cfg.fp32_bcr;
+    c->use_bcr64 = bcr64_wanted(c);
+    if (c->use_bcr64) {
+        const cudaError_t be = bcr64_build(c->bcr64, c->L, c->S, c->col.ld, c->st);
+        if (be != cudaSuccess) return fail(c, XK_ECUDA, "FP64 reduction plan: %s", cudaGetErrorString(be));
+    }
     c->use_cluster_solve64 = c->cfg.cluster_size >= 0 && solve_cluster_plan(c->S, 8, &c->splan64) == 0;
     set_preview(c, &c->plan64);
     if (sz == 8) set_preview(c, &c->plan);
@@ -1657,9 +1696,10 @@ int xk_hold_next_barrier(xk_ctx *c)
     int rc = need_ready(c);
     if (rc) return rc;
     // arrival counts that a grid of at most 2^30 CTAs never completes, for both counter pairs
-    // (the whole grid, and the second half of a two-chain elimination)
-    const unsigned held[4] = {1u << 30, 0u, 1u << 30, 0u};
-    cudaMemcpyAsync(c->bar, held, sizeof held, cudaMemcpyHostToDevice, c->st);
+    // (the whole grid, and the second half of a two-chain elimination); where the factorization has
+    // none, for the solve's, whose waits end at their count or above: as far below it
+    const unsigned held[6] = {1u << 30, 0u, 1u << 30, 0u, 3u << 30, 0u};
+    cudaMemcpyAsync(c->bar, held, (c->use_bcr64 ? 6 : 4) * sizeof(unsigned), cudaMemcpyHostToDevice, c->st);
     return finish_eval(c, "hold_next_barrier");
 }
 
@@ -1797,7 +1837,7 @@ int xk_batch_remove(xk_batch *b, int slot)
     s.ctx->st = s.saved_st;
     s.ctx->plan = s.saved_plan;
     s.ctx->plan64 = s.saved_plan64;
-    s.ctx->bcr.solve_ctas = s.saved_solve_ctas;
+    s.ctx->bcr.solve_ctas = s.ctx->bcr64.solve_ctas = s.saved_solve_ctas;
     if (s.ev) cudaEventDestroy(s.ev);
     cudaStreamDestroy(s.st);
     b->used -= s.bytes;
@@ -1863,7 +1903,7 @@ int xk_batch_add(xk_batch *b, xk_ctx *c, double dt0, int *slot)
     s.saved_plan = c->plan;
     s.saved_plan64 = c->plan64;
     s.saved_solve_ctas = c->bcr.solve_ctas;
-    c->bcr.solve_ctas = share;          // the reduction's cooperative solve on this column's share of the SMs
+    c->bcr.solve_ctas = c->bcr64.solve_ctas = share;          // the reduction's cooperative solve on this column's share of the SMs
     s.bytes = c->ws_bytes;
     s.finished = false;
     c->st = s.st;

@@ -535,16 +535,6 @@ struct Builder {
     }
     TcOut out_view(View v, int z, float alpha, int n) const { return out(v.arr, z, v.r0, v.c0, alpha, 0.0f, n, false); }
 
-    void mv_stage(std::vector<BcrMv> &ts, int level)
-    {
-        if (ts.empty()) return;
-        BcrStage s{kBcrMv, (int)p.mv.size(), (int)ts.size(), 0, 0, level};
-        p.mv.insert(p.mv.end(), ts.begin(), ts.end());
-        p.sol.push_back(s);
-    }
-    float *vec(float *a, int k) const { return a ? a + (size_t)k * Sp : nullptr; }
-    const float *row(const float *a, int k) const { return a ? a + (size_t)k * S : nullptr; }
-
     void build()
     {
         std::vector<int> w;
@@ -552,23 +542,11 @@ struct Builder {
         depth_col.assign(w.size() + 1, 0);
         for (size_t d = 0; d < w.size(); ++d) depth_col[d + 1] = depth_col[d] + w[d];
         p.Wt = std::max(32, (depth_col.back() + 31) / 32 * 32);
-        // the levels of the reduction
-        std::vector<std::vector<int>> lists{std::vector<int>(L)};
-        for (int k = 0; k < L; ++k) lists[0][k] = k;
-        while (lists.back().size() > 1) {
-            const auto &a = lists.back();
-            std::vector<int> kept;
-            for (size_t q = 0; q < a.size(); q += 2) kept.push_back(a[q]);
-            lists.push_back(kept);
-        }
+        const BcrLevels lv(L);
+        const auto &lists = lv.lists;
+        const auto &cp_off = lv.cp_off;
         p.levels = (int)lists.size() - 1;
-        std::vector<int> cp_off(lists.size(), 0);
-        int ncp = 0;
-        for (size_t l = 1; l < lists.size(); ++l) {
-            cp_off[l] = ncp;
-            ncp += (int)lists[l].size();
-        }
-        p.Ncp = std::max(ncp, 1);
+        p.Ncp = std::max(lv.ncp, 1);
         int zt = 1;
         for (int l = 0; l < p.levels; ++l) zt = std::max(zt, (int)lists[l].size() / 2);
         p.Zt = zt;
@@ -623,83 +601,109 @@ struct Builder {
         }
         const int root = lists.back()[0];
         inverse(Sp, Dfull, std::vector<int>{root}, Ifull, std::vector<int>{root}, 0, p.levels);
-        // solve: right-hand sides are read where they are first needed, and those of the layers kept
-        // at level 0 with the coupling terms to their eliminated neighbours taken off on the way
-        auto rhs0 = [&](int i, int &layer, const float *&c0, const float *&w0, const float *&c1, const float *&w1) {
-            layer = i;
-            if (i >= 1) { c0 = row(p.lo, i); w0 = vec(p.tw, i - 1); }
-            if (i + 1 < L) { c1 = row(p.up, i); w1 = vec(p.tw, i + 1); }
-        };
-        auto mv = [](const float *M, int ld, int K, float sign, float *y) {
-            BcrMv t{};
-            t.M = M; t.ld = ld; t.K = K; t.sign = sign; t.y = y;
-            t.in = t.bin = t.out = -1;
-            return t;
-        };
-        for (int l = 0; l < p.levels; ++l) {
-            const auto &a = lists[l];
-            std::vector<BcrMv> ts;
-            for (size_t q = 1; q < a.size(); q += 2) {       // t_j = D_j^-1 b_j
-                const int j = a[q];
-                BcrMv t = mv(ptr(kArrINV, j, 0, 0), Sp, Sp, 1.0f, vec(p.tw, j));
-                if (l == 0) t.in = j;
-                else if (l == 1) rhs0(j, t.in, t.d0, t.w0, t.d1, t.w1);
-                else t.v0 = vec(p.bw, j);
-                ts.push_back(t);
-            }
-            mv_stage(ts, l);
-            if (l == 0) continue;
-            ts.clear();
-            for (size_t q = 0; q < a.size(); q += 2) {       // b_i -= L_i t_l + U_i t_r
-                const int i = a[q];
-                const int cpi = cp_off[l] + (int)q;
-                const bool hl = q >= 1, hr = q + 1 < a.size();
-                if (!hl && !hr) continue;
-                BcrMv t = mv(ptr(kArrCP, cpi, 0, hl ? 0 : Sp), 2 * Sp, hl && hr ? 2 * Sp : Sp, -1.0f, vec(p.bw, i));
-                if (l == 1) rhs0(i, t.bin, t.e0, t.f0, t.e1, t.f1);
-                else t.base = vec(p.bw, i);
-                t.v0 = vec(p.tw, hl ? a[q - 1] : a[q + 1]);
-                if (hl && hr) t.v1 = vec(p.tw, a[q + 1]);
-                ts.push_back(t);
-            }
-            mv_stage(ts, l);
-        }
-        {
-            BcrMv t = mv(ptr(kArrINV, root, 0, 0), Sp, Sp, 1.0f, vec(p.xw, root));
-            if (p.levels == 0) t.in = root;
-            else if (p.levels == 1) rhs0(root, t.in, t.d0, t.w0, t.d1, t.w1);
-            else t.v0 = vec(p.bw, root);
-            t.out = root;
-            std::vector<BcrMv> ts{t};
-            mv_stage(ts, p.levels);
-        }
-        for (int l = p.levels - 1; l >= 0; --l) {
-            const auto &a = lists[l];
-            std::vector<BcrMv> ts;
-            for (size_t q = 1; q < a.size(); q += 2) {
-                const int j = a[q];
-                const bool hr = q + 1 < a.size();
-                BcrMv t;
-                if (l == 0) {      // x_j = D_j^-1 (b_j - lo_j x_{j-1} - up_j x_{j+1})
-                    t = mv(ptr(kArrINV, j, 0, 0), Sp, Sp, 1.0f, vec(p.xw, j));
-                    t.in = j;
-                    t.d0 = row(p.lo, j); t.w0 = vec(p.xw, a[q - 1]);
-                    if (hr) { t.d1 = row(p.up, j); t.w1 = vec(p.xw, a[q + 1]); }
-                } else {           // x_j = t_j - [P_j | Q_j] [x_l; x_r]
-                    t = mv(ptr(kArrPQ, j, 0, 0), 2 * Sp, hr ? 2 * Sp : Sp, -1.0f, vec(p.xw, j));
-                    t.v0 = vec(p.xw, a[q - 1]);
-                    t.v1 = hr ? vec(p.xw, a[q + 1]) : nullptr;
-                    t.base = vec(p.tw, j);
-                }
-                t.out = j;
-                ts.push_back(t);
-            }
-            mv_stage(ts, l);
-        }
+        bcr_solve_tasks(lv, BcrArrays<float>{p.INV, p.CP, p.PQ, p.lo, p.up, p.bw, p.tw, p.xw, L, S, Sp, Sp}, p.mv, p.sol);
     }
 };
 
 }  // namespace
+
+// Right-hand sides are read where they are first needed, and those of the layers kept at level 0 with
+// the coupling terms to their eliminated neighbours taken off on the way.
+template <typename T>
+void bcr_solve_tasks(const BcrLevels &lv, const BcrArrays<T> &p, std::vector<BcrMvT<T>> &out, std::vector<BcrStage> &sol)
+{
+    using Mv = BcrMvT<T>;
+    const auto &lists = lv.lists;
+    const auto &cp_off = lv.cp_off;
+    const int L = p.L, S = p.S, Sp = p.ld, levels = (int)lists.size() - 1, root = lists.back()[0];
+    const size_t blk = (size_t)p.rows * Sp;
+    // the lists are also sized before the arrays exist
+    auto inv = [&](int k) { return p.INV ? p.INV + k * blk : nullptr; };
+    auto cp = [&](int q, int c) { return p.CP ? p.CP + q * 2 * blk + c : nullptr; };
+    auto pq = [&](int k) { return p.PQ ? p.PQ + k * 2 * blk : nullptr; };
+    auto vec = [&](T *a, int k) { return a ? a + (size_t)k * Sp : nullptr; };
+    auto row = [&](const T *a, int k) { return a ? a + (size_t)k * S : nullptr; };
+    auto mv_stage = [&](std::vector<Mv> &ts, int level) {
+        if (ts.empty()) return;
+        sol.push_back(BcrStage{kBcrMv, (int)out.size(), (int)ts.size(), 0, 0, level});
+        out.insert(out.end(), ts.begin(), ts.end());
+    };
+    auto rhs0 = [&](int i, int &layer, const T *&c0, const T *&w0, const T *&c1, const T *&w1) {
+        layer = i;
+        if (i >= 1) { c0 = row(p.lo, i); w0 = vec(p.tw, i - 1); }
+        if (i + 1 < L) { c1 = row(p.up, i); w1 = vec(p.tw, i + 1); }
+    };
+    auto mv = [](const T *M, int ld, int K, T sign, T *y) {
+        Mv t{};
+        t.M = M; t.ld = ld; t.K = K; t.sign = sign; t.y = y;
+        t.in = t.bin = t.out = -1;
+        return t;
+    };
+    for (int l = 0; l < levels; ++l) {
+        const auto &a = lists[l];
+        std::vector<Mv> ts;
+        for (size_t q = 1; q < a.size(); q += 2) {       // t_j = D_j^-1 b_j
+            const int j = a[q];
+            Mv t = mv(inv(j), Sp, Sp, T(1), vec(p.tw, j));
+            if (l == 0) t.in = j;
+            else if (l == 1) rhs0(j, t.in, t.d0, t.w0, t.d1, t.w1);
+            else t.v0 = vec(p.bw, j);
+            ts.push_back(t);
+        }
+        mv_stage(ts, l);
+        if (l == 0) continue;
+        ts.clear();
+        for (size_t q = 0; q < a.size(); q += 2) {       // b_i -= L_i t_l + U_i t_r
+            const int i = a[q];
+            const int cpi = cp_off[l] + (int)q;
+            const bool hl = q >= 1, hr = q + 1 < a.size();
+            if (!hl && !hr) continue;
+            Mv t = mv(cp(cpi, hl ? 0 : Sp), 2 * Sp, hl && hr ? 2 * Sp : Sp, -T(1), vec(p.bw, i));
+            if (l == 1) rhs0(i, t.bin, t.e0, t.f0, t.e1, t.f1);
+            else t.base = vec(p.bw, i);
+            t.v0 = vec(p.tw, hl ? a[q - 1] : a[q + 1]);
+            if (hl && hr) t.v1 = vec(p.tw, a[q + 1]);
+            ts.push_back(t);
+        }
+        mv_stage(ts, l);
+    }
+    {
+        Mv t = mv(inv(root), Sp, Sp, T(1), vec(p.xw, root));
+        if (levels == 0) t.in = root;
+        else if (levels == 1) rhs0(root, t.in, t.d0, t.w0, t.d1, t.w1);
+        else t.v0 = vec(p.bw, root);
+        t.out = root;
+        std::vector<Mv> ts{t};
+        mv_stage(ts, levels);
+    }
+    for (int l = levels - 1; l >= 0; --l) {
+        const auto &a = lists[l];
+        std::vector<Mv> ts;
+        for (size_t q = 1; q < a.size(); q += 2) {
+            const int j = a[q];
+            const bool hr = q + 1 < a.size();
+            Mv t;
+            if (l == 0) {      // x_j = D_j^-1 (b_j - lo_j x_{j-1} - up_j x_{j+1})
+                t = mv(inv(j), Sp, Sp, T(1), vec(p.xw, j));
+                t.in = j;
+                t.d0 = row(p.lo, j); t.w0 = vec(p.xw, a[q - 1]);
+                if (hr) { t.d1 = row(p.up, j); t.w1 = vec(p.xw, a[q + 1]); }
+            } else {           // x_j = t_j - [P_j | Q_j] [x_l; x_r]
+                t = mv(pq(j), 2 * Sp, hr ? 2 * Sp : Sp, -T(1), vec(p.xw, j));
+                t.v0 = vec(p.xw, a[q - 1]);
+                t.v1 = hr ? vec(p.xw, a[q + 1]) : nullptr;
+                t.base = vec(p.tw, j);
+            }
+            t.out = j;
+            ts.push_back(t);
+        }
+        mv_stage(ts, l);
+    }
+}
+
+template void bcr_solve_tasks<float>(const BcrLevels &, const BcrArrays<float> &, std::vector<BcrMv> &, std::vector<BcrStage> &);
+template void bcr_solve_tasks<double>(const BcrLevels &, const BcrArrays<double> &, std::vector<BcrMvT<double>> &,
+                                      std::vector<BcrStage> &);
 
 BcrSizes bcr_sizes(int L, int S)
 {

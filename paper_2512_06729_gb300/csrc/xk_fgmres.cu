@@ -32,27 +32,45 @@ struct Rhs {
     double mult;
 };
 
+template <typename T>
 struct ApplyArgs {
     const BcrStage *stages;
-    const BcrMv *mv;
-    int nstages, L, S, Sp;
+    const BcrMvT<T> *mv;
+    int nstages, S, rows, ld;
+};
+// Four floats or two doubles of a row at a time.
+template <typename T>
+struct Wide;
+template <>
+struct Wide<float> {
+    using type = float4;
+    static __device__ __forceinline__ float dot(float acc, float4 a, float4 x)
+    {
+        return acc + (a.x * x.x + a.y * x.y + a.z * x.z + a.w * x.w);
+    }
+};
+template <>
+struct Wide<double> {
+    using type = double2;
+    static __device__ __forceinline__ double dot(double acc, double2 a, double2 x) { return fma(a.y, x.y, fma(a.x, x.x, acc)); }
 };
 
 // Entry k of a task's vector: the right-hand side of a layer or a work vector, less diagonal
 // coupling terms (level 0) on the first S entries.
-__device__ __forceinline__ float rhs_term(const Rhs &r, int layer, const float *v, int k, int S, const float *d0,
-                                          const float *w0, const float *d1, const float *w1)
+template <typename T>
+__device__ __forceinline__ T rhs_term(const Rhs &r, int layer, const T *v, int k, int S, const T *d0, const T *w0,
+                                      const T *d1, const T *w1)
 {
-    float val;
+    T val;
     if (layer >= 0) {
-        val = 0.0f;
+        val = T(0);
         if (k < S) {
             const long long q = (long long)layer * S + k;
             const double b = r.b[q] * r.mult;
-            val = (float)(r.bscale ? b * r.bscale[q] : b);
+            val = (T)(r.bscale ? b * r.bscale[q] : b);
         }
     } else {
-        val = v ? v[k] : 0.0f;
+        val = v ? v[k] : T(0);
     }
     if (k < S) {
         if (d0) val -= d0[k] * w0[k];
@@ -62,26 +80,24 @@ __device__ __forceinline__ float rhs_term(const Rhs &r, int layer, const float *
 }
 
 // Rows [row, row + RPW) of M v, one warp: all of a lane's loads of RPW rows in flight together.
-template <int RPW>
-__device__ __forceinline__ void mv_rows(const BcrMv &t, const float *v, int row, int nrow, float (&out)[RPW])
+template <int RPW, typename T>
+__device__ __forceinline__ void mv_rows(const BcrMvT<T> &t, const T *v, int row, int nrow, T (&out)[RPW])
 {
+    using V = typename Wide<T>::type;
     const int lane = threadIdx.x & 31;
-    const float4 *m[RPW];
-    float acc[RPW];
+    const V *m[RPW];
+    T acc[RPW];
 #pragma unroll
     for (int i = 0; i < RPW; ++i) {
-        m[i] = (const float4 *)(t.M + (long long)(row + min(i, nrow - 1)) * t.ld);
-        acc[i] = 0.0f;
+        m[i] = (const V *)(t.M + (long long)(row + min(i, nrow - 1)) * t.ld);
+        acc[i] = T(0);
     }
-    const int n4 = t.K / 4;
+    const int n4 = t.K * (int)sizeof(T) / 16;
 #pragma unroll 4
     for (int q = lane; q < n4; q += 32) {
-        const float4 x = *(const float4 *)(v + 4 * q);
+        const V x = ((const V *)v)[q];
 #pragma unroll
-        for (int i = 0; i < RPW; ++i) {
-            const float4 a = __ldg(m[i] + q);
-            acc[i] += a.x * x.x + a.y * x.y + a.z * x.z + a.w * x.w;
-        }
+        for (int i = 0; i < RPW; ++i) acc[i] = Wide<T>::dot(acc[i], __ldg(m[i] + q), x);
     }
 #pragma unroll
     for (int i = 0; i < RPW; ++i) {
@@ -93,38 +109,38 @@ __device__ __forceinline__ void mv_rows(const BcrMv &t, const float *v, int row,
 
 // One stage: chunks of kWarps * RPW rows of every task's block, contiguous chunks to a CTA so that
 // the task's vector in shared memory is filled once for several of them.
-template <int RPW>
-__device__ __forceinline__ void mv_stage(const ApplyArgs &a, const BcrStage &st, const Rhs &rhs, double *x,
-                                         const double *xscale, float *v)
+template <int RPW, typename T>
+__device__ __forceinline__ void mv_stage(const ApplyArgs<T> &a, const BcrStage &st, const Rhs &rhs, double *x,
+                                         const double *xscale, T *v)
 {
-    const int S = a.S, Sp = a.Sp, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rows = kWarps * RPW, chunks = (Sp + rows - 1) / rows, items = st.count * chunks;
+    const int S = a.S, Sp = a.ld, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rows = kWarps * RPW, chunks = (a.rows + rows - 1) / rows, items = st.count * chunks;
     const int G = gridDim.x, per = items / G, rest = items - per * G, b = blockIdx.x;
     const int i0 = b * per + min(b, rest), i1 = i0 + per + (b < rest ? 1 : 0);
     int have = -1;
     for (int item = i0; item < i1; ++item) {
         const int ti = item / chunks, chunk = item - ti * chunks;
-        const BcrMv &t = a.mv[st.off + ti];
+        const BcrMvT<T> &t = a.mv[st.off + ti];
         if (ti != have) {
             __syncthreads();
             for (int k = threadIdx.x; k < t.K; k += kThreads)
-                v[k] = k < Sp ? rhs_term(rhs, t.in, t.v0, k, S, t.d0, t.w0, t.d1, t.w1) : t.v1[k - Sp];
+                v[k] = k < Sp ? rhs_term<T>(rhs, t.in, t.v0, k, S, t.d0, t.w0, t.d1, t.w1) : t.v1[k - Sp];
             __syncthreads();
             have = ti;
         }
-        const int row = chunk * rows + warp * RPW, nrow = min(RPW, Sp - row);
+        const int row = chunk * rows + warp * RPW, nrow = min(RPW, a.rows - row);
         if (nrow <= 0) continue;
-        float out[RPW];
-        mv_rows<RPW>(t, v, row, nrow, out);
-        float mine = out[0];
+        T out[RPW];
+        mv_rows<RPW, T>(t, v, row, nrow, out);
+        T mine = out[0];
 #pragma unroll
         for (int i = 1; i < RPW; ++i)
             if (lane == i) mine = out[i];
         if (lane < nrow) {
             const int r = row + lane;
-            float base = 0.0f;
-            if (t.bin >= 0 || t.base) base = rhs_term(rhs, t.bin, t.base, r, S, t.e0, t.f0, t.e1, t.f1);
-            const float y = base + t.sign * mine;
+            T base = T(0);
+            if (t.bin >= 0 || t.base) base = rhs_term<T>(rhs, t.bin, t.base, r, S, t.e0, t.f0, t.e1, t.f1);
+            const T y = base + t.sign * mine;
             t.y[r] = y;
             if (t.out >= 0 && r < S) {
                 const long long q = (long long)t.out * S + r;
@@ -135,15 +151,16 @@ __device__ __forceinline__ void mv_stage(const ApplyArgs &a, const BcrStage &st,
 }
 
 // x = M^-1 rhs: every stage, a grid barrier after each but the last.  false: a wait gave up.
-__device__ __forceinline__ bool bcr_apply(const ApplyArgs &a, const Rhs &rhs, double *x, const double *xscale, float *v,
+template <typename T>
+__device__ __forceinline__ bool bcr_apply(const ApplyArgs<T> &a, const Rhs &rhs, double *x, const double *xscale, T *v,
                                           GridSync &gs)
 {
     for (int si = 0; si < a.nstages; ++si) {
         const BcrStage st = a.stages[si];
         // four rows to a warp where the stage has that much work for every CTA, else one
-        const int total = st.count * a.Sp;
-        if (total >= 4 * kWarps * (int)gridDim.x) mv_stage<4>(a, st, rhs, x, xscale, v);
-        else mv_stage<1>(a, st, rhs, x, xscale, v);
+        const int total = st.count * a.rows;
+        if (total >= 4 * kWarps * (int)gridDim.x) mv_stage<4, T>(a, st, rhs, x, xscale, v);
+        else mv_stage<1, T>(a, st, rhs, x, xscale, v);
         if (si + 1 < a.nstages && !gs.sync()) return false;
     }
     return true;
@@ -154,14 +171,15 @@ __device__ __forceinline__ bool stopped(const int *skip, const Ctl *ctl)
     return (ctl && (ctl->finished || ctl->err_timeout)) || (skip && *skip);
 }
 
+template <typename T>
 __global__ void __launch_bounds__(kThreads, 1)
-k_bcr_solve(ApplyArgs a, const double *b, const double *bscale, double *x, const double *xscale, unsigned *words,
+k_bcr_solve(ApplyArgs<T> a, const double *b, const double *bscale, double *x, const double *xscale, unsigned *words,
             const int *skip, Ctl *ctl)
 {
     if (stopped(skip, ctl)) return;
     extern __shared__ __align__(16) unsigned char dyn[];
     GridSync gs(words, ctl);
-    bcr_apply(a, Rhs{b, bscale, 1.0}, x, xscale, (float *)dyn, gs);
+    bcr_apply<T>(a, Rhs{b, bscale, 1.0}, x, xscale, (T *)dyn, gs);
     gs.leave();
 }
 
@@ -170,9 +188,10 @@ k_bcr_solve(ApplyArgs a, const double *b, const double *bscale, double *x, const
 // same iteration as enqueue_fgmres (cycles of m within max_iter, one short spare cycle, convergence
 // decided on the true residual at each cycle's start).  A CTA owns whole layers of every vector.
 // ---------------------------------------------------------------------------
+template <typename T>
 struct FgArgs {
     Col c;
-    ApplyArgs ap;
+    ApplyArgs<T> ap;
     const double *b, *rowd;
     double *x, *V, *Z, *w, *partials;
     unsigned *words;
@@ -180,7 +199,7 @@ struct FgArgs {
     Ctl *ctl;
     const int *skip;
     double tol;
-    int m, max_iter, rates_in_smem;
+    int m, max_iter, rates_in_smem, role;
 };
 
 struct FgShared {
@@ -201,7 +220,8 @@ __device__ __forceinline__ double warp_sum(double v)
 // CTA, then (after the barrier) every CTA adds the layers' parts in the same order, so that the sums
 // do not depend on how many CTAs the launch has.  The parts alternate between two buffers: a CTA past
 // the barrier may write its next parts while another still adds the last ones.
-__device__ __forceinline__ bool fg_dots(const FgArgs &a, int nv, const double *w, double *h, GridSync &gs, int &buf)
+template <typename T>
+__device__ __forceinline__ bool fg_dots(const FgArgs<T> &a, int nv, const double *w, double *h, GridSync &gs, int &buf)
 {
     const int S = a.c.S, L = a.c.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double *parts = a.partials + (long long)(buf ^= 1) * L * (kMaxBasis + 1);
@@ -230,7 +250,8 @@ __device__ __forceinline__ bool fg_dots(const FgArgs &a, int nv, const double *w
     return true;
 }
 
-__global__ void __launch_bounds__(kThreads, 1) k_fgmres(FgArgs a)
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1) k_fgmres(FgArgs<T> a)
 {
     if (stopped(a.skip, a.ctl)) return;
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -239,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fgmres(FgArgs a)
     const int S = c.S, L = c.L, G = gridDim.x, tid = threadIdx.x;
     const long long N = (long long)L * S;
     GridSync gs(a.words, a.ctl);
-    float *v = (float *)dyn;
+    T *v = (T *)dyn;
     double *jv = (double *)dyn;
 
     // f(e) for every element this CTA owns, the same thread for the same element each time
@@ -290,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fgmres(FgArgs a)
             // every CTA's part of w is written (the barrier of the norm above); V_j is this CTA's copy
             double *vj = a.V + (long long)j * N, *zj = a.Z + (long long)j * N;
             own([&](long long e) { vj[e] = a.w[e] * scale; });
-            if (!(ok = bcr_apply(a.ap, Rhs{a.w, a.rowd, scale}, zj, nullptr, v, gs))) break;
+            if (!(ok = bcr_apply<T>(a.ap, Rhs{a.w, a.rowd, scale}, zj, nullptr, v, gs))) break;
             if (!(ok = gs.sync())) break;
             matvec(zj);
             if (!(ok = fg_dots(a, j + 1, a.w, sh.h1, gs, buf))) break;
@@ -378,9 +399,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_fgmres(FgArgs a)
         ctl->solver_iters = iters;
         ctl->solver_resid = resid;
         ctl->total_iters += iters;
-        // a solve that did not reach the tolerance hands the step to the FP64 factorization, and so
-        // does every later step at this dt or above
-        if (failed || !(resid <= a.tol)) {
+        // a solve around the FP32 factors that did not reach the tolerance hands the step to the FP64
+        // factorization, and so does every later step at this dt or above
+        if (a.role == 0 && (failed || !(resid <= a.tol))) {
             ctl->skip64 = 0;
             ctl->used_fp64 = 1;
             if (ctl->dt < ctl->dt_fp64) ctl->dt_fp64 = ctl->dt;
@@ -401,16 +422,18 @@ int sm_count()
 }
 
 // One CTA per SM, or the column's share of them in a batch.
-int solve_ctas(const BcrPlan &p) { return p.solve_ctas > 0 ? std::min(p.solve_ctas, sm_count()) : sm_count(); }
+int solve_ctas(int share) { return share > 0 ? std::min(share, sm_count()) : sm_count(); }
 
-ApplyArgs apply_args(const BcrPlan &p) { return ApplyArgs{p.sol_d, p.mv_d, (int)p.sol.size(), p.L, p.S, p.Sp}; }
+template <typename T>
+ApplyArgs<T> apply_args(const BcrSolveT<T> &p) { return {p.stages, p.mv, p.nstages, p.S, p.rows, p.ld}; }
 
+template <typename T>
 cudaError_t smem_limits()
 {
     static const cudaError_t e = [] {
-        cudaError_t r = cudaFuncSetAttribute(k_bcr_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
+        cudaError_t r = cudaFuncSetAttribute(k_bcr_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
         if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_fgmres, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
+            r = cudaFuncSetAttribute(k_fgmres<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
         return r;
     }();
     return e;
@@ -418,25 +441,27 @@ cudaError_t smem_limits()
 
 }  // namespace
 
-cudaError_t bcr_solve(const BcrPlan &p, const double *b, double *x, const double *bscale, const double *xscale,
+template <typename T>
+cudaError_t bcr_solve(const BcrSolveT<T> &p, const double *b, double *x, const double *bscale, const double *xscale,
                       const int *skip, Ctl *ctl, cudaStream_t st)
 {
-    cudaError_t e = smem_limits();
+    cudaError_t e = smem_limits<T>();
     if (e != cudaSuccess) return e;
-    ApplyArgs a = apply_args(p);
+    ApplyArgs<T> a = apply_args(p);
     unsigned *words = p.bar;
     void *args[] = {(void *)&a, (void *)&b, (void *)&bscale, (void *)&x, (void *)&xscale, (void *)&words, (void *)&skip,
                     (void *)&ctl};
     count_launches(1);
-    return cudaLaunchCooperativeKernel((const void *)k_bcr_solve, dim3(solve_ctas(p)), dim3(kThreads), args,
-                                       (size_t)2 * p.Sp * sizeof(float), st);
+    return cudaLaunchCooperativeKernel((const void *)k_bcr_solve<T>, dim3(solve_ctas(p.ctas)), dim3(kThreads), args,
+                                       (size_t)2 * p.ld * sizeof(T), st);
 }
 
-cudaError_t bcr_fgmres(const BcrPlan &p, const Col &c, const GmArgs &g, const double *rowd, cudaStream_t st)
+template <typename T>
+cudaError_t bcr_fgmres(const BcrSolveT<T> &p, const Col &c, const GmArgs &g, const double *rowd, cudaStream_t st)
 {
-    cudaError_t e = smem_limits();
+    cudaError_t e = smem_limits<T>();
     if (e != cudaSuccess) return e;
-    FgArgs a;
+    FgArgs<T> a;
     a.c = c;
     a.ap = apply_args(p);
     a.b = g.b;
@@ -449,12 +474,20 @@ cudaError_t bcr_fgmres(const BcrPlan &p, const Col &c, const GmArgs &g, const do
     a.tol = g.tol;
     a.m = std::min(g.m, kMaxBasis);
     a.max_iter = g.max_iter;
+    a.role = g.role;
     a.rates_in_smem = jv_rates_in_smem(c) ? 1 : 0;
-    const size_t smem = std::max((size_t)2 * p.Sp * sizeof(float), jv_smem_doubles(c, a.rates_in_smem != 0) * sizeof(double));
+    const size_t smem = std::max((size_t)2 * p.ld * sizeof(T), jv_smem_doubles(c, a.rates_in_smem != 0) * sizeof(double));
     if (smem > kJvSmemMax) return cudaErrorInvalidValue;
     void *args[] = {(void *)&a};
     count_launches(1);
-    return cudaLaunchCooperativeKernel((const void *)k_fgmres, dim3(solve_ctas(p)), dim3(kThreads), args, smem, st);
+    return cudaLaunchCooperativeKernel((const void *)k_fgmres<T>, dim3(solve_ctas(p.ctas)), dim3(kThreads), args, smem, st);
 }
+
+template cudaError_t bcr_solve<float>(const BcrSolveT<float> &, const double *, double *, const double *, const double *,
+                                      const int *, Ctl *, cudaStream_t);
+template cudaError_t bcr_solve<double>(const BcrSolveT<double> &, const double *, double *, const double *, const double *,
+                                       const int *, Ctl *, cudaStream_t);
+template cudaError_t bcr_fgmres<float>(const BcrSolveT<float> &, const Col &, const GmArgs &, const double *, cudaStream_t);
+template cudaError_t bcr_fgmres<double>(const BcrSolveT<double> &, const Col &, const GmArgs &, const double *, cudaStream_t);
 
 }  // namespace xk
