@@ -353,31 +353,49 @@ cudaError_t launch_leaf(const BcrLeaf *tasks, int count, int n, const int *skip,
 // Level 0 (diagonal couplings), for each kept even layer i with eliminated neighbours l = i-1, r = i+1:
 //   D_i -= diag(lo_i) INV_l diag(up_l) + diag(up_i) INV_r diag(lo_r)
 //   CP(1, i/2) = [ -diag(lo_i) INV_l diag(lo_l) | -diag(up_i) INV_r diag(up_r) ]
-__global__ void k_bcr_level0(float *D, const float *INV, float *CP, const float *lo, const float *up, const int *kept,
-                             int L, int S, int Sp, const int *skip, const Ctl *ctl)
+// Four columns to a thread.  Bound by memory: at 594 species x 150 layers 555 MB, 81 us at the copy
+// rate if the second reading of each inverse comes from L2, and takes 98; entry by entry it took 221.
+__global__ void __launch_bounds__(256) k_bcr_level0(float *D, const float *INV, float *CP, const float *lo,
+                                                     const float *up, const int *kept, int L, int S, int Sp,
+                                                     const int *skip, const Ctl *ctl)
 {
     if (stop(skip, ctl)) return;
-    const int i = kept[blockIdx.y];
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)Sp * Sp) return;
-    const int y = (int)(e / Sp), c = (int)(e - (long long)y * Sp);
-    const long long blk = (long long)Sp * Sp;
+    const int i = kept[blockIdx.y], q = blockIdx.x * 256 + threadIdx.x, w4 = Sp / 4;
+    if (q >= Sp * w4) return;
+    const int y = q / w4, c = (q - y * w4) * 4;
+    const long long blk = (long long)Sp * Sp, e = (long long)y * Sp + c;
     const bool hasl = i >= 1, hasr = i + 1 < L;
+    float4 gl = make_float4(0, 0, 0, 0), gr = gl, d = *(const float4 *)(D + i * blk + e);
+    if (hasl) gl = *(const float4 *)(INV + (i - 1) * blk + e);
+    if (hasr) gr = *(const float4 *)(INV + (i + 1) * blk + e);
     const float loi = (hasl && y < S) ? lo[(long long)i * S + y] : 0.0f;
     const float upi = (hasr && y < S) ? up[(long long)i * S + y] : 0.0f;
-    float upd = 0.0f;
-    float *cp = CP + (long long)(i / 2) * Sp * 2 * Sp + (long long)y * 2 * Sp;
+    auto at = [&](const float *a, int k, int j) { return c + j < S ? a[(long long)k * S + c + j] : 0.0f; };
+    float *cp = CP + (long long)(i / 2) * Sp * 2 * Sp + (long long)y * 2 * Sp + c;
+    float upd[4] = {0.0f, 0.0f, 0.0f, 0.0f}, o[4];
     if (hasl) {
-        const float g = INV[(long long)(i - 1) * blk + e];
-        upd += loi * g * (c < S ? up[(long long)(i - 1) * S + c] : 0.0f);
-        if (i >= 2) cp[c] = -loi * g * (c < S ? lo[(long long)(i - 1) * S + c] : 0.0f);
+        const float g[4] = {gl.x, gl.y, gl.z, gl.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            upd[j] += loi * g[j] * at(up, i - 1, j);
+            o[j] = -loi * g[j] * at(lo, i - 1, j);
+        }
+        if (i >= 2) *(float4 *)cp = make_float4(o[0], o[1], o[2], o[3]);
     }
     if (hasr) {
-        const float g = INV[(long long)(i + 1) * blk + e];
-        upd += upi * g * (c < S ? lo[(long long)(i + 1) * S + c] : 0.0f);
-        if (i + 2 <= L - 1) cp[Sp + c] = -upi * g * (c < S ? up[(long long)(i + 1) * S + c] : 0.0f);
+        const float g[4] = {gr.x, gr.y, gr.z, gr.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            upd[j] += upi * g[j] * at(lo, i + 1, j);
+            o[j] = -upi * g[j] * at(up, i + 1, j);
+        }
+        if (i + 2 <= L - 1) *(float4 *)(cp + Sp) = make_float4(o[0], o[1], o[2], o[3]);
     }
-    D[(long long)i * blk + e] -= upd;
+    d.x -= upd[0];
+    d.y -= upd[1];
+    d.z -= upd[2];
+    d.w -= upd[3];
+    *(float4 *)(D + i * blk + e) = d;
 }
 
 __global__ void k_bcr_pad(float *D, int L, int S, int Sp)
@@ -807,7 +825,7 @@ cudaError_t bcr_factor(const BcrPlan &p, const int *skip, Ctl *ctl, cudaStream_t
         }
         case kBcrLevel0:
             count_launches(1);
-            k_bcr_level0<<<dim3(nblk((long long)p.Sp * p.Sp, 256), s.count), 256, 0, st>>>(
+            k_bcr_level0<<<dim3(nblk((long long)p.Sp * p.Sp / 4, 256), s.count), 256, 0, st>>>(
                 p.D, p.INV, p.CP, p.lo, p.up, p.l0_d, p.L, p.S, p.Sp, skip, ctl);
             break;
         default:

@@ -541,9 +541,11 @@ k_layer_terms(Col c, const double *n, double *F, const Ctl *ctl, double f_floor,
 // its lanes then sum whole columns of the row from there, each in a fixed order, eight rows to a
 // CTA; a species in more than kJacOcc reactions (the bath gas is in thousands) takes a whole CTA.
 // Gathering every term of every entry from global memory instead is bound by its latency: 1,290 us
-// at 594 species x 150 layers.  Bound now by the FP64 additions of the terms (4.2e7, about 75 us at
-// this part's two FP64 operations per clock and SM) beside the write of the blocks (222 MB in FP32,
-// 33 us); only non-zero entries are scaled and converted, which FP64 units do too.
+// at 594 species x 150 layers, this 390.  Bound by FP64 issue and latency: the additions of the terms
+// (4.2e7, about 75 us if every lane had the same number) and two products and a conversion per non-zero
+// entry; beside them the write of the blocks (222 MB in FP32, 33 us).  An entry of more than kJacLong
+// terms (the diagonal has one per reaction of the row) is summed by the warp, four of them together,
+// since one lane's chain held up the other 31 (541 us).
 template <typename T>
 __global__ void __launch_bounds__(kJacWarps * 32)
 k_jacobian(Col c, const Ctl *ctl, double dt_override, int scaled, T *A, T *lo, T *up, const int *skip, long long lstride)
@@ -562,28 +564,49 @@ k_jacobian(Col c, const Ctl *ctl, double dt_override, int scaled, T *A, T *lo, T
     // derivatives of tile t's reactions, by nt threads of which this is number id
     auto load_tile = [&](const double2 *dk, int t, double *dst, int id, int nt) {
         const int o0 = c.jto[t], n = (c.jto[t + 1] - o0) * 3;
-        for (int b = id; b < n; b += 4 * nt) {
-            double2 v[4];
+        for (int b = id; b < n; b += 8 * nt) {
+            double2 v[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < 8; ++u) {
                 const int e = min(b + u * nt, n - 1), occ = e / 3;
                 v[u] = dk[3 * (long long)(c.yent[o0 + occ] >> 4) + (e - 3 * occ)];
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < 8; ++u)
                 if (b + u * nt < n) ((double2 *)dst)[b + u * nt] = v[u];
         }
     };
-    auto group_sum = [&](const double *src, int g) {
+    // every step-th term from t to t1 (an addition of nothing costs as much as any other: the first
+    // term is taken as it is)
+    auto lane_sum = [&](const double *src, int t, int t1, int step) {
         double acc = 0.0;
-        const int t1 = c.jge[g + 1];
+        if (t < t1) {
+            const int code = c.jterm[t];
+            acc = signed_by(src[code >> 1], code & 1);
+            t += step;
+        }
 #pragma unroll 4
-        for (int t = c.jge[g]; t < t1; ++t) {
+        for (; t < t1; t += step) {
             const int code = c.jterm[t];
             acc += signed_by(src[code >> 1], code & 1);
         }
         return acc;
     };
+    auto group_sum = [&](const double *src, int g) { return lane_sum(src, c.jge[g], c.jge[g + 1], 1); };
+    // the sums of long groups g .. g + 3 (those below g1), by the warp: a lane's terms, then exchanges
+    // of which the first two halve the groups a lane holds; lane l gets group g + l / 8
+    auto long_sums = [&](const double *src, int g, int g1) {
+        double v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = g + q < g1 ? lane_sum(src, c.jge[g + q] + lane, c.jge[g + q + 1], 32) : 0.0;
+        const bool h16 = lane & 16, h8 = lane & 8;
+        const double a0 = (h16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
+        const double a1 = (h16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
+        double t = (h8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
+        for (int o = 4; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        return t;
+    };
+    auto is_long = [&](int g) { return c.jge[g + 1] - c.jge[g] > kJacLong; };
     auto couplings = [&](int k, int i) {
         const long long q = (long long)k * S + i;
         double lov = c.tlo[q], upv = c.tup[q];
@@ -612,12 +635,33 @@ k_jacobian(Col c, const Ctl *ctl, double dt_override, int scaled, T *A, T *lo, T
             if (t < c.jrt[i + 1]) {                       // one tile at most
                 load_tile(dk, t, dbuf, lane, 32);
                 __syncwarp();
-                for (int g = c.jtg[t] + lane; g < c.jtg[t + 1]; g += 32) {
-                    const int j = c.jgc[g];
-                    double v = group_sum(dbuf, g);
-                    if (j == i) v += diag;
-                    if (scaled && j != i) v = v * sk[j] * inv;
-                    row[j] = (T)v;
+                const int g1 = c.jtg[t + 1];
+                for (int g = c.jtg[t]; g < g1;) {
+                    // the longest come first: up to 32 of them one after the other, a lane keeping
+                    // each, then a lane for each of the next 32
+                    const int g0 = g;
+                    double v = 0.0;
+                    int n = 0;
+                    for (; n < 32 && g < g1 && is_long(g); n += 4, g += 4) {
+                        const double s = long_sums(dbuf, g, g1);
+                        const double mine = __shfl_sync(0xffffffffu, s, (lane & 3) * 8);
+                        if (lane >> 2 == n >> 2) v = mine;
+                    }
+                    if (g > g1) {
+                        n -= g - g1;
+                        g = g1;
+                    }
+                    if (n == 0) {
+                        n = min(32, g1 - g);
+                        if (lane < n) v = group_sum(dbuf, g + lane);
+                        g += n;
+                    }
+                    if (lane < n) {
+                        const int j = c.jgc[g0 + lane];
+                        if (j == i) v += diag;
+                        if (scaled && j != i) v = v * sk[j] * inv;
+                        row[j] = (T)v;
+                    }
                 }
             }
             if (lane == 0) {
@@ -638,8 +682,16 @@ k_jacobian(Col c, const Ctl *ctl, double dt_override, int scaled, T *A, T *lo, T
                 __syncthreads();
                 load_tile(dk, t, dall, threadIdx.x, blockDim.x);
                 __syncthreads();
-                for (int g = c.jtg[t] + threadIdx.x; g < c.jtg[t + 1]; g += blockDim.x)
-                    hrow[c.jgc[g]] += group_sum(dall, g);
+                // long groups four to a warp, the others a thread each (the longest come first)
+                const int g1 = c.jtg[t + 1];
+                const int g0 = c.jtg[t];
+                for (int g = g0 + 4 * warp; g < g1 && is_long(g); g += 4 * kJacWarps) {
+                    const double v = long_sums(dall, g, g1);
+                    if (!(lane & 7) && g + (lane >> 3) < g1) hrow[c.jgc[g + (lane >> 3)]] += v;
+                }
+                // (a group of four that began with a long one is done)
+                for (int g = g0 + threadIdx.x; g < g1; g += blockDim.x)
+                    if (!is_long(g0 + ((g - g0) & ~3))) hrow[c.jgc[g]] += group_sum(dall, g);
             }
             __syncthreads();
             T *Ar = A + (long long)k * lstride + (long long)i * ld;
@@ -1018,6 +1070,10 @@ void launch_layer_terms(const Col &c, const double *n, double *F, const Ctl *ctl
     k_layer_terms<<<std::min(c.L, kGatedBlocks), 512, sm, st>>>(c, n, F, ctl, f_floor, diag, bhat, rates ? 1 : 0);
 }
 
+// Blocks of few items each, the longest rows in the first: the hardware's order of them evens out what
+// rows of unequal length leave (1,216 blocks of three to an SM end in a third of a wave).
+constexpr long long kJacBlocks = 152 * 24;
+
 template <typename T>
 static void launch_jacobian_t(const Col &c, const Ctl *ctl, double dt_override, int scaled, T *A, T *lo, T *up,
                               cudaStream_t st, const int *skip, long long lstride)
@@ -1027,8 +1083,8 @@ static void launch_jacobian_t(const Col &c, const Ctl *ctl, double dt_override, 
     cudaFuncSetAttribute(k_jacobian<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const long long items = (long long)c.nji * c.L;
     count_launches(1);
-    k_jacobian<T><<<(int)std::min<long long>(items, kGatedBlocks), kJacWarps * 32, sm, st>>>(c, ctl, dt_override, scaled, A, lo,
-                                                                                           up, skip, lstride);
+    k_jacobian<T><<<(int)std::min<long long>(items, kJacBlocks), kJacWarps * 32, sm, st>>>(c, ctl, dt_override, scaled, A, lo,
+                                                                                         up, skip, lstride);
 }
 
 void launch_jacobian64(const Col &c, const Ctl *ctl, double dt_override, int scaled, double *A, double *lo, double *up,

@@ -113,6 +113,7 @@ struct Ctl {
     double dt_fp64;       // smallest dt at which the FP32-preconditioned solve did not converge
 };
 
+constexpr int kJacLong = 8;      // terms of a Jacobian entry above which a warp sums them
 constexpr int kJacWarps = 8, kJacOcc = 128, kJacHeavyOcc = kJacWarps * kJacOcc;
 constexpr int kEqSub = 24;      // terms of an equilibrium entry summed by one lane: the longest entry has some
                                 // 24 x 24 (hydrogen with itself), the two chains of FP64 additions are even
