@@ -27,7 +27,7 @@ namespace xk {
 namespace {
 
 constexpr int kInvThreads = 256;
-constexpr int kInvWorkers = kInvThreads / 32 - 1;
+constexpr int kInvBusy = 96;              // FP64 instructions of a step above which warp 4 works too
 constexpr size_t kInvSmemMax = 220 * 1024;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -222,11 +222,14 @@ __global__ void __launch_bounds__(kInvThreads, 1) k_inv64(const Bcr64Inv *tasks,
         }
     } else {
         // column l belongs to one warp throughout; of its columns, the ones due next come first
-        const int wk = warp - 1, own = (ncol - wk + kInvWorkers - 1) / kInvWorkers;
+        // (warp 4 shares the lead's FP64 unit: it works only where the units are what bounds the step)
+        const bool four = ncol * RPT > kInvBusy;
+        const int nwk = four ? 7 : 6, wk = warp == 4 ? (four ? 3 : ncol) : warp - 1 - (warp > 4 && !four);
+        const int own = wk < ncol ? (ncol - wk + nwk - 1) / nwk : 0;
         int first = 0, m0 = 0;                          // the lead's column (first after c), own's first behind it
         for (int c = 0; c < S; ++c) {
             if (rank + cs * first <= c) ++first;
-            while (m0 < own && wk + kInvWorkers * m0 <= first) ++m0;
+            while (m0 < own && wk + nwk * m0 <= first) ++m0;
             mbar_wait(ready0 + 8 * c, ctl);
             const double *v = slots + (size_t)c * lay.slot;
             const int p = prow[c];
@@ -236,7 +239,7 @@ __global__ void __launch_bounds__(kInvThreads, 1) k_inv64(const Bcr64Inv *tasks,
             for (int q = 0; q < own; ++q) {
                 int m = m0 + q;
                 if (m >= own) m -= own;
-                const int l = wk + kInvWorkers * m, j = rank + cs * l;
+                const int l = wk + nwk * m, j = rank + cs * l;
                 if (l == first || j == c) continue;     // the lead's
                 double *x = cols + l * S;
                 const double ap = x[p];
