@@ -24,13 +24,14 @@ namespace {
 
 constexpr int kMaxWarps = 32;
 constexpr int kRefineSweeps = 2;          // FP64 iterative-refinement sweeps of every implicit step
-constexpr size_t kSmemLimit = 200 * 1024; // dynamic shared memory the kernel may ask for
+constexpr size_t kSmemLimit = 208 * 1024; // dynamic shared memory the kernel may ask for
 
 struct Shared {
     double red[kMaxWarps];
     int ired[kMaxWarps];
     double h, t, hs;
     int last, done;
+    int piv[2];
 };
 
 __device__ __forceinline__ int nwarps() { return blockDim.x >> 5; }
@@ -317,13 +318,15 @@ __global__ void __launch_bounds__(1024, 1) k_parcel_iteration(Col c, ParcelArgs 
 // ---------------------------------------------------------------------------
 // systems of at most kSmallS species: matrices in shared memory
 // ---------------------------------------------------------------------------
-// A step is a chain of small dependent operations, and what it costs is their latency: an FP64 result
-// takes some 180 clocks, a division ten of them, a comparison as much as a product, a barrier thirty.
-// So pivots are compared as bit patterns, by every warp for itself; a column of the elimination has one
-// barrier; its reciprocals are kept for the triangular solves, which one warp does with the vector in
-// registers; and every sum is formed in the order of the general kernel, whose results these are bit
-// for bit (a parcel carries a rounding through hundreds of steps, grown many orders of magnitude).
-// A step of 40 species takes 71 us, on the general kernel (matrices in shared memory too) 185.
+// A step is a chain of small dependent operations.  An FP64 instruction holds its unit (one to four
+// warps) for 65 clocks, whatever the lanes do, and its result takes no longer; a division is ten of
+// them, a comparison as much as a product.  So pivots are compared as bit patterns; the column that is
+// pivoted next is a warp's own business while the others eliminate; its reciprocals are kept for the
+// triangular solves, which one warp does with the vector in registers; and every sum is formed in the
+// order of the general kernel, whose results these are bit for bit (a parcel carries a rounding
+// through hundreds of steps, grown many orders of magnitude).  A step of 40 species takes 60 us, on the
+// general kernel (its matrices in shared memory) 187: the elimination has two fifths of it, the three
+// solves over a third, the assembly and the residuals a tenth each.
 constexpr int kSmallS = 128;
 constexpr int kSmallThreads = 256;
 constexpr int kSmallWarps = kSmallThreads / 32;
@@ -340,102 +343,113 @@ __device__ __forceinline__ unsigned long long pivot_key(double v)
 // apart, so that 32 rows of a column lie in 32 banks.
 struct SmallLayout {
     int ld;
-    size_t vec, mats, rates, bytes;
+    size_t mats, rates, bytes;
 };
 __host__ __device__ inline SmallLayout small_layout(int S, int R, bool rates_in_smem)
 {
     SmallLayout l;
     l.ld = S | 1;
-    l.vec = 0;                                     // x, F, d, r, gain, loss, loss / dz, 1 / pivots; then the row order
-    l.mats = 8 * (size_t)S + (size_t)(S + 1) / 2;
+    // before the matrices: x, F, d, r, gain, loss, loss / dz, 1 / pivots, two columns; then the row order
+    l.mats = 10 * (size_t)S + (size_t)(S + 1) / 2;
     l.rates = l.mats + 2 * (size_t)S * l.ld;
     l.bytes = (l.rates + (rates_in_smem ? 7 * (size_t)R : 0)) * sizeof(double);
     return l;
 }
 
-// A <- its LU factors, order[i] the original row at place i, inv the pivots' reciprocals.  Every warp
-// finds the pivot and the multipliers of column c for itself and updates its own columns j > c, rows
-// along the lanes, reading the rows where they were and writing them where the exchange puts them; the
-// last warp keeps the columns up to c (a column's multipliers wait in its registers until all have read
-// it).  0, or -1 on a zero pivot column, in every thread.
-__device__ int small_factor(double *A, int ld, int *order, double *inv, int S)
+// A <- its LU factors, order[i] the original row at place i, inv the pivots' reciprocals; l: two columns
+// of multipliers.  Warp 0 runs one column ahead: while the others apply step c to the columns from c + 2
+// on, it applies it to column c + 1, finds that column's pivot (the first row of largest magnitude) and
+// multipliers, and leaves them for the next step.  It has its FP64 unit to itself: warp 4, on the same
+// one, only exchanges the rows of the finished columns.  Rows are read where they were and written where
+// the exchange puts them.  One barrier per column.  0, or -1 on a zero pivot column, in every thread.
+template <int kC>
+__device__ int small_factor_rows(double *A, int ld, int *order, double *inv, double *l, int S, Shared &sh)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kC = kSmallS / 32;
-    double held[kC];                               // multipliers of the column before (last warp)
-    for (int c = 0; c <= S; ++c) {
-        if (c && warp == kSmallWarps - 1) {
+    for (int c = -1; c + 1 < S; ++c) {
+        const int p = c >= 0 ? sh.piv[c & 1] : 0;
+        const double *lc = l + (c & 1) * S;
+        if (warp == 0) {
+            const int j = c + 1;
+            double *ln = l + (j & 1) * S;
+            const double ap = c >= 0 ? A[p * ld + j] : 0.0, ac = c >= 0 ? A[c * ld + j] : 0.0;
+            double v[kC];
+            unsigned long long best = 0ull;
+            int bi = S;
 #pragma unroll
             for (int t = 0; t < kC; ++t) {
-                const int i = c + t * 32 + lane;
-                if (i < S) A[i * ld + c - 1] = held[t];
+                v[t] = 0.0;
+                if (j + t * 32 >= S) continue;
+                const int i = j + t * 32 + lane, ii = min(i, S - 1);
+                v[t] = A[ii * ld + j];
+                if (c >= 0) v[t] = fma(-lc[ii], ap, ii == p ? ac : v[t]);
+                const unsigned long long k = i < S ? pivot_key(v[t]) : 0ull;
+                bi = k > best ? i : bi;
+                best = k > best ? k : best;
             }
-            __syncwarp();
-        }
-        if (c == S) break;
-        // the first row of largest magnitude
-        unsigned long long best = 0ull;
-        int bi = S;
+            const unsigned hi = (unsigned)(best >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+            const unsigned lo = hi == mh ? (unsigned)best : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+            const int q = (int)__reduce_min_sync(0xffffffffu, hi == mh && (unsigned)best == ml ? (unsigned)bi : 0xffffffffu);
+            if ((mh | ml) == 0u) {
+                if (lane == 0) sh.piv[j & 1] = -1;
+            } else {
+                double vp = v[0];
 #pragma unroll
-        for (int t = 0; t < kC; ++t) {
-            const int i = c + t * 32 + lane;
-            if (i < S) {
-                const unsigned long long k = pivot_key(A[i * ld + c]);
-                if (k > best) {
-                    best = k;
-                    bi = i;
+                for (int t = 1; t < kC; ++t)
+                    if (j + t * 32 < S && (q - j) >> 5 == t) vp = v[t];
+                vp = __shfl_sync(0xffffffffu, vp, (q - j) & 31);
+                const double vc = __shfl_sync(0xffffffffu, v[0], 0), ipv = reciprocal_rn(vp);
+                if (lane == 0) {
+                    if (c >= 0) A[c * ld + j] = ap;
+                    A[j * ld + j] = vp;
+                    inv[j] = ipv;
+                    const int o = order[j];
+                    order[j] = order[q];
+                    order[q] = o;
+                    sh.piv[j & 1] = q;
+                }
+#pragma unroll
+                for (int t = 0; t < kC; ++t) {
+                    if (j + t * 32 >= S) continue;
+                    const int i = j + t * 32 + lane;
+                    const double m = (i == q ? vc : v[t]) * ipv;
+                    if (i > j && i < S) A[i * ld + j] = ln[i] = m;
                 }
             }
-        }
-        const unsigned hi = (unsigned)(best >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
-        const unsigned lo = hi == mh ? (unsigned)best : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
-        if ((mh | ml) == 0u) return -1;
-        const int p = (int)__reduce_min_sync(0xffffffffu, hi == mh && (unsigned)best == ml ? (unsigned)bi : 0xffffffffu);
-        const double ipv = reciprocal_rn(A[p * ld + c]);
-        if (warp == kSmallWarps - 1) {
-            if (lane == 0) {
-                inv[c] = ipv;
-                const int o = order[c];
-                order[c] = order[p];
-                order[p] = o;
-            }
-            if (p != c)
+        } else if (warp == 4) {
+            if (c > 0 && p != c)
                 for (int j = lane; j < c; j += 32) {
                     const double t = A[c * ld + j];
                     A[c * ld + j] = A[p * ld + j];
                     A[p * ld + j] = t;
                 }
-        }
-        // multipliers of the rows c + 1 .. S - 1 as they will stand: row p's place takes row c
-        const double vc = A[c * ld + c], vp = A[p * ld + c];
-        double l[kC];
+        } else if (c >= 0) {
+            double m[kC];
 #pragma unroll
-        for (int t = 0; t < kC; ++t) {
-            const int i = c + 1 + t * 32 + lane;
-            l[t] = 0.0;
-            if (c + 1 + t * 32 < S && i < S) l[t] = (i == p ? vc : A[i * ld + c]) * ipv;
-        }
-        for (int j = c + 1 + warp; j < S; j += kSmallWarps) {
-            const double ap = A[p * ld + j], ac = A[c * ld + j];
-            __syncwarp();
-            if (lane == 0) A[c * ld + j] = ap;
+            for (int t = 0; t < kC; ++t) m[t] = c + 1 + t * 32 < S ? lc[min(c + 1 + t * 32 + lane, S - 1)] : 0.0;
+            for (int j = c + 2 + (warp < 4 ? warp - 1 : warp - 2); j < S; j += kSmallWarps - 2) {
+                const double ap = A[p * ld + j], ac = A[c * ld + j];
+                __syncwarp();
+                if (lane == 0) A[c * ld + j] = ap;
 #pragma unroll
-            for (int t = 0; t < kC; ++t) {
-                if (c + 1 + t * 32 >= S) break;
-                const int i = c + 1 + t * 32 + lane;
-                if (i < S) A[i * ld + j] = fma(-l[t], ap, i == p ? ac : A[i * ld + j]);
+                for (int t = 0; t < kC; ++t) {
+                    if (c + 1 + t * 32 >= S) continue;
+                    const int i = c + 1 + t * 32 + lane;
+                    if (i < S) A[i * ld + j] = fma(-m[t], ap, i == p ? ac : A[i * ld + j]);
+                }
             }
         }
         __syncthreads();
-        // all have read column c: the last warp writes it (with the next column's start)
-        if (warp == kSmallWarps - 1) {
-#pragma unroll
-            for (int t = 0; t < kC; ++t) held[t] = l[t];
-            if (lane == 0) A[c * ld + c] = vp;
-        }
+        if (sh.piv[(c + 1) & 1] < 0) return -1;
     }
-    __syncthreads();
     return 0;
+}
+
+__device__ int small_factor(double *A, int ld, int *order, double *inv, double *l, int S, Shared &sh)
+{
+    if (S <= 32) return small_factor_rows<1>(A, ld, order, inv, l, S, sh);
+    if (S <= 64) return small_factor_rows<2>(A, ld, order, inv, l, S, sh);
+    return small_factor_rows<4>(A, ld, order, inv, l, S, sh);
 }
 
 // x <- (LU)^-1 P f on one warp, T words of the vector to a lane.
@@ -510,7 +524,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_parcel_small(Col c, Parcel
     const SmallLayout lay = small_layout(S, R, rates_in_smem);
     const int ld = lay.ld;
     double *x = dyn, *F = x + S, *d = F + S, *r = d + S, *gain = r + S, *loss = gain + S, *ldz = loss + S, *inv = ldz + S;
-    int *order = (int *)(inv + S);
+    double *lbuf = inv + S;
+    int *order = (int *)(lbuf + 2 * S);
     double *A0 = dyn + lay.mats, *A = A0 + (size_t)S * ld;
     double *w = rates_in_smem ? dyn + lay.rates : a.w, *dd = rates_in_smem ? w + R : a.dd;
     // places of the pattern's entries in the matrices (-1 - place: on the diagonal); the general
@@ -526,8 +541,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_parcel_small(Col c, Parcel
     for (int y = tid; y < S; y += kSmallThreads) a.vmr[y] = a.N[y] / c.ngas[0];
     if (tid == 0) sh.h = st->h;
     long long steps = 0, rejected = 0;
-    // the species' sums go to the first warps, the matrix to the others
-    const int fw = min((S + 31) / 32, kSmallWarps / 2);
+    // the species' sums go to the first warp, the matrix to the others
+    const int fw = 1;
     __syncthreads();
     for (int v = 0; v < 2 * L - 1; ++v) {
         const int k = v < L ? v : 2 * L - 2 - v;
@@ -595,7 +610,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_parcel_small(Col c, Parcel
                 }
             }
             __syncthreads();
-            if (small_factor(A, ld, order, inv, S) != 0) {
+            if (small_factor(A, ld, order, inv, lbuf, S, sh) != 0) {
                 if (tid == 0) { st->status = XK_ESINGULAR; st->visit = v; }
                 return;
             }
