@@ -371,11 +371,18 @@ __global__ void k_photo_J_direct(Col c)
 // other), then the warps' in order.  Bound by FP64 issue, one multiply-add per layer, reaction and
 // wavelength (J dlambda comes ready from the kernel before): 65 us at 200 reactions, 1,000 wavelengths
 // and 150 layers (199 before), 513 at 10,000.
+//
+// Below kPhotoFaint the order of a product decides how many bits are left of it: a term loses at most
+// half the smallest double, 2.5e-324, times dlambda, and thousands of them are seen in sums below some
+// 1e-305 only.  There the sum is formed again with the products as the definition has them, (J sigma)
+// dlambda (a few rates in the layers where the beam ends, 10 us; sums of such numbers are exact or nearly).
 constexpr int kPhotoQ = 8;
+constexpr double kPhotoFaint = 1e-302;
 template <int KT>
 __global__ void __launch_bounds__(128) k_photo_k(Col c)
 {
     __shared__ double part[4][KT * kPhotoQ];
+    __shared__ int faint[KT * kPhotoQ];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nq = (c.Rph + kPhotoQ - 1) / kPhotoQ;
     const int k0 = blockIdx.x / nq * KT, q0 = blockIdx.x % nq * kPhotoQ;
     const double *J[KT], *sg[kPhotoQ];
@@ -423,7 +430,20 @@ __global__ void __launch_bounds__(128) k_photo_k(Col c)
         const int k = k0 + threadIdx.x / kPhotoQ, q = q0 + threadIdx.x % kPhotoQ;
         double t = 0.0;
         for (int i = 0; i < 4; ++i) t += part[i][threadIdx.x];
-        if (k < c.L && q < c.Rph) c.kph[(long long)k * c.Rph + q] = c.tf * t;
+        const bool in = k < c.L && q < c.Rph;
+        if (in) c.kph[(long long)k * c.Rph + q] = c.tf * t;
+        faint[threadIdx.x] = in && t > 0.0 && t < kPhotoFaint;
+    }
+    __syncthreads();
+    for (int e = warp; e < KT * kPhotoQ; e += 4) {
+        if (!faint[e]) continue;
+        const int k = k0 + e / kPhotoQ, q = q0 + e % kPhotoQ;
+        const double *Jk = c.Jw + (long long)k * c.W, *sq = c.sigma + (long long)q * c.W;
+        double t = 0.0;
+#pragma unroll 8
+        for (int w = lane; w < c.W; w += 32) t += Jk[w] * sq[w] * c.dlam[w];
+        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) c.kph[(long long)k * c.Rph + q] = c.tf * t;
     }
 }
 
@@ -433,21 +453,14 @@ __global__ void __launch_bounds__(128) k_photo_k(Col c)
 // reactions, 1,000 wavelengths and 150 layers, of an iteration's 260 ms.
 __global__ void k_photo_k_ordered(Col c)
 {
-    int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= c.L * c.Rph) return;
-    int k = warp / c.Rph, q = warp % c.Rph;
-    const double *J = c.Jw + (long long)k * c.W;
-    const double *sg = c.sigma + (long long)q * c.W;
+    const double *J = c.Jw + (long long)(warp / c.Rph) * c.W, *sg = c.sigma + (long long)(warp % c.Rph) * c.W;
     double s = 0.0;
-    for (int w = lane; w < c.W; w += 32)
-        s += J[w] * sg[w] * c.dlam[w];
+    for (int w = lane; w < c.W; w += 32) s += J[w] * sg[w] * c.dlam[w];
     double tot = 0.0;
-    for (int l = 0; l < 32; ++l) {
-        double v = __shfl_sync(0xffffffffu, s, l);
-        tot += v;
-    }
-    if (lane == 0) c.kph[(long long)k * c.Rph + q] = c.tf * tot;
+    for (int l = 0; l < 32; ++l) tot += __shfl_sync(0xffffffffu, s, l);
+    if (lane == 0) c.kph[warp] = c.tf * tot;
 }
 
 // ---------------------------------------------------------------------------
