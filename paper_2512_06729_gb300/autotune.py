@@ -18,7 +18,9 @@ import os
 from . import build as _build
 
 CANDIDATES = {
-    "fp64": [dict(panel_width=8, factor_ctas=152), dict(panel_width=16, factor_ctas=152),
+    # the first is the library's own choice (the reduction for small blocks), which an explicit number
+    # of CTAs rules out
+    "fp64": [dict(panel_width=8), dict(panel_width=8, factor_ctas=152), dict(panel_width=16, factor_ctas=152),
              dict(panel_width=8, factor_ctas=76), dict(fp64_panel=1, panel_width=8, factor_ctas=152)],
     "mixed": [dict(fp32_bcr=1),
               dict(fp32_bcr=0, cluster_size=16, panel_width=8), dict(fp32_bcr=0, cluster_size=16, panel_width=16),
@@ -44,7 +46,7 @@ def _load():
 
 
 def _key(S, precision):
-    return f"{_gpu_name()}|S={S}|{precision}|v3"
+    return f"{_gpu_name()}|S={S}|{precision}|v4"
 
 
 def measure(prob, precision, params, layers=None, reps=2):
