@@ -41,8 +41,8 @@ SAMPLE_LAYERS = 24          # CPU oracle sample: this many layers of the same co
 # a run in another configuration reports null.
 PROFILED_TRAFFIC = {
     ("mixed", 16, 8, 1): (371.3e6, "k_factor_cluster<8>, two-chain launch (profiles/k_factor_cluster_594x150.txt)"),
-    ("fp64", 152, 8, 0, 0): (833.5e6, "k_factor<double, 8> (profiles/k_factor_fp64_594x150.txt)"),
-    ("fp64", 152, 8, 0, 1): (818.6e6, "k_factor<double, 8>, two-chain launch (profiles/k_factor_fp64_594x150.txt)"),
+    ("fp64", 152, 8, 0, 0): (833.5e6, "k_factor<double, 8>, an earlier form (profiles/k_factor_fp64_594x150.txt)"),
+    ("fp64", 152, 8, 0, 1): (818.6e6, "k_factor<double, 8>, two-chain launch of an earlier form (profiles/k_factor_fp64_594x150.txt)"),
 }
 
 
@@ -483,7 +483,8 @@ def run_ours(args):
         twisted = int(cfg["twisted"] and not cfg["panel"] and L >= 3)
         key = ("fp64", cfg["ctas"], cfg["nb"], cfg["panel"], twisted)
         traffic, source = PROFILED_TRAFFIC.get(key, (None, None))
-        return {"kernel": f"k_factor<double, {cfg['nb']}>" + (" (two grid halves, then the middle layer)" if twisted else ""),
+        name = "k_factor64_flow" if cfg["nb"] == 8 and not cfg["panel"] else f"k_factor<double, {cfg['nb']}>"
+        return {"kernel": name + (" (two grid halves, then the middle layer)" if twisted else ""),
                 "bound": "alu", "achieved": achieved, "peak": live["f64"], "unit": "TFLOP/s",
                 "frac": achieved / live["f64"], "peak_kind": "FP64 matmul measured live (torch.matmul float64)",
                 "peak_derived": derived["f64"], "flops_per_factorization": flops,
@@ -795,7 +796,7 @@ def parcel_object(live, iterations=3, cpu=True, columns=152):
         "iterations_per_s": 1e3 / ms_it, "ms_per_iteration": ms_it, "implicit_steps_per_iteration": steps_it,
         "first_iteration": {"steps": int(first.steps), "rejected": int(first.rejected),
                             "max_change": float(first.max_change)},
-        "roofline": {"kernel": "k_parcel_iteration (one CTA, FP64 Gaussian elimination per implicit step)",
+        "roofline": {"kernel": "k_parcel_small / k_parcel_iteration (one CTA, FP64 Gaussian elimination per implicit step)",
                      "bound": "alu", "achieved": achieved, "peak": peak_sm, "unit": "TFLOP/s",
                      "frac": achieved / peak_sm,
                      "peak_kind": "FP64 matmul measured live / 152 SMs (the sweep is sequential: one SM)"},
@@ -984,7 +985,7 @@ def radiation_object(live, calls=5, cpu=True):
         ach = flops / (ms * 1e-3) / 1e12
         o = {"bins": W, "absorbers": n_abs, "scatterers": n_sca, "diffuse": int(prob.diffuse),
              "ms_per_evaluation": ms,
-             "roofline": {"kernels": "k_photo_alpha + k_photo_J + k_photo_k", "bound": "alu", "achieved": ach,
+             "roofline": {"kernels": "k_photo_alpha, beam and diffuse field, k_photo_k", "bound": "alu", "achieved": ach,
                           "peak": live["f64"], "unit": "TFLOP/s", "frac": ach / live["f64"],
                           "peak_kind": "FP64 matmul measured live; work = the two FP64 contractions"}}
         if cpu:

@@ -102,8 +102,8 @@ typedef struct {
                              layer (when two clusters fit and there are at least 3 layers); 0 keeps
                              the single top-down chain */
     int fp64_panel;       /* FP64 block inversion: 0 (default) runs Gauss-Jordan with partial
-                             pivoting on each panel column by column on one CTA (panel width 8 or
-                             16); 1 chooses each panel's pivots first on one CTA (elimination of the
+                             pivoting on each panel column by column, on a cluster (panel width 8)
+                             or one CTA (16); 1 chooses each panel's pivots first on one CTA (elimination of the
                              unpivoted rows only) and forms the panel's multipliers on all CTAs by
                              triangular solves with the pivot block's LU factors (8, 16 or 32) */
     int refine_max_iter;  /* FGMRES iterations in FP64 on the exact FP64 operator around an FP64
@@ -111,7 +111,10 @@ typedef struct {
                              mixed path's FP64 route (default 10; stops at gmres_tol).  A direct solve
                              with stored block inverses carries their backward error times the
                              system's condition number; the iterations bring the residual down to
-                             gmres_tol.  0 = direct solve only */
+                             gmres_tol.  0 = direct solve only.  With the refinement, at least 8 layers
+                             and cluster_size, panel_width (or 8), factor_ctas, twisted and fp64_panel at
+                             their defaults, the plain FP64 path factors blocks of at most 152 species by
+                             block cyclic reduction in FP64 */
     int fp32_bcr;         /* mixed mode: 1 factors the FP32 preconditioner by block cyclic reduction of
                              the layers (odd layers eliminated first, level by level) with every dense
                              product on the tensor cores (TF32 head/tail split, FP32 accuracy) and the
@@ -505,7 +508,8 @@ XK_API int xk_tc_gemm(int M, int N, int K, const float *A, int lda, const float 
 
 /* ---- tracing: CUDA events around each phase of every step ----
  * Phases: XK_PH_RATES (Gibbs energies + rate coefficients), XK_PH_PHOTO,
- * XK_PH_REACTION (w and its derivatives), XK_PH_RESIDUAL, XK_PH_JACOBIAN,
+ * XK_PH_REACTION (no time of its own: w and its derivatives are formed with the
+ * residual), XK_PH_RESIDUAL, XK_PH_JACOBIAN,
  * XK_PH_FACTOR (block inversions), XK_PH_SOLVE (block sweeps, or FGMRES with
  * its sweeps in mixed mode), XK_PH_CONTROL (accept/reject/update),
  * XK_PH_FALLBACK (mixed mode only: the FP64 Jacobian, factorization and

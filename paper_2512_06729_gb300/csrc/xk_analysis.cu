@@ -118,8 +118,8 @@ __device__ void warps_solve(EqShared &sh, int M)
 }
 
 // Dynamic shared memory: lnN, nj, mu [S] doubles, the entries' parts [2 nsub] doubles (sums of nj and
-// of nj mu), then the activity flags [S] as bytes.  Bound by FP64 latency and issue (a warp instruction
-// holds its unit some 75 clocks, a dependent one waits some 180): per iteration the exponentials, then
+// of nj mu), then the activity flags [S] as bytes.  Bound by FP64 issue (a warp instruction holds its
+// unit, one to four warps, for 65 clocks whatever its lanes do): per iteration the exponentials, then
 // the system's chain of M pivots.  At 594 species x 150 layers an iteration takes 25 us; with one thread
 // to an entry (the longest some 550 terms), divisions and a back substitution on one lane it took 110.
 __global__ void __launch_bounds__(kEqThreads) k_equilibrium(Col c, EqIndex ix, const double *b, double *x,

@@ -22,7 +22,6 @@ inline int nblocks(long long n, int t = kThreads) { return (int)((n + t - 1) / t
 // that a skipped launch (an FGMRES slot past convergence, an FP64 route not taken) schedules a
 // few thousand threads, not one per element.
 constexpr int kGatedBlocks = 152 * 8;
-inline int gated_blocks(long long n, int t = kThreads) { return (int)std::min<long long>((n + t - 1) / t, kGatedBlocks); }
 
 // ---------------------------------------------------------------------------
 // grid (Sec. 2.1): n_gas = P / (k_B T); hydrostatic altitudes; layer widths

@@ -175,9 +175,9 @@ __device__ __forceinline__ void reaction_terms_at(const Col &c, int k, int r, co
 }
 
 // 1 / x from the hardware's approximation (some 20 bits) by one third-order step, y (1 + e + e^2) with
-// e = 1 - x y: the series of 1 / (1 - e).  Three dependent FP64 operations; an FP64 result takes some
-// 180 clocks on this part, a division about ten of them.  The division where the approximation's range
-// ends (the exponent looked at as an integer).
+// e = 1 - x y: the series of 1 / (1 - e).  Three dependent FP64 operations of 65 clocks each on this
+// part, where a division takes about ten.  The division where the approximation's range ends (the
+// exponent looked at as an integer).
 __device__ __forceinline__ double reciprocal64(double x)
 {
     const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
