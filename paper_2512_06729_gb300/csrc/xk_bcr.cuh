@@ -172,7 +172,8 @@ struct Bcr64Sizes {
     size_t inv, cp, pq, vec;       // doubles
 };
 Bcr64Sizes bcr64_sizes(int L, int S);
-// Fill the plan for arrays already laid out; uploads the task lists and clears the arrays' padding.
+// Fill the plan for arrays already laid out (the task lists in the order inv, gemm, mv, sol); uploads the
+// lists and clears the arrays' padding.
 cudaError_t bcr64_build(Bcr64Plan &p, int L, int S, int ldd, cudaStream_t st);
 cudaError_t bcr64_factor(const Bcr64Plan &p, Ctl *ctl, cudaStream_t st);
 inline BcrSolveT<double> solve_of(const Bcr64Plan &p)

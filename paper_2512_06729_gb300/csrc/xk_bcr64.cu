@@ -18,6 +18,7 @@
 // reciprocal (beside the pivot search) and three dependent products: 1.2 us, which bounds every level
 // but the lowest two, where there are too few SMs for 96 columns of 75 blocks.
 #include <algorithm>
+#include <cstring>
 
 #include "xk_bcr.cuh"
 #include "xk_internal.cuh"
@@ -469,20 +470,27 @@ cudaError_t bcr64_build(Bcr64Plan &p, int L, int S, int ldd, cudaStream_t st)
 {
     if (S > kBcr64Max || ldd < S) return cudaErrorInvalidValue;
     build(p, L, S, ldd);
-    const Bcr64Sizes z = bcr64_sizes(L, S);
-    auto put = [&](auto *dst, const auto &v) {
-        return v.empty() ? cudaSuccess : cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, st);
+    // the task lists lie one behind the other (with the allocator's gaps): one copy for the four
+    std::vector<char> image;
+    auto put = [&](const auto *dst, const auto &v) {
+        const size_t at = (const char *)dst - (const char *)p.inv_d, bytes = v.size() * sizeof(v[0]);
+        if (image.size() < at + bytes) image.resize(at + bytes);
+        if (bytes) memcpy(image.data() + at, v.data(), bytes);
     };
-    cudaError_t e = put(p.inv_d, p.inv);
-    if (e == cudaSuccess) e = put(p.gemm_d, p.gemm);
-    if (e == cudaSuccess) e = put(p.mv_d, p.mv);
-    if (e == cudaSuccess) e = put(p.sol_d, p.sol);
-    // the padding columns are read by the solve and written by nobody
-    double *arr[] = {p.INV, p.CP, p.PQ, p.bw, p.tw, p.xw};
-    const size_t len[] = {z.inv, z.cp, z.pq, z.vec, z.vec, z.vec};
-    for (int i = 0; i < 6; ++i)
-        if (e == cudaSuccess) e = cudaMemsetAsync(arr[i], 0, len[i] * sizeof(double), st);
-    // the host copies of the task lists must outlive the asynchronous copies
+    put(p.inv_d, p.inv);
+    put(p.gemm_d, p.gemm);
+    put(p.mv_d, p.mv);
+    put(p.sol_d, p.sol);
+    cudaError_t e = cudaMemcpyAsync(p.inv_d, image.data(), image.size(), cudaMemcpyHostToDevice, st);
+    // a padding column is read by the solve and written by nobody
+    if (p.ld != S) {
+        const size_t blk = (size_t)S * p.ld, vec = (size_t)L * p.ld;
+        double *arr[] = {p.INV, p.CP, p.PQ, p.bw, p.tw, p.xw};
+        const size_t len[] = {L * blk, std::max(BcrLevels(L).ncp, 1) * 2 * blk, 2 * L * blk, vec, vec, vec};
+        for (int i = 0; i < 6; ++i)
+            if (e == cudaSuccess) e = cudaMemsetAsync(arr[i], 0, len[i] * sizeof(double), st);
+    }
+    // the host copy must outlive the asynchronous one
     return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
 }
 
