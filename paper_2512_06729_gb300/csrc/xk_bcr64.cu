@@ -2,11 +2,11 @@
 //
 // The block elimination from both ends (xk_factor64.cu) is a chain of L / 2 layers with S columns
 // each, and at these sizes it is all latency: 2,900 clocks per column, 11 ms for 96 species and 150
-// layers, of which the arithmetic would take 0.25.  The reduction does five times the arithmetic, but
+// layers, of which the arithmetic would take 0.25.  The reduction does four times the arithmetic, but
 // in a chain of log2 L inversions: every second layer of a level is inverted at once, and the products
 // that eliminate them are spread over the chip.  It pays while a block fits in the shared memory of a
-// cluster and the arithmetic stays short against the chain: the factorization takes 2.0 ms at 96
-// species and 150 layers (nine rounds of inversions of 194 to 116 us, products 0.83 ms), and a step
+// cluster and the arithmetic stays short against the chain: the factorization takes 1.8 ms at 96
+// species and 150 layers (nine inversions in a row of 195 to 90 us, products 0.84 ms), and a step
 // 11.9 ms with the elimination, 2.2 with the reduction (17.4 and 3.1 at 120 species and 90 layers).
 //
 // k_inv64: one block per cluster, columns dealt out over its CTAs, Gauss-Jordan in place with implicit
@@ -15,7 +15,7 @@
 // multipliers, applies them to the next column this CTA will have to send, and hands them to the other
 // warps, which update the rest of its columns behind it.  Every column has its own place and its own
 // barriers, each used once, so nobody waits for room.  A column costs one trip between CTAs, a
-// reciprocal (beside the pivot search) and three dependent products: 1.2 us, which bounds every level
+// reciprocal (beside the pivot search) and three dependent products: 0.9 us, which bounds every level
 // but the lowest two, where there are too few SMs for 96 columns of 75 blocks.
 #include <algorithm>
 #include <cstring>
