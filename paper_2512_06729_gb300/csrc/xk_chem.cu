@@ -197,15 +197,6 @@ __global__ void __launch_bounds__(128) k_photo_alpha(Col c, const double *n)
     }
 }
 
-// x / d by the (correctly rounded) reciprocal of d and one correction: a division takes some ten
-// dependent FP64 operations, this three, with the same result
-__device__ __forceinline__ double over(double x, double d, double rd)
-{
-    const double q = x * rd;
-    if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return q;   // the correction would be inf - inf
-    return fma(fma(-q, d, x), rd, q);
-}
-
 // The diffuse field.  In layer k the diffuse fluxes leaving it, D_k down through its bottom and U_k up
 // through its top, obey
 //     D_k = T_k D_{k+1} + r_k U_{k-1} + P_k / 2,   U_k = T_k U_{k-1} + r_k D_{k+1} + P_k / 2,
@@ -217,7 +208,7 @@ __device__ __forceinline__ double over(double x, double d, double rd)
 // above only through the optical depth.  A CTA takes 32 wavelengths, a warp a run of layers counted
 // from the top.  Bound by the FP64 issue of three exponentials a layer (a layer's bottom is the next
 // one's top).  Both kernels in one, a thread per wavelength, left half of the SMs' schedulers without
-// a warp and the rest waiting for one exponential after the other.  314 us at 10,000 wavelengths and
+// a warp and the rest waiting for one exponential after the other.  327 us at 10,000 wavelengths and
 // 150 layers, and 176 for the second.
 constexpr int kPhotoRuns = 16;
 __global__ void __launch_bounds__(32 * kPhotoRuns) k_photo_layers(Col c)

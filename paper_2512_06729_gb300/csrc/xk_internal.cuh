@@ -199,6 +199,22 @@ __device__ __forceinline__ double reciprocal_rn(double x)
     return fma(y, fma(-x, y, 1.0), y);
 }
 
+// x / d, correctly rounded, from rd = reciprocal_rn(d): the product q = x rd is within a unit of the
+// quotient, and q + rd (x - q d) rounds correctly (Markstein 1990) while the residual is exact and the
+// quotient a normal number, as it is for exponents of x and d within some 2^508 of one.  Three dependent
+// FP64 operations where a division takes some ten.  Elsewhere the division itself (a d below 2^-1024 has
+// an infinite reciprocal, and 0 x inf is no quotient); a zero x needs neither.
+__device__ __forceinline__ double over(double x, double d, double rd)
+{
+    const unsigned hx = (unsigned)__double2hiint(x) & 0x7fffffffu, hd = (unsigned)__double2hiint(d) & 0x7fffffffu;
+    const double q = x * rd;
+    if ((hd >> 20) - 515u <= 1015u) {
+        if ((hx >> 20) - 515u <= 1015u) return fma(fma(-q, d, x), rd, q);
+        if ((hx | (unsigned)__double2loint(x)) == 0u) return q;
+    }
+    return x / d;
+}
+
 // Entry q of the Jacobian pattern (row-grouped): sum of its terms, -dF_i/dn_j of one layer, in a
 // fixed order (dk: that layer's reaction derivatives [R][6]).
 __device__ __forceinline__ double jac_entry(const Col &c, int q, const double *dk)
