@@ -330,9 +330,8 @@ template <int RG>
 cudaError_t launch_leaf_rg(const BcrLeaf *tasks, int count, const int *skip, const Ctl *ctl, cudaStream_t st)
 {
     constexpr size_t smem = leaf_smem(RG);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_leaf_inverse<RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (attr != cudaSuccess) return attr;
+    const cudaError_t e = allow_smem(k_leaf_inverse<RG>, smem);
+    if (e != cudaSuccess) return e;
     count_launches(1);
     return launch_dependent(k_leaf_inverse<RG>, dim3(count), dim3(kLeafThreads), smem, st, tasks, skip, ctl);
 }

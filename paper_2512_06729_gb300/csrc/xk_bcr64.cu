@@ -434,9 +434,8 @@ cudaError_t launch_inv_rpt(const Bcr64Plan &p, const BcrStage &s, Ctl *ctl, cuda
     const int S = p.S, count = s.count;
     const int cs = inv_cluster(S, count);
     const InvLayout lay = inv_layout(S, cs);
-    static const cudaError_t once =
-        cudaFuncSetAttribute(k_inv64<RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvSmemMax);
-    if (once != cudaSuccess) return once;
+    const cudaError_t e = allow_smem(k_inv64<RPT>, kInvSmemMax);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(count * cs);
     cfg.blockDim = dim3(kInvThreads);
@@ -496,12 +495,10 @@ cudaError_t bcr64_build(Bcr64Plan &p, int L, int S, int ldd, cudaStream_t st)
 
 cudaError_t bcr64_factor(const Bcr64Plan &p, Ctl *ctl, cudaStream_t st)
 {
-    static const cudaError_t once =
-        cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_bytes(kBcr64Max));
-    if (once != cudaSuccess) return once;
+    cudaError_t e = allow_smem(k_gemm64, gemm_bytes(kBcr64Max));
+    if (e != cudaSuccess) return e;
     const int nt = (p.S + kTile - 1) / kTile;
     for (const BcrStage &s : p.fac) {
-        cudaError_t e = cudaSuccess;
         if (s.kind == kBcrLeafStage) {
             switch ((p.S + 31) / 32) {
             case 1: e = launch_inv_rpt<1>(p, s, ctl, st); break;

@@ -7,7 +7,6 @@
 #include <algorithm>
 
 #include <atomic>
-#include <mutex>
 
 #include "xk_layer.cuh"
 
@@ -1065,10 +1064,7 @@ void launch_layer_terms(const Col &c, const double *n, double *F, const Ctl *ctl
     if ((long long)c.L * c.S <= 0) return;
     const bool rates = jv_rates_in_smem(c);
     const size_t sm = jv_smem_doubles(c, rates) * sizeof(double);
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_layer_terms, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
-    });
+    allow_smem(k_layer_terms, kJvSmemMax);
     count_launches(1);
     k_layer_terms<<<std::min(c.L, kGatedBlocks), 512, sm, st>>>(c, n, F, ctl, f_floor, diag, bhat, rates ? 1 : 0);
 }
@@ -1115,10 +1111,7 @@ void launch_jv(const Col &c, const Ctl *ctl, const double *xs, double *ys, const
     }
     const bool rates = jv_rates_in_smem(c);
     const size_t sm = jv_smem_doubles(c, rates) * sizeof(double);
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_jv_layer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
-    });
+    allow_smem(k_jv_layer, kJvSmemMax);
     count_launches(1);
     k_jv_layer<<<std::min(c.L, kGatedBlocks), 512, sm, st>>>(c, ctl, xs, ys, rowdiv, skip, rates ? 1 : 0);
 }

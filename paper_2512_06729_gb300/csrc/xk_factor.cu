@@ -677,18 +677,6 @@ size_t factor_smem(int S, int ctas)
     return (m + 255) & ~(size_t)255;
 }
 
-int sm_count()
-{
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 1;
-    }
-    return n;
-}
-
 }  // namespace
 
 size_t barrier_words() { return 2; }
@@ -699,7 +687,7 @@ int factor_plan(int S, int precision_bytes, int nb_hint, int ctas_hint, FactorPl
     p.threads = kFactorThreads;
     p.nb = precision_bytes == 8 ? 8 : 32;
     if (nb_hint > 0) p.nb = nb_hint;
-    int sms = sm_count();
+    int sms = device_sms();
     // FP64 is ALU-bound on every SM; FP32 reads the panel per CTA, so fewer and wider slices
     if (S > kRowsPerThread * kFactorThreads) return -1;
     int want = sms;
@@ -811,7 +799,7 @@ cudaError_t launch_solve(const BlockSys<T> &sys, const FactorPlan &plan, const d
     size_t smem = ((size_t)sys.S * sizeof(T) + 255) & ~(size_t)255;
     int warps = kSolveThreads / 32;
     int ctas = (sys.S + warps - 1) / warps;
-    if (ctas > sm_count()) ctas = sm_count();
+    if (ctas > device_sms()) ctas = device_sms();
     if (plan.ctas > 0 && ctas > plan.ctas) ctas = plan.ctas;    // stay within the column's share of the SMs
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -13,7 +13,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "xk_bcr.cuh"
 #include "xk_gmres.cuh"
@@ -410,34 +409,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_fgmres(FgArgs<T> a)
     gs.leave();
 }
 
-int sm_count()
-{
-    static const int n = [] {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        return std::max(sms, 1);
-    }();
-    return n;
-}
-
 // One CTA per SM, or the column's share of them in a batch.
-int solve_ctas(int share) { return share > 0 ? std::min(share, sm_count()) : sm_count(); }
+int solve_ctas(int share) { return share > 0 ? std::min(share, device_sms()) : device_sms(); }
 
 template <typename T>
 ApplyArgs<T> apply_args(const BcrSolveT<T> &p) { return {p.stages, p.mv, p.nstages, p.S, p.rows, p.ld}; }
-
-template <typename T>
-cudaError_t smem_limits()
-{
-    static const cudaError_t e = [] {
-        cudaError_t r = cudaFuncSetAttribute(k_bcr_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_fgmres<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kJvSmemMax);
-        return r;
-    }();
-    return e;
-}
 
 }  // namespace
 
@@ -445,7 +421,7 @@ template <typename T>
 cudaError_t bcr_solve(const BcrSolveT<T> &p, const double *b, double *x, const double *bscale, const double *xscale,
                       const int *skip, Ctl *ctl, cudaStream_t st)
 {
-    cudaError_t e = smem_limits<T>();
+    cudaError_t e = allow_smem(k_bcr_solve<T>, kJvSmemMax);
     if (e != cudaSuccess) return e;
     ApplyArgs<T> a = apply_args(p);
     unsigned *words = p.bar;
@@ -459,7 +435,7 @@ cudaError_t bcr_solve(const BcrSolveT<T> &p, const double *b, double *x, const d
 template <typename T>
 cudaError_t bcr_fgmres(const BcrSolveT<T> &p, const Col &c, const GmArgs &g, const double *rowd, cudaStream_t st)
 {
-    cudaError_t e = smem_limits<T>();
+    cudaError_t e = allow_smem(k_fgmres<T>, kJvSmemMax);
     if (e != cudaSuccess) return e;
     FgArgs<T> a;
     a.c = c;

@@ -312,6 +312,23 @@ struct ParcelArgs {
 // One global iteration on one CTA (photolysis and rate coefficients already in c).
 cudaError_t launch_parcel_iteration(const Col &c, const ParcelArgs &a, cudaStream_t st);
 
+// Dynamic shared memory that a kernel may be launched with, on the current device: the limit is that
+// device's own (a process may hold contexts on several), so it is set where the kernel is launched.
+template <typename... P>
+cudaError_t allow_smem(void (*fn)(P...), size_t bytes)
+{
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// SMs of the current device.
+inline int device_sms()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();
+    return n > 0 ? n : 1;
+}
+
 // Launch a kernel that may start while its predecessor on the stream drains (programmatic dependent
 // launch): it must execute griddepcontrol.wait before it touches anything an earlier launch writes.
 template <typename... P, typename... A>

@@ -498,18 +498,10 @@ cudaError_t launch_tc_gemm(const TcTask *tasks, const int *tile_task, int total_
                            const int *skip, Ctl *ctl, cudaStream_t st)
 {
     if (total_tiles <= 0) return cudaSuccess;
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    static int sms = 1;
-    std::call_once(once, [] {
-        int dev = 0;
-        attr = cudaFuncSetAttribute(k_tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-        if (attr == cudaSuccess) attr = cudaGetDevice(&dev);
-        if (attr == cudaSuccess) attr = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    });
-    if (attr != cudaSuccess) return attr;
+    const cudaError_t e = allow_smem(k_tc_gemm, kSmemBytes);
+    if (e != cudaSuccess) return e;
     // a CTA per SM; more where one would get over kMaxTiles tiles
-    const int ctas = std::max(std::min(total_tiles, sms), (total_tiles + kMaxTiles - 1) / kMaxTiles);
+    const int ctas = std::max(std::min(total_tiles, device_sms()), (total_tiles + kMaxTiles - 1) / kMaxTiles);
     count_launches(1);
     return launch_dependent(k_tc_gemm, dim3(ctas), dim3(kThreads), kSmemBytes, st, tasks, tile_task, total_tiles, maps, skip,
                             ctl);

@@ -1,0 +1,84 @@
+"""What the library asks of the CUDA runtime, on a fake runtime of two devices (fake_cuda_runtime.cpp):
+the built objects are linked against it, device memory is host memory and kernels do nothing."""
+import ctypes
+import os
+import subprocess
+import types
+
+import numpy as np
+import pytest
+
+from paper_2512_06729_gb300 import build as xkbuild
+from paper_2512_06729_gb300 import synth, xk
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    pytest.importorskip("torch")
+    xkbuild.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libxk_fake.so")
+    objs = [os.path.join(xkbuild.BUILD, s.replace(".cu", ".o")) for s in xkbuild.SOURCES]
+    symbols = subprocess.run(["nm", "-u", *objs], capture_output=True, text=True, check=True).stdout
+    linked = {w for w in symbols.split() if w.startswith("__cudaRegisterLinkedBinary")}
+    include = os.path.join(os.path.dirname(os.path.dirname(xkbuild.nvcc())), "include")
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-Wl,-Bsymbolic", "-I", include, "-o", out,
+                    os.path.join(HERE, "fake_cuda_runtime.cpp"), *objs,
+                    *(f"-Wl,--defsym={s}=fake_linked_binary" for s in linked)], check=True)
+    lib = ctypes.CDLL(out)
+    for name, (res, args) in xk.SIGNATURES.items():
+        f = getattr(lib, name)
+        f.restype, f.argtypes = res, args
+    lib.fake_refused.restype = ctypes.c_char_p
+    return lib
+
+
+@pytest.fixture
+def column(fake, monkeypatch):
+    """column(problem, precision, device, **settings): a context with its workspace in host memory."""
+    monkeypatch.setattr(xk, "_lib", fake)
+    made = []
+
+    def make(p, precision, device, **kw):
+        c = xk.Column(p, precision, device=device, stream=types.SimpleNamespace(cuda_stream=0), allocate=False, **kw)
+        c.ws = np.zeros(c.workspace_bytes + 256, np.uint8)
+        base = (c.ws.ctypes.data + 255) & ~255
+        c._call("xk_set_workspace", ctypes.c_void_p(base), ctypes.c_size_t(c.workspace_bytes))
+        made.append(c)
+        return c
+
+    yield make
+    for c in made:
+        c.close()
+
+
+def _step(col):
+    n, d = np.zeros((col.L, col.S)), np.zeros((col.L, col.S))
+    it, resid = ctypes.c_int(), ctypes.c_double()
+    col._call("xk_step_delta", ctypes.c_void_p(n.ctypes.data), 1e-4, ctypes.c_void_p(d.ctypes.data), ctypes.byref(it),
+              ctypes.byref(resid))
+
+
+_PROBLEMS = {
+    "small": lambda: synth.small_column(L=12),
+    "chons": lambda: synth.chons_column(L=20),
+    "full": lambda: synth.full_column(L=6),
+}
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("name", list(_PROBLEMS))
+def test_every_device_of_a_process_runs_a_step(fake, column, name, precision):
+    """Contexts on two devices of one process, in both orders of creation and use: every kernel's
+    shared-memory limit is raised where it is launched, and persistent grids fit the device's own SMs."""
+    p = _PROBLEMS[name]()
+    first = column(p, precision, 0)
+    _step(first)
+    second = column(p, precision, 1)
+    before = fake.fake_launches(1)
+    _step(second)
+    _step(first)
+    _step(second)
+    assert fake.fake_refused() == b""
+    assert fake.fake_launches(1) > before
