@@ -1758,6 +1758,16 @@ void drop_round(xk_batch *b)
     b->round_kernels = 0;
 }
 
+// Graphs with IF nodes run over the device's connections, eight by default, where the branches of one
+// without them all run at once.  So columns that would wait for a connection are captured without:
+// a round of more than kNodeColumns, and what is submitted to the slots of a batch of more than
+// kNodeSlots (each a graph of its own).  ms a step with and without nodes, mixed 96 x 90: rounds of 8
+// columns 1.74 and 2.36, of 12 3.37 and 3.17, of 64 36.9 and 15.1; submitted to 6 slots 1.47 and 1.94,
+// to 8 2.64 and 2.35.  FP64 250 x 60: rounds of 8 34.6 and 35.0, of 12 68.6 and 36.3, of 64 1,137 and
+// 219; submitted to 6 slots 19.7 and 20.0, to 8 67.5 and 35.1.
+constexpr size_t kNodeColumns = 8;
+constexpr int kNodeSlots = 6;
+
 // Capture nsteps steps of every listed slot's column, each on its slot's stream, into b->round.
 int capture_round(xk_batch *b, const std::vector<int> &live, int nsteps)
 {
@@ -1788,7 +1798,9 @@ int capture_round(xk_batch *b, const std::vector<int> &live, int nsteps)
     for (int i : live) {
         BatchSlot &s = b->slots[i];
         cudaStreamWaitEvent(s.st, b->fork, 0);
+        s.ctx->cond.off = live.size() > kNodeColumns;
         if (rc == XK_OK && (rc = enqueue_chunk(s.ctx, nsteps, true)) != XK_OK) bad = s.ctx;
+        s.ctx->cond.off = false;
         cudaEventRecord(b->joins[i], s.st);
         cudaStreamWaitEvent(b->origin, b->joins[i], 0);
     }
@@ -2007,7 +2019,9 @@ int xk_batch_submit(xk_batch *b, int slot, int nsteps)
     if (s.finished) return XK_OK;
     cudaSetDevice(b->device);
     b->err.clear();
+    s.ctx->cond.off = b->max_slots > kNodeSlots;
     int rc = run_steps(s.ctx, nsteps, true);
+    s.ctx->cond.off = false;
     if (rc) {
         b->err = s.ctx->err;
         return rc;

@@ -82,3 +82,25 @@ def test_every_device_of_a_process_runs_a_step(fake, column, name, precision):
     _step(second)
     assert fake.fake_refused() == b""
     assert fake.fake_launches(1) > before
+
+
+def _batch(fake, column, slots, columns, p, precision):
+    b = xk.Batch(1 << 40, slots)
+    for _ in range(columns):
+        b.add(column(p, precision, 0), 1e-8)
+    return b
+
+
+@pytest.mark.parametrize("how,slots,columns,nodes", [("round", 8, 8, True), ("round", 16, 8, True), ("round", 9, 9, False),
+                                                     ("submit", 6, 2, True), ("submit", 7, 2, False)])
+def test_columns_of_a_batch_do_not_wait_for_connections(fake, column, how, slots, columns, nodes):
+    """Steps captured with conditional nodes run on the device's connections, eight by default: no more
+    columns than that are captured with them."""
+    b = _batch(fake, column, slots, columns, synth.small_column(L=9), "mixed")
+    before = fake.fake_conditional_nodes()
+    if how == "round":
+        b.step(1)
+    else:
+        b.submit(0, 1)
+    assert (fake.fake_conditional_nodes() > before) == nodes
+    b.close()
