@@ -6,7 +6,7 @@
 // rows factored by one CTA, with a block barrier pair per column, is most of the time: 51 us per
 // panel at 594 species (of which the other 75 SMs idle through about 40), 22 us at 96.  Here
 //  - the panel belongs to a thread-block cluster, its rows spread over the cluster's CTAs, one row
-//    per thread in registers.  Per column every warp sends its best candidate row (the reciprocal of
+//    per thread (two beyond 512 rows of a CTA) in registers.  Per column every warp sends its best candidate row (the reciprocal of
 //    its pivot and the row's panel entries) to all CTAs as asynchronous stores that complete on the
 //    receiver's mbarrier, and each picks the winner from its own copy: no barrier of the cluster or
 //    the block.  The loop over the panel's columns is rolled (the finished column moves to the end):
@@ -519,7 +519,6 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
 // panel q's columns over.  Panel p needs its columns with the panels before p - 1 applied; its G stays
 // in D's panel columns until the layer's end, when every CTA has read it, and the columns follow.
 constexpr int kMaxPanels = 2 * kThreads / kNB;
-template <int RPT>
 __global__ void __launch_bounds__(kThreads, 1)
 k_factor64_flow(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int cs)
 {
@@ -550,14 +549,14 @@ k_factor64_flow(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid
         double *D = a.D + (size_t)k * S * ld;
         int *perm = a.perm + (size_t)k * S, *iperm = a.iperm + (size_t)k * S;
         if (cidx == 0) {
-            unsigned used = unused_rows<RPT>(q);
+            unsigned used = unused_rows<1>(q);
             for (int p = 0; p < npan; ++p) {
                 if (tid == 0) {
                     const int c0 = p * kNB, owners = owner(min(c0 + kNB, S) - 1) - owner(c0) + 1;
                     wait_count(flag + 1 + p, (unsigned)(owners * (step + 1)), ctl);
                 }
                 __syncthreads();
-                panel_step<RPT>(q, D, perm, iperm, p, used);
+                panel_step<1>(q, D, perm, iperm, p, used);
                 __syncthreads();
                 if (tid == 0) raise_count(flag);
             }
@@ -700,9 +699,8 @@ size_t smem_flow(int S, int cs, int ntrail)
 using FactorFn = void (*)(BlockSys<double>, Ctl *, const int *, int, int, int);
 FactorFn kernel_of(int S, const FactorPlan &p)
 {
-    const bool one = (S + p.cs - 1) / p.cs <= kThreads;
-    if (p.flow64) return one ? k_factor64_flow<1> : k_factor64_flow<2>;
-    return one ? k_factor64<1> : k_factor64<2>;
+    if (p.flow64) return k_factor64_flow;
+    return (S + p.cs - 1) / p.cs <= kThreads ? k_factor64<1> : k_factor64<2>;
 }
 
 cudaError_t launch_mode(const BlockSys<double> &sys, const FactorPlan &plan, Ctl *ctl, cudaStream_t st, const int *skip,
@@ -743,50 +741,64 @@ int factor64_plan(int S, int want, FactorPlan *p)
     // taken from the updates.  Measured (ms with clusters of 1, 2, 4, 8): S = 20 (8 steps of 40 layers)
     // 8.4, 8.7, 8.7, 8.8; 96 (4 steps of 150) 52.6, 49.7, 48.6, 48.8; 131 (60 layers) 8.8, 7.8, 7.3, 7.2;
     // 250 (60) 21.1, 15.5, 13.7, 13.4; 400 (60) 46, 31, 22.9, 21.7; 594 (150) 275, 140, 102, 121.
-    for (int cs = S <= 32 ? 1 : S <= 128 || S > 500 ? 4 : 8; cs >= 1; cs /= 2) {
-        if (want < 4 * cs && cs > 1) continue;
-        if (cs > 1 && (S + cs - 1) / cs > kThreads) continue;
-        // columns to a CTA beyond the cluster: at least about four
-        const int chain = cs + std::max(1, (S + 3) / 4 / cs) * cs;
-        int ctas = std::min(want, 2 * chain) / cs * cs;
-        for (int flow = 1; flow >= 0; --flow) {
-            FactorPlan t = *p;
-            t.cs = cs;
-            t.flow64 = flow;
-            t.ctas64 = ctas;
-            for (int pass = 0; pass < 2; ++pass) {
-                const int half = chain_of(t.ctas64, cs);
-                if (flow && half <= cs) break;
-                t.smem64 = flow ? smem_flow(S, cs, half - cs) : smem_general(S, cs, std::max(1, half - cs));
-                if (t.smem64 > kSmemMax - sizeof(PanelShared)) break;
-                FactorFn fn = kernel_of(S, t);
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(cs);
-                cfg.blockDim = dim3(kThreads);
-                cfg.dynamicSmemBytes = t.smem64;
-                cudaLaunchAttribute attr[1];
-                attr[0].id = cudaLaunchAttributeClusterDimension;
-                attr[0].val.clusterDim.x = cs;
-                attr[0].val.clusterDim.y = 1;
-                attr[0].val.clusterDim.z = 1;
-                cfg.attrs = attr;
-                cfg.numAttrs = 1;
-                int n = 0;
-                if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem64) != cudaSuccess ||
-                    cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
-                    cudaGetLastError();
-                    break;
-                }
-                // fewer clusters than wanted fit at once: plan again for those
-                if (n * cs >= t.ctas64) {
-                    *p = t;
-                    return 0;
-                }
-                t.ctas64 = n * cs;
+    const int largest = S <= 32 ? 1 : S <= 128 || S > 500 ? 4 : 8;
+    // CTAs of a launch: to each beyond the cluster at least about four columns
+    auto ctas_of = [&](int cs) { return std::min(want, 2 * (cs + std::max(1, (S + 3) / 4 / cs) * cs)) / cs * cs; };
+    auto fits = [&](int cs, int flow) {
+        FactorPlan t = *p;
+        t.cs = cs;
+        t.flow64 = flow;
+        t.ctas64 = ctas_of(cs);
+        for (int pass = 0; pass < 2; ++pass) {
+            const int half = chain_of(t.ctas64, cs);
+            if (flow && half <= cs) return false;
+            t.smem64 = flow ? smem_flow(S, cs, half - cs) : smem_general(S, cs, std::max(1, half - cs));
+            if (t.smem64 > kSmemMax - sizeof(PanelShared)) return false;
+            FactorFn fn = kernel_of(S, t);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(cs);
+            cfg.blockDim = dim3(kThreads);
+            cfg.dynamicSmemBytes = t.smem64;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = cs;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (allow_smem(fn, t.smem64) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess ||
+                n < 1) {
+                cudaGetLastError();
+                return false;
             }
+            // fewer clusters than wanted fit at once: plan again for those
+            if (n * cs >= t.ctas64) {
+                *p = t;
+                return true;
+            }
+            t.ctas64 = n * cs;
         }
-    }
-    return -1;
+        return false;
+    };
+    // columns in shared memory where they fit, a quarter of the launch (half a chain) at most to the panel,
+    // before a larger cluster without (250 species, 40 layers on 8 CTAs 44 ms so, 30 with one CTA to the
+    // panel; 400, 30 layers on 16 64 and 46; 594, 24 layers on 38 62 and 51)
+    for (int cs = largest; cs >= 1; cs /= 2)
+        if ((S + cs - 1) / cs <= kThreads && (cs == 1 || want >= 4 * cs) && fits(cs, 1)) return 0;
+    // else in global memory, the CTAs of a small share of the SMs: the cluster that leaves a chain the
+    // most of them, the largest of equals (all of a chain's CTAs, if need be: the panel is then everyone's
+    // and so are the updates).  With half a chain to the panel, as above, and so: 250 species, 40 layers on
+    // 4 CTAs 82 and 53 ms; 400, 30 layers on 8 123 and 75; 594, 24 layers on 4 637 and 359, on 8 323 and
+    // 187.  A larger cluster that leaves CTAs over is no gain (on 6: 250 species
+    // 44 ms with 1, 52 with 2; 594 325 and 347; on 12 167 with 2, 181 with 4).
+    int best = 1, most = 0;
+    for (int cs = largest; cs >= 1; cs /= 2)
+        if (want >= 2 * cs && (cs == 1 || (S + cs - 1) / cs <= kThreads) && chain_of(ctas_of(cs), cs) > most) {
+            best = cs;
+            most = chain_of(ctas_of(cs), cs);
+        }
+    return fits(best, 0) || fits(1, 0) ? 0 : -1;
 }
 
 cudaError_t launch_factor64(const BlockSys<double> &sys, const FactorPlan &plan, Ctl *ctl, cudaStream_t st, const int *skip)

@@ -104,3 +104,27 @@ def test_columns_of_a_batch_do_not_wait_for_connections(fake, column, how, slots
         b.submit(0, 1)
     assert (fake.fake_conditional_nodes() > before) == nodes
     b.close()
+
+
+def _launches_of(fake, name):
+    grid, cluster = ctypes.c_int(), ctypes.c_int()
+    n = fake.fake_launches_of(name.encode(), ctypes.byref(grid), ctypes.byref(cluster))
+    return n, grid.value, cluster.value
+
+
+# (species, CTAs) -> kernel, its grid and cluster: shared-memory columns where they fit, else the cluster
+# that leaves each of two chains the most CTAs
+@pytest.mark.parametrize("S,ctas,kernel,grid,cluster", [
+    (40, 2, "k_factor64I", 2, 1), (40, 4, "k_factor64_flow", 4, 1), (96, 8, "k_factor64_flow", 8, 2),
+    (250, 2, "k_factor64I", 2, 1), (250, 4, "k_factor64I", 4, 2), (250, 6, "k_factor64I", 6, 1),
+    (250, 9, "k_factor64_flow", 8, 1), (250, 19, "k_factor64_flow", 16, 4), (400, 8, "k_factor64I", 8, 4),
+    (400, 16, "k_factor64_flow", 16, 2),
+    (594, 3, "k_factor64I", 2, 1), (594, 4, "k_factor64I", 4, 2), (594, 6, "k_factor64I", 6, 1), (594, 9, "k_factor64I", 8, 4),
+    (594, 12, "k_factor64I", 12, 2), (594, 38, "k_factor64_flow", 36, 2), (594, 152, "k_factor64_flow", 152, 4)])
+def test_elimination_on_few_ctas_keeps_them_busy(fake, column, S, ctas, kernel, grid, cluster):
+    p = synth.small_column(S=S, L=4, n_two=2 * S, n_three=S // 2, n_photo=5, W=40, elements="chons" if S < 110 else "full")
+    col = column(p, "fp64", 0, factor_ctas=ctas)
+    fake.fake_forget_launches()
+    _step(col)
+    assert _launches_of(fake, "k_factor64")[0] == 2
+    assert _launches_of(fake, kernel) == (2, grid, cluster)
