@@ -490,6 +490,14 @@ bool bcr64_wanted(const xk_ctx *c)
            g.factor_ctas == 0 && g.cluster_size == 0 && g.twisted == 1 && c->S <= kBcr64Max && c->L >= kBcr64MinLayers;
 }
 
+// Whether a column's share of the SMs in a batch is too small for the reduction: it does four times the
+// elimination's arithmetic to have the chain of a column alone short, and many columns have no use for
+// that.  Where the line lies (ms a step of 90 layers, reduction and elimination): 64 species in 64 slots
+// 14.4 and 17.1, 80 26.4 and 22.9; 96 in 16 10.7 and 13.5, in 32 21.1 and 23.4 (4 CTAs, half of a chain its panel's), in 64 41.8 and 30.0; 112 in 8
+// 9.7 and 9.6, in 12 13.9 and 11.1; 136 in 4 9.2 and 15.9, in 6 13.4 and 11.1; 152 in 4 14.6 and 17.7, in 5
+// 17.9 and 12.2, in 64 218 and 69.
+bool bcr64_outgrown(int S, int share) { return S > 96 ? (double)S * S * S > 1e5 * share : S > 72 && share < 4; }
+
 // Lay out the workspace; with base == nullptr only the size is computed.
 size_t layout(xk_ctx *c, char *base)
 {
@@ -1723,6 +1731,7 @@ struct BatchSlot {
     bool inflight = false;
     cudaStream_t saved_st = nullptr;
     FactorPlan saved_plan{}, saved_plan64{};
+    bool saved_use_bcr64 = false;
     int saved_solve_ctas = 0;
     size_t bytes = 0;
     bool finished = false;
@@ -1850,6 +1859,7 @@ int xk_batch_remove(xk_batch *b, int slot)
     s.ctx->plan = s.saved_plan;
     s.ctx->plan64 = s.saved_plan64;
     s.ctx->bcr.solve_ctas = s.ctx->bcr64.solve_ctas = s.saved_solve_ctas;
+    s.ctx->use_bcr64 = s.saved_use_bcr64;
     if (s.ev) cudaEventDestroy(s.ev);
     cudaStreamDestroy(s.st);
     b->used -= s.bytes;
@@ -1915,6 +1925,8 @@ int xk_batch_add(xk_batch *b, xk_ctx *c, double dt0, int *slot)
     s.saved_plan = c->plan;
     s.saved_plan64 = c->plan64;
     s.saved_solve_ctas = c->bcr.solve_ctas;
+    s.saved_use_bcr64 = c->use_bcr64;
+    if (bcr64_outgrown(c->S, share)) c->use_bcr64 = false;
     c->bcr.solve_ctas = c->bcr64.solve_ctas = share;          // the reduction's cooperative solve on this column's share of the SMs
     s.bytes = c->ws_bytes;
     s.finished = false;

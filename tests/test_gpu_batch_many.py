@@ -36,3 +36,29 @@ def test_many_columns_end_where_they_end_alone(precision):
         mask = n_alone > 1e-20 * n_alone.max(axis=1, keepdims=True)
         assert np.max(np.abs(n[mask] - n_alone[mask]) / n_alone[mask]) <= 1e-9
     b.close()
+
+
+def test_column_off_the_reduction_ends_where_it_ends_alone():
+    """A column of 120 species takes the block elimination in a batch of twelve slots and the reduction
+    alone: the same steps, and the same steady state to 1e-9."""
+    from paper_2512_06729_gb300 import synth, xk
+    from tests.test_gpu_batch import _alone
+    p = synth.small_column(S=120, L=20, n_two=960, n_three=240, n_photo=40, W=100, elements="full")
+    b = xk.Batch(64 << 30, 12)
+    cols = [xk.Column(p, "fp64") for _ in range(2)]
+    for c in cols:
+        c.set_mixing_ratios(p.f0)
+    slots = [b.add(c, 1e-8) for c in cols]
+    for _ in range(400):
+        b.step(8)
+        if all(b.poll(s)[1] for s in slots):
+            break
+    info, finished, status = b.poll(slots[0])
+    assert finished and status == 0
+    n_alone, ainfo = _alone(p, "fp64", info.steps)
+    assert ainfo.steps == info.steps
+    mask = n_alone > 1e-20 * n_alone.max(axis=1, keepdims=True)
+    for s in slots:
+        n = b.remove(s).get_state()
+        assert np.max(np.abs(n[mask] - n_alone[mask]) / n_alone[mask]) <= 1e-9
+    b.close()

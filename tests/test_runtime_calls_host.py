@@ -128,3 +128,23 @@ def test_elimination_on_few_ctas_keeps_them_busy(fake, column, S, ctas, kernel, 
     _step(col)
     assert _launches_of(fake, "k_factor64")[0] == 2
     assert _launches_of(fake, kernel) == (2, grid, cluster)
+
+
+@pytest.mark.parametrize("S,slots,reduction", [(64, 64, True), (80, 64, False), (96, 16, True), (96, 32, True), (96, 64, False), (120, 4, True),
+                                               (152, 4, True), (152, 5, False), (152, 64, False)])
+def test_small_shares_take_the_elimination(fake, column, S, slots, reduction):
+    """The FP64 route of a column in a batch goes by its share of the SMs; alone, before and after, it is
+    the reduction at these sizes."""
+    p = synth.small_column(S=S, L=9, n_two=2 * S, n_three=S // 2, n_photo=5, W=40, elements="chons" if S < 110 else "full")
+    b = xk.Batch(1 << 40, slots)
+    col = column(p, "fp64", 0)
+    slot = b.add(col, 1e-8)
+    fake.fake_forget_launches()
+    b.step(1)
+    assert (_launches_of(fake, "k_inv64")[0] > 0) == reduction
+    assert (_launches_of(fake, "k_factor64")[0] > 0) == (not reduction)
+    b.remove(slot)
+    fake.fake_forget_launches()
+    _step(col)
+    assert _launches_of(fake, "k_inv64")[0] > 0 and _launches_of(fake, "k_factor64")[0] == 0
+    b.close()
