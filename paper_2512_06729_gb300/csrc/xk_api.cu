@@ -1151,6 +1151,9 @@ int xk_create(xk_ctx **out, const xk_config *cfg)
         delete x;
         return XK_ECUDA;
     }
+    int mps = 0;
+    if (cudaDeviceGetAttribute(&mps, cudaDevAttrMpsEnabled, c.device) != cudaSuccess) cudaGetLastError();
+    x->cond.mps = mps != 0;
     *out = x;
     return XK_OK;
 }

@@ -354,16 +354,18 @@ struct CondStreams {
     cudaStream_t inner[2] = {nullptr, nullptr};
     int depth = 0;
     bool off = false;                    // no IF nodes: every part is enqueued
+    bool mps = false;                    // nor where the device is shared through MPS: the parts hold
+                                         // cooperative kernels, which IF nodes may not hold there
 };
 bool capturing(cudaStream_t st);
 cudaError_t cond_open(cudaStream_t st, cudaStream_t inner, const int *flag, int when, cudaGraphNode_t *node);
 cudaError_t cond_close(cudaStream_t st, cudaStream_t inner, cudaGraphNode_t node);
-// body(stream) as such a part while st is being captured (unless cs->off); otherwise body(st), whose kernels check the
+// body(stream) as such a part while st is being captured (unless cs->off or cs->mps); otherwise body(st), whose kernels check the
 // flag themselves.  Kernels of a part are not counted as launches: it may not run.
 template <typename F>
 cudaError_t enqueue_if(cudaStream_t st, CondStreams *cs, const int *flag, int when, F body)
 {
-    if (!cs || cs->off || cs->depth >= 2 || !capturing(st)) {
+    if (!cs || cs->off || cs->mps || cs->depth >= 2 || !capturing(st)) {
         body(st);
         return cudaSuccess;
     }

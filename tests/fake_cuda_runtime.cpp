@@ -12,6 +12,7 @@
 #include <set>
 #include <string>
 #include <utility>
+#include <vector>
 
 #define API extern "C" __attribute__((visibility("default")))
 #define FAKE extern "C"
@@ -22,6 +23,11 @@ int g_dev = 0, g_mps = 0, g_cond = 0, g_launches[kDevices] = {};
 std::map<std::pair<int, const void *>, size_t> g_limit;
 std::map<const void *, std::string> g_name;
 std::string g_refused;
+struct Launch {
+    std::string name;
+    int grid, cluster;
+};
+std::vector<Launch> g_log;
 std::set<cudaStream_t> g_capturing;
 std::set<cudaEvent_t> g_forked;
 cudaError_t g_last = cudaSuccess;
@@ -40,7 +46,7 @@ cudaError_t keep(cudaError_t e)
     if (e != cudaSuccess) g_last = e;
     return e;
 }
-cudaError_t launch(const void *fn, dim3 grid, size_t smem, bool cooperative)
+cudaError_t launch(const void *fn, dim3 grid, size_t smem, bool cooperative, int cluster = 1)
 {
     const auto it = g_limit.find({g_dev, fn});
     const size_t limit = it == g_limit.end() ? 48 * 1024 : std::max<size_t>(it->second, 48 * 1024);
@@ -49,6 +55,7 @@ cudaError_t launch(const void *fn, dim3 grid, size_t smem, bool cooperative)
         return keep(cudaErrorInvalidValue);
     }
     ++g_launches[g_dev];
+    g_log.push_back({g_name[fn], (int)grid.x, cluster});
     return cudaSuccess;
 }
 }  // namespace
@@ -57,7 +64,19 @@ API void fake_set_mps(int on) { g_mps = on; }
 API int fake_conditional_nodes() { return g_cond; }
 API int fake_launches(int dev) { return g_launches[dev]; }
 API const char *fake_refused() { return g_refused.c_str(); }
-API int fake_devices_sms(int dev) { return kSms[dev]; }
+// launches since fake_forget_launches of kernels whose (mangled) name holds `name`: their number, and the grid
+// and cluster of the first
+API int fake_launches_of(const char *name, int *grid, int *cluster)
+{
+    int n = 0;
+    for (const Launch &l : g_log)
+        if (l.name.find(name) != std::string::npos && n++ == 0) {
+            *grid = l.grid;
+            *cluster = l.cluster;
+        }
+    return n;
+}
+API void fake_forget_launches() { g_log.clear(); }
 
 FAKE cudaError_t cudaGetDeviceCount(int *n) { *n = kDevices; return cudaSuccess; }
 FAKE cudaError_t cudaGetDevice(int *d) { *d = g_dev; return cudaSuccess; }
@@ -157,8 +176,12 @@ FAKE cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cuda
 FAKE cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **)
 {
     bool coop = false;
-    for (unsigned i = 0; i < c->numAttrs; ++i) coop |= c->attrs[i].id == cudaLaunchAttributeCooperative && c->attrs[i].val.cooperative;
-    return launch(fn, c->gridDim, c->dynamicSmemBytes, coop);
+    int cluster = 1;
+    for (unsigned i = 0; i < c->numAttrs; ++i) {
+        coop |= c->attrs[i].id == cudaLaunchAttributeCooperative && c->attrs[i].val.cooperative;
+        if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[i].val.clusterDim.x;
+    }
+    return launch(fn, c->gridDim, c->dynamicSmemBytes, coop, cluster);
 }
 FAKE cudaError_t cudaLaunchCooperativeKernel(const void *fn, dim3 grid, dim3, void **, size_t smem, cudaStream_t) { return launch(fn, grid, smem, true); }
 FAKE unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t smem, struct CUstream_st *st) { g_pending = {grid, block, smem, st}; return 0; }

@@ -148,3 +148,24 @@ def test_small_shares_take_the_elimination(fake, column, S, slots, reduction):
     _step(col)
     assert _launches_of(fake, "k_inv64")[0] > 0 and _launches_of(fake, "k_factor64")[0] == 0
     b.close()
+
+
+@pytest.mark.parametrize("how", ["round", "submit", "run"])
+def test_no_conditional_nodes_under_mps(fake, column, how):
+    """Cooperative kernels, which the conditional parts hold, may stand in conditional nodes only while
+    the device is not shared through MPS: there the steps are captured without such nodes."""
+    fake.fake_set_mps(1)
+    b = _batch(fake, column, 2, 1, synth.small_column(L=9), "mixed")
+    try:
+        before = fake.fake_conditional_nodes()
+        if how == "round":
+            b.step(1)
+        elif how == "submit":
+            b.submit(0, 1)
+        else:
+            info = xk.StepInfo()
+            column(synth.small_column(L=9), "mixed", 0)._call("xk_step", 1e-8, ctypes.byref(info))
+        assert fake.fake_conditional_nodes() == before
+    finally:
+        b.close()
+        fake.fake_set_mps(0)
