@@ -121,10 +121,11 @@ typedef struct {
                              leaf block inversions in FP32 on the CUDA cores (the default); 0 by the
                              chain of block inversions
                              (cluster_size, panel_width, twisted, fp32_pivoting then apply) */
-    long long wait_polls; /* every device-side wait on other CTAs (the grid barriers of the FP64
-                             factorization) gives up after this many polls, about 0.1 us each, and
-                             the call returns XK_ETIMEOUT with the context still usable (0: 2^24
-                             polls, one to two seconds) */
+    long long wait_polls; /* every device-side wait on other CTAs (the barriers, flags and cluster
+                             exchanges of the FP64 factorizations, the barriers of the solves) gives
+                             up after this many polls, 0.1 to 0.4 us each, and the call returns
+                             XK_ETIMEOUT with the context still usable (0: 2^22 polls, or 2^24 of the
+                             shorter ones; about a second or two) */
     int use_graphs;       /* 1 (default): xk_run_to_steady and the batch calls capture a chunk of
                              controlled steps (every kernel of every step, with the device-side
                              gating of FGMRES iterations and of the FP64 route) in a CUDA graph once

@@ -21,7 +21,7 @@
 #include <cstring>
 
 #include "xk_bcr.cuh"
-#include "xk_internal.cuh"
+#include "xk_mbar.cuh"
 
 namespace xk {
 
@@ -31,54 +31,15 @@ constexpr int kInvThreads = 256;
 constexpr int kInvBusy = 96;              // FP64 instructions of a step above which warp 4 works too
 constexpr size_t kInvSmemMax = 220 * 1024;
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank)
-{
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
 // Asynchronous store of 8 bytes into a CTA of the cluster, counted by that CTA's mbarrier.
 __device__ __forceinline__ void st_async(uint32_t addr, unsigned long long v, uint32_t mbar)
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(mbar)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_init(uint32_t bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Bounded wait for a barrier's only phase.  Giving up is recorded, and the caller carries on (every
-// index it takes from what did not arrive is clamped) to the cluster's barrier at the end.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, Ctl *ctl)
-{
-    for (unsigned long long i = 0; i < kSyncPolls; ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar)
-            : "memory");
-        if (done) return;
-        if ((i & 63) == 63 && *(volatile int *)&ctl->err_timeout) return;
-    }
-    atomicExch(&ctl->err_timeout, 1);
 }
 __device__ __forceinline__ void cluster_sync()
 {
@@ -178,7 +139,7 @@ __global__ void __launch_bounds__(kInvThreads, 1) k_inv64(const Bcr64Inv *tasks,
                 }
             }
             double *v = slots + (size_t)c * lay.slot;
-            mbar_wait(bar0 + 8 * c, ctl);
+            mbar_wait(bar0 + 8 * c, 0u, ctl);
             const int p = min(max(((const int *)(v + S))[0], 0), S - 1);
             const double rp = v[S + 1];
             double w[RPT];
@@ -207,7 +168,7 @@ __global__ void __launch_bounds__(kInvThreads, 1) k_inv64(const Bcr64Inv *tasks,
                 j += cs;
                 ++l;
                 if (j < S) {
-                    if (c > 0) mbar_wait(handed0 + 8 * l, ctl);   // all steps before c are in it
+                    if (c > 0) mbar_wait(handed0 + 8 * l, 0u, ctl);   // all steps before c are in it
 #pragma unroll
                     for (int t = 0; t < RPT; ++t) a[t] = t * 32 + lane < S ? cols[l * S + t * 32 + lane] : 0.0;
                 }
@@ -231,7 +192,7 @@ __global__ void __launch_bounds__(kInvThreads, 1) k_inv64(const Bcr64Inv *tasks,
         for (int c = 0; c < S; ++c) {
             if (rank + cs * first <= c) ++first;
             while (m0 < own && wk + nwk * m0 <= first) ++m0;
-            mbar_wait(ready0 + 8 * c, ctl);
+            mbar_wait(ready0 + 8 * c, 0u, ctl);
             const double *v = slots + (size_t)c * lay.slot;
             const int p = prow[c];
             double w[RPT];

@@ -25,11 +25,10 @@
 // iperm_k its inverse.  After factorization D holds B_k with D'^-1_k[i][j] = B_k[perm_k(i)][iperm_k(j)].
 #include <cuda_runtime.h>
 #include <math.h>
-#include <stdint.h>
 
 #include <algorithm>
 
-#include "xk_internal.cuh"
+#include "xk_mbar.cuh"
 
 namespace xk {
 
@@ -51,19 +50,6 @@ struct __align__(16) Cand {
 };
 constexpr int kCandParts = sizeof(Cand) / 16;
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank)
-{
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
 __device__ __forceinline__ void st_cluster(uint32_t addr, int v)
 {
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
@@ -75,29 +61,7 @@ __device__ __forceinline__ void st_async(uint32_t addr, uint4 v, uint32_t mbar)
                  "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(mbar)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Bounded wait for a phase.  Giving up is recorded, and the caller carries on (every index it takes
-// from what did not arrive is clamped) to the next grid barrier, where the cluster leaves together.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, Ctl *ctl)
-{
-    for (unsigned long long i = 0; i < kSyncPolls; ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return;
-        if ((i & 63) == 63 && *(volatile int *)&ctl->err_timeout) return;
-    }
-    atomicExch(&ctl->err_timeout, 1);
-}
-// Bounded wait for a counter that other CTAs raise; as above.
+// Bounded wait for a counter that other CTAs raise, as mbar_wait.
 __device__ __forceinline__ void wait_count(const unsigned *word, unsigned target, Ctl *ctl)
 {
     const unsigned long long limit = ctl->wait_polls ? ctl->wait_polls : kSyncPolls;
@@ -390,7 +354,7 @@ __device__ __forceinline__ Panel make_panel(PanelShared &sh, double *dyn, const 
     q.ctl = ctl;
     // every CTA's mbarriers stand before another CTA sends to them
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 2; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(q.mbar + 8u * i) : "memory");
+        for (int i = 0; i < 2; ++i) mbar_init(q.mbar + 8u * i);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     cluster_sync(cs);
