@@ -36,16 +36,6 @@ WORKLOAD = "xodiac-594sp-7720rx-150L"
 SAMPLE_LAYERS = 24          # CPU oracle sample: this many layers of the same column
 
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the dominant
-# kernels, from the ncu captures summarized in profiles/, for the configuration captured there;
-# a run in another configuration reports null.
-PROFILED_TRAFFIC = {
-    ("mixed", 16, 8, 1): (371.3e6, "k_factor_cluster<8>, two-chain launch (profiles/k_factor_cluster_594x150.txt)"),
-    ("fp64", 152, 8, 0, 0): (833.5e6, "k_factor<double, 8>, an earlier form (profiles/k_factor_fp64_594x150.txt)"),
-    ("fp64", 152, 8, 0, 1): (818.6e6, "k_factor<double, 8>, two-chain launch of an earlier form (profiles/k_factor_fp64_594x150.txt)"),
-}
-
-
 def _peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     try:
@@ -357,6 +347,90 @@ def steady_runs(prob, tuning, caps):
     return out
 
 
+def fp64_factorization(S, L, settings):
+    """Name and flops of the FP64 factorization that a column of S species and L layers with these settings
+    takes: the reduction for small blocks unless a setting asks for an elimination, else Gauss-Jordan
+    inversions with Schur updates, layer by layer."""
+    nb, ctas = settings.get("panel_width", 0) or 8, settings.get("factor_ctas", 0)
+    flops = 2.0 * S ** 3 * L + 3.0 * S * S * (L - 1)
+    if settings.get("fp64_panel", 0):
+        return f"k_factor_pv<{nb}>", flops
+    two = " (two grid halves, then the middle layer)" if settings.get("twisted", 1) and L >= 3 else ""
+    if nb != 8:
+        return f"k_factor<double, {nb}>" + two, flops
+    if (S <= 152 and L >= 8 and not ctas and not settings.get("cluster_size", 0) and settings.get("twisted", 1) == 1
+            and settings.get("refine_max_iter", 10) > 0):
+        products, n = 0, (L + 1) // 2                 # level 0 has diagonal couplings
+        while n > 1:
+            elim, right = n // 2, (n - 1) // 2        # eliminated, and those with a neighbour above
+            # [P | Q], the Schur terms, and the couplings between the kept
+            products += 2 * (elim + right) + 2 * ((n + 1) // 2 - 1)
+            n = (n + 1) // 2
+        return "k_inv64, k_gemm64 (block cyclic reduction)", 2.0 * S ** 3 * (L + products)
+    half = (ctas or 152) // 2
+    cs = 1 if S <= 32 else 4 if S <= 128 or S > 500 else 8
+    cols = -(-S // max(half - cs, 1))
+    flow = half > cs and S * (cols | 1) * 8 <= 220 * 1024
+    return ("k_factor64_flow" if flow else "k_factor64") + two, flops
+
+
+def per_launch(ph, name):
+    ms_, calls = ph.get(name, (0.0, 0))
+    return ms_ / max(calls, 1), calls
+
+
+def a7_flops(S, L):
+    """LU and Schur work of block Thomas per step (the survey's count)."""
+    return 8.0 / 3.0 * S ** 3 * L
+
+
+def rooflines(res, S, L, derived, live):
+    """Per-kernel rooflines of the mixed step's FP32 factorization.  DRAM traffic is not measured here:
+    null."""
+    ph = res["phases"]
+    steps = res["steps"]
+    out = {}
+    if res["work"]:
+        mma, leaf = res["work"]
+        tc_ms, tc_calls = ph["tc"]
+        lf_ms, lf_calls = ph["leaf"]
+        nfac = max(ph["factor"][1], 1)            # factorizations timed
+        tc_s = tc_ms / nfac * 1e-3
+        lf_s = lf_ms / nfac * 1e-3
+        ach = 3.0 * mma / tc_s / 1e12            # the tensor pipe executes head x head, head x tail, tail x head
+        out["tc"] = {"kernel": "k_tc_gemm (tcgen05 kind::tf32, head/tail split)", "bound": "tensor",
+                     "achieved": ach, "peak": derived["tf32"], "unit": "TFLOP/s", "frac": ach / derived["tf32"],
+                     "peak_kind": derived["kind"] + " (tf32 1.1 / bf16 2.25)",
+                     "peak_live_tf32_matmul": live["tf32"], "frac_of_live": ach / live["tf32"],
+                     "useful_tflops": mma / tc_s / 1e12, "flops_per_factorization": mma,
+                     "ms_per_factorization": tc_s * 1e3, "launches_per_factorization": tc_calls / nfac,
+                     "ms_per_step": tc_ms / steps, "traffic": None}
+        ach = leaf / lf_s / 1e12
+        out["leaf"] = {"kernel": "k_leaf_inverse (FP32 Gauss-Jordan, partial pivoting, one CTA per block)",
+                       "bound": "alu", "achieved": ach, "peak": derived["f32"], "unit": "TFLOP/s",
+                       "frac": ach / derived["f32"], "peak_kind": derived["kind"],
+                       "peak_live_f32_matmul": live["f32"], "flops_per_factorization": leaf,
+                       "ms_per_factorization": lf_s * 1e3, "launches_per_factorization": lf_calls / nfac,
+                       "ms_per_step": lf_ms / steps, "traffic": None}
+    fac_ms, fac_calls = per_launch(ph, "factor")
+    out["a7"] = {"flops_per_factorization": a7_flops(S, L), "ms_per_factorization": fac_ms,
+                 "tflops": a7_flops(S, L) / (fac_ms * 1e-3) / 1e12,
+                 "note": "8/3 S^3 L (block Thomas LU + Schur) over the whole FP32 factorization phase"}
+    return out
+
+
+def roofline_fp64(res, S, L, derived, live):
+    """Roofline of the FP64 factorization that was run; DRAM traffic as above."""
+    fac_ms, fac_calls = per_launch(res["phases"], "factor")
+    avg_s = fac_ms * 1e-3
+    name, flops = fp64_factorization(S, L, res["settings"])
+    achieved = flops / avg_s / 1e12
+    return {"kernel": name, "bound": "alu", "achieved": achieved, "peak": live["f64"], "unit": "TFLOP/s",
+            "frac": achieved / live["f64"], "peak_kind": "FP64 matmul measured live (torch.matmul float64)",
+            "peak_derived": derived["f64"], "flops_per_factorization": flops,
+            "a7_survey_tflops": a7_flops(S, L) / avg_s / 1e12, "ms_per_factorization": avg_s * 1e3, "traffic": None}
+
+
 def run_ours(args):
     import numpy as np
     import torch
@@ -412,15 +486,11 @@ def run_ours(args):
         _barrier(ws)
         ms_traced, info_traced, phases, _, _ = time_steps(col, K, stream, prof=True)
         steps_done = max(int(info.steps), 1)
-        t = tuning[prec]
-        col_cfg = {"bcr": t.get("fp32_bcr", 1) if prec == "mixed" else 0, "cluster": t.get("cluster_size", 16),
-                   "nb": t.get("panel_width", 8) or 8, "twisted": t.get("twisted", 1),
-                   "ctas": t.get("factor_ctas", 152) or 152, "panel": t.get("fp64_panel", 0)}
-        work = col.factor_work() if (prec == "mixed" and col_cfg["bcr"]) else None
+        work = col.factor_work() if prec == "mixed" and tuning[prec].get("fp32_bcr", 1) else None
         results[prec] = dict(ms=ms, steps=steps_done, phases=phases, launches=launches, info=info, graphs=graphs,
                              start_state=start_state, start_dt=start_dt, K=K,
                              ms_traced=ms_traced, steps_traced=max(int(info_traced.steps), 1),
-                             col=col if prec == "mixed" else None, col_cfg=col_cfg, work=work)
+                             col=col if prec == "mixed" else None, settings=tuning[prec], work=work)
         if prec == "fp64":
             del col
             torch.cuda.empty_cache()
@@ -430,68 +500,7 @@ def run_ours(args):
     S, L = prob.S, prob.L
     value, ms_step = whole_job_rate(mixed["ms"] / mixed["steps"], ws, dev)
     fp64_value, fp64_ms_step = whole_job_rate(fp64["ms"] / fp64["steps"], ws, dev)
-    a7_flops = 8.0 / 3.0 * S ** 3 * L            # LU + Schur work of block Thomas per step (the survey's count)
-
-    def per_launch(ph, name):
-        ms_, calls = ph.get(name, (0.0, 0))
-        return ms_ / max(calls, 1), calls
-
-    def rooflines(res):
-        """Per-kernel rooflines of the mixed step's FP32 factorization and the FP64 one."""
-        ph = res["phases"]
-        steps = res["steps"]
-        out = {}
-        if res["work"]:
-            mma, leaf = res["work"]
-            tc_ms, tc_calls = ph["tc"]
-            lf_ms, lf_calls = ph["leaf"]
-            nfac = max(ph["factor"][1], 1)            # factorizations timed
-            tc_s = tc_ms / nfac * 1e-3
-            lf_s = lf_ms / nfac * 1e-3
-            ach = 3.0 * mma / tc_s / 1e12            # the tensor pipe executes head x head, head x tail, tail x head
-            out["tc"] = {"kernel": "k_tc_gemm (tcgen05 kind::tf32, head/tail split)", "bound": "tensor",
-                         "achieved": ach, "peak": derived["tf32"], "unit": "TFLOP/s", "frac": ach / derived["tf32"],
-                         "peak_kind": derived["kind"] + " (tf32 1.1 / bf16 2.25)",
-                         "peak_live_tf32_matmul": live["tf32"], "frac_of_live": ach / live["tf32"],
-                         "useful_tflops": mma / tc_s / 1e12, "flops_per_factorization": mma,
-                         "ms_per_factorization": tc_s * 1e3, "launches_per_factorization": tc_calls / nfac,
-                         "ms_per_step": tc_ms / steps, "traffic": 5.011e6,
-                         "traffic_launch": "one 72-tile launch (A and B operands first touched from DRAM)",
-                         "traffic_source": "profiles/k_tc_gemm_594x150.txt"}
-            ach = leaf / lf_s / 1e12
-            out["leaf"] = {"kernel": "k_leaf_inverse (FP32 Gauss-Jordan, partial pivoting, one CTA per block)",
-                           "bound": "alu", "achieved": ach, "peak": derived["f32"], "unit": "TFLOP/s",
-                           "frac": ach / derived["f32"], "peak_kind": derived["kind"],
-                           "peak_live_f32_matmul": live["f32"], "flops_per_factorization": leaf,
-                           "ms_per_factorization": lf_s * 1e3, "launches_per_factorization": lf_calls / nfac,
-                           "ms_per_step": lf_ms / steps, "traffic": 7.843e6,
-                           "traffic_launch": "one level-0 launch of 75 blocks of 160 (7.68 MB algorithmic read)",
-                           "traffic_source": "profiles/k_leaf_inverse_594x150.txt"}
-        fac_ms, fac_calls = per_launch(ph, "factor")
-        out["a7"] = {"flops_per_factorization": a7_flops, "ms_per_factorization": fac_ms,
-                     "tflops": a7_flops / (fac_ms * 1e-3) / 1e12,
-                     "note": "8/3 S^3 L (block Thomas LU + Schur) over the whole FP32 factorization phase"}
-        return out
-
-    def roofline_fp64(res):
-        ph = res["phases"]
-        fac_ms, fac_calls = per_launch(ph, "factor")
-        avg_s = fac_ms * 1e-3
-        flops = 2.0 * S ** 3 * L + 3.0 * S * S * (L - 1)     # Gauss-Jordan inversions + Schur updates
-        achieved = flops / avg_s / 1e12
-        cfg = res["col_cfg"]
-        twisted = int(cfg["twisted"] and not cfg["panel"] and L >= 3)
-        key = ("fp64", cfg["ctas"], cfg["nb"], cfg["panel"], twisted)
-        traffic, source = PROFILED_TRAFFIC.get(key, (None, None))
-        name = "k_factor64_flow" if cfg["nb"] == 8 and not cfg["panel"] else f"k_factor<double, {cfg['nb']}>"
-        return {"kernel": name + (" (two grid halves, then the middle layer)" if twisted else ""),
-                "bound": "alu", "achieved": achieved, "peak": live["f64"], "unit": "TFLOP/s",
-                "frac": achieved / live["f64"], "peak_kind": "FP64 matmul measured live (torch.matmul float64)",
-                "peak_derived": derived["f64"], "flops_per_factorization": flops,
-                "a7_survey_tflops": a7_flops / avg_s / 1e12, "ms_per_factorization": avg_s * 1e3,
-                "traffic": traffic, "traffic_source": source}
-
-    roof = rooflines(mixed)
+    roof = rooflines(mixed, S, L, derived, live)
     dom = max((k for k in ("tc", "leaf") if k in roof), key=lambda k: roof[k]["ms_per_step"], default=None)
 
     # end to end through the C-ABI with host buffers, over the same K steps as the timed region (same
@@ -567,7 +576,7 @@ def run_ours(args):
                      "steps": fp64["steps"], "speedup_mixed_over_fp64": fp64_ms_step / ms_step},
             "roofline": roof.get(dom) if dom else roof["a7"],
             "rooflines": roof,
-            "roofline_fp64": roofline_fp64(fp64),
+            "roofline_fp64": roofline_fp64(fp64, S, L, derived, live),
             "peaks": {"measured_file": {k: peaks.get(k) for k in ("hbm_gbs", "bf16_tflops", "bf16_tflops_sustained")},
                       "derived": derived, "live_matmul_tflops": live},
             "phases_ms": ph, "phases_ms_fp64": ph64,
