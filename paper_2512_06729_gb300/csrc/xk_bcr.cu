@@ -107,16 +107,6 @@ __device__ __forceinline__ void mul2(float2 &d, float2 a)
     asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(dd) : "l"(reinterpret_cast<unsigned long long &>(a)));
 }
 
-// 1 / x to an FP32 unit: the hardware's approximation and one Newton-Raphson step.  The division's
-// sequence is on the chain of every column (68 us against 63 for a block of 160).
-__device__ __forceinline__ float reciprocal(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    const float z = fmaf(y, fmaf(-x, y, 1.0f), y);
-    return fabsf(z) <= 3.402823466e38f ? z : 1.0f / x;      // subnormal or huge x
-}
-
 struct __align__(16) LeafCand {
     float row[kLeafPanel];        // 1 / pivot, then the rest of the row times it
 };
@@ -185,7 +175,7 @@ __global__ void __launch_bounds__(kLeafThreads, 1) k_leaf_inverse(const BcrLeaf 
                 // meanwhile this lane's own row, scaled (a singular block: the FP64 Krylov solve sees a
                 // poor preconditioner)
                 float s[NP];
-                s[0] = reciprocal(x[0] == 0.0f ? 1e-30f : x[0]);
+                s[0] = reciprocal32(x[0] == 0.0f ? 1e-30f : x[0]);
 #pragma unroll
                 for (int j = 1; j < NP; ++j) s[j] = x[j] * s[0];
                 LeafCand *cb = cand[c & 1];

@@ -89,18 +89,6 @@ __device__ __forceinline__ void cluster_sync(int cs)
     }
 }
 
-// 1 / x by two Newton-Raphson steps from the hardware's approximation; the quotient itself where the
-// approximation's range ends.
-__device__ __forceinline__ double reciprocal(double x)
-{
-    const double ax = fabs(x);
-    if (!(ax > 1e-290 && ax < 1e290)) return 1.0 / x;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-}
-
 // Barrier over the clusters of a chain.  The first CTA of each cluster arrives and polls (bounded, as
 // GridSync) and hands the outcome to the others, so that the CTAs of a cluster always leave together:
 // none writes into the shared memory of one that has gone.
@@ -234,7 +222,7 @@ __device__ __forceinline__ void panel_step(Panel &q, double *D, int *perm, int *
 #pragma unroll
             for (int j = 0; j < kNB; ++j) mine_row[j] = RPT > 1 && bi == RPT - 1 ? x[RPT - 1][j] : x[0][j];
             // (a column without a nonzero candidate is singular: the bookkeeping goes on)
-            mine_row[0] = key == 0u ? 0.0 : reciprocal(mine_row[0]);
+            mine_row[0] = key == 0u ? 0.0 : reciprocal_newton(mine_row[0]);
             const unsigned best = __reduce_max_sync(0xffffffffu, bi >= 0 ? key + 1u : 0u);
             const unsigned who = __ballot_sync(0xffffffffu, bi >= 0 && key + 1u == best);
             const int src = who ? __ffs(who) - 1 : 0;

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/xk.h"
+#include "xk_recip.cuh"
 
 namespace xk {
 
@@ -172,47 +173,6 @@ __device__ __forceinline__ void reaction_terms_at(const Col &c, int k, int r, co
         d[s] = df;
         d[3 + s] = db;
     }
-}
-
-// 1 / x from the hardware's approximation (some 20 bits) by one third-order step, y (1 + e + e^2) with
-// e = 1 - x y: the series of 1 / (1 - e).  Three dependent FP64 operations of 65 clocks each on this
-// part, where a division takes about ten.  The division where the approximation's range ends (the
-// exponent looked at as an integer).
-__device__ __forceinline__ double reciprocal64(double x)
-{
-    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-    if (ex - 32u > 1984u) return 1.0 / x;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
-// 1 / x correctly rounded, without the division's length: reciprocal64 is within one unit in the last
-// place, and from there y + y (1 - x y) rounds correctly (Markstein 1990) unless x's fraction is all
-// ones.  That case, and exponents at which the residual may not be exact, take the division.
-__device__ __forceinline__ double reciprocal_rn(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x), ex = (hi >> 20) & 0x7ffu;
-    if (ex - 64u > 1900u || ((hi & 0xfffffu) == 0xfffffu && __double2loint(x) == -1)) return 1.0 / x;
-    const double y = reciprocal64(x);
-    return fma(y, fma(-x, y, 1.0), y);
-}
-
-// x / d, correctly rounded, from rd = reciprocal_rn(d): the product q = x rd is within a unit of the
-// quotient, and q + rd (x - q d) rounds correctly (Markstein 1990) while the residual is exact and the
-// quotient a normal number, as it is for exponents of x and d within some 2^508 of one.  Three dependent
-// FP64 operations where a division takes some ten.  Elsewhere the division itself (a d below 2^-1024 has
-// an infinite reciprocal, and 0 x inf is no quotient); a zero x needs neither.
-__device__ __forceinline__ double over(double x, double d, double rd)
-{
-    const unsigned hx = (unsigned)__double2hiint(x) & 0x7fffffffu, hd = (unsigned)__double2hiint(d) & 0x7fffffffu;
-    const double q = x * rd;
-    if ((hd >> 20) - 515u <= 1015u) {
-        if ((hx >> 20) - 515u <= 1015u) return fma(fma(-q, d, x), rd, q);
-        if ((hx | (unsigned)__double2loint(x)) == 0u) return q;
-    }
-    return x / d;
 }
 
 // Entry q of the Jacobian pattern (row-grouped): sum of its terms, -dF_i/dn_j of one layer, in a
