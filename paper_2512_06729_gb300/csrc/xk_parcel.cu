@@ -11,8 +11,8 @@
 //
 // The sweep is sequential in the layers, so one CTA runs a whole iteration: every reduction,
 // pivot search and elimination step stays inside the block (no grid-wide wait).  Systems whose two
-// S x S matrices (the system and its factors) fit in shared memory (S up to 111) have a kernel of
-// their own; larger ones keep them in global memory, where they stay in L2.
+// S x S matrices (the system and its factors) fit in shared memory (S up to 112, small_layout against
+// kSmemLimit) have a kernel of their own; larger ones keep them in global memory, where they stay in L2.
 #include <cfloat>
 
 #include "xk_internal.cuh"

@@ -169,3 +169,14 @@ def test_no_conditional_nodes_under_mps(fake, column, how):
     finally:
         b.close()
         fake.fake_set_mps(0)
+
+
+@pytest.mark.parametrize("S,small", [(40, True), (111, True), (112, True), (113, False), (161, False)])
+def test_parcel_kernel_by_size(fake, column, S, small):
+    """The parcel's kernel for systems in shared memory ends where its layout does."""
+    p = synth.small_column(S=S, L=3, n_two=3 * S, n_three=3 * S // 4, n_photo=5, W=40, elements="chons" if S < 110 else "full")
+    col = column(p, "fp64", 0)
+    fake.fake_forget_launches()
+    col._call("xk_parcel_begin", 100, 1e-8)
+    assert (_launches_of(fake, "k_parcel_small")[0], _launches_of(fake, "k_parcel_iteration")[0]) == ((1, 0) if small else (0, 1))
+    assert fake.fake_refused() == b""
