@@ -114,7 +114,10 @@ typedef struct {
                              gmres_tol.  0 = direct solve only.  With the refinement, at least 8 layers
                              and cluster_size, panel_width (or 8), factor_ctas, twisted and fp64_panel at
                              their defaults, the plain FP64 path factors blocks of at most 152 species by
-                             block cyclic reduction in FP64 */
+                             block cyclic reduction in FP64.  Its arrays are five more S x S blocks a
+                             layer in the workspace (96 species, 150 layers: 104 MB instead of 48); any
+                             factor_ctas leaves them out, and a batch whose slots leave a column too few
+                             CTAs takes the elimination by itself */
     int fp32_bcr;         /* mixed mode: 1 factors the FP32 preconditioner by block cyclic reduction of
                              the layers (odd layers eliminated first, level by level) with every dense
                              product on the tensor cores (TF32 head/tail split, FP32 accuracy) and the

@@ -481,7 +481,9 @@ int basis_size(const xk_ctx *c)
 
 // Whether the plain FP64 path factors by the reduction: blocks it was made for, a refinement around it,
 // and no setting that asks for a particular elimination.  Below kBcr64MinLayers the elimination's chain
-// is as short as the reduction's.
+// is as short as the reduction's (a linear step of 152 species with the reduction and the elimination: 8
+// layers 1.40 and 1.66 ms, 9 1.80 and 1.64, 12 1.82 and 2.17, 40 3.3 and 5.7; of 96: 0.69 and 1.07 at 8,
+// 1.3 and 3.5 at 40; of 20: 0.57 and 1.31 at either).
 constexpr int kBcr64MinLayers = 8;
 bool bcr64_wanted(const xk_ctx *c)
 {
@@ -1863,6 +1865,7 @@ int xk_batch_remove(xk_batch *b, int slot)
     s.ctx->plan64 = s.saved_plan64;
     s.ctx->bcr.solve_ctas = s.ctx->bcr64.solve_ctas = s.saved_solve_ctas;
     s.ctx->use_bcr64 = s.saved_use_bcr64;
+    if (s.ctx->ctl_host->err_timeout) timed_out(s.ctx);      // the barrier words as the next call expects them
     if (s.ev) cudaEventDestroy(s.ev);
     cudaStreamDestroy(s.st);
     b->used -= s.bytes;

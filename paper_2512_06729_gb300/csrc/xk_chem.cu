@@ -879,7 +879,7 @@ __global__ void k_after_refactor(long long N, const double *s, double *s64, Ctl 
     long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx < N) s64[idx] = s[idx];
     if (idx == 0) {
-        ctl->have64 = 1;
+        ctl->have64 = !ctl->err_timeout;     // pivots and blocks of one that gave up are not complete
         ctl->refactors += 1;
     }
 }
@@ -978,7 +978,8 @@ void launch_set_mixing(const Col &c, const double *f, double *n, cudaStream_t st
 }
 
 // ---------------------------------------------------------------------------
-// Transport terms of the rows of I/dt - dF/dn (the same quotients k_jacobian forms per row).
+// Transport terms of the rows of I/dt - dF/dn, once per atmosphere: read by the rows' equilibration, the
+// Jacobian's assembly and J v.
 __global__ void k_transport_rows(Col c)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;

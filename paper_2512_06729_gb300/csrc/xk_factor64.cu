@@ -121,10 +121,23 @@ struct ChainSync {
                 }
             }
             __threadfence();
-            if (cs == 1) *go = ok;
-            else
-                for (int r = 0; r < cs; ++r) st_cluster(map_rank(smem_u32(go), r), ok);
+            // complete, but a wait of somebody's may have given up on the way here
+            tell(ok && !*vto);
         }
+        cluster_sync(cs);
+        return *go != 0;
+    }
+    __device__ __forceinline__ void tell(int ok)
+    {
+        if (cs == 1) *go = ok;
+        else
+            for (int r = 0; r < cs; ++r) st_cluster(map_rank(smem_u32(go), r), ok);
+    }
+    // at the start, after a barrier of the cluster: false if a wait of an earlier launch has given up.  One
+    // CTA looks: another that looked for itself might see a wait of this launch give up and leave alone.
+    __device__ __forceinline__ bool open()
+    {
+        if (crank == 0 && threadIdx.x == 0) tell(!*(volatile int *)&ctl->err_timeout);
         cluster_sync(cs);
         return *go != 0;
     }
@@ -288,6 +301,10 @@ __device__ __forceinline__ void panel_step(Panel &q, double *D, int *perm, int *
     }
 }
 
+// A pivot's row, or its place among them.  Where a wait has given up the list may hold anything: kept in
+// bounds until the chain's next barrier ends the launch.
+__device__ __forceinline__ int row_at(const int *p, int S) { return min(max(__ldcg(p), 0), S - 1); }
+
 // Which layers a chain takes, and in which order.
 struct Order {
     int nsteps, k0, dk;
@@ -366,7 +383,7 @@ template <int RPT>
 __global__ void __launch_bounds__(kThreads, 1)
 k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int cs)
 {
-    if (ctl->finished || ctl->err_timeout || (skip && *skip)) return;
+    if (ctl->finished || (skip && *skip)) return;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ PanelShared sh;
     const int S = a.S, ld = a.ld;
@@ -379,6 +396,7 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
     const int ntrail = nclus > 1 ? nblk - cs : nblk, tq = nclus > 1 ? bid - cs : bid;
     ChainSync chain{a.bar + 2 * half, a.bar + 6 + half, ctl, cs, nclus, crank, &sh.go, 0u};
     Panel q = make_panel(sh, (double *)dyn, a, ctl, cs, crank);
+    if (!chain.open()) return;
     double *U = q.G + (size_t)q.rpc * kPS;                // [kNB][cw]: pivot rows in this CTA's columns
     double *rowbuf = (double *)dyn + (size_t)warp * S;    // Schur term: a source row per warp
     const Order o = order_of(mode, half, a.L, mid);
@@ -392,13 +410,13 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
             const double *Bn = a.D + (size_t)nbr * S * ld;
             const int *pn = a.perm + (size_t)nbr * S, *ipn = a.iperm + (size_t)nbr * S;
             for (int i = bid * kWarps + warp; i < S; i += nblk * kWarps) {
-                const double *src = Bn + (size_t)__ldcg(pn + i) * ld;
+                const double *src = Bn + (size_t)row_at(pn + i, S) * ld;
                 const double rc = rowc[i];
                 __syncwarp();
                 for (int j = lane; j < S; j += 32) rowbuf[j] = __ldcg(src + j);
                 __syncwarp();
                 double *Di = D + (size_t)i * ld;
-                for (int j = lane; j < S; j += 32) Di[j] -= rc * rowbuf[__ldcg(ipn + j)] * colc[j];
+                for (int j = lane; j < S; j += 32) Di[j] -= rc * rowbuf[row_at(ipn + j, S)] * colc[j];
             }
         });
         if (touched && !chain.sync()) return;
@@ -414,12 +432,12 @@ k_factor64(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int
                 if (cw > 0) {
                     int pr[kNB];
 #pragma unroll
-                    for (int l = 0; l < kNB; ++l) pr[l] = l < nb ? min(max(__ldcg(perm + q0 + l), 0), S - 1) : -1;
+                    for (int l = 0; l < kNB; ++l) pr[l] = l < nb ? row_at(perm + q0 + l, S) : -1;
                     auto col = [&](int c) { return j0 + c < q0 ? j0 + c : j0 + c + (c1 - q0); };
                     __syncthreads();
                     for (int e = tid; e < kNB * cw; e += kThreads) {
                         const int l = e / cw, c = e - l * cw;
-                        U[e] = l < nb ? __ldcg(D + (size_t)min(max(__ldcg(perm + q0 + l), 0), S - 1) * ld + col(c)) : 0.0;
+                        U[e] = l < nb ? __ldcg(D + (size_t)row_at(perm + q0 + l, S) * ld + col(c)) : 0.0;
                     }
                     __syncthreads();
                     // one element per thread, three of them in flight
@@ -474,7 +492,7 @@ constexpr int kMaxPanels = 2 * kThreads / kNB;
 __global__ void __launch_bounds__(kThreads, 1)
 k_factor64_flow(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid, int cs)
 {
-    if (ctl->finished || ctl->err_timeout || (skip && *skip)) return;
+    if (ctl->finished || (skip && *skip)) return;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ PanelShared sh;
     const int S = a.S, ld = a.ld;
@@ -492,6 +510,7 @@ k_factor64_flow(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid
     const int j0 = tq * per + min(tq, rest), cw = tq >= 0 ? per + (tq < rest ? 1 : 0) : 0;
     auto owner = [&](int j) { return j < rest * (per + 1) ? j / (per + 1) : rest + (j - rest * (per + 1)) / max(per, 1); };
     Panel q = make_panel(sh, (double *)dyn, a, ctl, cs, crank);
+    if (!chain.open()) return;
     const int ws = cw | 1;                        // odd row stride: a row per thread without conflicts
     double *W = (double *)dyn;                    // [S][ws]: this CTA's columns
     double *U = W + (size_t)S * ws;               // [kNB][cw]
@@ -531,7 +550,7 @@ k_factor64_flow(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid
                 const int *pn = a.perm + (size_t)nbr * S, *ipn = a.iperm + (size_t)nbr * S;
                 for (int e = tid; e < S * cw; e += kThreads) {
                     const int i = e / cw, c = e - i * cw;
-                    W[i * ws + c] -= rowc[i] * __ldcg(Bn + (size_t)__ldcg(pn + i) * ld + __ldcg(ipn + j0 + c)) * colc[j0 + c];
+                    W[i * ws + c] -= rowc[i] * __ldcg(Bn + (size_t)row_at(pn + i, S) * ld + row_at(ipn + j0 + c, S)) * colc[j0 + c];
                 }
             });
             __syncthreads();
@@ -543,7 +562,7 @@ k_factor64_flow(BlockSys<double> a, Ctl *ctl, const int *skip, int mode, int mid
                 __syncthreads();
                 int pr[kNB];
 #pragma unroll
-                for (int l = 0; l < kNB; ++l) pr[l] = l < nb ? min(max(__ldcg(perm + c0 + l), 0), S - 1) : -1;
+                for (int l = 0; l < kNB; ++l) pr[l] = l < nb ? row_at(perm + c0 + l, S) : -1;
                 // G of this thread's first row on its way while the pivot rows are copied
                 double g[kNB];
                 auto load_g = [&](int r) {
