@@ -134,8 +134,8 @@ typedef struct {
                              gating of FGMRES iterations and of the FP64 route) in a CUDA graph once
                              and replay it, one graph launch per chunk; 0 launches every kernel from
                              the host.  Parts that the device may skip are conditional nodes of the
-                             graph, except in batches of more than 6 slots (submitted steps) or 8
-                             columns (rounds) and where the device is shared through MPS: there they
+                             graph, except in rounds of more than 8 columns, in steps submitted to
+                             batches of more slots than that (6 on the FP64 path) and where the device is shared through MPS: there they
                              are enqueued and their kernels return at once.  Tracing (xk_profile) launches from the host either way. */
     int photo_jacobian;   /* 1: the direct-beam photolysis rates are differentiated too (Sec. 2.3.3): the
                              operator of FGMRES (mixed path; the refinement iterations of the FP64 path)

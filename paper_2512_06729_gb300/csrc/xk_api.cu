@@ -1773,14 +1773,16 @@ void drop_round(xk_batch *b)
 }
 
 // Graphs with IF nodes run over the device's connections, eight by default, where the branches of one
-// without them all run at once.  So columns that would wait for a connection are captured without:
-// a round of more than kNodeColumns, and what is submitted to the slots of a batch of more than
-// kNodeSlots (each a graph of its own).  ms a step with and without nodes, mixed 96 x 90: rounds of 8
-// columns 1.74 and 2.36, of 12 3.37 and 3.17, of 64 36.9 and 15.1; submitted to 6 slots 1.47 and 1.94,
-// to 8 2.64 and 2.35.  FP64 250 x 60: rounds of 8 34.6 and 35.0, of 12 68.6 and 36.3, of 64 1,137 and
-// 219; submitted to 6 slots 19.7 and 20.0, to 8 67.5 and 35.1.
+// without them all run at once.  So columns that would wait for a connection are captured without: a
+// round of more than kNodeColumns, and what is submitted to the slots of a batch of more than that (each a
+// graph of its own), or of more than kNodeSlots64 where a column's FP64 elimination would wait and the
+// nodes only hold a few iterations.  ms a step with and without nodes, mixed 96 x 90: rounds of 8 columns
+// 1.74 and 2.36, of 12 3.37 and 3.17, of 64 36.9 and 15.1; late steps (64 to a column) submitted to 8 slots
+// 416 and 525 in all, to 32 2,031 and 1,389, of 250 x 60 to 8 677 and 800, to 16 1,671 and 1,350.  FP64
+// 250 x 60: rounds of 8 34.6 and 35.0, of 12 68.6 and 36.3, of 64 1,137 and 219; submitted to 6 slots 19.7
+// and 20.0, to 8 67.5 and 35.1.
 constexpr size_t kNodeColumns = 8;
-constexpr int kNodeSlots = 6;
+constexpr int kNodeSlots64 = 6;
 
 // Capture nsteps steps of every listed slot's column, each on its slot's stream, into b->round.
 int capture_round(xk_batch *b, const std::vector<int> &live, int nsteps)
@@ -2037,7 +2039,7 @@ int xk_batch_submit(xk_batch *b, int slot, int nsteps)
     if (s.finished) return XK_OK;
     cudaSetDevice(b->device);
     b->err.clear();
-    s.ctx->cond.off = b->max_slots > kNodeSlots;
+    s.ctx->cond.off = b->max_slots > (s.ctx->cfg.precision == XK_PREC_FP64 ? kNodeSlots64 : (int)kNodeColumns);
     int rc = run_steps(s.ctx, nsteps, true);
     s.ctx->cond.off = false;
     if (rc) {

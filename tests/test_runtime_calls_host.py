@@ -91,12 +91,16 @@ def _batch(fake, column, slots, columns, p, precision):
     return b
 
 
-@pytest.mark.parametrize("how,slots,columns,nodes", [("round", 8, 8, True), ("round", 16, 8, True), ("round", 9, 9, False),
-                                                     ("submit", 6, 2, True), ("submit", 7, 2, False)])
-def test_columns_of_a_batch_do_not_wait_for_connections(fake, column, how, slots, columns, nodes):
+@pytest.mark.parametrize("how,precision,slots,columns,nodes", [
+    ("round", "mixed", 8, 8, True), ("round", "mixed", 16, 8, True), ("round", "mixed", 9, 9, False),
+    ("submit", "mixed", 8, 2, True), ("submit", "mixed", 9, 2, False),
+    ("round", "fp64", 8, 2, True), ("submit", "fp64", 6, 2, True), ("submit", "fp64", 7, 2, False)])
+def test_columns_of_a_batch_do_not_wait_for_connections(fake, column, how, precision, slots, columns, nodes):
     """Steps captured with conditional nodes run on the device's connections, eight by default: no more
     columns than that are captured with them."""
-    b = _batch(fake, column, slots, columns, synth.small_column(L=9), "mixed")
+    S = 40 if precision == "mixed" else 160          # the FP64 elimination: the reduction has no nodes
+    p = synth.small_column(S=S, L=9, n_two=3 * S, n_three=S, elements="chons" if S < 110 else "full")
+    b = _batch(fake, column, slots, columns, p, precision)
     before = fake.fake_conditional_nodes()
     if how == "round":
         b.step(1)
