@@ -495,9 +495,9 @@ bool bcr64_wanted(const xk_ctx *c)
 // Whether a column's share of the SMs in a batch is too small for the reduction: it does four times the
 // elimination's arithmetic to have the chain of a column alone short, and many columns have no use for
 // that.  Where the line lies (ms a step of 90 layers, reduction and elimination): 64 species in 64 slots
-// 14.4 and 17.1, 80 26.4 and 22.9; 96 in 16 10.7 and 13.5, in 32 21.1 and 23.4 (4 CTAs, half of a chain its panel's), in 64 41.8 and 30.0; 112 in 8
-// 9.7 and 9.6, in 12 13.9 and 11.1; 136 in 4 9.2 and 15.9, in 6 13.4 and 11.1; 152 in 4 14.6 and 17.7, in 5
-// 17.9 and 12.2, in 64 218 and 69.
+// 14.4 and 17.1, 80 26.4 and 22.9; 96 in 16 10.7 and 13.5, in 32 21.1 and 23.4 (4 CTAs, half of a chain
+// its panel's), in 64 41.8 and 30.0; 112 in 8 9.7 and 9.6, in 12 13.9 and 11.1; 136 in 4 9.2 and 15.9, in 6
+// 13.4 and 11.1; 152 in 4 14.6 and 17.7, in 5 17.9 and 12.2, in 64 218 and 69.
 bool bcr64_outgrown(int S, int share) { return S > 96 ? (double)S * S * S > 1e5 * share : S > 72 && share < 4; }
 
 // Lay out the workspace; with base == nullptr only the size is computed.
