@@ -20,6 +20,8 @@ def fake(tmp_path_factory):
     xkbuild.build()
     out = str(tmp_path_factory.mktemp("fake") / "libxk_fake.so")
     objs = [os.path.join(xkbuild.BUILD, s.replace(".cu", ".o")) for s in xkbuild.SOURCES]
+    if not all(os.path.exists(o) for o in objs):
+        xkbuild.build(force=True)
     symbols = subprocess.run(["nm", "-u", *objs], capture_output=True, text=True, check=True).stdout
     linked = {w for w in symbols.split() if w.startswith("__cudaRegisterLinkedBinary")}
     include = os.path.join(os.path.dirname(os.path.dirname(xkbuild.nvcc())), "include")
